@@ -55,7 +55,9 @@ extern "C" {
 /* Storage / arithmetic formats (Sec. 3.2, Table "precision comparison";
  * Sec. 3.4: FP16 products accumulate in FP32, TF32 is never used). */
 typedef enum {
-    LRC_F64 = 0,      /* binary64 storage, binary64 arithmetic, binary64 output             */
+    LRC_F64 = 0,      /* binary64 storage and output; binary64 FMAs, or on larger problems
+                         exact products of 9-bit digits on the tensor cores rounded to
+                         binary64 once (no less accurate; see lrc_apply)                    */
     LRC_F32 = 1,      /* binary32 storage, binary32 FMA arithmetic, binary32 output         */
     LRC_F16 = 2,      /* binary16 storage, binary32 accumulation, binary32 output           */
     LRC_F16_O16 = 3,  /* binary16 storage, binary32 accumulation, binary16 workspaces and
@@ -142,8 +144,18 @@ LRC_API lrc_status lrc_widen_factors(const void* src, lrc_fmt fmt, int64_t rows,
  * columns of U, Vt and X are never read.  All five pointers must be 16-byte
  * aligned.  k may exceed min(m, n).  Asynchronous on `stream`.
  *
- * Intermediate: for LRC_F64 and LRC_F32 the b x k product (X V) diag(s)
- * stays in shared memory.  For LRC_F16 and LRC_F16_O16 the reduction over n
+ * LRC_F64: larger problems form both products from digits of the operands'
+ * rows.  A result is within about 2^-61 of (largest entry of the row of one
+ * operand) (largest entry of the row of the other) per term of the sum, plus
+ * one rounding; rows whose entries lie further apart than the digits reach
+ * (on average more than 2^-12 below the largest), or that hold an infinity, a
+ * NaN or a largest entry outside 2^-480 ... 2^495, are formed by binary64
+ * FMAs.  The digits (14 bytes an element, of at most 1 GiB of queries at a
+ * time) live in the stream's workspace; without memory for them, or while the
+ * stream is being captured with a smaller workspace, the FMA kernels run.
+ *
+ * Intermediate: for LRC_F64 (FMA kernels of more than 2048 queries) the b x k
+ * product (X V) diag(s) stays in shared memory.  For LRC_F16 and LRC_F16_O16 the reduction over n
  * is split over all multiprocessors, so its partial sums and the scaled
  * intermediate (binary16, a hi/lo pair for LRC_F16) pass through a device
  * workspace owned by the library: one buffer per (device, stream),

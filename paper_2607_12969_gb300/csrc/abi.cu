@@ -161,7 +161,8 @@ lrc_status check_apply(const void* U, const void* S, const void* Vt, const void*
 }
 
 lrc_status dispatch_apply(const ApplyProblem& p, lrc_fmt fmt, cudaStream_t s) {
-    if (apply_skinny_takes(plain_fmt(fmt), p.m, p.n, p.k, p.b))
+    if (!(fmt == LRC_F64 && apply_f64_tc_takes(p.m, p.n, p.k, p.b)) &&
+        apply_skinny_takes(plain_fmt(fmt), p.m, p.n, p.k, p.b))
         return launch_apply_skinny(p.U, p.S, p.Vt, p.X, p.Y, p.m, p.n, p.k, p.b, plain_fmt(fmt), s);
     switch (fmt) {
         case LRC_F64:
@@ -425,7 +426,7 @@ lrc_status lrc_device_status(lrc_stream_t stream) {
     const uint32_t t1 = take_tt_tc_error();
     const uint32_t t3 = take_tt3_tc_error();
     const uint32_t tn = take_ttn_tc_error();
-    const uint32_t sk = take_skinny_error();
+    const uint32_t sk = take_skinny_error() | take_split_error();
     const uint32_t t = t1 | t3 | tn;
     if (a == 0xffffffffu || t1 == 0xffffffffu || t3 == 0xffffffffu || tn == 0xffffffffu || sk == 0xffffffffu) {
         set_error("could not read the device error words");

@@ -18,9 +18,11 @@
 // reads of a warp are conflict-free; staging buffers are padded by one
 // element per row so that the transposing stores are conflict-free too.
 //
-// binary64 (DFMA-bound: the GB300 issues about 2 DFMA per clock per SM) uses
-// this kernel with thin 8-row tiles and many CTAs per SM, so the work spreads
-// evenly over the SMs.  binary32 (FFMA-bound) runs the two products on the
+// binary64 forms both products on the tensor cores from exact products of
+// digits (split_gemm.cu; 16384 x 8192, k = 128, b = 8192: 45.5 -> 1.62 ms);
+// this kernel (DFMA-bound: the GB300 issues about 2 DFMA per clock per SM),
+// with thin 8-row tiles and many CTAs per SM, so the work spreads evenly over
+// the SMs, takes what that path does not: no workspace to be had, n above 2^20.  binary32 (FFMA-bound) runs the two products on the
 // register-tiled kernel of gemm_cc.cu instead: phase 1 split over n (partial
 // sums of at most 1024 terms, added in split order by
 // reduce_scale_f32_kernel, which also applies diag(s)), phase 2 over
@@ -38,6 +40,7 @@
 #include <cuda_fp16.h>
 
 #include "common.cuh"
+#include "split_gemm.cuh"
 #include "tc.cuh"
 
 namespace lrc {
@@ -484,8 +487,98 @@ lrc_status launch_split_product(const float* A, int64_t a_rs, int64_t a_cs, cons
 // fill the GPU; they take the split path of apply_split.cu (ranks up to 1024).
 constexpr int64_t kSplitMaxBatchF64 = 2048, kSplitMaxBatchF32 = 32, kSplitMaxRank = 1024;
 
+// ---------------------------------------------------------------- binary64 on the tensor cores
+namespace {
+
+// First operand of a product: the one whose tiles waste less (tiles of 128
+// rows of the first, of at most kNTMax of the second).
+bool swap_sides(int64_t M, int64_t N) {
+    const int64_t a = sg::image_tiles(M, 128) * sg::image_tiles(N, sg::n_tile(N));
+    const int64_t b = sg::image_tiles(N, 128) * sg::image_tiles(M, sg::n_tile(M));
+    return b < a;
+}
+
+constexpr int64_t kPanelBytes = (int64_t)1 << 30;     // digit images of a panel of queries
+
+}  // namespace
+
+// Where the digits' fixed cost (eight launches, about 45 us) pays.  Measured
+// on square matrices, digits / FMA kernels: against the kernels for at most 16
+// queries 16384^2, k = 256: b = 8 180 / 164 us, b = 16 178 / 284 us, and k =
+// 128, b = 16 166 / 166 us; against the others 512^2, k = 32, b = 64 57 / 55 us
+// and b = 256 58 / 59 us, 2048^2, k = 128, b = 64 62 / 160 us.
+bool apply_f64_tc_takes(int64_t m, int64_t n, int64_t k, int64_t b) {
+    if (n > sg::kMaxK || k > 4096 || m >= (1ll << 31) || b >= (1ll << 31)) return false;
+    const double work = (double)(m + n) * (double)k * (double)b;
+    return work >= (apply_skinny_takes(LRC_F64, m, n, k, b) ? 8e7 : 4e6);
+}
+
+// *handled = false: no workspace for the digits (nothing launched).
+static lrc_status launch_apply_f64_tc(const double* U, const double* S, const double* Vt, const double* X, double* Y,
+                                      int64_t m, int64_t n, int64_t k, int64_t b, cudaStream_t s, bool* handled) {
+    *handled = false;
+    const int64_t ldn = lrc_packed_ld(n), ldk = lrc_packed_ld(k);
+    // queries in panels of whole tiles, whose images stay below kPanelBytes
+    int64_t pb = kPanelBytes / (sg::kParts64 * 2 * sg::kKB * sg::image_blocks(n)) / 128 * 128;
+    if (pb < 128) pb = 128;
+    if (pb > b) pb = b;
+    const bool sw1 = swap_sides(pb, k), sw2 = swap_sides(pb, m);
+    const int R_x = sw1 ? sg::n_tile(pb) : 128, R_v = sw1 ? 128 : sg::n_tile(k);
+    const int R_w = sw2 ? sg::n_tile(pb) : 128, R_u = sw2 ? 128 : sg::n_tile(m);
+    sg::Operand64 oV{{Vt, ldn, 1, nullptr, 0}, k, n, R_v};
+    sg::Operand64 oU{{U, ldk, 1, S, 1}, m, k, R_u};
+    sg::Operand64 oX{{X, ldn, 1, nullptr, 0}, pb, n, R_x};
+    sg::Operand64 oW{{nullptr, ldk, 1, S, -1}, pb, k, R_w};
+    size_t off = 0;
+    auto take = [&](size_t bytes) {
+        const size_t o = off;
+        off += (bytes + 255) & ~(size_t)255;
+        return o;
+    };
+    const size_t o_v = take(sg::operand_bytes(k, n, R_v)), o_u = take(sg::operand_bytes(m, k, R_u));
+    const size_t o_x = take(sg::operand_bytes(pb, n, R_x)), o_w = take(sg::operand_bytes(pb, k, R_w));
+    const size_t o_wd = take((size_t)pb * ldk * 8);
+    const size_t o_p = take(sw1 ? sg::part_bytes(k, pb, n, R_x) : sg::part_bytes(pb, k, n, R_v));
+    void* ws = nullptr;
+    lrc_status st = stream_workspace_try(s, off, &ws);
+    if (st != LRC_OK || !ws) return st;
+    *handled = true;
+    unsigned char* base = static_cast<unsigned char*>(ws);
+    double* W = reinterpret_cast<double*>(base + o_wd);
+    double* part = reinterpret_cast<double*>(base + o_p);
+    sg::operand_carve(&oV, base + o_v);
+    sg::operand_carve(&oU, base + o_u);
+    oW.src.p = W;
+    for (int64_t r0 = 0; r0 < b; r0 += pb) {
+        const int64_t rows = b - r0 < pb ? b - r0 : pb;
+        oX.src.p = X + r0 * ldn;
+        oX.rows = oW.rows = rows;
+        sg::operand_carve(&oX, base + o_x);
+        sg::operand_carve(&oW, base + o_w);
+        oW.cleared = true;
+        const sg::Operand64* px[3] = {&oX, &oV, &oU};      // V and U with the first panel
+        const sg::Operand64* pw[1] = {&oW};
+        if ((st = sg::slice(px, r0 == 0 ? 3 : 1, s)) != LRC_OK) return st;
+        const sg::Out64 ow = sw1 ? sg::Out64{W, 1, ldk, S, nullptr, oW.hard} : sg::Out64{W, ldk, 1, nullptr, S, oW.hard};
+        if ((st = sw1 ? sg::product(oV, oX, ow, true, part, s) : sg::product(oX, oV, ow, true, part, s)) != LRC_OK)
+            return st;
+        if ((st = sg::slice(pw, 1, s)) != LRC_OK) return st;
+        double* Yr = Y + r0 * m;
+        const sg::Out64 oy = sw2 ? sg::Out64{Yr, 1, m, nullptr, nullptr} : sg::Out64{Yr, m, 1, nullptr, nullptr};
+        if ((st = sw2 ? sg::product(oU, oW, oy, false, nullptr, s) : sg::product(oW, oU, oy, false, nullptr, s)) != LRC_OK)
+            return st;
+    }
+    return LRC_OK;
+}
+
 lrc_status launch_apply_f64(const double* U, const double* S, const double* Vt, const double* X,
                             double* Y, int64_t m, int64_t n, int64_t k, int64_t b, cudaStream_t s) {
+    if (apply_f64_tc_takes(m, n, k, b)) {
+        bool handled = false;
+        const lrc_status st = launch_apply_f64_tc(U, S, Vt, X, Y, m, n, k, b, s, &handled);
+        if (st != LRC_OK || handled) return st;
+        if (apply_skinny_takes(LRC_F64, m, n, k, b)) return launch_apply_skinny(U, S, Vt, X, Y, m, n, k, b, LRC_F64, s);
+    }
     if (b <= kSplitMaxBatchF64 && k <= kSplitMaxRank) return launch_apply_split_f64(U, S, Vt, X, Y, m, n, k, b, s);
     return launch_apply_cc<double>(U, S, Vt, X, Y, m, n, k, b, s, "apply_cc_kernel<f64>");
 }

@@ -78,6 +78,8 @@ lrc_status launch_widen(const void* src, lrc_fmt fmt, int64_t rows, int64_t cols
                         double* dst, int64_t ld_dst, cudaStream_t s);
 lrc_status launch_apply_f64(const double* U, const double* S, const double* Vt, const double* X,
                             double* Y, int64_t m, int64_t n, int64_t k, int64_t b, cudaStream_t s);
+// binary64 applies whose products run on the tensor cores (split_gemm.cu)
+bool apply_f64_tc_takes(int64_t m, int64_t n, int64_t k, int64_t b);
 // LRC_F32_TC output product C (P x Q, row pitch Q) = A B^T on the tensor
 // cores through the scaled binary16 split (apply_cc.cu): A(i, j) =
 // A[i a_rs + j a_cs] is P x k (a scale per row), B(i, j) = B[i b_rs + j b_cs]
@@ -205,6 +207,7 @@ lrc_status launch_tt3_f16_tc(const TTShape& sh, bool out16, void* out, cudaStrea
 lrc_status launch_ttn_f16_tc(const TTShape& sh, bool out16, void* out, cudaStream_t s, bool* handled);
 uint32_t take_ttn_tc_error();
 uint32_t take_skinny_error();
+uint32_t take_split_error();
 lrc_status launch_wait_timeout_probe(int64_t limit_ns, cudaStream_t s);
 
 lrc_status run_fro_diff(const void* A, lrc_fmt fa, const void* B, lrc_fmt fb, int64_t count,
@@ -212,6 +215,10 @@ lrc_status run_fro_diff(const void* A, lrc_fmt fa, const void* B, lrc_fmt fb, in
 void release_scratch();
 // Per-(device, stream) workspace, grown on demand; freed by release_workspaces().
 lrc_status stream_workspace(cudaStream_t s, size_t bytes, void** out);
+// The same where another path can do without: *out = nullptr when the buffer
+// cannot be made (no memory, or the stream is being captured and the present
+// one is too small).
+lrc_status stream_workspace_try(cudaStream_t s, size_t bytes, void** out);
 // Per-(device, stream) arrival counters, zero between kernels: kStreamCounters
 // of them, made (and zeroed in stream order) on first use.
 constexpr int kStreamCounters = 1024;

@@ -1,0 +1,981 @@
+// split_gemm.cu -- binary64 products C = A B^T on the tensor cores.
+//
+// This GPU multiplies bfloat16 numbers on its tensor cores about 1300 times
+// as fast as it multiplies binary64 numbers (1.26 TFLOP/s), so a binary64
+// product is formed from exact products of short pieces (the error-free
+// splitting of Ozaki, Ogita, Oishi and Rump, "Error-free transformations of
+// matrix multiplication by using fast routines of matrix multiplication and
+// its applications", Numer. Algorithms 59, 2012):
+//
+//   * every row of A and of B is scaled by a power of two to at most 1/2 and
+//     cut into seven signed 9-bit digits d_0 ... d_6 (|d_0| <= 128, |d_i| <=
+//     256), x = 2^(e - 7) sum_i d_i 2^(-9 i): 62 bits below the row's largest
+//     entry, so entries down to 2^-9 of it are carried without error.  A
+//     digit is a bfloat16 number.
+//   * C = sum over classes t = i + j of 2^(-9 t) D_i E_j^T, each class in an
+//     accumulator of its own.  Within 64 terms of the reduction the sums of
+//     classes 0 to 4 are integers of at most 2^20, 2^22, 2^23, 2^23.6 and
+//     2^24, so the tensor cores' binary32 accumulation forms them without
+//     error; those of classes 5 and 6 are as a rule, and where not the error
+//     is 2^-24 of a class that lies 2^-45 below the first.  Classes from 7 on
+//     are below 2^-62 and are left out (28 products of 49).
+//   * every 64 terms (`period`: less often where the bound allows) the
+//     accumulators are drained into two 64-bit integers per entry, and the
+//     whole sum is rounded to binary64 once.
+//
+// So the result is as close as the best rounded one for rows whose entries
+// lie within about 2^-9 of each other's scale, and the error never exceeds
+// about 2^-61 of (largest of row i)(largest of row j) per term.  Rows that
+// this does not describe well -- their entries lie on average more than
+// 2^-kMaxGap below the largest, or they hold an infinity, a NaN or a largest
+// entry outside 2^-480 ... 2^495 -- get zero digits and are
+// recomputed by a kernel of binary64 FMAs (`repair`).
+//
+// Kernels: row statistics (row_stats_kernel), digits (slice_kernel, which
+// writes them as the product's operand images), the product (product_kernel,
+// persistent, one CTA a SM), the ordered sum of split reductions
+// (part_sum_kernel) and the repair (repair_kernel).
+#include <algorithm>
+
+#include "split_gemm.cuh"
+#include "tc.cuh"
+
+namespace lrc {
+namespace sg {
+
+namespace {
+
+using namespace tc;
+
+__device__ unsigned int g_err_split;
+
+constexpr int64_t kOwnStatsK = 512;    // reductions up to this long: slice_kernel takes the row statistics itself
+constexpr int kMaxGap = 12;            // mean distance (in bits) of a row's entries below its largest
+constexpr int kNonFinite = 1 << 20;    // marks a row with an infinity or NaN in its statistics
+// Biased exponents of a row's largest entry that digits carry: with both rows
+// inside, every result is zero or a normal number (round96).
+constexpr int kMinExp = 544, kMaxExp = 1518;
+
+// ---------------------------------------------------------------- sources
+struct View64 {
+    Src64 s;
+    __device__ double at(int64_t r, int64_t k) const { return __ldg(s.p + r * s.rs + k * s.cs); }
+    __device__ int shift(int64_t k) const {
+        if (!s.scale) return 0;
+        const int e = (int)((uint64_t)__double_as_longlong(__ldg(s.scale + k)) >> 52) & 0x7ff;
+        return e == 0 || e == 0x7ff ? 0 : s.sign * ((e - 1023) / 2);
+    }
+};
+
+// Biased exponent of |x| (bits), a subnormal's as if the range went on; x != 0.
+__device__ __forceinline__ int biased_exp(uint64_t bits) {
+    const int e = (int)(bits >> 52) & 0x7ff;
+    if (e != 0) return e == 0x7ff ? kNonFinite : e;
+    return 12 - __clzll((long long)(bits & 0xfffffffffffffull));
+}
+
+// ---------------------------------------------------------------- statistics
+// Per row: the largest biased exponent, the sum of the exponents of the
+// nonzero entries and their number.
+struct RowStat {
+    int mx = -(1 << 20), sum = 0, cnt = 0;
+    __device__ __forceinline__ void add(double x, int shift) {
+        const uint64_t bits = (uint64_t)__double_as_longlong(x) & 0x7fffffffffffffffull;
+        if (bits != 0) {
+            const int e = biased_exp(bits) + shift;
+            mx = max(mx, e);
+            sum += e >= kNonFinite / 2 ? 0 : e;
+            cnt += 1;
+        }
+    }
+    __device__ __forceinline__ void merge(int4 o) {
+        mx = max(mx, o.x);
+        sum += o.y;
+        cnt += o.z;
+    }
+};
+
+// What the kernels below take of an operand, and its share of the blocks.
+struct Job {
+    View64 v;
+    int64_t rows, K, img_rows, kblocks;
+    int64_t b0;              // first block
+    int64_t kchunk;          // columns a block takes
+    int R, kparts, splits, vec;
+    int4* stats;             // splits > 0: statistics per slice of K; else slice_kernel takes its own
+    unsigned char* img;
+    int* exps;
+    int* hard;
+};
+struct Jobs {
+    Job j[kMaxOps];
+    int n;
+    int* clear[kMaxOps];     // row lists to empty
+};
+__device__ __forceinline__ const Job& job_of(const Jobs& js, int64_t block) {
+    int i = 0;
+    while (i + 1 < js.n && block >= js.j[i + 1].b0) ++i;
+    return js.j[i];
+}
+
+// Statistics of 32 rows over columns [k0, k1), by 256 threads; row r0 + lane's
+// in warp 0.  K contiguous: a warp per row, lanes along K; else a lane per
+// row, so that either way a warp reads consecutive addresses.
+__device__ __forceinline__ RowStat block_stats(const View64& v, int64_t r0, int64_t rows, int64_t k0, int64_t k1,
+                                               int4 (&sm)[8][32]) {
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    if (v.s.cs == 1) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int64_t r = r0 + warp + 8 * q;
+            RowStat a;
+            if (r < rows) {
+                int64_t k = k0 + lane;
+                for (; k + 96 < k1; k += 128) {
+                    double x[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) x[u] = v.at(r, k + 32 * u);
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) a.add(x[u], v.shift(k + 32 * u));
+                }
+                for (; k < k1; k += 32) a.add(v.at(r, k), v.shift(k));
+            }
+            a.mx = __reduce_max_sync(0xffffffffu, a.mx);
+            a.sum = __reduce_add_sync(0xffffffffu, a.sum);
+            a.cnt = __reduce_add_sync(0xffffffffu, a.cnt);
+            if (lane == 0) sm[0][warp + 8 * q] = make_int4(a.mx, a.sum, a.cnt, 0);
+        }
+    } else {
+        const int64_t r = r0 + lane;
+        RowStat a;
+        if (r < rows) {
+            int64_t k = k0 + warp;
+            for (; k + 24 < k1; k += 32) {
+                double x[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) x[u] = v.at(r, k + 8 * u);
+#pragma unroll
+                for (int u = 0; u < 4; ++u) a.add(x[u], v.shift(k + 8 * u));
+            }
+            for (; k < k1; k += 8) a.add(v.at(r, k), v.shift(k));
+        }
+        sm[warp][lane] = make_int4(a.mx, a.sum, a.cnt, 0);
+    }
+    __syncthreads();
+    RowStat t;
+    if (warp == 0) {
+        t.merge(sm[0][lane]);
+        if (v.s.cs != 1) {
+#pragma unroll
+            for (int w = 1; w < 8; ++w) t.merge(sm[w][lane]);
+        }
+    }
+    return t;
+}
+
+__global__ void __launch_bounds__(256) row_stats_kernel(const __grid_constant__ Jobs js) {
+    __shared__ int4 sm[8][32];
+    pdl_wait();
+    pdl_trigger();
+    const Job& o = job_of(js, blockIdx.x);
+    const int64_t lb = (int64_t)blockIdx.x - o.b0, rg = lb / o.splits, z = lb - rg * o.splits;
+    const int64_t r0 = rg * 32, k0 = z * o.kchunk;
+    if (blockIdx.x == 0 && threadIdx.x < kMaxOps && js.clear[threadIdx.x]) *js.clear[threadIdx.x] = 0;
+    const RowStat a = block_stats(o.v, r0, o.rows, k0, min(o.K, k0 + o.kchunk), sm);
+    if (threadIdx.x < 32 && r0 + threadIdx.x < o.rows)
+        o.stats[z * o.rows + r0 + threadIdx.x] = make_int4(a.mx, a.sum, a.cnt, 0);
+}
+
+// ---------------------------------------------------------------- digits
+// The seven digits of eight values as bfloat16: w[p][q] holds digits
+// p of values 2q (low half) and 2q + 1.  em: biased exponent of the row's
+// largest entry.  The value is rounded to a multiple of 2^-61 of 2^(em -
+// 1022), the power of two above it, and the digits are those of that integer
+// plus 256 at every place but the first, minus 256 again: a number read with
+// digits in [-256, 255].
+__device__ __forceinline__ void digits8(const double (&x)[8], const int (&sh)[8], int em, uint32_t (&w)[kParts64][4]) {
+    constexpr uint64_t kBias = 256ull * (1ull + (1ull << 9) + (1ull << 18) + (1ull << 27) + (1ull << 36) + (1ull << 45));
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        float f[2][kParts64];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int64_t b = __double_as_longlong(x[2 * q + h]);
+            const int e = (int)((uint64_t)b >> 52) & 0x7ff;
+            const int64_t mant = (b & 0xfffffffffffffll) | (e ? (1ll << 52) : 0);
+            const int s = (e ? e : 1) + sh[2 * q + h] - em + 8;      // <= 8
+            int64_t v;
+            if (s >= 0) v = mant << s;
+            else v = s > -55 ? (mant + (1ll << (-s - 1))) >> -s : 0;
+            if (b < 0) v = -v;
+            const uint64_t t = (uint64_t)v + kBias;
+            const int d0 = (int)((int64_t)t >> 54);
+            f[h][0] = __int_as_float(0x4b400000 + d0) - 12582912.0f;
+#pragma unroll
+            for (int i = 1; i < kParts64; ++i) {
+                const uint32_t d = (uint32_t)(t >> (9 * (6 - i))) & 511u;
+                f[h][i] = __int_as_float(0x4b400000u | d) - (12582912.0f + 256.0f);
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < kParts64; ++i)
+            w[i][q] = __byte_perm(__float_as_uint(f[0][i]), __float_as_uint(f[1][i]), 0x7632);
+    }
+}
+
+// Digit images: [row tile][block of 16 columns][digit][R rows x 16 columns in
+// the canonical K-major layout: 8-row x 16-byte core matrices, row groups 128
+// bytes apart, column octets 16 R bytes apart].  A CTA takes 32 image rows
+// and `kchunk` columns (of an operand with a short reduction all of them, and
+// takes the row statistics itself); a lane is a row, so that a warp's 16-byte
+// stores of one digit are four runs of 128 bytes.
+__global__ void __launch_bounds__(256) slice_kernel(const __grid_constant__ Jobs js) {
+    __shared__ int4 sm[8][32];
+    __shared__ int s_em[32];
+    pdl_wait();
+    pdl_trigger();
+    const Job& o = job_of(js, blockIdx.x);
+    const View64 v = o.v;
+    const int64_t rows = o.rows, K = o.K;
+    const int R = o.R;
+    const int64_t lb = (int64_t)blockIdx.x - o.b0, rg = lb / o.kparts, kp = lb - rg * o.kparts;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int64_t r0 = rg * 32;
+    RowStat own;
+    if (o.splits == 0) own = block_stats(v, r0, rows, 0, K, sm);
+    if (tid < 32) {
+        const int64_t r = r0 + lane;
+        int em = 1023;
+        bool zero = true;
+        if (r < rows) {
+            int mx = own.mx;
+            int64_t sum = own.sum, cnt = own.cnt;
+            for (int z = 0; z < o.splits; ++z) {
+                const int4 a = o.stats[(int64_t)z * rows + r];
+                mx = max(mx, a.x);
+                sum += a.y;
+                cnt += a.z;
+            }
+            if (cnt > 0) {
+                zero = mx < kMinExp || mx > kMaxExp || (int64_t)mx * cnt - sum > (int64_t)kMaxGap * cnt;
+                if (!zero) em = mx;
+                else if (kp == 0) o.hard[1 + atomicAdd(o.hard, 1)] = (int)r;
+            }
+        }
+        s_em[lane] = zero ? -1 : em;
+        if (kp == 0 && r < o.img_rows) o.exps[r] = em;
+    }
+    __syncthreads();
+    const int64_t r = r0 + lane;
+    if (r >= o.img_rows) return;
+    const int em = s_em[lane];
+    const int64_t tile = r / R;
+    const int rr = (int)(r - tile * R);
+    const size_t block_bytes = (size_t)kParts64 * R * (kKB * 2);
+    unsigned char* row_base = o.img + (size_t)tile * o.kblocks * block_bytes + (rr >> 3) * 128 + (rr & 7) * 16;
+    const int64_t o1 = min((kp + 1) * o.kchunk, o.kblocks * kKB) / 8;
+    for (int64_t oc = kp * o.kchunk / 8 + warp; oc < o1; oc += 8) {
+        double x[8];
+        int sh[8];
+        const int64_t k0 = oc * 8;
+        if (em < 0) {
+#pragma unroll
+            for (int j = 0; j < 8; ++j) x[j] = 0.0;
+        } else if (o.vec && k0 + 8 <= K) {
+            const double2* p = reinterpret_cast<const double2*>(v.s.p + r * v.s.rs + k0);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const double2 d = __ldg(p + j);
+                x[2 * j] = d.x;
+                x[2 * j + 1] = d.y;
+            }
+        } else {
+#pragma unroll
+            for (int j = 0; j < 8; ++j) x[j] = k0 + j < K ? v.at(r, k0 + j) : 0.0;
+        }
+#pragma unroll
+        for (int j = 0; j < 8; ++j) sh[j] = (v.s.scale && k0 + j < K) ? v.shift(k0 + j) : 0;
+        uint32_t w[kParts64][4];
+        digits8(x, sh, em < 0 ? 1023 : em, w);
+        unsigned char* dst = row_base + (size_t)(oc >> 1) * block_bytes + (size_t)(oc & 1) * (R * 16);
+#pragma unroll
+        for (int i = 0; i < kParts64; ++i)
+            *reinterpret_cast<uint4*>(dst + (size_t)i * R * (kKB * 2)) = make_uint4(w[i][0], w[i][1], w[i][2], w[i][3]);
+    }
+}
+
+// ---------------------------------------------------------------- product
+struct GemmArgs {
+    const unsigned char* A;
+    const unsigned char* B;
+    const int* ea;
+    const int* eb;
+    double* C;               // split: partial tiles [slot][column][128 rows]
+    int64_t cr, cc, M, N;
+    int ntiles, tiles;       // tiles of B; all tiles
+    int chunks;              // 64-column chunks of the reduction
+    int kblocks;             // 16-column blocks
+    int split, group, stages, vec;
+    uint32_t a_bytes, b_bytes;
+    uint32_t tmem_cols;
+};
+
+// The (tile, chunk range) pieces of a CTA, in order.  A split reduction is cut
+// over groups of `group` CTAs, one per tile of B: a group walks one range of
+// (tile of A, chunk), laid end to end, so that its CTAs read the same blocks of
+// A at about the same time and only the first read comes from HBM.
+struct Pieces {
+    int left, t, c, step;      // split: chunks left, first chunk of the next piece
+    __device__ explicit Pieces(const GemmArgs& a) {
+        if (a.split) {
+            const int groups = gridDim.x / a.group, gi = blockIdx.x / a.group;
+            const int64_t Q = (int64_t)(a.tiles / a.group) * a.chunks;
+            const int64_t q0 = Q * gi / groups, q1 = Q * (gi + 1) / groups;
+            const int mt = (int)(q0 / a.chunks);
+            t = mt * a.group + (int)(blockIdx.x - gi * a.group);
+            c = (int)(q0 - (int64_t)mt * a.chunks);
+            left = (int)(q1 - q0);
+            step = a.group;
+        } else {
+            t = blockIdx.x;
+            c = 0;
+            step = gridDim.x;
+            left = t < a.tiles ? 1 : 0;
+        }
+    }
+    // false: no piece left
+    __device__ bool next(const GemmArgs& a, int* tile, int* c0, int* c1) {
+        if (left <= 0) return false;
+        *tile = t;
+        *c0 = c;
+        *c1 = a.chunks;
+        t += step;
+        if (a.split) {
+            *c1 = min(a.chunks, c + left);
+            left -= *c1 - c;
+            c = 0;
+        } else {
+            left = t < a.tiles ? 1 : 0;
+        }
+        return true;
+    }
+};
+// Partial tile of a piece: distinct for every (group, tile).
+__device__ __forceinline__ int64_t part_slot(const GemmArgs& a, int tile) {
+    return (int64_t)(blockIdx.x / a.group) * a.group + tile;
+}
+
+// Sixteen epilogue warps, four per quarter of the tensor-memory lanes, each
+// with a quarter of the columns: with eight, two a scheduler, the drain's and
+// the rounding's dependent steps were not covered (a 128 x 64 tile of two
+// chunks took 26000 clocks, its MMAs 10750).
+constexpr int kEpiWarps = 16;
+constexpr int kThreads = 32 * (4 + kEpiWarps);
+// Registers: the first four warps (producer, MMA issuer, two idle) hand some
+// of theirs to the epilogue's, which keep two 64-bit sums per entry: 128 x 64
+// + 512 x 104 = 61440, the 640 x 96 = 61440 of the launch.
+constexpr int kRegsLow = 64, kRegsEpi = 104;
+constexpr int kChunkBlocks = 64 / kKB;
+constexpr uint32_t kCtrlBytes = 1024;
+
+// Chunks between drains of a class's accumulator: its sums stay at most 2^24
+// (classes 5 and 6: see above).  A converting drain costs an entry 8 clocks of
+// a scheduler's F2I rate per class and chunk.
+__host__ __device__ constexpr int period(int t) { return t == 0 ? 16 : t == 2 ? 2 : t == 3 || t == 4 ? 1 : 4; }
+
+__device__ __forceinline__ void tmem_ld_cols(uint32_t taddr, uint32_t (&r)[8]) { tmem_ld8(taddr, r); }
+__device__ __forceinline__ void tmem_ld_cols(uint32_t taddr, uint32_t (&r)[4]) { tmem_ld4(taddr, r); }
+
+// Adds HC columns of an accumulator, times `weight`, to the sums.
+template <int HC>
+__device__ __forceinline__ void drain(uint32_t taddr, int weight, int64_t (&sum)[HC]) {
+    constexpr int G = HC % 8 == 0 ? 8 : 4;
+    uint32_t v[HC / G][G];
+#pragma unroll
+    for (int q = 0; q < HC / G; ++q) tmem_ld_cols(taddr + q * G, v[q]);
+    tmem_ld_wait();
+#pragma unroll
+    for (int j = 0; j < HC; ++j) sum[j] += (int64_t)__float2int_rn(__uint_as_float(v[j / G][j % G])) * weight;
+}
+
+// Classes 5 and 6 together, in units of 2^-4 of class 5's.
+template <int HC>
+__device__ __forceinline__ void drain56(uint32_t t5, uint32_t t6, int64_t (&sum)[HC]) {
+    constexpr int G = 4;
+#pragma unroll
+    for (int q = 0; q < HC; q += G) {
+        uint32_t u[G], v[G];
+        tmem_ld_cols(t5 + q, u);
+        tmem_ld_cols(t6 + q, v);
+        tmem_ld_wait();
+#pragma unroll
+        for (int j = 0; j < G; ++j)
+            sum[q + j] += __float2int_rn(fmaf(__uint_as_float(v[j]), 0.03125f, __uint_as_float(u[j]) * 16.0f));
+    }
+}
+
+// P 2^-27 + Q 2^-49 times 2^(esum - 2058), rounded to nearest; esum is the sum
+// of the biased exponents of the two rows' largest entries (a row's value is
+// its digit sum times 2^(e - 1029)).  |P| < 2^63, |Q| < 2^62; the sum's
+// integer, in units of 2^-59, is below 2^95 (reductions of up to 2^20 terms),
+// so kMinExp and kMaxExp keep the result's exponent within 1 ... 2046.
+// Straight-line code, so that a thread's entries interleave: it runs on the
+// integer pipe, at half an instruction a clock, and with K = 128 takes about
+// as long per tile as the MMAs.
+__device__ __forceinline__ double round_pq(int64_t p, int64_t q, int esum) {
+    p += q >> 22;
+    uint32_t a = (uint32_t)((uint64_t)p >> 32), b = (uint32_t)p, c = (uint32_t)q << 10;
+    const uint32_t neg = (uint32_t)((int32_t)a >> 31);
+    a ^= neg;
+    b ^= neg;
+    c ^= neg;
+    asm("sub.cc.u32 %0, %0, %3;\n\tsubc.cc.u32 %1, %1, %3;\n\tsubc.u32 %2, %2, %3;" : "+r"(c), "+r"(b), "+r"(a) : "r"(neg));
+    int n = esum - 1000;
+#pragma unroll
+    for (int z = 0; z < 2; ++z) {
+        const bool up = a == 0;
+        a = up ? b : a;
+        b = up ? c : b;
+        c = up ? 0 : c;
+        n -= up ? 32 : 0;
+    }
+    const int s = __clz((int)a);
+    const uint32_t e = a ? (uint32_t)(n - s) << 20 : 0u;       // (exponent - 1) << 20; a == 0: the sum is zero
+    const uint32_t hi = __funnelshift_l(b, a, s), mid = __funnelshift_l(c, b, s);
+    uint32_t r0 = __funnelshift_r(mid, hi, 11), r1 = hi >> 11, t = mid << 21;
+    // + the first bit dropped (to nearest, ties away from zero)
+    asm("add.cc.u32 %2, %2, %2;\n\taddc.cc.u32 %0, %0, 0;\n\taddc.u32 %1, %1, %3;" : "+r"(r0), "+r"(r1), "+r"(t) : "r"(e));
+    return __hiloint2double((int)(r1 | (neg & 0x80000000u)), (int)r0);
+}
+
+// The same through two binary64 additions: p' = p + (q >> 22) and the rest of q
+// as binary64 numbers by their encodings, 1.5 2^52 + p' and 2^30 + rest 2^-22,
+// added with the constants' sum taken off first (exact).  For |p'| < 2^51.  The
+// binary64 pipe takes 128 clocks of a scheduler for it, the integer pipe about
+// 80 for round_pq, so the epilogue gives three entries of eight to it.
+__device__ __forceinline__ double round_pq_fp64(int64_t p, int64_t q, int esum) {
+    p += q >> 22;
+    const double a = __hiloint2double((int)((uint64_t)p >> 32) + 0x43380000, (int)p);
+    const double b = __hiloint2double(0x41d00000, (int)((uint32_t)q & 0x3fffffu));
+    const double y = __dadd_rn(__dsub_rn(a, 6755399441055744.0 + 1073741824.0), b);
+    const int hi = __double2hiint(y);
+    return __hiloint2double(hi ? hi + ((esum - 2085) << 20) : 0, __double2loint(y));
+}
+
+// The products of classes [T0, T1) of one block from digit I of A on,
+// straight-line (a branch between two MMAs costs about as much as one).  All
+// that share a digit of A follow one another: A stays in the collector buffer
+// (an MMA of 64 columns is bound by its reads of shared memory, 48 clocks with
+// A's 4 KB read and 35 with them kept), and no MMA adds to the accumulator of
+// the one before it, which would wait for its result (about 120 clocks).
+// fresh: bit t is set where class t starts a new sum.
+template <int NT, int T0, int T1, int I = 0, int J = (T0 > 0 ? T0 : 0)>
+__device__ __forceinline__ void issue(uint32_t tmem, uint32_t fresh, uint32_t alo, uint32_t ahi, uint32_t blo,
+                                      uint32_t bhi) {
+    constexpr int kAPart = 128 * kKB * 2 / 16, kBPart = NT * kKB * 2 / 16;      // one digit
+    constexpr int J0 = T0 > I ? T0 - I : 0, J1 = T1 - I;                        // digits of B for this one of A
+    constexpr int kMmaUse = J1 - J0 == 1 ? kNoReuse : J == J0 ? kFill : J == J1 - 1 ? kLast : kUse;
+    mma_f16_col<kMmaUse>(tmem + (I + J) * NT, alo + I * kAPart, ahi, blo + J * kBPart, bhi,
+                          idesc_f16_f32(128, NT) | kIdescBF16, I > 0 ? 1u : ((fresh >> (I + J)) & 1u) ^ 1u);
+    if constexpr (J + 1 < J1) issue<NT, T0, T1, I, J + 1>(tmem, fresh, alo, ahi, blo, bhi);
+    else if constexpr (I + 1 < T1) issue<NT, T0, T1, I + 1, (T0 > I + 1 ? T0 - I - 1 : 0)>(tmem, fresh, alo, ahi, blo, bhi);
+}
+
+template <int NT>
+__global__ void __launch_bounds__(kThreads, 1) product_kernel(const __grid_constant__ GemmArgs a) {
+    constexpr int HC = NT / 4;          // columns a thread drains
+    extern __shared__ __align__(128) unsigned char smem[];
+    uint64_t* full = reinterpret_cast<uint64_t*>(smem);
+    uint64_t* empty = full + 8;
+    uint64_t* gfull = empty + 8;        // accumulator groups complete
+    uint64_t* gempty = gfull + 2;       // accumulator groups drained
+    uint64_t* mma_done = gempty + 2;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(mma_done + 1);
+    volatile int* abort = reinterpret_cast<volatile int*>(tmem_slot + 1);
+    unsigned char* ring = smem + kCtrlBytes;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t stage_bytes = a.a_bytes + a.b_bytes;
+    unsigned int* err = &g_err_split;
+
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < a.stages; ++i) {
+            mbar_init(&full[i], 1);
+            mbar_init(&empty[i], 1);
+        }
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(&gfull[i], 1);
+            mbar_init(&gempty[i], 32 * kEpiWarps);
+        }
+        mbar_init(mma_done, 1);
+        *abort = 0;
+        fence_barrier_init();
+    }
+    if (warp == 1) tmem_alloc(tmem_slot, a.tmem_cols);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *tmem_slot;
+    pdl_wait();
+    pdl_trigger();
+
+    if (warp >= 4) {
+        reg_inc<kRegsEpi>();
+        // ------------------------------------------------------------ epilogue
+        const int g = warp & 3, quarter = (warp - 4) >> 2;      // of the lanes, of the columns
+        const uint32_t tbase = tmem + ((uint32_t)(g * 32) << 16) + quarter * HC;
+        const int r = g * 32 + lane;
+        Pieces pc(a);
+        int tile, c0, c1;
+        int ch = 0;
+        bool ok = true;
+        // one warp polls the mbarrier, the others sleep at the named barrier
+        // (512 polling threads would take the MMA issuer's issue slots)
+        auto epi_wait = [&](uint64_t* bar, uint32_t parity) {
+            if (warp == 4) mbar_wait(bar, parity, abort, err, 4u);
+            named_bar_sync(1, 32 * kEpiWarps);
+            return *abort == 0;
+        };
+        while (ok && pc.next(a, &tile, &c0, &c1)) {
+            const int mt = tile / a.ntiles, nt = tile - mt * a.ntiles;
+            const int64_t row = (int64_t)mt * 128 + r, col0 = (int64_t)nt * NT + quarter * HC;
+            // exponents: of the thread's row, and of column `lane`
+            const int ea = row < a.M ? a.ea[row] : 0;
+            const int eb = lane < HC && col0 + lane < a.N ? a.eb[col0 + lane] : 0;
+            int64_t P[HC], Q[HC];
+#pragma unroll
+            for (int j = 0; j < HC; ++j) P[j] = Q[j] = 0;
+            for (int c = c0; c < c1; ++c, ++ch) {
+                const int n = c - c0 + 1;
+                auto due = [&](int t) { return c + 1 == c1 || n % period(t) == 0; };
+                if (!(ok = epi_wait(&gfull[0], ch & 1))) break;
+                tc_fence_after();
+                drain<HC>(tbase + 3 * NT, 1, P);
+                if (due(2)) drain<HC>(tbase + 2 * NT, 1 << 9, P);
+                if (due(1)) drain<HC>(tbase + NT, 1 << 18, P);
+                if (due(0)) drain<HC>(tbase, 1 << 27, P);
+                tc_fence_before();
+                mbar_arrive(&gempty[0]);
+                if (!(ok = epi_wait(&gfull[1], ch & 1))) break;
+                tc_fence_after();
+                drain<HC>(tbase + 4 * NT, 1 << 13, Q);
+                if (due(5)) drain56<HC>(tbase + 5 * NT, tbase + 6 * NT, Q);
+                tc_fence_before();
+                mbar_arrive(&gempty[1]);
+            }
+            if (!ok) break;
+            if (a.split) {
+                double* dst = a.C + part_slot(a, tile) * (128 * NT) + (int64_t)(quarter * HC) * 128 + r;
+#pragma unroll
+                for (int j = 0; j < HC; ++j) dst[j * 128] = round_pq(P[j], Q[j], ea + __shfl_sync(0xffffffffu, eb, j));
+                continue;
+            }
+            double* dst = a.C + row * a.cr + col0 * a.cc;
+            const bool shallow = a.chunks <= 8;      // |P| stays below 2^50
+#pragma unroll
+            for (int j0 = 0; j0 < HC; j0 += 4) {
+                double y[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const int es = ea + __shfl_sync(0xffffffffu, eb, j0 + j);
+                    y[j] = shallow && ((0x52 >> ((j0 + j) & 7)) & 1) ? round_pq_fp64(P[j0 + j], Q[j0 + j], es)
+                                                                     : round_pq(P[j0 + j], Q[j0 + j], es);
+                }
+                if (row < a.M) {
+                    // a whole 32-byte sector a lane where the rows allow it
+                    if (a.vec == 2 && col0 + j0 + 4 <= a.N) {
+                        asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};"
+                                     ::"l"(dst + j0), "d"(y[0]), "d"(y[1]), "d"(y[2]), "d"(y[3]) : "memory");
+                    } else if (a.vec == 1 && col0 + j0 + 4 <= a.N) {
+                        reinterpret_cast<double2*>(dst + j0)[0] = make_double2(y[0], y[1]);
+                        reinterpret_cast<double2*>(dst + j0)[1] = make_double2(y[2], y[3]);
+                    } else {
+#pragma unroll
+                        for (int j = 0; j < 4; ++j)
+                            if (col0 + j0 + j < a.N) dst[(j0 + j) * a.cc] = y[j];
+                    }
+                }
+            }
+        }
+    } else {
+        reg_dec<kRegsLow>();
+        if (warp == 0) {
+        // ------------------------------------------------------------ producer
+        if (lane == 0) {
+            Pieces pc(a);
+            int tile, c0, c1;
+            int it = 0, slot = 0;
+            uint32_t phase = 1;
+            bool ok = true;
+            while (ok && pc.next(a, &tile, &c0, &c1)) {
+                const int mt = tile / a.ntiles, nt = tile - mt * a.ntiles;
+                const int b1 = min(kChunkBlocks * c1, a.kblocks);
+                for (int kb = kChunkBlocks * c0; kb < b1; ++kb, ++it) {
+                    if (!(ok = mbar_wait(&empty[slot], phase, abort, err, 1u))) break;
+                    unsigned char* dst = ring + (size_t)slot * stage_bytes;
+                    mbar_arrive_expect_tx(&full[slot], stage_bytes);
+                    bulk_load(dst, a.A + ((size_t)mt * a.kblocks + kb) * a.a_bytes, a.a_bytes, &full[slot]);
+                    bulk_load(dst + a.a_bytes, a.B + ((size_t)nt * a.kblocks + kb) * a.b_bytes, a.b_bytes, &full[slot]);
+                    if (++slot == a.stages) {
+                        slot = 0;
+                        phase ^= 1;
+                    }
+                }
+            }
+            if (!ok) {
+                volatile int no_abort = 0;
+                for (int j = it - a.stages > 0 ? it - a.stages : 0; j < it; ++j)
+                    mbar_wait(&full[j % a.stages], (j / a.stages) & 1, &no_abort, err, 0u, 100000000ull);
+            }
+        }
+    } else if (warp == 1) {
+        // ------------------------------------------------------------ MMA issuer
+        // The whole warp walks the loop and waits; one lane issues, in one branch
+        // per block (with a branch or an election per MMA the warp, which shares
+        // its scheduler with busy epilogue warps, issued one in 49 to 100 clocks).
+        Pieces pc(a);
+        int tile, c0, c1;
+        int slot = 0, ch = 0;
+        uint32_t phase = 0;            // parity of the ring's current pass
+        bool ok = true;
+        // waits agree on every lane before the warp goes on
+        auto wait = [&](uint64_t* bar, uint32_t parity) {
+            return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort, err, 2u)) != 0;
+        };
+        const uint32_t ahi = (uint32_t)(smem_desc(0, 2048, 128, 0) >> 32);
+        const uint32_t bhi = (uint32_t)(smem_desc(0, NT * 16, 128, 0) >> 32);
+        const uint32_t alo0 = (uint32_t)smem_desc(smem_u32(ring), 2048, 128, 0);
+        const uint32_t blo0 = (uint32_t)smem_desc(smem_u32(ring) + a.a_bytes, NT * 16, 128, 0);
+        while (ok && pc.next(a, &tile, &c0, &c1)) {
+            for (int c = c0; c < c1 && ok; ++c, ++ch) {
+                const int nb = min(kChunkBlocks, a.kblocks - kChunkBlocks * c);
+                uint32_t fresh = 0;
+#pragma unroll
+                for (int t = 0; t < kParts64; ++t) fresh |= (c - c0) % period(t) == 0 ? 1u << t : 0u;
+                // classes 0 to 3 of the whole chunk, drained while the others run
+                if (!(ok = wait(&gempty[0], (ch & 1) ^ 1))) break;
+                for (int b0 = 0; b0 < nb; b0 += 2) {
+                    // two blocks per wait, half the lanes polling each
+                    const int b1 = min(b0 + 2, nb);
+                    int sl = slot + min(b0 + (lane & 1), b1 - 1);
+                    const uint32_t ph = sl >= a.stages ? phase ^ 1 : phase;
+                    if (sl >= a.stages) sl -= a.stages;
+                    if (!(ok = wait(&full[sl], ph))) break;
+                    tc_fence_after();
+                    if (elect_one()) {
+                        sl = slot + b0 >= a.stages ? slot + b0 - a.stages : slot + b0;
+                        for (int b = b0; b < b1; ++b) {
+                            const uint32_t off = (uint32_t)sl * stage_bytes / 16;
+                            if (b == 0) issue<NT, 0, 4>(tmem, fresh, alo0 + off, ahi, blo0 + off, bhi);
+                            else issue<NT, 0, 4>(tmem, 0u, alo0 + off, ahi, blo0 + off, bhi);
+                            if (++sl == a.stages) sl = 0;
+                        }
+                        if (b1 == nb) mma_commit(&gfull[0]);
+                    }
+                    __syncwarp();
+                }
+                if (!ok) break;
+                if (!(ok = wait(&gempty[1], (ch & 1) ^ 1))) break;
+                tc_fence_after();
+                if (elect_one()) {
+                    int sl = slot;
+                    for (int b = 0; b < nb; ++b) {
+                        const uint32_t off = (uint32_t)sl * stage_bytes / 16;
+                        if (b == 0) issue<NT, 4, 7>(tmem, fresh, alo0 + off, ahi, blo0 + off, bhi);
+                        else issue<NT, 4, 7>(tmem, 0u, alo0 + off, ahi, blo0 + off, bhi);
+                        mma_commit(&empty[sl]);
+                        if (++sl == a.stages) sl = 0;
+                    }
+                    mma_commit(&gfull[1]);
+                }
+                __syncwarp();
+                slot += nb;
+                if (slot >= a.stages) {
+                    slot -= a.stages;
+                    phase ^= 1;
+                }
+            }
+        }
+        if (elect_one()) mma_commit(mma_done);
+        __syncwarp();
+        volatile int no_abort = 0;
+        mbar_wait(mma_done, 0, &no_abort, err, 2u, 100000000ull);
+    }
+    }
+    __syncwarp();
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    if (warp == 1) tmem_dealloc(tmem, a.tmem_cols);
+}
+
+// The partial tiles of a split reduction, added in the order of the groups.
+__host__ __device__ __forceinline__ int64_t group_of_chunk(int64_t u, int64_t Q, int64_t G) {
+    return ((u + 1) * G + Q - 1) / Q - 1;
+}
+
+__global__ void __launch_bounds__(256) part_sum_kernel(const double* __restrict__ part, int NT, int64_t ntiles,
+                                                       int64_t chunks, int64_t Q, int64_t G, int group,
+                                                       double* __restrict__ C, int64_t cr, int64_t cc, int64_t M,
+                                                       int64_t N, const double* __restrict__ rscale,
+                                                       const double* __restrict__ cscale, int* __restrict__ clear) {
+    pdl_wait();
+    pdl_trigger();
+    if (clear && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *clear = 0;
+    const int64_t tile = blockIdx.x;
+    const int64_t mt = tile / ntiles, nt = tile - mt * ntiles, u = tile / group * chunks;
+    const int64_t p0 = group_of_chunk(u, Q, G), p1 = group_of_chunk(u + chunks - 1, Q, G);
+    for (int e = blockIdx.y * 256 + threadIdx.x; e < 128 * NT; e += 256 * gridDim.y) {
+        const int64_t row = mt * 128 + (e & 127), col = nt * NT + (e >> 7);
+        if (row >= M || col >= N) continue;
+        double s = 0.0;
+#pragma unroll 4
+        for (int64_t p = p0; p <= p1; ++p) s += part[(p * group + tile) * (128 * NT) + e];
+        if (rscale) s *= __ldg(rscale + row);
+        if (cscale) s *= __ldg(cscale + col);
+        C[row * cr + col * cc] = s;
+    }
+}
+
+// ---------------------------------------------------------------- repair
+// Rows listed as hard: their part of C by binary64 FMAs, 64 x 64 tiles of
+// gathered rows, 4 x 4 entries a thread.
+__global__ void __launch_bounds__(256) repair_kernel(View64 A, const int* __restrict__ ha, int64_t M, View64 B,
+                                                     const int* __restrict__ hb, int64_t N, int64_t K,
+                                                     double* __restrict__ C, int64_t cr, int64_t cc,
+                                                     const double* __restrict__ rscale,
+                                                     const double* __restrict__ cscale) {
+    __shared__ double As[16][65];
+    __shared__ double Bs[16][65];
+    pdl_wait();
+    pdl_trigger();
+    const int64_t na = ha[0], nb = hb[0];
+    const int64_t ta = (na + 63) / 64 * ((N + 63) / 64), tb = (nb + 63) / 64 * ((M + 63) / 64);
+    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+    for (int64_t t = blockIdx.x; t < ta + tb; t += gridDim.x) {
+        // tile of C rows (first list entry or row) and columns
+        const bool ga = t < ta;
+        const int64_t u = ga ? t : t - ta;
+        const int64_t other = ga ? (N + 63) / 64 : (M + 63) / 64;
+        const int64_t l0 = u / other * 64, o0 = (u % other) * 64;
+        const int64_t i0 = ga ? l0 : o0, j0 = ga ? o0 : l0;
+        const int64_t ni = ga ? na : M, nj = ga ? N : nb;
+        auto row_of = [&](int i) { return i0 + i < ni ? (ga ? (int64_t)ha[1 + i0 + i] : i0 + i) : (int64_t)-1; };
+        auto col_of = [&](int j) { return j0 + j < nj ? (ga ? j0 + j : (int64_t)hb[1 + j0 + j]) : (int64_t)-1; };
+        double acc[4][4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
+        for (int64_t k0 = 0; k0 < K; k0 += 16) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int e = tid + 256 * q;
+                const int kk = e & 15, x = e >> 4;
+                const int64_t ri = row_of(x), cj = col_of(x);
+                As[kk][x] = (ri >= 0 && k0 + kk < K) ? A.at(ri, k0 + kk) : 0.0;
+                Bs[kk][x] = (cj >= 0 && k0 + kk < K) ? B.at(cj, k0 + kk) : 0.0;
+            }
+            __syncthreads();
+            const int kn = (int)min((int64_t)16, K - k0);
+#pragma unroll 4
+            for (int kk = 0; kk < kn; ++kk) {
+                double x[4], y[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) x[i] = As[kk][ty + 16 * i];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) y[j] = Bs[kk][tx + 16 * j];
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) acc[i][j] = fma(x[i], y[j], acc[i][j]);
+            }
+            __syncthreads();
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int64_t row = row_of(ty + 16 * i);
+            if (row < 0) continue;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int64_t col = col_of(tx + 16 * j);
+                if (col < 0) continue;
+                double s = acc[i][j];
+                if (rscale) s *= __ldg(rscale + row);
+                if (cscale) s *= __ldg(cscale + col);
+                C[row * cr + col * cc] = s;
+            }
+        }
+    }
+}
+
+size_t up256(size_t v) { return (v + 255) & ~(size_t)255; }
+
+int stat_splits(int64_t rows, int64_t K) {
+    // enough CTAs for two per SM, at least 256 columns each
+    const int64_t groups = (rows + 31) / 32;
+    int64_t z = (2 * (int64_t)sm_count() + groups - 1) / groups;
+    z = std::min<int64_t>(z, (K + 255) / 256);
+    return (int)std::max<int64_t>(1, std::min<int64_t>(z, kStatSplits));
+}
+
+template <int NT>
+lrc_status launch_product(const GemmArgs& a, int64_t grid, size_t smem, cudaStream_t s) {
+    cudaError_t e = cudaFuncSetAttribute(product_kernel<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return cuda_fail(e, "split product_kernel smem attribute");
+    e = launch_pdl(product_kernel<NT>, dim3((unsigned)grid), dim3(kThreads), smem, s, a);
+    if (e != cudaSuccess) return cuda_fail(e, "split product_kernel launch");
+    return after_launch("split product_kernel");
+}
+
+}  // namespace
+
+size_t operand_bytes(int64_t rows, int64_t K, int R) {
+    const int64_t tiles = image_tiles(rows, R);
+    return up256((size_t)tiles * image_blocks(K) * kParts64 * R * kKB * 2) + up256((size_t)tiles * R * 4) +
+           up256((size_t)rows * kStatSplits * sizeof(int4)) + up256((size_t)(rows + 1) * 4);
+}
+
+void operand_carve(Operand64* o, unsigned char* ws) {
+    const int64_t tiles = image_tiles(o->rows, o->R);
+    o->img = ws;
+    ws += up256((size_t)tiles * image_blocks(o->K) * kParts64 * o->R * kKB * 2);
+    o->exps = reinterpret_cast<int*>(ws);
+    ws += up256((size_t)tiles * o->R * 4);
+    o->stats = reinterpret_cast<int4*>(ws);
+    ws += up256((size_t)o->rows * kStatSplits * sizeof(int4));
+    o->hard = reinterpret_cast<int*>(ws);
+}
+
+lrc_status slice(const Operand64* const* ops, int count, cudaStream_t s) {
+    Jobs st{}, sl{};
+    int64_t bs = 0, bl = 0;
+    for (int i = 0; i < count; ++i) {
+        const Operand64& o = *ops[i];
+        Job j{};
+        j.v = View64{o.src};
+        j.rows = o.rows;
+        j.K = o.K;
+        j.R = o.R;
+        j.img_rows = image_tiles(o.rows, o.R) * o.R;
+        j.kblocks = image_blocks(o.K);
+        j.vec = o.src.cs == 1 && o.src.rs % 2 == 0 && aligned16(o.src.p);
+        j.stats = o.stats;
+        j.img = o.img;
+        j.exps = o.exps;
+        j.hard = o.hard;
+        if (o.K > kOwnStatsK) {
+            const int z = stat_splits(o.rows, o.K);
+            j.kchunk = ((o.K + z - 1) / z + 31) / 32 * 32;
+            j.splits = (int)((o.K + j.kchunk - 1) / j.kchunk);
+            j.b0 = bs;
+            bs += (o.rows + 31) / 32 * j.splits;
+            st.j[st.n++] = j;
+            j.kchunk = 256;
+        } else {
+            j.kchunk = j.kblocks * kKB;
+        }
+        j.kparts = (int)((j.kblocks * kKB + j.kchunk - 1) / j.kchunk);
+        j.b0 = bl;
+        bl += (j.img_rows + 31) / 32 * j.kparts;
+        sl.j[sl.n++] = j;
+        if (!o.cleared) st.clear[i] = o.hard;
+    }
+    if (bs > 0x7fffffff || bl > 0x7fffffff) {
+        set_error("split product: operand too large");
+        return LRC_ERR_UNSUPPORTED;
+    }
+    lrc_status r;
+    cudaError_t e;
+    if (st.n == 0) {
+        for (int i = 0; i < count; ++i)
+            if (st.clear[i] && (e = cudaMemsetAsync(st.clear[i], 0, sizeof(int), s)) != cudaSuccess)
+                return cuda_fail(e, "cudaMemsetAsync (row list)");
+    } else {
+        e = launch_pdl(row_stats_kernel, dim3((unsigned)bs), dim3(256), 0, s, st);
+        if (e != cudaSuccess) return cuda_fail(e, "row_stats_kernel launch");
+        if ((r = after_launch("row_stats_kernel")) != LRC_OK) return r;
+    }
+    e = launch_pdl(slice_kernel, dim3((unsigned)bl), dim3(256), 0, s, sl);
+    if (e != cudaSuccess) return cuda_fail(e, "slice_kernel launch");
+    return after_launch("slice_kernel");
+}
+
+size_t part_bytes(int64_t M, int64_t N, int64_t K, int R_b) {
+    (void)K;
+    const int64_t tiles = image_tiles(M, 128) * image_tiles(N, R_b);
+    return up256((size_t)(tiles + sm_count()) * 128 * R_b * 8);
+}
+
+lrc_status product(const Operand64& A, const Operand64& B, const Out64& out, bool split, double* part, cudaStream_t s) {
+    const int NT = B.R;
+    GemmArgs a{};
+    a.A = A.img;
+    a.B = B.img;
+    a.ea = A.exps;
+    a.eb = B.exps;
+    a.C = split ? part : out.C;
+    a.cr = out.cr;
+    a.cc = out.cc;
+    a.M = A.rows;
+    a.N = B.rows;
+    const int64_t tiles = image_tiles(A.rows, 128) * image_tiles(B.rows, NT);
+    if (tiles > 0x3fffffff || A.K > kMaxK) {
+        set_error("split product too large (%lld tiles, reduction of %lld)", (long long)tiles, (long long)A.K);
+        return LRC_ERR_UNSUPPORTED;
+    }
+    a.ntiles = (int)image_tiles(B.rows, NT);
+    a.tiles = (int)tiles;
+    a.kblocks = (int)image_blocks(A.K);
+    a.chunks = (a.kblocks + kChunkBlocks - 1) / kChunkBlocks;
+    a.split = split;
+    a.a_bytes = kParts64 * 128 * kKB * 2;
+    a.b_bytes = (uint32_t)(kParts64 * NT * kKB * 2);
+    a.stages = (int)std::min<int64_t>(8, (int64_t)(227 * 1024 - kCtrlBytes) / (a.a_bytes + a.b_bytes));
+    a.vec = out.cc != 1 || out.cr % 2 != 0 || !aligned16(out.C) ? 0
+            : out.cr % 4 == 0 && (reinterpret_cast<uintptr_t>(out.C) & 31u) == 0 ? 2 : 1;
+    uint32_t cols = 32;
+    while (cols < (uint32_t)(7 * NT)) cols *= 2;
+    a.tmem_cols = cols;
+    const int64_t sms = sm_count();
+    // groups of one CTA per tile of B while that leaves at least eight groups
+    a.group = split && (int64_t)a.ntiles * 8 <= sms ? a.ntiles : 1;
+    const int64_t Q = tiles / a.group * a.chunks;
+    const int64_t groups = std::min<int64_t>(Q, sms / a.group);
+    const int64_t grid = split ? groups * a.group : std::min<int64_t>(tiles, sms);
+    const size_t smem = kCtrlBytes + (size_t)a.stages * (a.a_bytes + a.b_bytes);
+    lrc_status st;
+    switch (NT) {
+        case 16: st = launch_product<16>(a, grid, smem, s); break;
+        case 32: st = launch_product<32>(a, grid, smem, s); break;
+        case 48: st = launch_product<48>(a, grid, smem, s); break;
+        default: st = launch_product<64>(a, grid, smem, s); break;
+        
+    }
+    if (st != LRC_OK) return st;
+    cudaError_t e;
+    if (split) {
+        const unsigned gy = (unsigned)std::max<int64_t>(1, std::min<int64_t>(128 * NT / 256, 4 * sms / tiles));
+        e = launch_pdl(part_sum_kernel, dim3((unsigned)tiles, gy), dim3(256), 0, s, (const double*)part, NT, (int64_t)a.ntiles,
+                       (int64_t)a.chunks, Q, groups, a.group, out.C, out.cr, out.cc, A.rows, B.rows, out.rscale, out.cscale, out.clear);
+        if (e != cudaSuccess) return cuda_fail(e, "part_sum_kernel launch");
+        if ((st = after_launch("part_sum_kernel")) != LRC_OK) return st;
+    }
+    e = launch_pdl(repair_kernel, dim3((unsigned)(2 * sms)), dim3(256), 0, s, View64{A.src}, (const int*)A.hard, A.rows,
+                   View64{B.src}, (const int*)B.hard, B.rows, A.K, out.C, out.cr, out.cc, out.rscale, out.cscale);
+    if (e != cudaSuccess) return cuda_fail(e, "repair_kernel launch");
+    return after_launch("repair_kernel");
+}
+
+}  // namespace sg
+
+uint32_t take_split_error() {
+    unsigned int v = 0;
+    if (cudaMemcpyFromSymbol(&v, sg::g_err_split, sizeof v) != cudaSuccess) return 0xffffffffu;
+    if (v) {
+        const unsigned int z = 0;
+        cudaMemcpyToSymbol(sg::g_err_split, &z, sizeof z);
+    }
+    return v;
+}
+
+}  // namespace lrc

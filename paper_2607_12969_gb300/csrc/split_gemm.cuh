@@ -1,0 +1,74 @@
+// split_gemm.cuh -- products of binary64 matrices on the tensor cores
+// (split_gemm.cu): operands, images and the product itself.
+#pragma once
+
+#include "common.cuh"
+
+namespace lrc {
+namespace sg {
+
+constexpr int kParts64 = 7;        // 9-bit digits a binary64 value is cut into
+constexpr int kKB = 16;            // columns of the reduction per image block
+constexpr int64_t kMaxK = 1 << 20; // longest reduction the 64-bit sums hold
+constexpr int kStatSplits = 32;    // most slices of the reduction in the row statistics
+
+// Rows a digit image is tiled by: 128 for the first operand; for the second
+// the rows split evenly over tiles of at most kNTMax rows, a multiple of 16.
+constexpr int kNTMax = 64;
+inline int n_tile(int64_t rows) {
+    const int64_t tiles = (rows + kNTMax - 1) / kNTMax;
+    return (int)(((rows + tiles - 1) / tiles + 15) / 16 * 16);
+}
+
+// A matrix whose rows are cut into digits: entry (r, c) is p[r rs + c cs]
+// times 2^(sh sign) with sh half the exponent of scale[c] (scale may be null).
+// For W = (X V) diag(s) and U of a second product W U^T with scale = s and
+// signs -1 and +1: with s_j decaying over many orders the entries of a row of
+// W would lie far below its first ones; this halves that distance on either
+// side, exactly.
+struct Src64 {
+    const double* p;
+    int64_t rs, cs;
+    const double* scale;
+    int sign;
+};
+
+// One operand of a product.  `rows` x K; tiles of R rows.
+struct Operand64 {
+    Src64 src;
+    int64_t rows, K;
+    int R;
+    unsigned char* img;      // digits
+    int* exps;               // exponent of every row (image rows)
+    int4* stats;             // row statistics per slice of K
+    int* hard;               // hard[0] = rows that the digits cannot carry; then their indices
+    bool cleared = false;    // an earlier kernel of the call has set hard[0] = 0
+};
+constexpr int kMaxOps = 3;   // operands per slice()
+
+inline int64_t image_tiles(int64_t rows, int R) { return (rows + R - 1) / R; }
+inline int64_t image_blocks(int64_t K) { return (K + kKB - 1) / kKB; }
+size_t operand_bytes(int64_t rows, int64_t K, int R);
+// Carves an operand's buffers out of `ws` (256-byte aligned).
+void operand_carve(Operand64* o, unsigned char* ws);
+
+// Digits of up to kMaxOps operands (at most two launches for all of them).
+lrc_status slice(const Operand64* const* ops, int count, cudaStream_t s);
+
+// C(i, j) at C[i cr + j cc], i < A.rows, j < B.rows: the product A B^T times
+// rscale[i] cscale[j] (each may be null).  `split` splits the reduction over
+// the CTAs (few, deep tiles); its partial sums are added in a fixed order.
+// `part` holds part_bytes() bytes.  Rows that the digits cannot carry are
+// recomputed with binary64 FMAs.
+struct Out64 {
+    double* C;
+    int64_t cr, cc;
+    const double* rscale;
+    const double* cscale;
+    int* clear = nullptr;    // a later operand's hard[0], set to 0 on the way (split only)
+};
+size_t part_bytes(int64_t M, int64_t N, int64_t K, int R_b);
+lrc_status product(const Operand64& A, const Operand64& B, const Out64& out, bool split, double* part, cudaStream_t s);
+
+}  // namespace sg
+}  // namespace lrc

@@ -175,6 +175,14 @@ __device__ __forceinline__ void bulk_wait() {
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// ---------------------------------------------------------------- registers
+// Every warp of a warpgroup gives up (dec) or takes (inc, from what the
+// block's other warpgroups gave up) registers, to N a thread.
+template <int N>
+__device__ __forceinline__ void reg_dec() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N)); }
+template <int N>
+__device__ __forceinline__ void reg_inc() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N)); }
+
 // ---------------------------------------------------------------- tensor memory
 // Allocates `ncols` (power of two >= 32) columns; the whole warp must call.
 __device__ __forceinline__ void tmem_alloc(uint32_t* slot_smem, uint32_t ncols) {
@@ -200,6 +208,19 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
           "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]),
           "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
         : "r"(taddr));
+}
+
+// The same with 8 columns.
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr));
+}
+
+// ... and with 4.
+__device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t (&r)[4]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(taddr));
 }
 
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
@@ -256,6 +277,32 @@ __device__ __forceinline__ void mma_f16(uint32_t d_tmem, uint64_t a_desc, uint64
         : "memory");
 }
 
+// True on one lane of a converged warp (the same one each time).
+__device__ __forceinline__ bool elect_one() {
+    uint32_t r;
+    asm volatile("{\n .reg .pred q;\n elect.sync _|q, 0xffffffff;\n selp.u32 %0, 1, 0, q;\n}\n" : "=r"(r));
+    return r != 0;
+}
+
+// mma_f16 with descriptors given as their low and high words.  USE names what
+// the MMA does with the collector buffer of A: kept for the next MMA (kFill),
+// taken from it (kUse, kLast for the last time) or neither.
+enum CollectorUse { kNoReuse, kFill, kUse, kLast };
+#define LRC_MMA_COL(OP)                                                                                          \
+    asm volatile("{\n .reg .pred p;\n .reg .b64 da, db;\n mov.b64 da, {%1, %2};\n mov.b64 db, {%3, %4};\n"        \
+                 " setp.ne.b32 p, %6, 0;\n"                                                                       \
+                 " tcgen05.mma.cta_group::1.kind::f16" OP " [%0], da, db, %5, p;\n}\n" ::"r"(d_tmem),            \
+                 "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate)                         \
+                 : "memory")
+template <int USE>
+__device__ __forceinline__ void mma_f16_col(uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo,
+                                            uint32_t b_hi, uint32_t idesc, uint32_t accumulate) {
+    if constexpr (USE == kFill) LRC_MMA_COL(".collector::a::fill");
+    else if constexpr (USE == kUse) LRC_MMA_COL(".collector::a::use");
+    else if constexpr (USE == kLast) LRC_MMA_COL(".collector::a::lastuse");
+    else LRC_MMA_COL("");
+}
+#undef LRC_MMA_COL
 // Arrives once on `bar` when every previously issued tcgen05.mma of this
 // thread has completed.
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {

@@ -66,6 +66,28 @@ lrc_status stream_workspace(cudaStream_t s, size_t bytes, void** out) {
     return LRC_OK;
 }
 
+lrc_status stream_workspace_try(cudaStream_t s, size_t bytes, void** out) {
+    *out = nullptr;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return cuda_fail(e, "cudaGetDevice");
+    bool grow = true;
+    {
+        std::lock_guard<std::mutex> lock(g_ws_mu);
+        const auto it = g_ws.find(std::make_pair(dev, s));
+        grow = it == g_ws.end() || it->second.bytes < bytes;
+    }
+    if (grow) {
+        // a buffer cannot be made or replaced while the stream is being captured
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) cudaGetLastError();
+        if (cap != cudaStreamCaptureStatusNone) return LRC_OK;
+    }
+    const lrc_status st = stream_workspace(s, bytes, out);
+    if (st == LRC_ERR_NOMEM) *out = nullptr;
+    return st == LRC_ERR_NOMEM ? LRC_OK : st;
+}
+
 lrc_status stream_counters(cudaStream_t s, unsigned int** out) {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);

@@ -1,0 +1,115 @@
+"""binary64 products on the tensor cores (split_gemm.cu): values cut into
+seven 9-bit digits, 28 exact digit products, one rounding.
+
+Integer data whose sums stay below 2^53 must come out exactly, whatever the
+tiling; rows that the digits cannot carry (wide ranges, infinities, NaN,
+extreme magnitudes) go through binary64 FMAs and must come out as they do."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import workloads as W
+from parity import packed, rel_fro
+
+pytestmark = pytest.mark.gpu
+
+U64 = 2.0 ** -53
+
+
+def run(lrc, dev, U, s, Vt, X):
+    m, k = U.shape
+    n, b = Vt.shape[1], X.shape[0]
+    ops = [packed(lrc, a, "f64", dev) for a in (U, s, Vt, X)]
+    Y = torch.full((b, m), float("nan"), dtype=torch.float64, device=dev)
+    lrc.lrc_apply(*ops, Y, m, n, k, b, "f64")
+    torch.cuda.synchronize()
+    assert lrc.lrc_device_status() == 0
+    return Y.cpu().numpy()
+
+
+# tile edges of both orientations (128 rows by 16, 32, 48 or 64), reductions of
+# one block, a partial chunk, several chunks with every drain period, odd sizes
+SHAPES = [(129, 65, 33, 700), (1000, 64, 64, 128), (257, 1100, 300, 127), (4096, 17, 16, 200), (301, 2049, 40, 128),
+          (64, 5000, 128, 17), (2051, 700, 97, 33), (127, 40000, 16, 129)]
+
+
+@pytest.mark.parametrize("m,n,k,b", SHAPES)
+def test_integers_are_exact(lrc, cuda, m, n, k, b):
+    rng = np.random.default_rng(m + n)
+    hi = max(2, int(2.0 ** (51 - 2 - np.log2(k) - 3 - np.log2(n) - 7)))     # the sums stay below 2^53
+    X = rng.integers(-hi, hi + 1, (b, n)).astype(np.float64)
+    Vt = rng.integers(-64, 65, (k, n)).astype(np.float64)
+    U = rng.integers(-8, 9, (m, k)).astype(np.float64)
+    s = rng.integers(-2, 3, k).astype(np.float64)
+    want = ((X @ Vt.T) * s) @ U.T
+    assert np.max(np.abs(want)) < 2.0 ** 53
+    assert np.array_equal(run(lrc, cuda, U, s, Vt, X), want)
+
+
+@pytest.mark.parametrize("m,n,k,b", SHAPES[:5])
+def test_close_to_the_exact_product(lrc, cuda, m, n, k, b):
+    """W and Y are each rounded once; digits and the classes left out add less:
+    relative Frobenius error below 4 u against a product in extended precision."""
+    f = W.random_factors(m, n, k, seed=7)
+    X = W.gaussian((b, n), 8)
+    got = run(lrc, cuda, f.U, f.s, f.Vt, X)
+    L = np.longdouble
+    want = ((X.astype(L) @ f.Vt.T.astype(L)) * f.s.astype(L)) @ f.U.T.astype(L)
+    assert float(np.linalg.norm((got - want).astype(np.float64))) <= 4 * U64 * float(np.linalg.norm(want.astype(np.float64)))
+
+
+def test_rows_the_digits_cannot_carry(lrc, cuda):
+    m, n, k, b = 300, 777, 64, 130
+    f = W.random_factors(m, n, k, seed=9)
+    X = W.gaussian((b, n), 10)
+    U, Vt = f.U.copy(), f.Vt.copy()
+    rng = np.random.default_rng(11)
+    X[3] *= 2.0 ** rng.integers(-200, 200, n)        # a wide row
+    X[4] = 0.0
+    X[5] *= 2.0 ** 600                               # beyond the digits' exponents
+    U[17] *= 2.0 ** rng.integers(-90, 90, k)
+    U[18] *= 2.0 ** -700
+    Vt[2] *= 2.0 ** rng.integers(-90, 90, n)
+    got = run(lrc, cuda, U, f.s, Vt, X)
+    want = oracle.apply(U, f.s, Vt, X)
+    bound = (np.abs(X) @ np.abs(Vt).T * np.abs(f.s)) @ np.abs(U).T
+    assert np.all(np.abs(got - want) <= 2 * (n + k + 2) * U64 * bound)
+
+
+@pytest.mark.parametrize("v", [np.inf, -np.inf, np.nan])
+def test_nonfinite_values_spread_as_in_fma_sums(lrc, cuda, v):
+    m, n, k, b = 200, 300, 64, 300
+    f = W.random_factors(m, n, k, seed=12)
+    X = W.gaussian((b, n), 13)
+    U = f.U.copy()
+    X[7, 5] = v
+    U[9, 2] = v
+    got = run(lrc, cuda, U, f.s, f.Vt, X)
+    with np.errstate(invalid="ignore"):
+        want = ((X @ f.Vt.T) * f.s) @ U.T
+    assert np.array_equal(np.isnan(got), np.isnan(want))
+    inf = np.isinf(want)
+    assert np.array_equal(got[inf], want[inf])
+    ok = np.isfinite(want)
+    assert rel_fro(got[ok], want[ok]) <= 1e-14
+
+
+def test_captured_call_and_repeat_are_the_same_bits(lrc, cuda):
+    m, n, k, b = 600, 900, 48, 256
+    f = W.random_factors(m, n, k, seed=14)
+    X = W.gaussian((b, n), 15)
+    ops = [packed(lrc, a, "f64", cuda) for a in (f.U, f.s, f.Vt, X)]
+    Y = torch.empty((b, m), dtype=torch.float64, device=cuda)
+    st = torch.cuda.Stream()
+    with torch.cuda.stream(st):
+        lrc.lrc_apply(*ops, Y, m, n, k, b, "f64", stream=st)
+    torch.cuda.synchronize()
+    want = Y.clone()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=st):
+        lrc.lrc_apply(*ops, Y, m, n, k, b, "f64", stream=st)
+    Y.zero_()
+    g.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(Y.view(torch.int64), want.view(torch.int64))
