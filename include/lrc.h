@@ -223,7 +223,10 @@ LRC_API lrc_status lrc_apply_batched(int count, const void* const* U, const void
  * Element types: LRC_F64 cores/out binary64; LRC_F32 binary32; LRC_F16
  * binary16 cores, binary32 out; LRC_F16_O16 binary16 cores, workspaces and
  * out.  Cores must be aligned to their element size, out to 16 bytes.
- * Intermediate products Z_l stay on chip.  Asynchronous on `stream`.
+ * Intermediate products Z_l of the FMA kernels stay on chip; LRC_F64 chains of
+ * at least 4e7 flops form every product from digits on the tensor cores (see
+ * lrc_apply), with Z_l, S_l and the digits in the stream's workspace, or where
+ * there is no memory for them by the FMA kernels.  Asynchronous on `stream`.
  */
 /* LRC_F32_TC: binary32 cores and output; the chain's output product on the
  * tensor cores when the chain's sides fit its one-pass side kernel
@@ -338,9 +341,10 @@ LRC_API lrc_status lrc_fro_diff_noalloc(const void* A, lrc_fmt fa, const void* B
  * of the size of ||A|| cancels: the result is accurate relative to eta,
  * where the dense route (lrc_apply with X = I, lrc_fro_diff) is accurate
  * relative to ||A||.  Work: about 2 (m + n) k (2k + 1) binary64 flops.
- * All arithmetic binary64; deterministic on a device.  k <= 4096.  Pointers
- * 16-byte aligned.  Scratch: the stream's library workspace (see
- * lrc_apply), 16 (m + n) k bytes plus O(k^2); the results come back through
+ * All arithmetic binary64 (the Gram matrices of larger factors from digits on
+ * the tensor cores, see lrc_apply); deterministic on a device.  k <= 4096.
+ * Pointers 16-byte aligned.  Scratch: the stream's library workspace (see
+ * lrc_apply), 16 (m + n) k bytes, with digits 44 (m + n) k, plus O(k^2); the results come back through
  * the stream's mapped host slot (see lrc_fro_diff).  SYNCHRONISES `stream`.
  */
 LRC_API lrc_status lrc_lowrank_eta(const double* U, const double* S, const double* Vt,

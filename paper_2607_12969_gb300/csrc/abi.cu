@@ -256,6 +256,11 @@ lrc_status tt_reconstruct(const void* const* cores, const int64_t* dims, const i
         return launch_tt_chain_f32tc(sh, static_cast<float*>(out), s);
     }
     if (fmt == LRC_F32 || fmt == LRC_F32_TC) return launch_tt_chain_f32(sh, static_cast<float*>(out), s);
+    if (tt_chain_f64_tc_takes(sh)) {
+        bool handled = false;
+        st = launch_tt_chain_f64_tc(sh, static_cast<double*>(out), s, &handled);
+        if (st != LRC_OK || handled) return st;
+    }
     if (tt_chain_saves(sh)) return launch_tt_chain_f64(sh, static_cast<double*>(out), s);
     return launch_tt_cc(sh, fmt, out, s);
 }

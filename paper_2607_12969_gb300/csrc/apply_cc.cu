@@ -490,14 +490,6 @@ constexpr int64_t kSplitMaxBatchF64 = 2048, kSplitMaxBatchF32 = 32, kSplitMaxRan
 // ---------------------------------------------------------------- binary64 on the tensor cores
 namespace {
 
-// First operand of a product: the one whose tiles waste less (tiles of 128
-// rows of the first, of at most kNTMax of the second).
-bool swap_sides(int64_t M, int64_t N) {
-    const int64_t a = sg::image_tiles(M, 128) * sg::image_tiles(N, sg::n_tile(N));
-    const int64_t b = sg::image_tiles(N, 128) * sg::image_tiles(M, sg::n_tile(M));
-    return b < a;
-}
-
 constexpr int64_t kPanelBytes = (int64_t)1 << 30;     // digit images of a panel of queries
 
 }  // namespace
@@ -522,23 +514,22 @@ static lrc_status launch_apply_f64_tc(const double* U, const double* S, const do
     int64_t pb = kPanelBytes / (sg::kParts64 * 2 * sg::kKB * sg::image_blocks(n)) / 128 * 128;
     if (pb < 128) pb = 128;
     if (pb > b) pb = b;
-    const bool sw1 = swap_sides(pb, k), sw2 = swap_sides(pb, m);
-    const int R_x = sw1 ? sg::n_tile(pb) : 128, R_v = sw1 ? 128 : sg::n_tile(k);
-    const int R_w = sw2 ? sg::n_tile(pb) : 128, R_u = sw2 ? 128 : sg::n_tile(m);
-    sg::Operand64 oV{{Vt, ldn, 1, nullptr, 0}, k, n, R_v};
-    sg::Operand64 oU{{U, ldk, 1, S, 1}, m, k, R_u};
-    sg::Operand64 oX{{X, ldn, 1, nullptr, 0}, pb, n, R_x};
-    sg::Operand64 oW{{nullptr, ldk, 1, S, -1}, pb, k, R_w};
+    sg::Operand64 oV{{Vt, ldn, 1, nullptr, 0}, k, n};
+    sg::Operand64 oU{{U, ldk, 1, S, 1}, m, k};
+    sg::Operand64 oX{{X, ldn, 1, nullptr, 0}, pb, n};
+    sg::Operand64 oW{{nullptr, ldk, 1, S, -1}, pb, k};
     size_t off = 0;
     auto take = [&](size_t bytes) {
         const size_t o = off;
         off += (bytes + 255) & ~(size_t)255;
         return o;
     };
-    const size_t o_v = take(sg::operand_bytes(k, n, R_v)), o_u = take(sg::operand_bytes(m, k, R_u));
-    const size_t o_x = take(sg::operand_bytes(pb, n, R_x)), o_w = take(sg::operand_bytes(pb, k, R_w));
+    const size_t o_v = take(sg::operand_bytes(k, n)), o_u = take(sg::operand_bytes(m, k));
+    const size_t o_x = take(sg::operand_bytes(pb, n)), o_w = take(sg::operand_bytes(pb, k));
     const size_t o_wd = take((size_t)pb * ldk * 8);
-    const size_t o_p = take(sw1 ? sg::part_bytes(k, pb, n, R_x) : sg::part_bytes(pb, k, n, R_v));
+    size_t pbytes = sg::part_bytes(pb, k);
+    if (b % pb) pbytes = sg::part_bytes(b % pb, k) > pbytes ? sg::part_bytes(b % pb, k) : pbytes;     // the last panel
+    const size_t o_p = take(pbytes);
     void* ws = nullptr;
     lrc_status st = stream_workspace_try(s, off, &ws);
     if (st != LRC_OK || !ws) return st;
@@ -559,13 +550,9 @@ static lrc_status launch_apply_f64_tc(const double* U, const double* S, const do
         const sg::Operand64* px[3] = {&oX, &oV, &oU};      // V and U with the first panel
         const sg::Operand64* pw[1] = {&oW};
         if ((st = sg::slice(px, r0 == 0 ? 3 : 1, s)) != LRC_OK) return st;
-        const sg::Out64 ow = sw1 ? sg::Out64{W, 1, ldk, S, nullptr, oW.hard} : sg::Out64{W, ldk, 1, nullptr, S, oW.hard};
-        if ((st = sw1 ? sg::product(oV, oX, ow, true, part, s) : sg::product(oX, oV, ow, true, part, s)) != LRC_OK)
-            return st;
+        if ((st = sg::product(oX, oV, sg::Out64{W, ldk, 1, nullptr, S, oW.hard}, true, part, s)) != LRC_OK) return st;
         if ((st = sg::slice(pw, 1, s)) != LRC_OK) return st;
-        double* Yr = Y + r0 * m;
-        const sg::Out64 oy = sw2 ? sg::Out64{Yr, 1, m, nullptr, nullptr} : sg::Out64{Yr, m, 1, nullptr, nullptr};
-        if ((st = sw2 ? sg::product(oU, oW, oy, false, nullptr, s) : sg::product(oW, oU, oy, false, nullptr, s)) != LRC_OK)
+        if ((st = sg::product(oW, oU, sg::Out64{Y + r0 * m, m, 1, nullptr, nullptr}, false, nullptr, s)) != LRC_OK)
             return st;
     }
     return LRC_OK;

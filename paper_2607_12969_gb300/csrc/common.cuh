@@ -164,6 +164,10 @@ lrc_status launch_tt_cc(const TTShape& sh, lrc_fmt fmt, void* out, cudaStream_t 
 lrc_status launch_tt_chain_f32(const TTShape& sh, float* out, cudaStream_t s);
 lrc_status launch_tt_chain_f64(const TTShape& sh, double* out, cudaStream_t s);
 bool tt_chain_saves(const TTShape& sh);
+// the binary64 chain with its products on the tensor cores (split_gemm.cu);
+// *handled = false when there is no workspace for it (nothing launched)
+bool tt_chain_f64_tc_takes(const TTShape& sh);
+lrc_status launch_tt_chain_f64_tc(const TTShape& sh, double* out, cudaStream_t s, bool* handled);
 // multiply count (x2) of that chain at its cheapest bond
 double tt_chain_flops(const TTShape& sh);
 lrc_status launch_tt_f16(const TTShape& sh, bool out16, void* out, cudaStream_t s);

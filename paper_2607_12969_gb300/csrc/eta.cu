@@ -23,8 +23,9 @@
 // follows from M_l = sum_i C_l(i)^T M_{l-1} C_l(i), so eta_TT^2 =
 // sum_i [G_d(i); dG_d(i)]^T M_{d-1} [G_d(i); dG_d(i)].
 //
-// All arithmetic is binary64 (CUDA-core DFMA); the sums are deterministic
-// (fixed per-CTA ranges, partials added in a fixed order).
+// All arithmetic is binary64 (CUDA-core DFMA; the Gram matrices of larger
+// factors through exact digit products on the tensor cores, split_gemm.cu); the
+// sums are deterministic (fixed per-CTA ranges, partials added in a fixed order).
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
@@ -32,6 +33,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "split_gemm.cuh"
 
 namespace lrc {
 
@@ -412,13 +414,17 @@ __global__ void __launch_bounds__(256) eta_tt_combine_kernel(const double* __res
     }
 }
 
-__global__ void eta_finish_kernel(const double* __restrict__ part, int nparts, double* __restrict__ res) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
+// One block adds the block sums, each thread every 256th in order, then the
+// threads' in a fixed tree.
+__global__ void __launch_bounds__(256) eta_finish_kernel(const double* __restrict__ part, int nparts,
+                                                         double* __restrict__ res) {
     double e2 = 0.0, n2 = 0.0;
-    for (int b = 0; b < nparts; ++b) {
+    for (int b = threadIdx.x; b < nparts; b += 256) {
         e2 += part[2 * b];
         n2 += part[2 * b + 1];
     }
+    block_sum2(e2, n2);
+    if (threadIdx.x != 0) return;
     res[0] = sqrt(fmax(e2, 0.0));
     res[1] = sqrt(fmax(n2, 0.0));
 }
@@ -555,7 +561,7 @@ lrc_status finish_eta(const double* cpart, int nparts, double* eta_out, double* 
     double* dev = nullptr;
     lrc_status st = stream_result_slot(s, &host, &dev);
     if (st != LRC_OK) return st;
-    eta_finish_kernel<<<1, 32, 0, s>>>(cpart, nparts, dev);
+    eta_finish_kernel<<<1, 256, 0, s>>>(cpart, nparts, dev);
     if ((st = after_launch("eta_finish_kernel")) != LRC_OK) return st;
     const cudaError_t e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return cuda_fail(e, "cudaStreamSynchronize (eta)");
@@ -576,6 +582,30 @@ struct Carve {
     }
 };
 
+// The Gram matrix C (p x p, pitch p) of the columns of a matrix of L rows
+// (pitch p) through digits (split_gemm.cu): its columns are the rows of both
+// operands, the reduction runs over L.
+struct DigitGram {
+    sg::Operand64 a;
+    double* part;
+};
+size_t digit_gram_bytes(int p, int64_t L) { return sg::operand_bytes(p, L) + sg::part_bytes(p, p); }
+DigitGram digit_gram(const double* A, int p, int64_t L, unsigned char* ws) {
+    DigitGram g{};
+    g.a.src = sg::Src64{A, 1, p, nullptr, 0};
+    g.a.rows = p;
+    g.a.K = L;
+    sg::operand_carve(&g.a, ws);
+    g.part = reinterpret_cast<double*>(ws + sg::operand_bytes(p, L));
+    return g;
+}
+
+// Multiply-adds from which the Gram matrices of a matrix eta go through digits:
+// their eight launches cost about 60 us, the DFMA kernel 2 us per 1e6 until it
+// fills the GPU and 1.6 us per 1e6 from there (16384 x 8192, k = 144: 2.0e9,
+// 1887 -> 324 us with the rounding of the factors).
+constexpr double kDigitGramWork = 3e7;
+
 template <typename T>
 lrc_status lowrank_eta_t(const double* U, const double* S, const double* Vt, const void* Uh, const void* Sh,
                          const void* Vht, int64_t m, int64_t n, int64_t k, double* eta_out, double* norm_out,
@@ -590,9 +620,16 @@ lrc_status lowrank_eta_t(const double* U, const double* S, const double* Vt, con
     const size_t o_gu = c.take((size_t)w * w * 8), o_gv = c.take((size_t)w * w * 8);
     const size_t o_part = c.take((size_t)gram_slots(sp, 2) * 8);
     const size_t o_cp = c.take((size_t)2 * kCombineBlocks * 8);
+    const size_t plain = c.off;
     void* ws = nullptr;
-    lrc_status st = stream_workspace(s, c.off, &ws);
-    if (st != LRC_OK) return st;
+    lrc_status st = LRC_OK;
+    bool digits = (double)(m + n) * w * w >= kDigitGramWork && m <= sg::kMaxK && n <= sg::kMaxK;
+    const size_t o_du = c.take(digit_gram_bytes(w, m)), o_dv = c.take(digit_gram_bytes(w, n));
+    if (digits) {
+        if ((st = stream_workspace_try(s, c.off, &ws)) != LRC_OK) return st;
+        digits = ws != nullptr;
+    }
+    if (!digits && (st = stream_workspace(s, plain, &ws)) != LRC_OK) return st;
     char* base = (char*)ws;
     double* Pu = (double*)(base + o_pu);
     double* Pv = (double*)(base + o_pv);
@@ -606,7 +643,18 @@ lrc_status lowrank_eta_t(const double* U, const double* S, const double* Vt, con
 
     if ((st = pack_rows<T>(U, ldk, Uh, ldk, m, kk, 0, Pu, s)) != LRC_OK) return st;
     if ((st = pack_cols<T>(Vt, ldn, Vht, ldn, n, kk, 0, Pv, s)) != LRC_OK) return st;
-    if ((st = run_gram(sp, 2, (double*)(base + o_part), s)) != LRC_OK) return st;
+    if (digits) {
+        const DigitGram g[2] = {digit_gram(Pu, w, m, (unsigned char*)base + o_du),
+                                digit_gram(Pv, w, n, (unsigned char*)base + o_dv)};
+        const sg::Operand64* ops[2] = {&g[0].a, &g[1].a};
+        if ((st = sg::slice(ops, 2, s)) != LRC_OK) return st;
+        for (int i = 0; i < 2; ++i) {
+            const sg::Out64 out{sp[i].C, w, 1, nullptr, nullptr};
+            if ((st = sg::product(g[i].a, g[i].a, out, true, g[i].part, s)) != LRC_OK) return st;
+        }
+    } else if ((st = run_gram(sp, 2, (double*)(base + o_part), s)) != LRC_OK) {
+        return st;
+    }
     const int cb = std::min(kCombineBlocks, kk);
     eta_lowrank_combine_kernel<T><<<cb, 256, 0, s>>>(Gu, Gv, S, (const T*)Sh, kk, cpart);
     if ((st = after_launch("eta_lowrank_combine_kernel")) != LRC_OK) return st;

@@ -32,10 +32,11 @@
 // recomputed by a kernel of binary64 FMAs (`repair`).
 //
 // Kernels: row statistics (row_stats_kernel), digits (slice_kernel, which
-// writes them as the product's operand images), the product (product_kernel,
+// writes them as images that either side of a product loads by bulk copies), the product (product_kernel,
 // persistent, one CTA a SM), the ordered sum of split reductions
 // (part_sum_kernel) and the repair (repair_kernel).
 #include <algorithm>
+#include <utility>
 
 #include "split_gemm.cuh"
 #include "tc.cuh"
@@ -101,7 +102,7 @@ struct Job {
     int64_t rows, K, img_rows, kblocks;
     int64_t b0;              // first block
     int64_t kchunk;          // columns a block takes
-    int R, kparts, splits, vec;
+    int kparts, splits, vec;
     int4* stats;             // splits > 0: statistics per slice of K; else slice_kernel takes its own
     unsigned char* img;
     int* exps;
@@ -223,9 +224,7 @@ __device__ __forceinline__ void digits8(const double (&x)[8], const int (&sh)[8]
     }
 }
 
-// Digit images: [row tile][block of 16 columns][digit][R rows x 16 columns in
-// the canonical K-major layout: 8-row x 16-byte core matrices, row groups 128
-// bytes apart, column octets 16 R bytes apart].  A CTA takes 32 image rows
+// Digits into the image (split_gemm.cuh).  A CTA takes 32 image rows
 // and `kchunk` columns (of an operand with a short reduction all of them, and
 // takes the row statistics itself); a lane is a row, so that a warp's 16-byte
 // stores of one digit are four runs of 128 bytes.
@@ -237,7 +236,6 @@ __global__ void __launch_bounds__(256) slice_kernel(const __grid_constant__ Jobs
     const Job& o = job_of(js, blockIdx.x);
     const View64 v = o.v;
     const int64_t rows = o.rows, K = o.K;
-    const int R = o.R;
     const int64_t lb = (int64_t)blockIdx.x - o.b0, rg = lb / o.kparts, kp = lb - rg * o.kparts;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int64_t r0 = rg * 32;
@@ -269,10 +267,8 @@ __global__ void __launch_bounds__(256) slice_kernel(const __grid_constant__ Jobs
     const int64_t r = r0 + lane;
     if (r >= o.img_rows) return;
     const int em = s_em[lane];
-    const int64_t tile = r / R;
-    const int rr = (int)(r - tile * R);
-    const size_t block_bytes = (size_t)kParts64 * R * (kKB * 2);
-    unsigned char* row_base = o.img + (size_t)tile * o.kblocks * block_bytes + (rr >> 3) * 128 + (rr & 7) * 16;
+    const size_t block_bytes = (size_t)(o.img_rows / 8) * kGroupBytes;
+    unsigned char* row_base = o.img + (size_t)(r >> 3) * kGroupBytes + (r & 7) * 16;
     const int64_t o1 = min((kp + 1) * o.kchunk, o.kblocks * kKB) / 8;
     for (int64_t oc = kp * o.kchunk / 8 + warp; oc < o1; oc += 8) {
         double x[8];
@@ -297,10 +293,10 @@ __global__ void __launch_bounds__(256) slice_kernel(const __grid_constant__ Jobs
         for (int j = 0; j < 8; ++j) sh[j] = (v.s.scale && k0 + j < K) ? v.shift(k0 + j) : 0;
         uint32_t w[kParts64][4];
         digits8(x, sh, em < 0 ? 1023 : em, w);
-        unsigned char* dst = row_base + (size_t)(oc >> 1) * block_bytes + (size_t)(oc & 1) * (R * 16);
+        unsigned char* dst = row_base + (size_t)(oc >> 1) * block_bytes + (size_t)(oc & 1) * 128;
 #pragma unroll
         for (int i = 0; i < kParts64; ++i)
-            *reinterpret_cast<uint4*>(dst + (size_t)i * R * (kKB * 2)) = make_uint4(w[i][0], w[i][1], w[i][2], w[i][3]);
+            *reinterpret_cast<uint4*>(dst + i * (8 * kKB * 2)) = make_uint4(w[i][0], w[i][1], w[i][2], w[i][3]);
     }
 }
 
@@ -316,7 +312,8 @@ struct GemmArgs {
     int chunks;              // 64-column chunks of the reduction
     int kblocks;             // 16-column blocks
     int split, group, stages, vec;
-    uint32_t a_bytes, b_bytes;
+    int64_t a_block, b_block;    // bytes of a block of either image
+    uint32_t a_bytes, b_bytes;   // of a tile's part of it
     uint32_t tmem_cols;
 };
 
@@ -472,10 +469,10 @@ __device__ __forceinline__ double round_pq_fp64(int64_t p, int64_t q, int esum) 
 template <int NT, int T0, int T1, int I = 0, int J = (T0 > 0 ? T0 : 0)>
 __device__ __forceinline__ void issue(uint32_t tmem, uint32_t fresh, uint32_t alo, uint32_t ahi, uint32_t blo,
                                       uint32_t bhi) {
-    constexpr int kAPart = 128 * kKB * 2 / 16, kBPart = NT * kKB * 2 / 16;      // one digit
+    constexpr int kPart = 8 * kKB * 2 / 16;                                     // one digit
     constexpr int J0 = T0 > I ? T0 - I : 0, J1 = T1 - I;                        // digits of B for this one of A
     constexpr int kMmaUse = J1 - J0 == 1 ? kNoReuse : J == J0 ? kFill : J == J1 - 1 ? kLast : kUse;
-    mma_f16_col<kMmaUse>(tmem + (I + J) * NT, alo + I * kAPart, ahi, blo + J * kBPart, bhi,
+    mma_f16_col<kMmaUse>(tmem + (I + J) * NT, alo + I * kPart, ahi, blo + J * kPart, bhi,
                           idesc_f16_f32(128, NT) | kIdescBF16, I > 0 ? 1u : ((fresh >> (I + J)) & 1u) ^ 1u);
     if constexpr (J + 1 < J1) issue<NT, T0, T1, I, J + 1>(tmem, fresh, alo, ahi, blo, bhi);
     else if constexpr (I + 1 < T1) issue<NT, T0, T1, I + 1, (T0 > I + 1 ? T0 - I - 1 : 0)>(tmem, fresh, alo, ahi, blo, bhi);
@@ -613,8 +610,8 @@ __global__ void __launch_bounds__(kThreads, 1) product_kernel(const __grid_const
                     if (!(ok = mbar_wait(&empty[slot], phase, abort, err, 1u))) break;
                     unsigned char* dst = ring + (size_t)slot * stage_bytes;
                     mbar_arrive_expect_tx(&full[slot], stage_bytes);
-                    bulk_load(dst, a.A + ((size_t)mt * a.kblocks + kb) * a.a_bytes, a.a_bytes, &full[slot]);
-                    bulk_load(dst + a.a_bytes, a.B + ((size_t)nt * a.kblocks + kb) * a.b_bytes, a.b_bytes, &full[slot]);
+                    bulk_load(dst, a.A + kb * a.a_block + (size_t)mt * a.a_bytes, a.a_bytes, &full[slot]);
+                    bulk_load(dst + a.a_bytes, a.B + kb * a.b_block + (size_t)nt * a.b_bytes, a.b_bytes, &full[slot]);
                     if (++slot == a.stages) {
                         slot = 0;
                         phase ^= 1;
@@ -641,10 +638,10 @@ __global__ void __launch_bounds__(kThreads, 1) product_kernel(const __grid_const
         auto wait = [&](uint64_t* bar, uint32_t parity) {
             return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort, err, 2u)) != 0;
         };
-        const uint32_t ahi = (uint32_t)(smem_desc(0, 2048, 128, 0) >> 32);
-        const uint32_t bhi = (uint32_t)(smem_desc(0, NT * 16, 128, 0) >> 32);
-        const uint32_t alo0 = (uint32_t)smem_desc(smem_u32(ring), 2048, 128, 0);
-        const uint32_t blo0 = (uint32_t)smem_desc(smem_u32(ring) + a.a_bytes, NT * 16, 128, 0);
+        // column octets 128 bytes apart, row groups kGroupBytes
+        const uint64_t ad = smem_desc(smem_u32(ring), 128, kGroupBytes, 0);
+        const uint64_t bd = smem_desc(smem_u32(ring) + a.a_bytes, 128, kGroupBytes, 0);
+        const uint32_t ahi = (uint32_t)(ad >> 32), bhi = (uint32_t)(bd >> 32), alo0 = (uint32_t)ad, blo0 = (uint32_t)bd;
         while (ok && pc.next(a, &tile, &c0, &c1)) {
             for (int c = c0; c < c1 && ok; ++c, ++ch) {
                 const int nb = min(kChunkBlocks, a.kblocks - kChunkBlocks * c);
@@ -829,20 +826,20 @@ lrc_status launch_product(const GemmArgs& a, int64_t grid, size_t smem, cudaStre
 
 }  // namespace
 
-size_t operand_bytes(int64_t rows, int64_t K, int R) {
-    const int64_t tiles = image_tiles(rows, R);
-    return up256((size_t)tiles * image_blocks(K) * kParts64 * R * kKB * 2) + up256((size_t)tiles * R * 4) +
-           up256((size_t)rows * kStatSplits * sizeof(int4)) + up256((size_t)(rows + 1) * 4);
+size_t operand_bytes(int64_t rows, int64_t K) {
+    const int64_t ir = image_rows(rows);
+    return up256((size_t)(ir / 8) * image_blocks(K) * kGroupBytes) + up256((size_t)ir * 4) +
+           up256((size_t)rows * (K > kOwnStatsK ? kStatSplits : 0) * sizeof(int4)) + hard_bytes(rows);
 }
 
 void operand_carve(Operand64* o, unsigned char* ws) {
-    const int64_t tiles = image_tiles(o->rows, o->R);
+    const int64_t ir = image_rows(o->rows);
     o->img = ws;
-    ws += up256((size_t)tiles * image_blocks(o->K) * kParts64 * o->R * kKB * 2);
+    ws += up256((size_t)(ir / 8) * image_blocks(o->K) * kGroupBytes);
     o->exps = reinterpret_cast<int*>(ws);
-    ws += up256((size_t)tiles * o->R * 4);
+    ws += up256((size_t)ir * 4);
     o->stats = reinterpret_cast<int4*>(ws);
-    ws += up256((size_t)o->rows * kStatSplits * sizeof(int4));
+    ws += up256((size_t)o->rows * (o->K > kOwnStatsK ? kStatSplits : 0) * sizeof(int4));
     o->hard = reinterpret_cast<int*>(ws);
 }
 
@@ -855,8 +852,7 @@ lrc_status slice(const Operand64* const* ops, int count, cudaStream_t s) {
         j.v = View64{o.src};
         j.rows = o.rows;
         j.K = o.K;
-        j.R = o.R;
-        j.img_rows = image_tiles(o.rows, o.R) * o.R;
+        j.img_rows = image_rows(o.rows);
         j.kblocks = image_blocks(o.K);
         j.vec = o.src.cs == 1 && o.src.rs % 2 == 0 && aligned16(o.src.p);
         j.stats = o.stats;
@@ -900,14 +896,32 @@ lrc_status slice(const Operand64* const* ops, int count, cudaStream_t s) {
     return after_launch("slice_kernel");
 }
 
-size_t part_bytes(int64_t M, int64_t N, int64_t K, int R_b) {
-    (void)K;
-    const int64_t tiles = image_tiles(M, 128) * image_tiles(N, R_b);
-    return up256((size_t)(tiles + sm_count()) * 128 * R_b * 8);
+namespace {
+
+int64_t n_tiles(int64_t rows) { return (rows + n_tile(rows) - 1) / n_tile(rows); }
+
+// Tiles of a product with M rows on the first side; the side whose tiles waste
+// less goes there.
+int64_t tiles_of(int64_t M, int64_t N) { return (M + 127) / 128 * n_tiles(N); }
+
+}  // namespace
+
+size_t part_bytes(int64_t M, int64_t N) {
+    if (tiles_of(N, M) < tiles_of(M, N)) std::swap(M, N);
+    return up256((size_t)(tiles_of(M, N) + sm_count()) * 128 * n_tile(N) * 8);
 }
 
-lrc_status product(const Operand64& A, const Operand64& B, const Out64& out, bool split, double* part, cudaStream_t s) {
-    const int NT = B.R;
+lrc_status product(const Operand64& A0, const Operand64& B0, const Out64& out0, bool split, double* part,
+                   cudaStream_t s) {
+    const bool swap = tiles_of(B0.rows, A0.rows) < tiles_of(A0.rows, B0.rows);
+    const Operand64& A = swap ? B0 : A0;
+    const Operand64& B = swap ? A0 : B0;
+    Out64 out = out0;
+    if (swap) {
+        std::swap(out.cr, out.cc);
+        std::swap(out.rscale, out.cscale);
+    }
+    const int NT = n_tile(B.rows);
     GemmArgs a{};
     a.A = A.img;
     a.B = B.img;
@@ -918,18 +932,20 @@ lrc_status product(const Operand64& A, const Operand64& B, const Out64& out, boo
     a.cc = out.cc;
     a.M = A.rows;
     a.N = B.rows;
-    const int64_t tiles = image_tiles(A.rows, 128) * image_tiles(B.rows, NT);
+    const int64_t tiles = tiles_of(A.rows, B.rows);
     if (tiles > 0x3fffffff || A.K > kMaxK) {
         set_error("split product too large (%lld tiles, reduction of %lld)", (long long)tiles, (long long)A.K);
         return LRC_ERR_UNSUPPORTED;
     }
-    a.ntiles = (int)image_tiles(B.rows, NT);
+    a.ntiles = (int)n_tiles(B.rows);
     a.tiles = (int)tiles;
     a.kblocks = (int)image_blocks(A.K);
     a.chunks = (a.kblocks + kChunkBlocks - 1) / kChunkBlocks;
     a.split = split;
-    a.a_bytes = kParts64 * 128 * kKB * 2;
-    a.b_bytes = (uint32_t)(kParts64 * NT * kKB * 2);
+    a.a_block = image_rows(A.rows) / 8 * kGroupBytes;
+    a.b_block = image_rows(B.rows) / 8 * kGroupBytes;
+    a.a_bytes = 128 / 8 * kGroupBytes;
+    a.b_bytes = (uint32_t)(NT / 8 * kGroupBytes);
     a.stages = (int)std::min<int64_t>(8, (int64_t)(227 * 1024 - kCtrlBytes) / (a.a_bytes + a.b_bytes));
     a.vec = out.cc != 1 || out.cr % 2 != 0 || !aligned16(out.C) ? 0
             : out.cr % 4 == 0 && (reinterpret_cast<uintptr_t>(out.C) & 31u) == 0 ? 2 : 1;

@@ -12,8 +12,8 @@ constexpr int kKB = 16;            // columns of the reduction per image block
 constexpr int64_t kMaxK = 1 << 20; // longest reduction the 64-bit sums hold
 constexpr int kStatSplits = 32;    // most slices of the reduction in the row statistics
 
-// Rows a digit image is tiled by: 128 for the first operand; for the second
-// the rows split evenly over tiles of at most kNTMax rows, a multiple of 16.
+// Tiles of the product: 128 rows of the first side, and of the second the rows
+// split evenly over tiles of at most kNTMax, a multiple of 16.
 constexpr int kNTMax = 64;
 inline int n_tile(int64_t rows) {
     const int64_t tiles = (rows + kNTMax - 1) / kNTMax;
@@ -33,11 +33,13 @@ struct Src64 {
     int sign;
 };
 
-// One operand of a product.  `rows` x K; tiles of R rows.
+// One operand of a product, `rows` x K, and its digits.  The image is
+// [block of kKB columns][group of 8 rows][digit][column octet][8 rows x 16
+// bytes]: the blocks of any run of row groups are contiguous, so the same image
+// serves as either side of a product, with tiles of any height.
 struct Operand64 {
     Src64 src;
     int64_t rows, K;
-    int R;
     unsigned char* img;      // digits
     int* exps;               // exponent of every row (image rows)
     int4* stats;             // row statistics per slice of K
@@ -46,17 +48,20 @@ struct Operand64 {
 };
 constexpr int kMaxOps = 3;   // operands per slice()
 
-inline int64_t image_tiles(int64_t rows, int R) { return (rows + R - 1) / R; }
+constexpr int kGroupBytes = kParts64 * 8 * kKB * 2;      // one row group of one block
+inline int64_t image_rows(int64_t rows) { return (rows + 127) / 128 * 128; }
 inline int64_t image_blocks(int64_t K) { return (K + kKB - 1) / kKB; }
-size_t operand_bytes(int64_t rows, int64_t K, int R);
-// Carves an operand's buffers out of `ws` (256-byte aligned).
+size_t operand_bytes(int64_t rows, int64_t K);
+// Carves an operand's buffers out of `ws` (256-byte aligned); its row list is
+// the last part, hard_bytes() of it.
 void operand_carve(Operand64* o, unsigned char* ws);
+inline size_t hard_bytes(int64_t rows) { return ((size_t)(rows + 1) * 4 + 255) & ~(size_t)255; }
 
 // Digits of up to kMaxOps operands (at most two launches for all of them).
 lrc_status slice(const Operand64* const* ops, int count, cudaStream_t s);
 
 // C(i, j) at C[i cr + j cc], i < A.rows, j < B.rows: the product A B^T times
-// rscale[i] cscale[j] (each may be null).  `split` splits the reduction over
+// rscale[i] cscale[j] (each may be null, and both are with `split` false).  `split` splits the reduction over
 // the CTAs (few, deep tiles); its partial sums are added in a fixed order.
 // `part` holds part_bytes() bytes.  Rows that the digits cannot carry are
 // recomputed with binary64 FMAs.
@@ -67,7 +72,7 @@ struct Out64 {
     const double* cscale;
     int* clear = nullptr;    // a later operand's hard[0], set to 0 on the way (split only)
 };
-size_t part_bytes(int64_t M, int64_t N, int64_t K, int R_b);
+size_t part_bytes(int64_t M, int64_t N);
 lrc_status product(const Operand64& A, const Operand64& B, const Out64& out, bool split, double* part, cudaStream_t s);
 
 }  // namespace sg

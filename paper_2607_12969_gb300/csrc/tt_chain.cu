@@ -17,7 +17,10 @@
 // workspace (two buffers per side, alternating).
 #include <math.h>
 
+#include <vector>
+
 #include "common.cuh"
+#include "split_gemm.cuh"
 
 namespace lrc {
 
@@ -147,6 +150,93 @@ lrc_status launch_tt_chain_f32tc(const TTShape& sh, float* out, cudaStream_t s) 
 
 lrc_status launch_tt_chain_f64(const TTShape& sh, double* out, cudaStream_t s) {
     return launch_chain<double>(sh, out, s);
+}
+
+// The binary64 chain with every product on the tensor cores (split_gemm.cu).
+// Both operands of a product are cut into digits first: rows of Z, columns of
+// the core (or of S).
+lrc_status launch_tt_chain_f64_tc(const TTShape& sh, double* out, cudaStream_t s, bool* handled) {
+    *handled = false;
+    const int d = sh.d, c = plan_chain(sh).c;
+    const double* const* G = reinterpret_cast<const double* const*>(sh.cores);
+    struct Step {
+        const double* A;
+        const double* B;
+        double* C;
+        int64_t M, N, K;
+        sg::Operand64 a, b;
+        size_t oa, ob, oc;
+    };
+    std::vector<Step> steps;
+    size_t off = 0;
+    auto take = [&](size_t bytes) {
+        const size_t o = off;
+        off += round256(bytes);
+        return o;
+    };
+    // A is M x K, B is K x N, both row-major (null: the step before's C on that side)
+    auto add = [&](const double* A, const double* B, int64_t M, int64_t N, int64_t K, bool last) {
+        Step t{A, B, nullptr, M, N, K, {}, {}, 0, 0, 0};
+        t.a.rows = M;
+        t.b.rows = N;
+        t.a.K = t.b.K = K;
+        t.oa = take(sg::operand_bytes(M, K) - sg::hard_bytes(M));
+        t.ob = take(sg::operand_bytes(N, K) - sg::hard_bytes(N));
+        t.oc = last ? 0 : take((size_t)M * (size_t)N * 8);
+        steps.push_back(t);
+    };
+    int64_t P = sh.dims[0], Q = sh.dims[d - 1];
+    for (int j = 1; j <= c - 1; ++j) {
+        add(j == 1 ? G[0] : nullptr, G[j], P, sh.dims[j] * sh.ranks[j + 1], sh.ranks[j], false);
+        P *= sh.dims[j];
+    }
+    const int left = (int)steps.size();
+    for (int j = d - 2; j >= c; --j) {
+        add(G[j], j == d - 2 ? G[d - 1] : nullptr, sh.ranks[j] * sh.dims[j], Q, sh.ranks[j + 1], false);
+        Q *= sh.dims[j];
+    }
+    const int right = (int)steps.size();
+    add(left ? nullptr : G[0], right > left ? nullptr : G[d - 1], P, Q, sh.ranks[c], true);
+    // the row lists of all operands side by side, emptied at once
+    const size_t o_hard = off;
+    for (const Step& t : steps) off += sg::hard_bytes(t.M) + sg::hard_bytes(t.N);
+    void* p = nullptr;
+    lrc_status st = stream_workspace_try(s, off, &p);
+    if (st != LRC_OK || !p) return st;
+    *handled = true;
+    unsigned char* ws = static_cast<unsigned char*>(p);
+    cudaError_t e = cudaMemsetAsync(ws + o_hard, 0, off - o_hard, s);
+    if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync (row lists)");
+    size_t hard = o_hard;
+    for (int i = 0; i < (int)steps.size(); ++i) {
+        Step& t = steps[i];
+        const bool last = i + 1 == (int)steps.size();
+        const double* A = t.A ? t.A : (last ? steps[left - 1].C : steps[i - 1].C);
+        const double* B = t.B ? t.B : (last ? steps[right - 1].C : steps[i - 1].C);
+        t.C = last ? out : reinterpret_cast<double*>(ws + t.oc);
+        sg::operand_carve(&t.a, ws + t.oa);
+        sg::operand_carve(&t.b, ws + t.ob);
+        t.a.hard = reinterpret_cast<int*>(ws + hard);
+        hard += sg::hard_bytes(t.M);
+        t.b.hard = reinterpret_cast<int*>(ws + hard);
+        hard += sg::hard_bytes(t.N);
+        t.a.cleared = t.b.cleared = true;
+        t.a.src = sg::Src64{A, t.K, 1, nullptr, 0};
+        t.b.src = sg::Src64{B, 1, t.N, nullptr, 0};
+        const sg::Operand64* ops[2] = {&t.a, &t.b};
+        if ((st = sg::slice(ops, 2, s)) != LRC_OK) return st;
+        if ((st = sg::product(t.a, t.b, sg::Out64{t.C, t.N, 1, nullptr, nullptr}, false, nullptr, s)) != LRC_OK)
+            return st;
+    }
+    return LRC_OK;
+}
+
+// Where the digits' fixed cost (three launches a product, about 20 us a chain)
+// pays: the FMA kernels take about 1 us per 1e6 flops (256^3, rank 34: 1.2e9
+// flops, 1.1 ms -> 0.15 ms).
+bool tt_chain_f64_tc_takes(const TTShape& sh) {
+    constexpr double kTTDigitFlops = 4e7;
+    return plan_chain(sh).flops >= kTTDigitFlops;
 }
 
 bool tt_chain_saves(const TTShape& sh) { return plan_chain(sh).flops <= 0.8 * chain_flops(sh, sh.d - 1); }

@@ -1,5 +1,6 @@
-"""binary64 products on the tensor cores (split_gemm.cu): values cut into
-seven 9-bit digits, 28 exact digit products, one rounding.
+"""binary64 products on the tensor cores (split_gemm.cu; the apply, the TT
+chain, the Gram matrices of eta): values cut into seven 9-bit digits, 28 exact
+digit products, one rounding.
 
 Integer data whose sums stay below 2^53 must come out exactly, whatever the
 tiling; rows that the digits cannot carry (wide ranges, infinities, NaN,
@@ -113,3 +114,55 @@ def test_captured_call_and_repeat_are_the_same_bits(lrc, cuda):
     g.replay()
     torch.cuda.synchronize()
     assert torch.equal(Y.view(torch.int64), want.view(torch.int64))
+
+
+TT_SHAPES = [((130, 70, 90), (1, 20, 33, 1)), ((16, 16, 16, 16), (1, 16, 24, 16, 1)), ((300, 40, 129), (1, 7, 64, 1)),
+             ((64, 2000), (1, 65, 1)), ((33, 17, 29, 31), (1, 30, 40, 20, 1))]
+
+
+@pytest.mark.parametrize("dims,ranks", TT_SHAPES)
+def test_tt_chain(lrc, cuda, dims, ranks):
+    """Integer cores come out exactly; Gaussian ones within a few roundings of
+    the chain's products of absolute values."""
+    rng = np.random.default_rng(len(dims))
+    d = len(dims)
+    for integer in (True, False):
+        cores = [rng.integers(-9, 10, (ranks[l], dims[l], ranks[l + 1])).astype(np.float64) if integer
+                 else rng.standard_normal((ranks[l], dims[l], ranks[l + 1])) for l in range(d)]
+        dev = [torch.from_numpy(c).to(cuda) for c in cores]
+        out = torch.empty(int(np.prod(dims)), dtype=torch.float64, device=cuda)
+        lrc.tt_reconstruct(dev, dims, ranks, "f64", out)
+        torch.cuda.synchronize()
+        assert lrc.lrc_device_status() == 0
+
+        def chain(cs):
+            z = cs[0].reshape(dims[0], -1)
+            for c in cs[1:]:
+                z = (z @ c.reshape(c.shape[0], -1)).reshape(-1, c.shape[2])
+            return z.reshape(-1)
+        want = chain(cores)
+        got = out.cpu().numpy()
+        if integer:
+            assert np.array_equal(got, want)
+        else:
+            bound = chain([np.abs(c) for c in cores])
+            assert np.all(np.abs(got - want) <= (sum(ranks) + 2 * d) * U64 * bound)
+
+
+@pytest.mark.parametrize("fmt", ["f16", "f32"])
+@pytest.mark.parametrize("m,n,k", [(1500, 700, 65), (300, 2100, 130), (20000, 400, 32)])
+def test_eta_through_digit_gram_matrices(lrc, cuda, fmt, m, n, k):
+    f = W.random_factors(m, n, k, seed=21)
+    wide = [packed(lrc, a, "f64", cuda) for a in (f.U, f.s, f.Vt)]
+    low = [packed(lrc, a, fmt, cuda) for a in (f.U, f.s, f.Vt)]
+    eta, norm = lrc.lrc_lowrank_eta(*wide, *low, fmt, m, n, k)
+    L = np.longdouble
+    Uh, sh, Vh = (oracle.rounded(a, fmt).astype(L) for a in (f.U, f.s, f.Vt))
+    U, s, Vt = (a.astype(L) for a in (f.U, f.s, f.Vt))
+    Pu, Pv = np.hstack([U - Uh, Uh]), np.vstack([Vt - Vh, Vh])
+    M = np.zeros((2 * k, 2 * k), L)
+    i = np.arange(k)
+    M[i, i], M[i, k + i], M[k + i, i], M[k + i, k + i] = s, s, s, s - sh
+    want = np.sqrt(np.sum((M.T @ (Pu.T @ Pu) @ M) * (Pv @ Pv.T)))
+    assert abs(eta - float(want)) <= 1e-13 * float(want)
+    assert abs(norm - float(np.linalg.norm(f.s))) <= 1e-12 * norm or k > min(m, n)
