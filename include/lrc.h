@@ -58,7 +58,9 @@ typedef enum {
     LRC_F64 = 0,      /* binary64 storage and output; binary64 FMAs, or on larger problems
                          exact products of 9-bit digits on the tensor cores rounded to
                          binary64 once (no less accurate; see lrc_apply)                    */
-    LRC_F32 = 1,      /* binary32 storage, binary32 FMA arithmetic, binary32 output         */
+    LRC_F32 = 1,      /* binary32 storage and output; binary32 FMAs, or in larger applies
+                         products of three bfloat16 parts of every operand on the tensor
+                         cores, accumulated in binary32 (no less accurate)                   */
     LRC_F16 = 2,      /* binary16 storage, binary32 accumulation, binary32 output           */
     LRC_F16_O16 = 3,  /* binary16 storage, binary32 accumulation, binary16 workspaces and
                          output: the method-precision FP16 path of Sec. 3.4                 */
@@ -173,8 +175,14 @@ LRC_API lrc_status lrc_widen_factors(const void* src, lrc_fmt fmt, int64_t rows,
  * not take the call (more than 64 queries, n > 32768), else
  * LRC_ERR_UNSUPPORTED.
  */
-/* LRC_F32_TC: as LRC_F32, with the second product (W U^T) on the tensor
- * cores when b > 32 and k <= 192; otherwise the LRC_F32 kernels. */
+/* LRC_F32: larger problems form both products from bfloat16 parts (x = hi +
+ * mid + lo exactly; the six largest of the nine products of parts, which leaves
+ * out 2^-26 of a term); a row that holds a nonzero entry outside 2^-100 ...
+ * 2^126, an infinity or a NaN is formed by binary32 FMAs.  The parts (6 bytes
+ * an element, of at most 1 GiB of queries at a time) live in the stream's
+ * workspace; without it (see above) the FMA kernels run.
+ * LRC_F32_TC: the same; on smaller problems as LRC_F32 with the second product
+ * (W U^T) on the tensor cores when b > 32 and k <= 192. */
 LRC_API lrc_status lrc_apply(const void* U, const void* S, const void* Vt, const void* X, void* Y,
                      int64_t m, int64_t n, int64_t k, int64_t b, lrc_fmt fmt,
                      lrc_stream_t stream);

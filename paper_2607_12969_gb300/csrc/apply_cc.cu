@@ -28,7 +28,7 @@
 // reduce_scale_f32_kernel, which also applies diag(s)), phase 2 over
 // 128 x 128 tiles of Y.  W (b x k') passes through the stream's workspace.
 //
-// LRC_F32_TC (a variant): phase 2 on the tensor cores.  W (per row: queries
+// LRC_F32_TC (a variant): on those smaller problems phase 2 on the tensor cores.  W (per row: queries
 // may differ in magnitude by any factor) and U (per 32 rows) are scaled by
 // powers of two that bring each group's largest magnitude into [2^14, 2^15)
 // and split into binary16 parts hi = fp16(x), lo = fp16(x - hi)
@@ -41,6 +41,7 @@
 
 #include "common.cuh"
 #include "split_gemm.cuh"
+#include "split_gemm32.cuh"
 #include "tc.cuh"
 
 namespace lrc {
@@ -570,8 +571,84 @@ lrc_status launch_apply_f64(const double* U, const double* S, const double* Vt, 
     return launch_apply_cc<double>(U, S, Vt, X, Y, m, n, k, b, s, "apply_cc_kernel<f64>");
 }
 
+// binary32 applies whose products run on the tensor cores (split_gemm32.cu):
+// where the parts' fixed cost (eight launches and their images) pays.  Measured,
+// parts / FMA kernels: 1138^2, k = 41, b = 1024 (9.5e7) 40 / 31 us and b = 8192
+// (7.6e8) 73 / 99 us; 16384 x 600, k = 40, b = 256 (1.7e8) 38 / 31 us and b =
+// 1024 47 / 64 us; 2048^2, k = 136, b = 256 (1.4e8) 41 / 39 us; with a long
+// reduction earlier: 600 x 16384, k = 40, b = 256 50 / 87 us, 16384^2, k = 272,
+// b = 20 (1.8e8) 75 / 92 us.
+static bool apply_f32_tc_takes(int64_t m, int64_t n, int64_t k, int64_t b) {
+    if (n >= (1ll << 30) || k > 4096 || m >= (1ll << 31) || b >= (1ll << 31)) return false;
+    const double work = (double)(m + n) * (double)k * (double)b;
+    return work >= (n >= 4096 ? 1e8 : 2.2e8);
+}
+
+// *handled = false: no workspace for the parts (nothing launched).
+static lrc_status launch_apply_f32_tc(const float* U, const float* S, const float* Vt, const float* X, float* Y,
+                                      int64_t m, int64_t n, int64_t k, int64_t b, cudaStream_t s, bool* handled) {
+    *handled = false;
+    const int64_t ldn = lrc_packed_ld(n), ldk = lrc_packed_ld(k);
+    // queries in panels of whole tiles, whose images stay below kPanelBytes
+    int64_t pb = kPanelBytes / (sg32::kParts * 2 * sg32::kKB * sg32::image_blocks(n)) / 256 * 256;
+    if (pb < 256) pb = 256;
+    if (pb > b) pb = b;
+    sg32::Operand oV{Vt, ldn, 1, k, n, nullptr, nullptr}, oU{U, ldk, 1, m, k, nullptr, nullptr};
+    sg32::Operand oX{X, ldn, 1, pb, n, nullptr, nullptr}, oW{nullptr, ldk, 1, pb, k, nullptr, nullptr};
+    size_t off = 0;
+    auto take = [&](size_t bytes) {
+        const size_t o = off;
+        off += (bytes + 255) & ~(size_t)255;
+        return o;
+    };
+    const size_t o_v = take(sg32::image_bytes(k, n)), o_u = take(sg32::image_bytes(m, k));
+    const size_t o_x = take(sg32::image_bytes(pb, n)), o_w = take(sg32::image_bytes(pb, k));
+    const size_t o_wd = take((size_t)pb * ldk * 4);
+    size_t pbytes = sg32::part_bytes(pb, k);
+    if (b % pb && sg32::part_bytes(b % pb, k) > pbytes) pbytes = sg32::part_bytes(b % pb, k);     // the last panel
+    const size_t o_p = take(pbytes);
+    const size_t o_h = off;                                  // row lists: V, U, then X and W of a panel
+    const size_t h_vu = sg32::hard_bytes(k) + sg32::hard_bytes(m), h_xw = 2 * sg32::hard_bytes(pb);
+    off += h_vu + h_xw;
+    void* ws = nullptr;
+    lrc_status st = stream_workspace_try(s, off, &ws);
+    if (st != LRC_OK || !ws) return st;
+    *handled = true;
+    unsigned char* base = static_cast<unsigned char*>(ws);
+    float* W = reinterpret_cast<float*>(base + o_wd);
+    float* part = reinterpret_cast<float*>(base + o_p);
+    oV.img = base + o_v;
+    oU.img = base + o_u;
+    oX.img = base + o_x;
+    oW.img = base + o_w;
+    oW.p = W;
+    oV.hard = reinterpret_cast<int*>(base + o_h);
+    oU.hard = reinterpret_cast<int*>(base + o_h + sg32::hard_bytes(k));
+    oX.hard = reinterpret_cast<int*>(base + o_h + h_vu);
+    oW.hard = reinterpret_cast<int*>(base + o_h + h_vu + sg32::hard_bytes(pb));
+    for (int64_t r0 = 0; r0 < b; r0 += pb) {
+        oX.p = X + r0 * ldn;
+        oX.rows = oW.rows = b - r0 < pb ? b - r0 : pb;
+        const size_t skip = r0 ? h_vu : 0;
+        const cudaError_t e = cudaMemsetAsync(base + o_h + skip, 0, h_vu + h_xw - skip, s);
+        if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync (row lists)");
+        const sg32::Operand* px[3] = {&oX, &oV, &oU};      // V and U with the first panel
+        const sg32::Operand* pw[1] = {&oW};
+        if ((st = sg32::split(px, r0 == 0 ? 3 : 1, s)) != LRC_OK) return st;
+        if ((st = sg32::product(oX, oV, W, ldk, S, true, part, s)) != LRC_OK) return st;
+        if ((st = sg32::split(pw, 1, s)) != LRC_OK) return st;
+        if ((st = sg32::product(oW, oU, Y + r0 * m, m, nullptr, false, nullptr, s)) != LRC_OK) return st;
+    }
+    return LRC_OK;
+}
+
 lrc_status launch_apply_f32(const float* U, const float* S, const float* Vt, const float* X,
                             float* Y, int64_t m, int64_t n, int64_t k, int64_t b, bool tc, cudaStream_t s) {
+    if (apply_f32_tc_takes(m, n, k, b)) {
+        bool handled = false;
+        const lrc_status st = launch_apply_f32_tc(U, S, Vt, X, Y, m, n, k, b, s, &handled);
+        if (st != LRC_OK || handled) return st;
+    }
     if (b <= kSplitMaxBatchF32 && k <= kSplitMaxRank) return launch_apply_split_f32(U, S, Vt, X, Y, m, n, k, b, s);
     // phase 1: partial products of W = X V over n-splits, with V = (V^T)^T read
     // from the stored V^T rows; phase 2 after the ordered reduction and diag(s)

@@ -212,6 +212,7 @@ lrc_status launch_ttn_f16_tc(const TTShape& sh, bool out16, void* out, cudaStrea
 uint32_t take_ttn_tc_error();
 uint32_t take_skinny_error();
 uint32_t take_split_error();
+uint32_t take_split32_error();
 lrc_status launch_wait_timeout_probe(int64_t limit_ns, cudaStream_t s);
 
 lrc_status run_fro_diff(const void* A, lrc_fmt fa, const void* B, lrc_fmt fb, int64_t count,

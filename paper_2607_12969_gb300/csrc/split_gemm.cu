@@ -39,6 +39,7 @@
 #include <utility>
 
 #include "split_gemm.cuh"
+#include "split_pieces.cuh"
 #include "tc.cuh"
 
 namespace lrc {
@@ -317,51 +318,6 @@ struct GemmArgs {
     uint32_t tmem_cols;
 };
 
-// The (tile, chunk range) pieces of a CTA, in order.  A split reduction is cut
-// over groups of `group` CTAs, one per tile of B: a group walks one range of
-// (tile of A, chunk), laid end to end, so that its CTAs read the same blocks of
-// A at about the same time and only the first read comes from HBM.
-struct Pieces {
-    int left, t, c, step;      // split: chunks left, first chunk of the next piece
-    __device__ explicit Pieces(const GemmArgs& a) {
-        if (a.split) {
-            const int groups = gridDim.x / a.group, gi = blockIdx.x / a.group;
-            const int64_t Q = (int64_t)(a.tiles / a.group) * a.chunks;
-            const int64_t q0 = Q * gi / groups, q1 = Q * (gi + 1) / groups;
-            const int mt = (int)(q0 / a.chunks);
-            t = mt * a.group + (int)(blockIdx.x - gi * a.group);
-            c = (int)(q0 - (int64_t)mt * a.chunks);
-            left = (int)(q1 - q0);
-            step = a.group;
-        } else {
-            t = blockIdx.x;
-            c = 0;
-            step = gridDim.x;
-            left = t < a.tiles ? 1 : 0;
-        }
-    }
-    // false: no piece left
-    __device__ bool next(const GemmArgs& a, int* tile, int* c0, int* c1) {
-        if (left <= 0) return false;
-        *tile = t;
-        *c0 = c;
-        *c1 = a.chunks;
-        t += step;
-        if (a.split) {
-            *c1 = min(a.chunks, c + left);
-            left -= *c1 - c;
-            c = 0;
-        } else {
-            left = t < a.tiles ? 1 : 0;
-        }
-        return true;
-    }
-};
-// Partial tile of a piece: distinct for every (group, tile).
-__device__ __forceinline__ int64_t part_slot(const GemmArgs& a, int tile) {
-    return (int64_t)(blockIdx.x / a.group) * a.group + tile;
-}
-
 // Sixteen epilogue warps, four per quarter of the tensor-memory lanes, each
 // with a quarter of the columns: with eight, two a scheduler, the drain's and
 // the rounding's dependent steps were not covered (a 128 x 64 tile of two
@@ -521,7 +477,7 @@ __global__ void __launch_bounds__(kThreads, 1) product_kernel(const __grid_const
         const int g = warp & 3, quarter = (warp - 4) >> 2;      // of the lanes, of the columns
         const uint32_t tbase = tmem + ((uint32_t)(g * 32) << 16) + quarter * HC;
         const int r = g * 32 + lane;
-        Pieces pc(a);
+        Pieces<GemmArgs> pc(a);
         int tile, c0, c1;
         int ch = 0;
         bool ok = true;
@@ -598,7 +554,7 @@ __global__ void __launch_bounds__(kThreads, 1) product_kernel(const __grid_const
         if (warp == 0) {
         // ------------------------------------------------------------ producer
         if (lane == 0) {
-            Pieces pc(a);
+            Pieces<GemmArgs> pc(a);
             int tile, c0, c1;
             int it = 0, slot = 0;
             uint32_t phase = 1;
@@ -629,7 +585,7 @@ __global__ void __launch_bounds__(kThreads, 1) product_kernel(const __grid_const
         // The whole warp walks the loop and waits; one lane issues, in one branch
         // per block (with a branch or an election per MMA the warp, which shares
         // its scheduler with busy epilogue warps, issued one in 49 to 100 clocks).
-        Pieces pc(a);
+        Pieces<GemmArgs> pc(a);
         int tile, c0, c1;
         int slot = 0, ch = 0;
         uint32_t phase = 0;            // parity of the ring's current pass
@@ -706,10 +662,6 @@ __global__ void __launch_bounds__(kThreads, 1) product_kernel(const __grid_const
 }
 
 // The partial tiles of a split reduction, added in the order of the groups.
-__host__ __device__ __forceinline__ int64_t group_of_chunk(int64_t u, int64_t Q, int64_t G) {
-    return ((u + 1) * G + Q - 1) / Q - 1;
-}
-
 __global__ void __launch_bounds__(256) part_sum_kernel(const double* __restrict__ part, int NT, int64_t ntiles,
                                                        int64_t chunks, int64_t Q, int64_t G, int group,
                                                        double* __restrict__ C, int64_t cr, int64_t cc, int64_t M,

@@ -1,0 +1,110 @@
+"""binary32 products on the tensor cores (split_gemm32.cu): three bfloat16
+parts of every value, six products of parts.
+
+Integer data whose sums stay below 2^24 must come out exactly, whatever the
+tiling; rows with entries that the parts cannot carry go through binary32 FMAs
+and must come out as they do."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import workloads as W
+from parity import packed
+
+pytestmark = pytest.mark.gpu
+
+U32 = 2.0 ** -24
+
+
+def run(lrc, dev, U, s, Vt, X, fmt="f32"):
+    m, k = U.shape
+    n, b = Vt.shape[1], X.shape[0]
+    ops = [packed(lrc, a, fmt, dev) for a in (U, s, Vt, X)]
+    Y = torch.full((b, m), float("nan"), dtype=torch.float32, device=dev)
+    lrc.lrc_apply(*ops, Y, m, n, k, b, fmt)
+    torch.cuda.synchronize()
+    assert lrc.lrc_device_status() == 0
+    return Y.double().cpu().numpy()
+
+
+# row and column tiles' edges, output rows with and without a 16-byte pitch,
+# reductions of one block, a partial chunk, past one drain of the lower products
+SHAPES = [(300, 7777, 33, 520), (129, 4100, 65, 380), (4097, 4096, 16, 900), (1000, 1030, 129, 900), (256, 16384, 40, 200),
+          (2050, 5000, 17, 1025), (515, 4099, 272, 128)]
+
+
+@pytest.mark.parametrize("m,n,k,b", SHAPES)
+def test_integers_are_exact(lrc, cuda, m, n, k, b):
+    rng = np.random.default_rng(m + n)
+    X = rng.integers(-1, 2, (b, n)).astype(np.float64) * (rng.random((b, n)) < 0.05) * 17
+    Vt = rng.integers(-3, 4, (k, n)).astype(np.float64)
+    U = rng.integers(-2, 3, (m, k)).astype(np.float64) * (rng.random((m, k)) < 0.2)
+    s = rng.integers(0, 2, k).astype(np.float64)
+    W1 = X @ Vt.T
+    want = (W1 * s) @ U.T
+    assert max(np.max(np.abs(X) @ np.abs(Vt).T), np.max((np.abs(W1) * s) @ np.abs(U).T)) < 2.0 ** 24
+    assert np.array_equal(run(lrc, cuda, U, s, Vt, X), want)
+
+
+@pytest.mark.parametrize("fmt", ["f32", "f32tc"])
+@pytest.mark.parametrize("m,n,k,b", SHAPES)
+def test_no_further_from_the_exact_product_than_fma_sums(lrc, cuda, m, n, k, b, fmt):
+    """A sum of K binary32 FMAs in blocks of 1024 is off by about 0.2 sqrt(1024)
+    roundings of random sign; allow 8 u relative Frobenius (n + k terms)."""
+    f = W.random_factors(m, n, k, seed=7)
+    X = W.gaussian((b, n), 8)
+    U, s, Vt, X = (oracle.rounded(a, "f32") for a in (f.U, f.s, f.Vt, X))
+    want = ((X @ Vt.T) * s) @ U.T
+    got = run(lrc, cuda, U, s, Vt, X, fmt)
+    assert np.linalg.norm(got - want) <= 8 * U32 * np.linalg.norm(want)
+
+
+def test_rows_the_parts_cannot_carry(lrc, cuda):
+    m, n, k, b = 300, 4100, 64, 520
+    f = W.random_factors(m, n, k, seed=9)
+    X = W.gaussian((b, n), 10)
+    U, Vt = f.U.copy(), f.Vt.copy()
+    X[3] *= 2.0 ** -110
+    X[4] = 0.0
+    X[5, 7] = 2.0 ** 127
+    X[6, 9] = 2.0 ** -140
+    U[17, 3] = 2.0 ** -130
+    Vt[2] *= 2.0 ** -20
+    U, s, Vt, X = (oracle.rounded(a, "f32") for a in (U, f.s, Vt, X))
+    got = run(lrc, cuda, U, s, Vt, X)
+    want = oracle.apply(U, s, Vt, X)
+    bound = ((np.abs(X) @ np.abs(Vt).T) * np.abs(s)) @ np.abs(U).T
+    assert np.all(np.abs(got - want) <= 64 * U32 * bound + 2.0 ** -140)
+
+
+@pytest.mark.parametrize("v", [np.inf, -np.inf, np.nan, 3.0e38])
+def test_nonfinite_values_spread_as_in_fma_sums(lrc, cuda, v):
+    m, n, k, b = 200, 4300, 64, 400
+    f = W.random_factors(m, n, k, seed=12)
+    X = W.gaussian((b, n), 13)
+    U = f.U.copy()
+    X[7, 5] = v
+    U[9, 2] = v
+    U, s, Vt, X = (oracle.rounded(a, "f32") for a in (U, f.s, f.Vt, X))
+    got = run(lrc, cuda, U, s, Vt, X)
+    with np.errstate(invalid="ignore", over="ignore"):
+        want = (((X @ Vt.T).astype(np.float32) * s.astype(np.float32)).astype(np.float64) @ U.T).astype(np.float32).astype(np.float64)
+    if np.isfinite(v):          # sums near the end of the range: only their neighbours are compared
+        keep = np.ones(b, bool)
+        keep[7] = False
+        ok = np.isfinite(want) & keep[:, None]
+    else:
+        assert np.array_equal(np.isnan(got), np.isnan(want))
+        inf = np.isinf(want)
+        assert np.array_equal(got[inf], want[inf])
+        ok = np.isfinite(want)
+    ok[:, 9] = False
+    assert np.linalg.norm(got[ok] - want[ok]) <= 8 * U32 * np.linalg.norm(want[ok])
+
+
+def test_repeat_is_the_same_bits(lrc, cuda):
+    m, n, k, b = 700, 5000, 48, 500
+    f = W.random_factors(m, n, k, seed=14)
+    X = W.gaussian((b, n), 15)
+    assert np.array_equal(run(lrc, cuda, f.U, f.s, f.Vt, X), run(lrc, cuda, f.U, f.s, f.Vt, X))
