@@ -96,6 +96,26 @@ def load() -> ctypes.CDLL:
     return L
 
 
+# torch and what the calls need of it, looked up once (an import statement and
+# torch.cuda.current_stream() cost a small call more than its launches)
+_torch = None
+_raw_stream = None
+_STORE = _OUT = _GATHER = ()
+
+
+def _T():
+    global _torch, _raw_stream, _STORE, _OUT, _GATHER
+    if _torch is None:
+        import torch
+        f64, f32, f16, bf16 = torch.float64, torch.float32, torch.float16, torch.bfloat16
+        _STORE = (f64, f32, f16, f16, f32, bf16)
+        _OUT = (f64, f32, f32, f16, f32, bf16)
+        _GATHER = (f64, f32, f32, f16, f32, bf16)
+        _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        _torch = torch
+    return _torch
+
+
 def _fmt(fmt) -> int:
     if isinstance(fmt, str):
         return FORMATS[fmt]
@@ -103,17 +123,19 @@ def _fmt(fmt) -> int:
 
 
 def storage_dtype(fmt):
-    import torch
+    _T()
     f = _fmt(fmt)
-    return {F64: torch.float64, F32: torch.float32, F16: torch.float16, F16_O16: torch.float16,
-            F32_TC: torch.float32, BF16: torch.bfloat16}[f]
+    if not 0 <= f < len(_STORE):
+        raise KeyError(f)
+    return _STORE[f]
 
 
 def output_dtype(fmt):
-    import torch
+    _T()
     f = _fmt(fmt)
-    return {F64: torch.float64, F32: torch.float32, F16: torch.float32, F16_O16: torch.float16,
-            F32_TC: torch.float32, BF16: torch.bfloat16}[f]
+    if not 0 <= f < len(_OUT):
+        raise KeyError(f)
+    return _OUT[f]
 
 
 def _check(status: int) -> None:
@@ -131,7 +153,9 @@ def np_prod(xs) -> int:
 
 def _stream(stream) -> int:
     if stream is None:
-        import torch
+        torch = _T()
+        if _raw_stream is not None:
+            return _raw_stream(torch.cuda.current_device())
         return torch.cuda.current_stream().cuda_stream
     if isinstance(stream, int):
         return stream
@@ -154,8 +178,7 @@ def _call_device(stream) -> int:
     dev = getattr(stream, "device", None)
     if dev is not None:
         return dev.index if hasattr(dev, "index") else int(dev)
-    import torch
-    return torch.cuda.current_device()
+    return _T().cuda.current_device()
 
 
 def _need(t, what: str, dtype=None, elems: int = 0, stream=None) -> None:
@@ -179,9 +202,30 @@ def _need(t, what: str, dtype=None, elems: int = 0, stream=None) -> None:
                          f"writes {elems}")
 
 
+def _check_arg(t, what: str, dtype, elems: int, dev: int, stream) -> None:
+    """_need's checks, in one expression where they hold (the checks by name,
+    in their order, where one fails)."""
+    if not (t is not None and t.is_cuda and t.dtype is dtype and t.device.index == dev and
+            (elems <= 0 or
+             (t.storage_offset() + elems) * dtype.itemsize <= t.untyped_storage().nbytes())):
+        _need(t, what, dtype, elems, stream)
+
+
 def _extent(rows: int, cols: int, ld: int) -> int:
     """Elements a rows x cols array with row pitch ld spans."""
     return (rows - 1) * ld + cols if rows > 0 and cols > 0 else 0
+
+
+_ARRAYS = {}
+
+
+def _array(ctype, xs):
+    """ctypes array of xs (the array types are made once per length)."""
+    key = (ctype, len(xs))
+    at = _ARRAYS.get(key)
+    if at is None:
+        at = _ARRAYS[key] = ctype * max(len(xs), 1)
+    return at(*xs)
 
 
 # --------------------------------------------------------------------------
@@ -193,31 +237,35 @@ def lrc_packed_ld(cols: int) -> int:
 
 
 def lrc_round_factors(src, rows: int, cols: int, ld_src: int, dst, ld_dst: int, fmt, stream=None):
-    import torch
-    _need(src, "src", torch.float64, _extent(rows, cols, ld_src), stream=stream)
-    _need(dst, "dst", storage_dtype(fmt), _extent(rows, ld_dst, ld_dst), stream=stream)
-    _check(load().lrc_round_factors(_ptr(src), rows, cols, ld_src, _ptr(dst), ld_dst, _fmt(fmt),
-                                    _stream(stream)))
+    f64, dev = _T().float64, _call_device(stream)
+    _check_arg(src, "src", f64, _extent(rows, cols, ld_src), dev, stream)
+    _check_arg(dst, "dst", storage_dtype(fmt), _extent(rows, ld_dst, ld_dst), dev, stream)
+    _check(load().lrc_round_factors(_ptr(src), rows, cols, ld_src, _ptr(dst), ld_dst, _fmt(fmt), _stream(stream)))
 
 
 def lrc_widen_factors(src, fmt, rows: int, cols: int, ld_src: int, dst, ld_dst: int, stream=None):
-    import torch
-    _need(src, "src", storage_dtype(fmt), _extent(rows, cols, ld_src), stream=stream)
-    _need(dst, "dst", torch.float64, _extent(rows, ld_dst, ld_dst), stream=stream)
-    _check(load().lrc_widen_factors(_ptr(src), _fmt(fmt), rows, cols, ld_src, _ptr(dst), ld_dst,
-                                    _stream(stream)))
+    f64, dev = _T().float64, _call_device(stream)
+    _check_arg(src, "src", storage_dtype(fmt), _extent(rows, cols, ld_src), dev, stream)
+    _check_arg(dst, "dst", f64, _extent(rows, ld_dst, ld_dst), dev, stream)
+    _check(load().lrc_widen_factors(_ptr(src), _fmt(fmt), rows, cols, ld_src, _ptr(dst), ld_dst, _stream(stream)))
+
+
+def _apply_args(U, S, Vt, X, Y, m, n, k, b, f, dev, stream, tag=""):
+    """Addresses of one apply's tensors, checked where its sizes are positive."""
+    if m > 0 and n > 0 and k > 0 and b > 0:
+        st, ldk, ldn = storage_dtype(f), (k + 15) // 16 * 16, (n + 15) // 16 * 16
+        _check_arg(U, "U" + tag, st, (m - 1) * ldk + k, dev, stream)
+        _check_arg(S, "S" + tag, st, k, dev, stream)
+        _check_arg(Vt, "Vt" + tag, st, (k - 1) * ldn + n, dev, stream)
+        _check_arg(X, "X" + tag, st, (b - 1) * ldn + n, dev, stream)
+        _check_arg(Y, "Y" + tag, output_dtype(f), b * m, dev, stream)
+    return _ptr(U), _ptr(S), _ptr(Vt), _ptr(X), _ptr(Y)
 
 
 def lrc_apply(U, S, Vt, X, Y, m: int, n: int, k: int, b: int, fmt, stream=None):
-    if m > 0 and n > 0 and k > 0 and b > 0:
-        st, ldk, ldn = storage_dtype(fmt), lrc_packed_ld(k), lrc_packed_ld(n)
-        _need(U, "U", st, _extent(m, k, ldk), stream=stream)
-        _need(S, "S", st, k, stream=stream)
-        _need(Vt, "Vt", st, _extent(k, n, ldn), stream=stream)
-        _need(X, "X", st, _extent(b, n, ldn), stream=stream)
-        _need(Y, "Y", output_dtype(fmt), b * m, stream=stream)
-    _check(load().lrc_apply(_ptr(U), _ptr(S), _ptr(Vt), _ptr(X), _ptr(Y), m, n, k, b, _fmt(fmt),
-                            _stream(stream)))
+    f = _fmt(fmt)
+    p = _apply_args(U, S, Vt, X, Y, m, n, k, b, f, _call_device(stream), stream)
+    _check(load().lrc_apply(*p, m, n, k, b, f, _stream(stream)))
 
 
 def lrc_apply_batched(U: Sequence, S: Sequence, Vt: Sequence, X: Sequence, Y: Sequence, m: Sequence[int],
@@ -227,62 +275,51 @@ def lrc_apply_batched(U: Sequence, S: Sequence, Vt: Sequence, X: Sequence, Y: Se
     count = len(U)
     if not all(len(a) == count for a in (S, Vt, X, Y, m, n, k, b)):
         raise ValueError("every argument needs one entry per problem")
-    st, ot = storage_dtype(fmt), output_dtype(fmt)
-    for p in range(count):
-        mp, np_, kp, bp = int(m[p]), int(n[p]), int(k[p]), int(b[p])
-        if mp > 0 and np_ > 0 and kp > 0 and bp > 0:
-            ldk, ldn = lrc_packed_ld(kp), lrc_packed_ld(np_)
-            _need(U[p], f"U[{p}]", st, _extent(mp, kp, ldk), stream=stream)
-            _need(S[p], f"S[{p}]", st, kp, stream=stream)
-            _need(Vt[p], f"Vt[{p}]", st, _extent(kp, np_, ldn), stream=stream)
-            _need(X[p], f"X[{p}]", st, _extent(bp, np_, ldn), stream=stream)
-            _need(Y[p], f"Y[{p}]", ot, bp * mp, stream=stream)
-    arr = lambda ts: (ctypes.c_void_p * max(count, 1))(*[_ptr(t) for t in ts])  # noqa: E731
-    i64s = lambda xs: (ctypes.c_int64 * max(count, 1))(*[int(x) for x in xs])   # noqa: E731
-    pu, ps, pv, px, py = arr(U), arr(S), arr(Vt), arr(X), arr(Y)
-    am, an, ak, ab = i64s(m), i64s(n), i64s(k), i64s(b)
-    c = lambda a: ctypes.cast(a, ctypes.c_void_p)   # noqa: E731
-    _check(load().lrc_apply_batched(count, c(pu), c(ps), c(pv), c(px), c(py), c(am), c(an), c(ak), c(ab),
-                                    _fmt(fmt), _stream(stream)))
+    f = _fmt(fmt)
+    storage_dtype(f)          # an unknown format is refused whatever the count
+    dev = _call_device(stream)
+    m, n, k, b = ([int(x) for x in xs] for xs in (m, n, k, b))
+    rows = [_apply_args(U[p], S[p], Vt[p], X[p], Y[p], m[p], n[p], k[p], b[p], f, dev, stream, f"[{p}]")
+            for p in range(count)]
+    ptrs = [_array(ctypes.c_void_p, col) for col in zip(*rows)] if rows else [_array(ctypes.c_void_p, ())] * 5
+    sizes = [_array(ctypes.c_int64, xs) for xs in (m, n, k, b)]
+    _check(load().lrc_apply_batched(count, *ptrs, *sizes, f, _stream(stream)))
 
 
-def _need_cores(cores, dims, ranks, fmt, stream=None) -> bool:
+def _check_cores(cores, dims, ranks, dtype, dev, stream) -> bool:
     """Checks the cores; True when dims and ranks describe them (else the
     library's validation reports the mismatch)."""
     d = len(cores)
-    shaped = len(dims) == d and len(ranks) == d + 1 and all(int(x) > 0 for x in list(dims) + list(ranks))
+    shaped = len(dims) == d and len(ranks) == d + 1 and all(int(x) > 0 for x in dims) and all(int(x) > 0 for x in ranks)
     for l, c in enumerate(cores):
-        _need(c, f"cores[{l}]", storage_dtype(fmt),
-              int(ranks[l]) * int(dims[l]) * int(ranks[l + 1]) if shaped else 0, stream=stream)
+        _check_arg(c, f"cores[{l}]", dtype, int(ranks[l]) * int(dims[l]) * int(ranks[l + 1]) if shaped else 0, dev, stream)
     return shaped
 
 
-def tt_reconstruct(cores: Sequence, dims: Sequence[int], ranks: Sequence[int], fmt, out, stream=None):
-    if _need_cores(cores, dims, ranks, fmt, stream):
-        _need(out, "out", output_dtype(fmt), int(np_prod(dims)), stream=stream)
+def _shape_args(cores, dims, ranks):
     d = len(cores)
-    ptrs = (ctypes.c_void_p * d)(*[c.data_ptr() for c in cores])
-    dd = (ctypes.c_int64 * d)(*[int(x) for x in dims])
-    rr = (ctypes.c_int64 * (d + 1))(*[int(x) for x in ranks])
-    _check(load().tt_reconstruct(ctypes.cast(ptrs, ctypes.c_void_p), ctypes.cast(dd, ctypes.c_void_p),
-                                 ctypes.cast(rr, ctypes.c_void_p), d, _fmt(fmt), _ptr(out),
-                                 _stream(stream)))
+    return (_array(ctypes.c_void_p, [c.data_ptr() for c in cores]), (ctypes.c_int64 * d)(*[int(x) for x in dims]),
+            (ctypes.c_int64 * (d + 1))(*[int(x) for x in ranks]))
+
+
+def tt_reconstruct(cores: Sequence, dims: Sequence[int], ranks: Sequence[int], fmt, out, stream=None):
+    f = _fmt(fmt)
+    dev = _call_device(stream)
+    if _check_cores(cores, dims, ranks, storage_dtype(f), dev, stream):
+        _check_arg(out, "out", output_dtype(f), np_prod(dims), dev, stream)
+    ptrs, dd, rr = _shape_args(cores, dims, ranks)
+    _check(load().tt_reconstruct(ptrs, dd, rr, len(cores), f, _ptr(out), _stream(stream)))
 
 
 def tt_gather(cores: Sequence, dims: Sequence[int], ranks: Sequence[int], fmt, idx, out, stream=None):
     """Entries of the TT at the flat indices `idx` (int64 CUDA tensor) into `out`."""
-    import torch
-    _need_cores(cores, dims, ranks, fmt, stream)
-    _need(idx, "idx", torch.int64, stream=stream)
-    gather_dtype = {F64: torch.float64, F16_O16: torch.float16, BF16: torch.bfloat16}.get(_fmt(fmt), torch.float32)
-    _need(out, "out", gather_dtype, int(idx.numel()), stream=stream)
-    d = len(cores)
-    ptrs = (ctypes.c_void_p * d)(*[c.data_ptr() for c in cores])
-    dd = (ctypes.c_int64 * d)(*[int(x) for x in dims])
-    rr = (ctypes.c_int64 * (d + 1))(*[int(x) for x in ranks])
-    _check(load().tt_gather(ctypes.cast(ptrs, ctypes.c_void_p), ctypes.cast(dd, ctypes.c_void_p),
-                            ctypes.cast(rr, ctypes.c_void_p), d, _fmt(fmt), _ptr(idx), int(idx.numel()),
-                            _ptr(out), _stream(stream)))
+    f = _fmt(fmt)
+    dev = _call_device(stream)
+    _check_cores(cores, dims, ranks, storage_dtype(f), dev, stream)
+    _check_arg(idx, "idx", _T().int64, 0, dev, stream)
+    _check_arg(out, "out", _GATHER[f], int(idx.numel()), dev, stream)
+    ptrs, dd, rr = _shape_args(cores, dims, ranks)
+    _check(load().tt_gather(ptrs, dd, rr, len(cores), f, _ptr(idx), int(idx.numel()), _ptr(out), _stream(stream)))
 
 
 def lrc_fro_diff(A, fa, B, fb, count: int, stream=None, want_norm: bool = True) -> Tuple[float, float]:
@@ -322,7 +359,7 @@ def lrc_lowrank_eta(U, S, Vt, Uh, Sh, Vht, fmt, m: int, n: int, k: int, stream=N
     eta = ctypes.c_double(0.0)
     norm = ctypes.c_double(float("nan"))
     if m > 0 and n > 0 and k > 0:
-        import torch
+        torch = _T()
         ldk, ldn, st = lrc_packed_ld(k), lrc_packed_ld(n), storage_dtype(fmt)
         for t, what, dt in ((U, "U", torch.float64), (Uh, "Uh", st)):
             _need(t, what, dt, _extent(m, k, ldk), stream=stream)
@@ -339,14 +376,11 @@ def lrc_lowrank_eta(U, S, Vt, Uh, Sh, Vht, fmt, m: int, n: int, k: int, stream=N
 def lrc_tt_eta(cores: Sequence, cores_hat: Sequence, dims: Sequence[int], ranks: Sequence[int], fmt,
                stream=None, want_norm: bool = True) -> Tuple[float, float]:
     """Returns (eta_TT, ||T||_F) for binary64 cores and stored cores of format fmt."""
-    import torch
     d = len(cores)
-    shaped = len(dims) == d and len(ranks) == d + 1 and all(int(x) > 0 for x in list(dims) + list(ranks))
-    for l, c in enumerate(cores):
-        _need(c, f"cores[{l}]", torch.float64,
-              int(ranks[l]) * int(dims[l]) * int(ranks[l + 1]) if shaped else 0, stream=stream)
+    dev = _call_device(stream)
+    _check_cores(cores, dims, ranks, _T().float64, dev, stream)
     if len(cores_hat) == d:
-        _need_cores(cores_hat, dims, ranks, fmt, stream)
+        _check_cores(cores_hat, dims, ranks, storage_dtype(fmt), dev, stream)
     d = len(cores)
     if len(cores_hat) != d:
         raise ValueError("cores and cores_hat differ in length")
@@ -406,12 +440,12 @@ def lrc_tt_svd(T, dims: Sequence[int], ranks: Sequence[int], cores: Sequence, st
     (delta2, spectra): the discarded squared singular values per bond and,
     if asked, every bond's singular values (a list of arrays)."""
     import numpy as np
-    import torch
+    torch = _T()
     d = len(dims)
     if len(cores) != d or len(ranks) != d + 1:
         raise ValueError("cores needs d entries and ranks d + 1")
     _need(T, "T", torch.float64, np_prod(dims), stream=stream)
-    _need_cores(cores, dims, ranks, "f64", stream)
+    _check_cores(cores, dims, ranks, _T().float64, _call_device(stream), stream)
     sizes, rest = [], np_prod(dims)
     for l in range(d - 1):
         rest //= int(dims[l])
@@ -436,7 +470,7 @@ def lrc_tt_svd(T, dims: Sequence[int], ranks: Sequence[int], cores: Sequence, st
 def lrc_tt_left_orthogonalize(cores: Sequence, dims: Sequence[int], ranks: Sequence[int], stream=None) -> None:
     """Left-orthogonal gauge of binary64 cores, in place."""
     d = len(cores)
-    _need_cores(cores, dims, ranks, "f64", stream)
+    _check_cores(cores, dims, ranks, _T().float64, _call_device(stream), stream)
     ptrs = (ctypes.c_void_p * d)(*[c.data_ptr() for c in cores])
     dd = (ctypes.c_int64 * d)(*[int(x) for x in dims])
     rr = (ctypes.c_int64 * (d + 1))(*[int(x) for x in ranks])
