@@ -19,7 +19,7 @@
 // element per row so that the transposing stores are conflict-free too.
 //
 // binary64 forms both products on the tensor cores from exact products of
-// digits (split_gemm.cu; 16384 x 8192, k = 128, b = 8192: 45.5 -> 1.62 ms);
+// digits (split_gemm.cu; 16384 x 8192, k = 128, b = 8192: 45.5 -> 1.54 ms);
 // this kernel (DFMA-bound: the GB300 issues about 2 DFMA per clock per SM),
 // with thin 8-row tiles and many CTAs per SM, so the work spreads evenly over
 // the SMs, takes what that path does not: no workspace to be had, n above 2^20.  binary32 (FFMA-bound) runs the two products on the
@@ -495,15 +495,16 @@ constexpr int64_t kPanelBytes = (int64_t)1 << 30;     // digit images of a panel
 
 }  // namespace
 
-// Where the digits' fixed cost (eight launches, about 45 us) pays.  Measured
+// Where the digits' fixed cost (eight launches, about 35 us) pays.  Measured
 // on square matrices, digits / FMA kernels: against the kernels for at most 16
-// queries 16384^2, k = 256: b = 8 180 / 164 us, b = 16 178 / 284 us, and k =
-// 128, b = 16 166 / 166 us; against the others 512^2, k = 32, b = 64 57 / 55 us
-// and b = 256 58 / 59 us, 2048^2, k = 128, b = 64 62 / 160 us.
+// queries 16384^2, b = 16, k = 256: 136 / 284 us, k = 32 (1.7e7): 66 / 70 us, and
+// 2048^2, k = 256, b = 16 (1.7e7): 66 / 112 us, k = 128 (8e6): 50 / 48 us; against
+// the others 512^2, k = 32, b = 64 (2e6) 53 / 55 us, 2048^2, k = 32, b = 64
+// 46 / 56 us and k = 128, b = 64 60 / 160 us.
 bool apply_f64_tc_takes(int64_t m, int64_t n, int64_t k, int64_t b) {
     if (n > sg::kMaxK || k > 4096 || m >= (1ll << 31) || b >= (1ll << 31)) return false;
     const double work = (double)(m + n) * (double)k * (double)b;
-    return work >= (apply_skinny_takes(LRC_F64, m, n, k, b) ? 8e7 : 4e6);
+    return work >= (apply_skinny_takes(LRC_F64, m, n, k, b) ? 1.5e7 : 4e6);
 }
 
 // *handled = false: no workspace for the digits (nothing launched).

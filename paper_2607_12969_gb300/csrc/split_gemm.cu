@@ -82,13 +82,15 @@ __device__ __forceinline__ int biased_exp(uint64_t bits) {
 struct RowStat {
     int mx = -(1 << 20), sum = 0, cnt = 0;
     __device__ __forceinline__ void add(double x, int shift) {
-        const uint64_t bits = (uint64_t)__double_as_longlong(x) & 0x7fffffffffffffffull;
-        if (bits != 0) {
-            const int e = biased_exp(bits) + shift;
-            mx = max(mx, e);
-            sum += e >= kNonFinite / 2 ? 0 : e;
-            cnt += 1;
+        const uint32_t h = (uint32_t)__double2hiint(x) & 0x7fffffffu, e = h >> 20;
+        int v = (int)e + shift, one = 1;
+        if (e - 1u >= 0x7feu) {            // zero, subnormal, infinity or NaN
+            one = (h | (uint32_t)__double2loint(x)) != 0 ? 1 : 0;
+            v = one ? biased_exp(((uint64_t)h << 32) | (uint32_t)__double2loint(x)) + shift : -(1 << 20);
         }
+        mx = max(mx, v);
+        sum += one && v < kNonFinite / 2 ? v : 0;
+        cnt += one;
     }
     __device__ __forceinline__ void merge(int4 o) {
         mx = max(mx, o.x);
@@ -123,24 +125,35 @@ __device__ __forceinline__ const Job& job_of(const Jobs& js, int64_t block) {
 // Statistics of 32 rows over columns [k0, k1), by 256 threads; row r0 + lane's
 // in warp 0.  K contiguous: a warp per row, lanes along K; else a lane per
 // row, so that either way a warp reads consecutive addresses.
+template <bool SCALED>
 __device__ __forceinline__ RowStat block_stats(const View64& v, int64_t r0, int64_t rows, int64_t k0, int64_t k1,
-                                               int4 (&sm)[8][32]) {
+                                               bool vec, int4 (&sm)[8][32]) {
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    auto shift = [&](int64_t k) { return SCALED ? v.shift(k) : 0; };
     if (v.s.cs == 1) {
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const int64_t r = r0 + warp + 8 * q;
             RowStat a;
             if (r < rows) {
-                int64_t k = k0 + lane;
-                for (; k + 96 < k1; k += 128) {
-                    double x[4];
+                int64_t k = k0 + 2 * lane;
+                if (vec) {
+                    for (; k + 194 <= k1; k += 256) {
+                        double2 x[4];
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) x[u] = v.at(r, k + 32 * u);
+                        for (int u = 0; u < 4; ++u)
+                            x[u] = __ldg(reinterpret_cast<const double2*>(v.s.p + r * v.s.rs + k + 64 * u));
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) a.add(x[u], v.shift(k + 32 * u));
+                        for (int u = 0; u < 4; ++u) {
+                            a.add(x[u].x, shift(k + 64 * u));
+                            a.add(x[u].y, shift(k + 64 * u + 1));
+                        }
+                    }
                 }
-                for (; k < k1; k += 32) a.add(v.at(r, k), v.shift(k));
+                for (; k < k1; k += 64) {
+                    a.add(v.at(r, k), shift(k));
+                    if (k + 1 < k1) a.add(v.at(r, k + 1), shift(k + 1));
+                }
             }
             a.mx = __reduce_max_sync(0xffffffffu, a.mx);
             a.sum = __reduce_add_sync(0xffffffffu, a.sum);
@@ -157,9 +170,9 @@ __device__ __forceinline__ RowStat block_stats(const View64& v, int64_t r0, int6
 #pragma unroll
                 for (int u = 0; u < 4; ++u) x[u] = v.at(r, k + 8 * u);
 #pragma unroll
-                for (int u = 0; u < 4; ++u) a.add(x[u], v.shift(k + 8 * u));
+                for (int u = 0; u < 4; ++u) a.add(x[u], shift(k + 8 * u));
             }
-            for (; k < k1; k += 8) a.add(v.at(r, k), v.shift(k));
+            for (; k < k1; k += 8) a.add(v.at(r, k), shift(k));
         }
         sm[warp][lane] = make_int4(a.mx, a.sum, a.cnt, 0);
     }
@@ -183,7 +196,9 @@ __global__ void __launch_bounds__(256) row_stats_kernel(const __grid_constant__ 
     const int64_t lb = (int64_t)blockIdx.x - o.b0, rg = lb / o.splits, z = lb - rg * o.splits;
     const int64_t r0 = rg * 32, k0 = z * o.kchunk;
     if (blockIdx.x == 0 && threadIdx.x < kMaxOps && js.clear[threadIdx.x]) *js.clear[threadIdx.x] = 0;
-    const RowStat a = block_stats(o.v, r0, o.rows, k0, min(o.K, k0 + o.kchunk), sm);
+    const int64_t k1 = min(o.K, k0 + o.kchunk);
+    const RowStat a = o.v.s.scale ? block_stats<true>(o.v, r0, o.rows, k0, k1, o.vec != 0, sm)
+                                  : block_stats<false>(o.v, r0, o.rows, k0, k1, o.vec != 0, sm);
     if (threadIdx.x < 32 && r0 + threadIdx.x < o.rows)
         o.stats[z * o.rows + r0 + threadIdx.x] = make_int4(a.mx, a.sum, a.cnt, 0);
 }
@@ -241,7 +256,7 @@ __global__ void __launch_bounds__(256) slice_kernel(const __grid_constant__ Jobs
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int64_t r0 = rg * 32;
     RowStat own;
-    if (o.splits == 0) own = block_stats(v, r0, rows, 0, K, sm);
+    if (o.splits == 0) own = block_stats<true>(v, r0, rows, 0, K, o.vec != 0, sm);
     if (tid < 32) {
         const int64_t r = r0 + lane;
         int em = 1023;
@@ -302,6 +317,7 @@ __global__ void __launch_bounds__(256) slice_kernel(const __grid_constant__ Jobs
 }
 
 // ---------------------------------------------------------------- product
+constexpr int kMaxListed = 120;
 struct GemmArgs {
     const unsigned char* A;
     const unsigned char* B;
@@ -315,6 +331,8 @@ struct GemmArgs {
     int split, group, stages, vec;
     int64_t a_block, b_block;    // bytes of a block of either image
     uint32_t a_bytes, b_bytes;   // of a tile's part of it
+    int listed;                  // > 0: the tiles are list[0 ... listed), row << 8 | column
+    uint16_t list[kMaxListed];
     uint32_t tmem_cols;
 };
 
@@ -328,6 +346,13 @@ constexpr int kThreads = 32 * (4 + kEpiWarps);
 // of theirs to the epilogue's, which keep two 64-bit sums per entry: 128 x 64
 // + 512 x 104 = 61440, the 640 x 96 = 61440 of the launch.
 constexpr int kRegsLow = 64, kRegsEpi = 104;
+// Row and column of a tile.
+__device__ __forceinline__ int2 tile_at(const GemmArgs& a, int tile) {
+    if (a.listed) return make_int2(a.list[tile] >> 8, a.list[tile] & 255);
+    const int mt = tile / a.ntiles;
+    return make_int2(mt, tile - mt * a.ntiles);
+}
+
 constexpr int kChunkBlocks = 64 / kKB;
 constexpr uint32_t kCtrlBytes = 1024;
 
@@ -422,16 +447,18 @@ __device__ __forceinline__ double round_pq_fp64(int64_t p, int64_t q, int esum) 
 // A's 4 KB read and 35 with them kept), and no MMA adds to the accumulator of
 // the one before it, which would wait for its result (about 120 clocks).
 // fresh: bit t is set where class t starts a new sum.
+// col3: column of class 3's accumulator.
 template <int NT, int T0, int T1, int I = 0, int J = (T0 > 0 ? T0 : 0)>
-__device__ __forceinline__ void issue(uint32_t tmem, uint32_t fresh, uint32_t alo, uint32_t ahi, uint32_t blo,
-                                      uint32_t bhi) {
+__device__ __forceinline__ void issue(uint32_t tmem, uint32_t col3, uint32_t fresh, uint32_t alo, uint32_t ahi,
+                                      uint32_t blo, uint32_t bhi) {
     constexpr int kPart = 8 * kKB * 2 / 16;                                     // one digit
     constexpr int J0 = T0 > I ? T0 - I : 0, J1 = T1 - I;                        // digits of B for this one of A
     constexpr int kMmaUse = J1 - J0 == 1 ? kNoReuse : J == J0 ? kFill : J == J1 - 1 ? kLast : kUse;
-    mma_f16_col<kMmaUse>(tmem + (I + J) * NT, alo + I * kPart, ahi, blo + J * kPart, bhi,
+    mma_f16_col<kMmaUse>(tmem + (I + J == 3 ? col3 : (uint32_t)(I + J) * NT), alo + I * kPart, ahi, blo + J * kPart, bhi,
                           idesc_f16_f32(128, NT) | kIdescBF16, I > 0 ? 1u : ((fresh >> (I + J)) & 1u) ^ 1u);
-    if constexpr (J + 1 < J1) issue<NT, T0, T1, I, J + 1>(tmem, fresh, alo, ahi, blo, bhi);
-    else if constexpr (I + 1 < T1) issue<NT, T0, T1, I + 1, (T0 > I + 1 ? T0 - I - 1 : 0)>(tmem, fresh, alo, ahi, blo, bhi);
+    if constexpr (J + 1 < J1) issue<NT, T0, T1, I, J + 1>(tmem, col3, fresh, alo, ahi, blo, bhi);
+    else if constexpr (I + 1 < T1) issue<NT, T0, T1, I + 1, (T0 > I + 1 ? T0 - I - 1 : 0)>(tmem, col3, fresh, alo, ahi,
+                                                                                                  blo, bhi);
 }
 
 template <int NT>
@@ -440,9 +467,9 @@ __global__ void __launch_bounds__(kThreads, 1) product_kernel(const __grid_const
     extern __shared__ __align__(128) unsigned char smem[];
     uint64_t* full = reinterpret_cast<uint64_t*>(smem);
     uint64_t* empty = full + 8;
-    uint64_t* gfull = empty + 8;        // accumulator groups complete
-    uint64_t* gempty = gfull + 2;       // accumulator groups drained
-    uint64_t* mma_done = gempty + 2;
+    uint64_t* gfull = empty + 8;        // classes 0 to 3 of an even or odd chunk complete; classes 4 to 6
+    uint64_t* gempty = gfull + 3;       // ... drained
+    uint64_t* mma_done = gempty + 3;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(mma_done + 1);
     volatile int* abort = reinterpret_cast<volatile int*>(tmem_slot + 1);
     unsigned char* ring = smem + kCtrlBytes;
@@ -455,7 +482,7 @@ __global__ void __launch_bounds__(kThreads, 1) product_kernel(const __grid_const
             mbar_init(&full[i], 1);
             mbar_init(&empty[i], 1);
         }
-        for (int i = 0; i < 2; ++i) {
+        for (int i = 0; i < 3; ++i) {
             mbar_init(&gfull[i], 1);
             mbar_init(&gempty[i], 32 * kEpiWarps);
         }
@@ -489,7 +516,8 @@ __global__ void __launch_bounds__(kThreads, 1) product_kernel(const __grid_const
             return *abort == 0;
         };
         while (ok && pc.next(a, &tile, &c0, &c1)) {
-            const int mt = tile / a.ntiles, nt = tile - mt * a.ntiles;
+            const int2 at = tile_at(a, tile);
+                const int mt = at.x, nt = at.y;
             const int64_t row = (int64_t)mt * 128 + r, col0 = (int64_t)nt * NT + quarter * HC;
             // exponents: of the thread's row, and of column `lane`
             const int ea = row < a.M ? a.ea[row] : 0;
@@ -500,20 +528,20 @@ __global__ void __launch_bounds__(kThreads, 1) product_kernel(const __grid_const
             for (int c = c0; c < c1; ++c, ++ch) {
                 const int n = c - c0 + 1;
                 auto due = [&](int t) { return c + 1 == c1 || n % period(t) == 0; };
-                if (!(ok = epi_wait(&gfull[0], ch & 1))) break;
+                if (!(ok = epi_wait(&gfull[ch & 1], (ch >> 1) & 1))) break;
                 tc_fence_after();
-                drain<HC>(tbase + 3 * NT, 1, P);
+                drain<HC>(tbase + (ch & 1 ? 7 : 3) * NT, 1, P);
                 if (due(2)) drain<HC>(tbase + 2 * NT, 1 << 9, P);
                 if (due(1)) drain<HC>(tbase + NT, 1 << 18, P);
                 if (due(0)) drain<HC>(tbase, 1 << 27, P);
                 tc_fence_before();
-                mbar_arrive(&gempty[0]);
-                if (!(ok = epi_wait(&gfull[1], ch & 1))) break;
+                mbar_arrive(&gempty[ch & 1]);
+                if (!(ok = epi_wait(&gfull[2], ch & 1))) break;
                 tc_fence_after();
                 drain<HC>(tbase + 4 * NT, 1 << 13, Q);
                 if (due(5)) drain56<HC>(tbase + 5 * NT, tbase + 6 * NT, Q);
                 tc_fence_before();
-                mbar_arrive(&gempty[1]);
+                mbar_arrive(&gempty[2]);
             }
             if (!ok) break;
             if (a.split) {
@@ -560,7 +588,8 @@ __global__ void __launch_bounds__(kThreads, 1) product_kernel(const __grid_const
             uint32_t phase = 1;
             bool ok = true;
             while (ok && pc.next(a, &tile, &c0, &c1)) {
-                const int mt = tile / a.ntiles, nt = tile - mt * a.ntiles;
+                const int2 at = tile_at(a, tile);
+            const int mt = at.x, nt = at.y;
                 const int b1 = min(kChunkBlocks * c1, a.kblocks);
                 for (int kb = kChunkBlocks * c0; kb < b1; ++kb, ++it) {
                     if (!(ok = mbar_wait(&empty[slot], phase, abort, err, 1u))) break;
@@ -604,8 +633,15 @@ __global__ void __launch_bounds__(kThreads, 1) product_kernel(const __grid_const
                 uint32_t fresh = 0;
 #pragma unroll
                 for (int t = 0; t < kParts64; ++t) fresh |= (c - c0) % period(t) == 0 ? 1u << t : 0u;
-                // classes 0 to 3 of the whole chunk, drained while the others run
-                if (!(ok = wait(&gempty[0], (ch & 1) ^ 1))) break;
+                // Classes 0 to 3 of the whole chunk, drained while the others run.  Class
+                // 3, the only one of them drained every chunk, has two accumulators, so
+                // the chunk waits for the drain before the last one, and for the last
+                // one only where it emptied one of classes 0 to 2 (128 x 64 tiles of two
+                // chunks: the second chunk's MMAs no longer wait for the rounding and
+                // stores of the tile before).
+                if (!(ok = wait(&gempty[ch & 1], ((ch >> 1) & 1) ^ 1))) break;
+                if ((fresh & 7) && ch > 0 && !(ok = wait(&gempty[(ch - 1) & 1], ((ch - 1) >> 1) & 1))) break;
+                const uint32_t col3 = (uint32_t)(ch & 1 ? 7 : 3) * NT;
                 for (int b0 = 0; b0 < nb; b0 += 2) {
                     // two blocks per wait, half the lanes polling each
                     const int b1 = min(b0 + 2, nb);
@@ -618,27 +654,27 @@ __global__ void __launch_bounds__(kThreads, 1) product_kernel(const __grid_const
                         sl = slot + b0 >= a.stages ? slot + b0 - a.stages : slot + b0;
                         for (int b = b0; b < b1; ++b) {
                             const uint32_t off = (uint32_t)sl * stage_bytes / 16;
-                            if (b == 0) issue<NT, 0, 4>(tmem, fresh, alo0 + off, ahi, blo0 + off, bhi);
-                            else issue<NT, 0, 4>(tmem, 0u, alo0 + off, ahi, blo0 + off, bhi);
+                            if (b == 0) issue<NT, 0, 4>(tmem, col3, fresh, alo0 + off, ahi, blo0 + off, bhi);
+                            else issue<NT, 0, 4>(tmem, col3, 0u, alo0 + off, ahi, blo0 + off, bhi);
                             if (++sl == a.stages) sl = 0;
                         }
-                        if (b1 == nb) mma_commit(&gfull[0]);
+                        if (b1 == nb) mma_commit(&gfull[ch & 1]);
                     }
                     __syncwarp();
                 }
                 if (!ok) break;
-                if (!(ok = wait(&gempty[1], (ch & 1) ^ 1))) break;
+                if (!(ok = wait(&gempty[2], (ch & 1) ^ 1))) break;
                 tc_fence_after();
                 if (elect_one()) {
                     int sl = slot;
                     for (int b = 0; b < nb; ++b) {
                         const uint32_t off = (uint32_t)sl * stage_bytes / 16;
-                        if (b == 0) issue<NT, 4, 7>(tmem, fresh, alo0 + off, ahi, blo0 + off, bhi);
-                        else issue<NT, 4, 7>(tmem, 0u, alo0 + off, ahi, blo0 + off, bhi);
+                        if (b == 0) issue<NT, 4, 7>(tmem, 0u, fresh, alo0 + off, ahi, blo0 + off, bhi);
+                        else issue<NT, 4, 7>(tmem, 0u, 0u, alo0 + off, ahi, blo0 + off, bhi);
                         mma_commit(&empty[sl]);
                         if (++sl == a.stages) sl = 0;
                     }
-                    mma_commit(&gfull[1]);
+                    mma_commit(&gfull[2]);
                 }
                 __syncwarp();
                 slot += nb;
@@ -662,26 +698,57 @@ __global__ void __launch_bounds__(kThreads, 1) product_kernel(const __grid_const
 }
 
 // The partial tiles of a split reduction, added in the order of the groups.
-__global__ void __launch_bounds__(256) part_sum_kernel(const double* __restrict__ part, int NT, int64_t ntiles,
-                                                       int64_t chunks, int64_t Q, int64_t G, int group,
-                                                       double* __restrict__ C, int64_t cr, int64_t cc, int64_t M,
-                                                       int64_t N, const double* __restrict__ rscale,
-                                                       const double* __restrict__ cscale, int* __restrict__ clear) {
+constexpr int kManyParts = 24;
+// (Of a listed, symmetric product the entries above the diagonal, both ways.)
+__global__ void __launch_bounds__(256) part_sum_kernel(const __grid_constant__ GemmArgs a, int NT, int64_t Q, int64_t G,
+                                                       double* __restrict__ C, const double* __restrict__ rscale,
+                                                       const double* __restrict__ cscale, int* __restrict__ clear,
+                                                       double* __restrict__ mirror) {
     pdl_wait();
     pdl_trigger();
     if (clear && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *clear = 0;
-    const int64_t tile = blockIdx.x;
-    const int64_t mt = tile / ntiles, nt = tile - mt * ntiles, u = tile / group * chunks;
-    const int64_t p0 = group_of_chunk(u, Q, G), p1 = group_of_chunk(u + chunks - 1, Q, G);
-    for (int e = blockIdx.y * 256 + threadIdx.x; e < 128 * NT; e += 256 * gridDim.y) {
-        const int64_t row = mt * 128 + (e & 127), col = nt * NT + (e >> 7);
-        if (row >= M || col >= N) continue;
-        double s = 0.0;
-#pragma unroll 4
-        for (int64_t p = p0; p <= p1; ++p) s += part[(p * group + tile) * (128 * NT) + e];
+    const int tile = blockIdx.x;
+    const int2 at = tile_at(a, tile);
+    const int64_t u = (int64_t)(tile / a.group) * a.chunks;
+    const int64_t p0 = group_of_chunk(u, Q, G), p1 = group_of_chunk(u + a.chunks - 1, Q, G);
+    const double* part = a.C + (int64_t)tile * (128 * NT);
+    const int64_t step = (int64_t)a.group * (128 * NT);
+    auto put = [&](int e, double s) {
+        const int64_t row = at.x * 128 + (e & 127), col = (int64_t)at.y * NT + (e >> 7);
+        if (row >= a.M || col >= a.N || (a.listed && row > col)) return;
         if (rscale) s *= __ldg(rscale + row);
         if (cscale) s *= __ldg(cscale + col);
-        C[row * cr + col * cc] = s;
+        C[row * a.cr + col * a.cc] = s;
+        if (a.listed) C[col * a.cr + row * a.cc] = s;
+        if (mirror) mirror[col * a.cr + row * a.cc] = s;
+    };
+    if (p1 - p0 < kManyParts) {
+        for (int e = blockIdx.y * 256 + threadIdx.x; e < 128 * NT; e += 256 * gridDim.y) {
+            double s = 0.0;
+#pragma unroll 4
+            for (int64_t p = p0; p <= p1; ++p) s += part[p * step + e];
+            put(e, s);
+        }
+        return;
+    }
+    // many partial tiles (one tile spread over all SMs: 152, 27 us one after the
+    // other): eight warps take an eighth each, their sums are added in order
+    __shared__ double sm[8][32];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t np = p1 - p0 + 1, q0 = p0 + np * w / 8, q1 = p0 + np * (w + 1) / 8;
+    for (int e0 = blockIdx.y * 32; e0 < 128 * NT; e0 += 32 * gridDim.y) {
+        double s = 0.0;
+#pragma unroll 4
+        for (int64_t p = q0; p < q1; ++p) s += part[p * step + e0 + lane];
+        __syncthreads();
+        sm[w][lane] = s;
+        __syncthreads();
+        if (w == 0) {
+            s = sm[0][lane];
+#pragma unroll
+            for (int i = 1; i < 8; ++i) s += sm[i][lane];
+            put(e0 + lane, s);
+        }
     }
 }
 
@@ -692,7 +759,7 @@ __global__ void __launch_bounds__(256) repair_kernel(View64 A, const int* __rest
                                                      const int* __restrict__ hb, int64_t N, int64_t K,
                                                      double* __restrict__ C, int64_t cr, int64_t cc,
                                                      const double* __restrict__ rscale,
-                                                     const double* __restrict__ cscale) {
+                                                     const double* __restrict__ cscale, double* __restrict__ mirror) {
     __shared__ double As[16][65];
     __shared__ double Bs[16][65];
     pdl_wait();
@@ -752,6 +819,7 @@ __global__ void __launch_bounds__(256) repair_kernel(View64 A, const int* __rest
                 if (rscale) s *= __ldg(rscale + row);
                 if (cscale) s *= __ldg(cscale + col);
                 C[row * cr + col * cc] = s;
+                if (mirror) mirror[col * cr + row * cc] = s;
             }
         }
     }
@@ -760,9 +828,9 @@ __global__ void __launch_bounds__(256) repair_kernel(View64 A, const int* __rest
 size_t up256(size_t v) { return (v + 255) & ~(size_t)255; }
 
 int stat_splits(int64_t rows, int64_t K) {
-    // enough CTAs for two per SM, at least 256 columns each
+    // eight CTAs a SM, at least 256 columns each
     const int64_t groups = (rows + 31) / 32;
-    int64_t z = (2 * (int64_t)sm_count() + groups - 1) / groups;
+    int64_t z = (8 * (int64_t)sm_count() + groups - 1) / groups;
     z = std::min<int64_t>(z, (K + 255) / 256);
     return (int)std::max<int64_t>(1, std::min<int64_t>(z, kStatSplits));
 }
@@ -780,14 +848,14 @@ lrc_status launch_product(const GemmArgs& a, int64_t grid, size_t smem, cudaStre
 
 size_t operand_bytes(int64_t rows, int64_t K) {
     const int64_t ir = image_rows(rows);
-    return up256((size_t)(ir / 8) * image_blocks(K) * kGroupBytes) + up256((size_t)ir * 4) +
+    return up256((size_t)(ir / 8) * image_blocks(K) * kGroupBytes + kTailBytes) + up256((size_t)ir * 4) +
            up256((size_t)rows * (K > kOwnStatsK ? kStatSplits : 0) * sizeof(int4)) + hard_bytes(rows);
 }
 
 void operand_carve(Operand64* o, unsigned char* ws) {
     const int64_t ir = image_rows(o->rows);
     o->img = ws;
-    ws += up256((size_t)(ir / 8) * image_blocks(o->K) * kGroupBytes);
+    ws += up256((size_t)(ir / 8) * image_blocks(o->K) * kGroupBytes + kTailBytes);
     o->exps = reinterpret_cast<int*>(ws);
     ws += up256((size_t)ir * 4);
     o->stats = reinterpret_cast<int4*>(ws);
@@ -863,8 +931,10 @@ size_t part_bytes(int64_t M, int64_t N) {
     return up256((size_t)(tiles_of(M, N) + sm_count()) * 128 * n_tile(N) * 8);
 }
 
-lrc_status product(const Operand64& A0, const Operand64& B0, const Out64& out0, bool split, double* part,
-                   cudaStream_t s) {
+namespace {
+
+lrc_status run_product(const Operand64& A0, const Operand64& B0, const Out64& out0, bool split, double* part, bool sym,
+                       cudaStream_t s) {
     const bool swap = tiles_of(B0.rows, A0.rows) < tiles_of(A0.rows, B0.rows);
     const Operand64& A = swap ? B0 : A0;
     const Operand64& B = swap ? A0 : B0;
@@ -884,12 +954,25 @@ lrc_status product(const Operand64& A0, const Operand64& B0, const Out64& out0, 
     a.cc = out.cc;
     a.M = A.rows;
     a.N = B.rows;
-    const int64_t tiles = tiles_of(A.rows, B.rows);
+    int64_t tiles = tiles_of(A.rows, B.rows);
     if (tiles > 0x3fffffff || A.K > kMaxK) {
         set_error("split product too large (%lld tiles, reduction of %lld)", (long long)tiles, (long long)A.K);
         return LRC_ERR_UNSUPPORTED;
     }
     a.ntiles = (int)n_tiles(B.rows);
+    if (sym && tiles <= 2 * kMaxListed) {
+        int n = 0;
+        for (int mt = 0; mt < (int)(tiles / a.ntiles); ++mt)
+            for (int nt = 0; nt < a.ntiles; ++nt)
+                if ((nt + 1) * NT > mt * 128) {
+                    if (n < kMaxListed) a.list[n] = (uint16_t)(mt << 8 | nt);
+                    ++n;
+                }
+        if (n <= kMaxListed) {
+            a.listed = n;
+            tiles = n;
+        }
+    }
     a.tiles = (int)tiles;
     a.kblocks = (int)image_blocks(A.K);
     a.chunks = (a.kblocks + kChunkBlocks - 1) / kChunkBlocks;
@@ -902,11 +985,11 @@ lrc_status product(const Operand64& A0, const Operand64& B0, const Out64& out0, 
     a.vec = out.cc != 1 || out.cr % 2 != 0 || !aligned16(out.C) ? 0
             : out.cr % 4 == 0 && (reinterpret_cast<uintptr_t>(out.C) & 31u) == 0 ? 2 : 1;
     uint32_t cols = 32;
-    while (cols < (uint32_t)(7 * NT)) cols *= 2;
+    while (cols < (uint32_t)(8 * NT)) cols *= 2;
     a.tmem_cols = cols;
     const int64_t sms = sm_count();
     // groups of one CTA per tile of B while that leaves at least eight groups
-    a.group = split && (int64_t)a.ntiles * 8 <= sms ? a.ntiles : 1;
+    a.group = split && !a.listed && (int64_t)a.ntiles * 8 <= sms ? a.ntiles : 1;
     const int64_t Q = tiles / a.group * a.chunks;
     const int64_t groups = std::min<int64_t>(Q, sms / a.group);
     const int64_t grid = split ? groups * a.group : std::min<int64_t>(tiles, sms);
@@ -922,16 +1005,28 @@ lrc_status product(const Operand64& A0, const Operand64& B0, const Out64& out0, 
     if (st != LRC_OK) return st;
     cudaError_t e;
     if (split) {
-        const unsigned gy = (unsigned)std::max<int64_t>(1, std::min<int64_t>(128 * NT / 256, 4 * sms / tiles));
-        e = launch_pdl(part_sum_kernel, dim3((unsigned)tiles, gy), dim3(256), 0, s, (const double*)part, NT, (int64_t)a.ntiles,
-                       (int64_t)a.chunks, Q, groups, a.group, out.C, out.cr, out.cc, A.rows, B.rows, out.rscale, out.cscale, out.clear);
+        const bool many = groups / (tiles / a.group) >= kManyParts;
+        const unsigned gy = (unsigned)std::max<int64_t>(1, std::min<int64_t>(128 * NT / (many ? 32 : 256), (many ? 8 : 4) * sms / tiles));
+        e = launch_pdl(part_sum_kernel, dim3((unsigned)tiles, gy), dim3(256), 0, s, a, NT, Q, groups, out.C, out.rscale,
+                       out.cscale, out.clear, out.mirror);
         if (e != cudaSuccess) return cuda_fail(e, "part_sum_kernel launch");
         if ((st = after_launch("part_sum_kernel")) != LRC_OK) return st;
     }
     e = launch_pdl(repair_kernel, dim3((unsigned)(2 * sms)), dim3(256), 0, s, View64{A.src}, (const int*)A.hard, A.rows,
-                   View64{B.src}, (const int*)B.hard, B.rows, A.K, out.C, out.cr, out.cc, out.rscale, out.cscale);
+                   View64{B.src}, (const int*)B.hard, B.rows, A.K, out.C, out.cr, out.cc, out.rscale, out.cscale,
+                   out.mirror);
     if (e != cudaSuccess) return cuda_fail(e, "repair_kernel launch");
     return after_launch("repair_kernel");
+}
+
+}  // namespace
+
+lrc_status product(const Operand64& A, const Operand64& B, const Out64& out, bool split, double* part, cudaStream_t s) {
+    return run_product(A, B, out, split, part, false, s);
+}
+
+lrc_status gram(const Operand64& A, double* C, int64_t ldc, double* part, cudaStream_t s) {
+    return run_product(A, A, Out64{C, ldc, 1, nullptr, nullptr}, true, part, true, s);
 }
 
 }  // namespace sg

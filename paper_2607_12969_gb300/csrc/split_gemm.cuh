@@ -10,7 +10,7 @@ namespace sg {
 constexpr int kParts64 = 7;        // 9-bit digits a binary64 value is cut into
 constexpr int kKB = 16;            // columns of the reduction per image block
 constexpr int64_t kMaxK = 1 << 20; // longest reduction the 64-bit sums hold
-constexpr int kStatSplits = 32;    // most slices of the reduction in the row statistics
+constexpr int kStatSplits = 128;    // most slices of the reduction in the row statistics
 
 // Tiles of the product: 128 rows of the first side, and of the second the rows
 // split evenly over tiles of at most kNTMax, a multiple of 16.
@@ -46,10 +46,14 @@ struct Operand64 {
     int* hard;               // hard[0] = rows that the digits cannot carry; then their indices
     bool cleared = false;    // an earlier kernel of the call has set hard[0] = 0
 };
-constexpr int kMaxOps = 3;   // operands per slice()
+constexpr int kMaxOps = 5;   // operands per slice()
 
 constexpr int kGroupBytes = kParts64 * 8 * kKB * 2;      // one row group of one block
-inline int64_t image_rows(int64_t rows) { return (rows + 127) / 128 * 128; }
+// Rows are padded to 16; a tile that reaches past them reads the next block's
+// first rows (or the kTailBytes behind the image), which only reach entries
+// that are not stored.
+inline int64_t image_rows(int64_t rows) { return (rows + 15) / 16 * 16; }
+constexpr int kTailBytes = 16 * kGroupBytes;
 inline int64_t image_blocks(int64_t K) { return (K + kKB - 1) / kKB; }
 size_t operand_bytes(int64_t rows, int64_t K);
 // Carves an operand's buffers out of `ws` (256-byte aligned); its row list is
@@ -71,9 +75,13 @@ struct Out64 {
     const double* rscale;
     const double* cscale;
     int* clear = nullptr;    // a later operand's hard[0], set to 0 on the way (split only)
+    double* mirror = nullptr;    // C(i, j) also at mirror[j cr + i cc] (split only)
 };
 size_t part_bytes(int64_t M, int64_t N);
 lrc_status product(const Operand64& A, const Operand64& B, const Out64& out, bool split, double* part, cudaStream_t s);
+// C(i, j) = C(j, i) at C[i ldc + j]: A A^T, `part` as above.  Tiles below the
+// diagonal are left out.
+lrc_status gram(const Operand64& A, double* C, int64_t ldc, double* part, cudaStream_t s);
 
 }  // namespace sg
 }  // namespace lrc
