@@ -44,6 +44,8 @@
 
 #include <mutex>
 
+#include <type_traits>
+
 #include "common.cuh"
 #include "tc.cuh"
 
@@ -847,24 +849,55 @@ __device__ __forceinline__ void y_body(const CUtensorMap* tm_u, const CUtensorMa
                                 sb + rr * 128 + (((lane >> 2) ^ (rr & 7)) * 16) + (lane & 3) * 4);
                         if (a.out16) {
                             const int c = 2 * lane;
-#pragma unroll
-                            for (int rr = 0; rr < 32; ++rr) {
-                                if (rr >= nrows) break;
-                                uint16_t* y = static_cast<uint16_t*>(a.Y) + (rbase + rr) * a.m + col0 + c;
-                                const uint32_t w = wv[rr];
-                                if (c + 1 < nvalid && ((reinterpret_cast<uintptr_t>(y) & 3u) == 0)) {
-                                    *reinterpret_cast<uint32_t*>(y) = w;
+                            uint16_t* y = static_cast<uint16_t*>(a.Y) + rbase * a.m + col0 + c;
+                            // full 32 x 64 boxes without a branch per row: the rows of an
+                            // odd-pitched Y alternate between word-aligned and not
+                            auto put = [&](auto aligned, uint16_t* q, uint32_t w) {
+                                if constexpr (decltype(aligned)::value) {
+                                    *reinterpret_cast<uint32_t*>(q) = w;
                                 } else {
-                                    if (c < nvalid) y[0] = (uint16_t)(w & 0xffffu);
-                                    if (c + 1 < nvalid) y[1] = (uint16_t)(w >> 16);
+                                    q[0] = (uint16_t)(w & 0xffffu);
+                                    q[1] = (uint16_t)(w >> 16);
+                                }
+                            };
+                            auto full = [&](auto even_rows, auto odd_rows) {
+#pragma unroll
+                                for (int rr = 0; rr < 32; rr += 2) {
+                                    put(even_rows, y + (int64_t)rr * a.m, wv[rr]);
+                                    put(odd_rows, y + (int64_t)(rr + 1) * a.m, wv[rr + 1]);
+                                }
+                            };
+                            const bool al = (reinterpret_cast<uintptr_t>(y) & 3u) == 0;
+                            if (nrows == 32 && nvalid == ecols) {
+                                if (a.m & 1) {
+                                    if (al) full(std::true_type{}, std::false_type{});
+                                    else full(std::false_type{}, std::true_type{});
+                                } else if (al) {
+                                    full(std::true_type{}, std::true_type{});
+                                } else {
+                                    full(std::false_type{}, std::false_type{});
+                                }
+                            } else {
+#pragma unroll
+                                for (int rr = 0; rr < 32; ++rr) {
+                                    if (rr >= nrows) break;
+                                    uint16_t* q = y + (int64_t)rr * a.m;
+                                    const uint32_t w = wv[rr];
+                                    if (c < nvalid) q[0] = (uint16_t)(w & 0xffffu);
+                                    if (c + 1 < nvalid) q[1] = (uint16_t)(w >> 16);
                                 }
                             }
                         } else if (lane < nvalid) {
                             uint32_t* y = static_cast<uint32_t*>(a.Y) + rbase * a.m + col0 + lane;
+                            if (nrows == 32) {
 #pragma unroll
-                            for (int rr = 0; rr < 32; ++rr) {
-                                if (rr >= nrows) break;
-                                y[(int64_t)rr * a.m] = wv[rr];
+                                for (int rr = 0; rr < 32; ++rr) y[(int64_t)rr * a.m] = wv[rr];
+                            } else {
+#pragma unroll
+                                for (int rr = 0; rr < 32; ++rr) {
+                                    if (rr >= nrows) break;
+                                    y[(int64_t)rr * a.m] = wv[rr];
+                                }
                             }
                         }
                     }
