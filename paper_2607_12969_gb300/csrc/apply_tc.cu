@@ -1362,6 +1362,13 @@ lrc_status encode_map_2d(CUtensorMap* map, CUtensorMapDataType dt, const void* b
                     swizzle128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE);
 }
 
+lrc_status encode_map_2d_sw64(CUtensorMap* map, CUtensorMapDataType dt, const void* base, int64_t cols, int64_t rows,
+                              int64_t pitch_bytes, uint32_t box_cols, uint32_t box_rows, const char* what) {
+    lrc_status st = get_encoder();
+    if (st != LRC_OK) return st;
+    return make_map(map, dt, base, cols, rows, pitch_bytes, box_cols, box_rows, what, CU_TENSOR_MAP_SWIZZLE_64B);
+}
+
 lrc_status y_product_plan(int64_t m, int64_t b, int kp, bool out16, int* n2) {
     YArgs a{};
     size_t smem = 0;

@@ -198,6 +198,10 @@ lrc_status encode_map_2d(CUtensorMap* map, CUtensorMapDataType dt, const void* b
                          int64_t pitch_bytes, uint32_t box_cols, uint32_t box_rows, bool swizzle128,
                          const char* what);
 
+// The same with the 64-byte swizzle.
+lrc_status encode_map_2d_sw64(CUtensorMap* map, CUtensorMapDataType dt, const void* base, int64_t cols, int64_t rows,
+                              int64_t pitch_bytes, uint32_t box_cols, uint32_t box_rows, const char* what);
+
 // Device error words of the tensor-core kernels (bounded waits that gave up);
 // read and cleared by lrc_device_status().  0xffffffff = could not be read.
 uint32_t take_apply_tc_error();

@@ -328,7 +328,7 @@ struct GemmArgs {
     int ntiles, tiles;       // tiles of B; all tiles
     int chunks;              // 64-column chunks of the reduction
     int kblocks;             // 16-column blocks
-    int split, group, stages, vec;
+    int split, group, stages, tma;
     int64_t a_block, b_block;    // bytes of a block of either image
     uint32_t a_bytes, b_bytes;   // of a tile's part of it
     int listed;                  // > 0: the tiles are list[0 ... listed), row << 8 | column
@@ -355,6 +355,7 @@ __device__ __forceinline__ int2 tile_at(const GemmArgs& a, int tile) {
 
 constexpr int kChunkBlocks = 64 / kKB;
 constexpr uint32_t kCtrlBytes = 1024;
+constexpr int kStageBytes = 32 * 64;           // a warp's rows on their way out
 
 // Chunks between drains of a class's accumulator: its sums stay at most 2^24
 // (classes 5 and 6: see above).  A converting drain costs an entry 8 clocks of
@@ -462,9 +463,10 @@ __device__ __forceinline__ void issue(uint32_t tmem, uint32_t col3, uint32_t fre
 }
 
 template <int NT>
-__global__ void __launch_bounds__(kThreads, 1) product_kernel(const __grid_constant__ GemmArgs a) {
+__global__ void __launch_bounds__(kThreads, 1) product_kernel(const __grid_constant__ GemmArgs a,
+                                                              const __grid_constant__ CUtensorMap tm_c) {
     constexpr int HC = NT / 4;          // columns a thread drains
-    extern __shared__ __align__(128) unsigned char smem[];
+    extern __shared__ __align__(1024) unsigned char smem[];
     uint64_t* full = reinterpret_cast<uint64_t*>(smem);
     uint64_t* empty = full + 8;
     uint64_t* gfull = empty + 8;        // classes 0 to 3 of an even or odd chunk complete; classes 4 to 6
@@ -504,16 +506,18 @@ __global__ void __launch_bounds__(kThreads, 1) product_kernel(const __grid_const
         const int g = warp & 3, quarter = (warp - 4) >> 2;      // of the lanes, of the columns
         const uint32_t tbase = tmem + ((uint32_t)(g * 32) << 16) + quarter * HC;
         const int r = g * 32 + lane;
+        unsigned char* stage = ring + (size_t)a.stages * stage_bytes + (size_t)(warp - 4) * kStageBytes;
         Pieces<GemmArgs> pc(a);
         int tile, c0, c1;
         int ch = 0;
         bool ok = true;
-        // one warp polls the mbarrier, the others sleep at the named barrier
-        // (512 polling threads would take the MMA issuer's issue slots)
+        // One lane of a warp polls (512 polling threads would take the MMA issuer's
+        // issue slots), and the warps do not wait for one another: while one drains,
+        // on the conversion and FMA pipes, another rounds, on the integer pipe.
         auto epi_wait = [&](uint64_t* bar, uint32_t parity) {
-            if (warp == 4) mbar_wait(bar, parity, abort, err, 4u);
-            named_bar_sync(1, 32 * kEpiWarps);
-            return *abort == 0;
+            bool got = true;
+            if (lane == 0) got = mbar_wait(bar, parity, abort, err, 4u);
+            return __all_sync(0xffffffffu, got) != 0;
         };
         while (ok && pc.next(a, &tile, &c0, &c1)) {
             const int2 at = tile_at(a, tile);
@@ -550,33 +554,61 @@ __global__ void __launch_bounds__(kThreads, 1) product_kernel(const __grid_const
                 for (int j = 0; j < HC; ++j) dst[j * 128] = round_pq(P[j], Q[j], ea + __shfl_sync(0xffffffffu, eb, j));
                 continue;
             }
-            double* dst = a.C + row * a.cr + col0 * a.cc;
             const bool shallow = a.chunks <= 8;      // |P| stays below 2^50
+            auto value = [&](int j) {
+                const int es = ea + __shfl_sync(0xffffffffu, eb, j);
+                return shallow && ((0x52 >> (j & 7)) & 1) ? round_pq_fp64(P[j], Q[j], es) : round_pq(P[j], Q[j], es);
+            };
+            if (a.cc == 1) {
+                // 32 rows x CG columns at a time through shared memory (64-byte rows in
+                // the 64-byte swizzle, or 32-byte rows) and out by TMA, or where a row's pitch does
+                // not allow that by runs of CG: stores straight from the registers, 32
+                // bytes a row, filled the load/store unit
+                constexpr int CG = HC % 8 == 0 ? 8 : 4;
 #pragma unroll
-            for (int j0 = 0; j0 < HC; j0 += 4) {
-                double y[4];
+                for (int j0 = 0; j0 < HC; j0 += CG) {
+                    double y[CG];
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const int es = ea + __shfl_sync(0xffffffffu, eb, j0 + j);
-                    y[j] = shallow && ((0x52 >> ((j0 + j) & 7)) & 1) ? round_pq_fp64(P[j0 + j], Q[j0 + j], es)
-                                                                     : round_pq(P[j0 + j], Q[j0 + j], es);
-                }
-                if (row < a.M) {
-                    // a whole 32-byte sector a lane where the rows allow it
-                    if (a.vec == 2 && col0 + j0 + 4 <= a.N) {
-                        asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};"
-                                     ::"l"(dst + j0), "d"(y[0]), "d"(y[1]), "d"(y[2]), "d"(y[3]) : "memory");
-                    } else if (a.vec == 1 && col0 + j0 + 4 <= a.N) {
-                        reinterpret_cast<double2*>(dst + j0)[0] = make_double2(y[0], y[1]);
-                        reinterpret_cast<double2*>(dst + j0)[1] = make_double2(y[2], y[3]);
-                    } else {
+                    for (int j = 0; j < CG; ++j) y[j] = value(j0 + j);
+                    if (a.tma && lane == 0) bulk_wait_read<0>();      // the store before has read the buffer
+                    __syncwarp();
 #pragma unroll
-                        for (int j = 0; j < 4; ++j)
-                            if (col0 + j0 + j < a.N) dst[(j0 + j) * a.cc] = y[j];
+                    for (int j = 0; j < CG; j += 2) {
+                        const int c = CG == 8 ? (j >> 1) ^ ((lane >> 1) & 3) : j >> 1;
+                        *reinterpret_cast<double2*>(stage + lane * (CG * 8) + c * 16) = make_double2(y[j], y[j + 1]);
                     }
+                    const int64_t rb = (int64_t)mt * 128 + g * 32;
+                    if (a.tma) {
+                        fence_proxy_async_smem();
+                        __syncwarp();
+                        if (lane == 0 && rb < a.M && col0 + j0 < a.N) {
+                            tma_store_2d(&tm_c, (int32_t)(col0 + j0), (int32_t)rb, stage);
+                            bulk_commit();
+                        }
+                    } else {
+                        __syncwarp();
+                        const int q = lane % CG, r0 = lane / CG;
+                        double* dst = a.C + (rb + r0) * a.cr + col0 + j0 + q;
+                        const bool mine = col0 + j0 + q < a.N;
+#pragma unroll
+                        for (int i = 0; i < CG; ++i) {
+                            const int rr = i * (32 / CG) + r0;
+                            const int c = CG == 8 ? (q >> 1) ^ ((rr >> 1) & 3) : q >> 1;
+                            const double d = *reinterpret_cast<const double*>(stage + rr * (CG * 8) + c * 16 + (q & 1) * 8);
+                            if (mine && rb + rr < a.M) dst[(int64_t)i * (32 / CG) * a.cr] = d;
+                        }
+                    }
+                }
+            } else {
+                double* dst = a.C + row * a.cr + col0 * a.cc;
+#pragma unroll
+                for (int j = 0; j < HC; ++j) {
+                    const double y = value(j);
+                    if (row < a.M && col0 + j < a.N) dst[j * a.cc] = y;
                 }
             }
         }
+        if (a.tma && lane == 0) bulk_wait<0>();
     } else {
         reg_dec<kRegsLow>();
         if (warp == 0) {
@@ -836,10 +868,10 @@ int stat_splits(int64_t rows, int64_t K) {
 }
 
 template <int NT>
-lrc_status launch_product(const GemmArgs& a, int64_t grid, size_t smem, cudaStream_t s) {
+lrc_status launch_product(const GemmArgs& a, const CUtensorMap& tm, int64_t grid, size_t smem, cudaStream_t s) {
     cudaError_t e = cudaFuncSetAttribute(product_kernel<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return cuda_fail(e, "split product_kernel smem attribute");
-    e = launch_pdl(product_kernel<NT>, dim3((unsigned)grid), dim3(kThreads), smem, s, a);
+    e = launch_pdl(product_kernel<NT>, dim3((unsigned)grid), dim3(kThreads), smem, s, a, tm);
     if (e != cudaSuccess) return cuda_fail(e, "split product_kernel launch");
     return after_launch("split product_kernel");
 }
@@ -981,9 +1013,20 @@ lrc_status run_product(const Operand64& A0, const Operand64& B0, const Out64& ou
     a.b_block = image_rows(B.rows) / 8 * kGroupBytes;
     a.a_bytes = 128 / 8 * kGroupBytes;
     a.b_bytes = (uint32_t)(NT / 8 * kGroupBytes);
-    a.stages = (int)std::min<int64_t>(8, (int64_t)(227 * 1024 - kCtrlBytes) / (a.a_bytes + a.b_bytes));
-    a.vec = out.cc != 1 || out.cr % 2 != 0 || !aligned16(out.C) ? 0
-            : out.cr % 4 == 0 && (reinterpret_cast<uintptr_t>(out.C) & 31u) == 0 ? 2 : 1;
+    CUtensorMap tm{};
+    a.tma = !split && out.cc == 1 && out.cr % 2 == 0 && aligned16(out.C);
+    lrc_status st;
+    if (a.tma) {
+        const bool wide = NT % 32 == 0;      // columns a warp stores at a time: 8, else 4
+        st = wide ? encode_map_2d_sw64(&tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, out.C, B.rows, A.rows, out.cr * 8, 8, 32,
+                                       "split product output")
+                  : encode_map_2d(&tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, out.C, B.rows, A.rows, out.cr * 8, 4, 32, false,
+                                  "split product output");
+        if (st != LRC_OK) return st;
+    }
+    // (a chunk's blocks are all in the ring at once: at least kChunkBlocks stages)
+    const size_t staging = !split && out.cc == 1 ? (size_t)kEpiWarps * kStageBytes : 0;
+    a.stages = (int)std::min<int64_t>(8, (int64_t)(227 * 1024 - kCtrlBytes - staging) / (a.a_bytes + a.b_bytes));
     uint32_t cols = 32;
     while (cols < (uint32_t)(8 * NT)) cols *= 2;
     a.tmem_cols = cols;
@@ -993,13 +1036,12 @@ lrc_status run_product(const Operand64& A0, const Operand64& B0, const Out64& ou
     const int64_t Q = tiles / a.group * a.chunks;
     const int64_t groups = std::min<int64_t>(Q, sms / a.group);
     const int64_t grid = split ? groups * a.group : std::min<int64_t>(tiles, sms);
-    const size_t smem = kCtrlBytes + (size_t)a.stages * (a.a_bytes + a.b_bytes);
-    lrc_status st;
+    const size_t smem = kCtrlBytes + (size_t)a.stages * (a.a_bytes + a.b_bytes) + staging;
     switch (NT) {
-        case 16: st = launch_product<16>(a, grid, smem, s); break;
-        case 32: st = launch_product<32>(a, grid, smem, s); break;
-        case 48: st = launch_product<48>(a, grid, smem, s); break;
-        default: st = launch_product<64>(a, grid, smem, s); break;
+        case 16: st = launch_product<16>(a, tm, grid, smem, s); break;
+        case 32: st = launch_product<32>(a, tm, grid, smem, s); break;
+        case 48: st = launch_product<48>(a, tm, grid, smem, s); break;
+        default: st = launch_product<64>(a, tm, grid, smem, s); break;
         
     }
     if (st != LRC_OK) return st;
