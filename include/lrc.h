@@ -64,8 +64,9 @@ typedef enum {
     LRC_F16 = 2,      /* binary16 storage, binary32 accumulation, binary32 output           */
     LRC_F16_O16 = 3,  /* binary16 storage, binary32 accumulation, binary16 workspaces and
                          output: the method-precision FP16 path of Sec. 3.4                 */
-    LRC_F32_TC = 4,   /* binary32 storage and output; the output product of lrc_apply and
-                         tt_reconstruct on the tensor cores: each binary32 operand is scaled
+    LRC_F32_TC = 4,   /* binary32 storage and output; where LRC_F32 uses FMAs the output
+                         product of lrc_apply and tt_reconstruct on the tensor cores: each
+                         binary32 operand is scaled
                          by a power of two per 32 rows and split into binary16 parts
                          hi + lo, and Z S ~ Z_hi S_hi + Z_lo S_hi + Z_hi S_lo accumulates in
                          binary32 (about 22 significand bits per operand).  A variant of
@@ -236,9 +237,10 @@ LRC_API lrc_status lrc_apply_batched(int count, const void* const* U, const void
  * lrc_apply), with Z_l, S_l and the digits in the stream's workspace, or where
  * there is no memory for them by the FMA kernels.  Asynchronous on `stream`.
  */
-/* LRC_F32_TC: binary32 cores and output; the chain's output product on the
- * tensor cores when the chain's sides fit its one-pass side kernel
- * (bond rank <= 64), otherwise the LRC_F32 kernels. */
+/* LRC_F32: chains whose cores fit the one-pass side kernel (bond rank <= 64)
+ * and output products of at least 2.5e9 flops run on the tensor cores from
+ * bfloat16 parts (see lrc_apply), others on FMAs.
+ * LRC_F32_TC: the same; other output products from scaled binary16 parts. */
 LRC_API lrc_status tt_reconstruct(const void* const* cores, const int64_t* dims, const int64_t* ranks,
                           int d, lrc_fmt fmt, void* out, lrc_stream_t stream);
 

@@ -251,7 +251,7 @@ lrc_status tt_reconstruct(const void* const* cores, const int64_t* dims, const i
     if (fmt == LRC_BF16) return launch_tt_bf16(sh, out, s);
     if (fmt == LRC_F32_TC) {
         bool handled = false;
-        st = launch_tt_split_f32tc(sh, static_cast<float*>(out), s, &handled);
+        st = launch_tt_split_f32(sh, static_cast<float*>(out), s, &handled);
         if (st != LRC_OK || handled) return st;
         return launch_tt_chain_f32tc(sh, static_cast<float*>(out), s);
     }

@@ -174,9 +174,9 @@ lrc_status launch_tt_f16(const TTShape& sh, bool out16, void* out, cudaStream_t 
 // binary16 TT as a product chain with the output product on the tensor cores
 // (tt_split.cu); *handled = false when the shape is outside it (nothing launched)
 lrc_status launch_tt_split_f16(const TTShape& sh, bool out16, void* out, cudaStream_t s, bool* handled);
-// the same product chain for binary32 cores (LRC_F32_TC): both operands split
-// into scaled hi/lo binary16 parts; *handled = false when the shape is outside it
-lrc_status launch_tt_split_f32tc(const TTShape& sh, float* out, cudaStream_t s, bool* handled);
+// the same product chain for binary32 cores: both operands in three bfloat16
+// parts; *handled = false when the shape is outside it
+lrc_status launch_tt_split_f32(const TTShape& sh, float* out, cudaStream_t s, bool* handled);
 // bfloat16 cores, bfloat16 workspaces and output: the same product chain with
 // bfloat16 tensor-core operands where the shape fits it, else the CUDA-core
 // chain of tt_cc.cu

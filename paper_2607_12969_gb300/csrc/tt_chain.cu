@@ -21,6 +21,7 @@
 
 #include "common.cuh"
 #include "split_gemm.cuh"
+#include "split_gemm32.cuh"
 
 namespace lrc {
 
@@ -75,7 +76,11 @@ lrc_status product(const double* A, int64_t lda, const double* B, int64_t ldb, d
     return gemm_cc_f64(A, lda, B, ldb, C, ldc, M, N, K, s);
 }
 
-// tc_final (binary32 only): the output product on the tensor cores through
+// Output products of binary32 chains go through bfloat16 parts from here on
+// (512 x 512 x 224, ranks 70, 52: 6.1e9 flops).
+constexpr double kPartsFlops = 2.5e9;
+
+// tc_final (binary32 only): a smaller output product on the tensor cores through
 // the scaled binary16 split (LRC_F32_TC) when the product kernel takes it.
 template <typename T>
 lrc_status launch_chain(const TTShape& sh, T* out, cudaStream_t s, bool tc_final = false) {
@@ -99,12 +104,25 @@ lrc_status launch_chain(const TTShape& sh, T* out, cudaStream_t s, bool tc_final
     }
     unsigned char* ws = nullptr;
     const int64_t rc = sh.ranks[c];
-    const bool tc = tc_final && sizeof(T) == 4 && split_product_fits(P[c], Q[c], rc);
-    const size_t tsz = tc ? round256(split_product_bytes(P[c], Q[c], rc)) : 0;
-    const size_t total = lsz[0] + lsz[1] + rsz[0] + rsz[1] + tsz;
-    if (total > 0) {
+    const size_t sides = lsz[0] + lsz[1] + rsz[0] + rsz[1];
+    // binary32: a large output product in bfloat16 parts (split_gemm32.cu), where
+    // there is workspace for them
+    sg32::Operand oz{nullptr, rc, 1, P[c], rc, nullptr, nullptr}, os{nullptr, 1, Q[c], Q[c], rc, nullptr, nullptr};
+    const size_t zi = round256(sg32::image_bytes(P[c], rc)), si = round256(sg32::image_bytes(Q[c], rc));
+    bool parts = sizeof(T) == 4 && 2.0 * (double)P[c] * (double)Q[c] * (double)rc >= kPartsFlops;
+    if (parts) {
         void* p = nullptr;
-        lrc_status st = stream_workspace(s, total, &p);
+        const lrc_status st = stream_workspace_try(
+            s, sides + zi + si + sg32::hard_bytes(P[c]) + sg32::hard_bytes(Q[c]), &p);
+        if (st != LRC_OK) return st;
+        parts = p != nullptr;
+        ws = static_cast<unsigned char*>(p);
+    }
+    const bool tc = !parts && tc_final && sizeof(T) == 4 && split_product_fits(P[c], Q[c], rc);
+    const size_t tsz = tc ? round256(split_product_bytes(P[c], Q[c], rc)) : 0;
+    if (!parts && sides + tsz > 0) {
+        void* p = nullptr;
+        lrc_status st = stream_workspace(s, sides + tsz, &p);
         if (st != LRC_OK) return st;
         ws = static_cast<unsigned char*>(p);
     }
@@ -127,6 +145,20 @@ lrc_status launch_chain(const TTShape& sh, T* out, cudaStream_t s, bool tc_final
         S = dst;
     }
     if constexpr (sizeof(T) == 4) {
+        if (parts) {
+            unsigned char* q = ws + sides;
+            oz.p = Z;
+            os.p = S;
+            oz.img = q;
+            os.img = q + zi;
+            oz.hard = reinterpret_cast<int*>(q + zi + si);
+            os.hard = reinterpret_cast<int*>(q + zi + si + sg32::hard_bytes(P[c]));
+            const cudaError_t e = cudaMemsetAsync(oz.hard, 0, sg32::hard_bytes(P[c]) + sg32::hard_bytes(Q[c]), s);
+            if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync (row lists)");
+            const sg32::Operand* ops[2] = {&oz, &os};
+            if ((st = sg32::split(ops, 2, s)) != LRC_OK) return st;
+            return sg32::product(oz, os, out, Q[c], nullptr, false, nullptr, s);
+        }
         // Z is P x r (row pitch r), S is r x Q (row pitch Q): B = S^T
         if (tc)
             return launch_split_product(Z, rc, 1, S, 1, Q[c], P[c], Q[c], rc,
@@ -139,8 +171,10 @@ lrc_status launch_chain(const TTShape& sh, T* out, cudaStream_t s, bool tc_final
 
 lrc_status launch_tt_chain_f32(const TTShape& sh, float* out, cudaStream_t s) {
     bool handled = false;
-    const lrc_status st = launch_tt_side_f32(sh, out, s, &handled);
-    if (handled) return st;
+    lrc_status st = launch_tt_split_f32(sh, out, s, &handled);
+    if (st != LRC_OK || handled) return st;
+    st = launch_tt_side_f32(sh, out, s, &handled);
+    if (st != LRC_OK || handled) return st;
     return launch_chain<float>(sh, out, s);
 }
 

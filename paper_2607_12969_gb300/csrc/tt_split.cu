@@ -13,8 +13,7 @@
 // the output traffic.
 //
 // Operands of that product are binary16 with binary32 accumulation (Sec. 3.4).
-// An operand that is a stored binary16 core is exact in binary16; binary32
-// cores (the LRC_F32_TC variant) take the hi/lo split below on both sides.  An operand the
+// An operand that is a stored binary16 core is exact in binary16.  An operand the
 // chain computed is binary32; for a binary32 output it enters the product as
 // a pair hi = fp16(x), lo = fp16(x - hi) laid side by side along the
 // reduction, so one product of concatenated operands forms
@@ -29,6 +28,14 @@
 // bfloat16 cores (LRC_BF16) take the same chain with bfloat16 operand images
 // rounded once (the format's method-precision workspace) and a bfloat16
 // tensor-core product.
+// binary32 cores take it with three bfloat16 parts of both operands, x = hi +
+// mid + lo (exactly), and the six largest products of parts along one
+// reduction, hi hi last: the tensor cores cut sums off at every step of 16
+// terms, in one direction, so the steps at the result's full size are few (16^6,
+// rank 26: distance from the exact tensor 1.8e-7, with an FMA product 2.0e-7, in
+// 39 us instead of 42).  Units
+// of Z or S that hold an infinity or a NaN are marked in their scale, and the
+// entries they reach are formed from the images by tt_repair_kernel.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
@@ -41,14 +48,15 @@ namespace lrc {
 namespace {
 
 constexpr int BM = 128;
-constexpr int kMaxParts = 3;
+constexpr int kMaxParts = 3, kMaxParts32 = 6;
+constexpr int kBadUnit = 1000;     // scale that marks a unit with an infinity or a NaN
 constexpr int kUnit = 32;      // rows of Z or columns of S per CTA of the side kernel (one scale group)
 
-// Part kinds of an operand laid along the reduction: bit p of `lomask` set =
-// part p is the lo half, otherwise the hi half (or the single rounding).
+// Part kinds of an operand laid along the reduction, two bits a part: 0 the hi
+// part (or the single rounding), 1 the next, 2 the one after that.
 struct Parts {
     int n;
-    int lomask;
+    int kinds;
 };
 
 // e with max * 2^e in [2^14, 2^15), clamped to [-60, 60] (so that the
@@ -61,20 +69,51 @@ __device__ __forceinline__ int scale_exp(float maxabs) {
     return e < -60 ? -60 : (e > 60 ? 60 : e);
 }
 
+// Does a unit of a binary32 chain with this largest magnitude hold an infinity or
+// a NaN (or come so near the range's end that hi would overflow)?
+template <typename TC>
+__device__ __forceinline__ bool marked(float maxabs) {
+    return std::is_same_v<TC, float> && !(maxabs <= 3.0e38f);
+}
+
 // 2^e for |e| <= 126
 __device__ __forceinline__ float pow2(int e) { return __int_as_float((127 + e) << 23); }
 
-__device__ __forceinline__ __half part_value(float y, bool lo) {
+__device__ __forceinline__ __half part_value(float y, int kind) {
     const __half hi = __float2half_rn(y);
-    return lo ? __float2half_rn(y - __half2float(hi)) : hi;
+    return kind ? __float2half_rn(y - __half2float(hi)) : hi;
 }
 
-// Encoding of one operand-image element: binary16 parts, or one bfloat16
-// rounding (the bfloat16 chain has a single part).
-template <bool BF>
-__device__ __forceinline__ uint16_t image_bits(float y, bool lo) {
-    if constexpr (BF) return tc::to_bf16_bits(y);
-    else return __half_as_ushort(part_value(y, lo));
+// Part `kind` of the three bfloat16 parts of y (an infinity or NaN is all hi;
+// where the nearest hi would be infinite, the one below).
+__device__ __forceinline__ uint16_t part32_bits(float y, int kind) {
+    const bool finite = fabsf(y) <= 3.402823466e38f;
+    uint32_t hi = tc::to_bf16_bits(y);
+    if (finite && (hi & 0x7fffu) == 0x7f80u) hi = __float_as_uint(y) >> 16;
+    if (kind == 0) return (uint16_t)hi;
+    if (!finite) return 0;
+    const float r = y - tc::bf16_bits_to_float(hi);
+    const uint32_t mid = tc::to_bf16_bits(r);
+    return kind == 1 ? (uint16_t)mid : tc::to_bf16_bits(r - tc::bf16_bits_to_float(mid));
+}
+
+// Running maximum of magnitudes; of binary32 chains an infinity or NaN counts as
+// infinite (fmaxf would drop a NaN).
+template <typename TC>
+__device__ __forceinline__ float max_mag(float m, float y) {
+    const float v = fabsf(y);
+    if constexpr (std::is_same_v<TC, float>) return v <= 3.0e38f ? fmaxf(m, v) : INFINITY;
+    else return fmaxf(m, v);
+}
+
+// Encoding of one operand-image element: binary16 parts of binary16 cores'
+// chains, one bfloat16 rounding (a single part) of bfloat16 cores', bfloat16
+// parts of binary32 cores'.
+template <typename TC>
+__device__ __forceinline__ uint16_t image_bits(float y, int kind) {
+    if constexpr (std::is_same_v<TC, float>) return part32_bits(y, kind);
+    else if constexpr (std::is_same_v<TC, __nv_bfloat16>) return tc::to_bf16_bits(y);
+    else return __half_as_ushort(part_value(y, kind));
 }
 
 __device__ __forceinline__ float block_max(float v, float* sh) {
@@ -280,7 +319,6 @@ __device__ float* right_cols(const SideArgs& a, int64_t q0, int64_t qend, float*
 template <typename TC, bool IMG>
 __global__ void __launch_bounds__(256)
 tt_side_kernel(const SideArgs a) {
-    constexpr bool BF = std::is_same_v<TC, __nv_bfloat16>;
     extern __shared__ float sbuf[];
     __shared__ float red[8];
     tc::pdl_wait();
@@ -302,24 +340,24 @@ tt_side_kernel(const SideArgs a) {
         }
         float mx = 0.0f;
         for (int e = threadIdx.x; e < nrow * a.r; e += blockDim.x)
-            mx = fmaxf(mx, fabsf(z[(e / a.r) * a.ldb + e % a.r]));
+            mx = max_mag<TC>(mx, z[(e / a.r) * a.ldb + e % a.r]);
         const float tmax = block_max(mx, red);
         const int ex = a.scale_w ? scale_exp(tmax) : 0;
         const float f = pow2(ex);
         tc::pdl_trigger();
-        if (threadIdx.x == 0) a.esc_w[t] = ex;
+        if (threadIdx.x == 0) a.esc_w[t] = marked<TC>(tmax) ? kBadUnit : ex;
         unsigned char* tile = a.Wimg + (size_t)(p0 / BM) * BM * kp * 2;
         const int ro = (int)(p0 % BM);
         // one thread per (row, 8-column group), rows fastest: a warp writes 512 contiguous bytes
         for (int i = threadIdx.x; i < kUnit * (kp / 8); i += blockDim.x) {
             const int row = i % kUnit, c0 = (i / kUnit) * 8;
             const int p = c0 / a.rp, a0 = c0 - p * a.rp;
-            const bool lo = (a.pw.lomask >> p) & 1;
+            const int kind = (a.pw.kinds >> (2 * p)) & 3;
             __align__(16) uint16_t h[8];
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
                 const int k = a0 + j;
-                h[j] = (k < a.r && row < nrow) ? image_bits<BF>(z[row * a.ldb + k] * f, lo) : (uint16_t)0;
+                h[j] = (k < a.r && row < nrow) ? image_bits<TC>(z[row * a.ldb + k] * f, kind) : (uint16_t)0;
             }
             *reinterpret_cast<uint4*>(tile + tc::w_image_off((uint32_t)(ro + row), (uint32_t)c0)) =
                 *reinterpret_cast<const uint4*>(h);
@@ -342,26 +380,64 @@ tt_side_kernel(const SideArgs a) {
         }
         float mx = 0.0f;
         for (int e = threadIdx.x; e < nq * a.r; e += blockDim.x)
-            mx = fmaxf(mx, fabsf(sc[(base + e / a.r) * a.ldb + e % a.r]));
+            mx = max_mag<TC>(mx, sc[(base + e / a.r) * a.ldb + e % a.r]);
         const float tmax = block_max(mx, red);
         const int ex = a.scale_u ? scale_exp(tmax) : 0;
         const float f = pow2(ex);
         tc::pdl_trigger();
-        if (threadIdx.x == 0) a.esc_u[t] = ex;
+        if (threadIdx.x == 0) a.esc_u[t] = marked<TC>(tmax) ? kBadUnit : ex;
         const int groups = kp / 8;
         // one thread per (row of U, 8-column group), groups fastest: a warp writes contiguous rows
         for (int i = threadIdx.x; i < nq * groups; i += blockDim.x) {
             const int q = i / groups, c0 = (i - q * groups) * 8;
             const int p = c0 / a.rp, a0 = c0 - p * a.rp;
-            const bool lo = (a.pu.lomask >> p) & 1;
+            const int kind = (a.pu.kinds >> (2 * p)) & 3;
             const float* col = sc + (base + q) * a.ldb;
             __align__(16) uint16_t h[8];
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
                 const int k = a0 + j;
-                h[j] = (k < a.r) ? image_bits<BF>(col[k] * f, lo) : (uint16_t)0;
+                h[j] = (k < a.r) ? image_bits<TC>(col[k] * f, kind) : (uint16_t)0;
             }
             *reinterpret_cast<uint4*>(a.Uimg + (q0 + q) * kp + c0) = *reinterpret_cast<const uint4*>(h);
+        }
+    }
+}
+
+// Entries whose row or column lies in a marked unit, from the images: binary32
+// FMAs over hi + mid + lo (parts 2, 1, 0 of a row of Z; 0, 1, 2 of one of S).
+__global__ void __launch_bounds__(256) tt_repair_kernel(const SideArgs a, float* __restrict__ out) {
+    tc::pdl_wait();
+    tc::pdl_trigger();
+    const int64_t units = a.wunits + (a.Q + kUnit - 1) / kUnit;      // esc_u follows esc_w
+    bool any = false;
+    for (int64_t i = threadIdx.x; i < units; i += 256) any |= a.esc_w[i] == kBadUnit;
+    if (!__syncthreads_or(any)) return;
+    const int kp = kMaxParts32 * a.rp;
+    auto part = [](uint16_t h) { return tc::bf16_bits_to_float(h); };
+    auto scale = [](int e) { return pow2(e == kBadUnit ? 0 : -e); };
+    for (int64_t u = 0; u < units; ++u) {
+        if (a.esc_w[u] != kBadUnit) continue;
+        const bool ws = u < a.wunits;
+        const int64_t f0 = (ws ? u : u - a.wunits) * kUnit, lim = ws ? a.P : a.Q, other = ws ? a.Q : a.P;
+        const int64_t n = lim - f0 < kUnit ? lim - f0 : kUnit;
+        for (int64_t e = blockIdx.x * 256ll + threadIdx.x; e < n * other; e += gridDim.x * 256ll) {
+            const int64_t f = f0 + e % n, o = e / n, p = ws ? f : o, q = ws ? o : f;
+            const unsigned char* w = a.Wimg + (size_t)(p / BM) * BM * kp * 2;
+            const uint16_t* s = a.Uimg + q * kp;
+            const float fw = scale(a.esc_w[p / kUnit]), fs = scale(a.esc_u[q / kUnit]);
+            float acc = 0.0f;
+            for (int k = 0; k < a.r; ++k) {
+                float x[3];
+#pragma unroll
+                for (int i = 0; i < 3; ++i)
+                    x[i] = part(*reinterpret_cast<const uint16_t*>(
+                        w + tc::w_image_off((uint32_t)(p % BM), (uint32_t)((2 - i) * a.rp + k))));
+                const float z = (x[0] + (x[1] + x[2])) * fw;
+                const float y = (part(s[k]) + (part(s[a.rp + k]) + part(s[2 * a.rp + k]))) * fs;
+                acc = fmaf(z, y, acc);
+            }
+            out[p * a.Q + q] = acc;
         }
     }
 }
@@ -416,11 +492,13 @@ size_t side_smem(const TTShape& sh, const SideArgs& a) {
 namespace {
 
 // The split product chain for binary16 cores (TC = __half, stored cores exact
-// in binary16) or binary32 cores (TC = float: every operand split and scaled).
+// in binary16), bfloat16 cores, or binary32 cores (TC = float: every operand in
+// three bfloat16 parts).
 template <typename TC>
 lrc_status launch_split_t(const TTShape& sh, bool out16, void* out, cudaStream_t s, bool* handled) {
     constexpr bool kExactCores = sizeof(TC) == 2;
-    constexpr bool kBF = std::is_same_v<TC, __nv_bfloat16>;
+    constexpr bool kF32 = std::is_same_v<TC, float>;
+    constexpr bool kBF = !std::is_same_v<TC, __half>;      // bfloat16 operands of the product
     *handled = false;
     const int d = sh.d;
     if (d > 16) return LRC_OK;
@@ -430,23 +508,26 @@ lrc_status launch_split_t(const TTShape& sh, bool out16, void* out, cudaStream_t
     const bool z_core = kExactCores && (c == 1), s_core = kExactCores && (c == d - 1);   // operands exact in binary16
     // parts along the reduction (see the file comment)
     Parts pw{1, 0}, pu{1, 0};
-    if (!out16) {
+    if (kF32) {
+        pw = Parts{6, 2 | 1 << 2 | 1 << 6};           // [Z_lo | Z_mid | Z_hi | Z_mid | Z_hi | Z_hi]
+        pu = Parts{6, 1 << 2 | 2 << 4 | 1 << 8};      // [S_hi | S_mid | S_lo | S_hi | S_mid | S_hi]
+    } else if (!out16) {
         if (!z_core && !s_core) {
-            pw = Parts{3, 0b010};   // [Z_hi | Z_lo | Z_hi]
-            pu = Parts{3, 0b100};   // [S_hi | S_hi | S_lo]
+            pw = Parts{3, 1 << 2};   // [Z_hi | Z_lo | Z_hi]
+            pu = Parts{3, 1 << 4};   // [S_hi | S_hi | S_lo]
         } else if (!z_core) {
-            pw = Parts{2, 0b10};    // [Z_hi | Z_lo]
-            pu = Parts{2, 0b00};    // [S | S]
+            pw = Parts{2, 1 << 2};   // [Z_hi | Z_lo]
+            pu = Parts{2, 0};        // [S | S]
         } else if (!s_core) {
-            pw = Parts{2, 0b00};    // [Z | Z]
-            pu = Parts{2, 0b10};    // [S_hi | S_lo]
+            pw = Parts{2, 0};        // [Z | Z]
+            pu = Parts{2, 1 << 2};   // [S_hi | S_lo]
         }
     }
     const int kp = pw.n * rp;
     SideArgs a{};
     const int rmax = fill_side(sh, c, a);
     int n2 = 0;
-    if (kp > kMaxParts * 64 || rmax > 64 || y_product_plan(a.Q, a.P, kp, out16, &n2) != LRC_OK) return LRC_OK;
+    if (kp > (kF32 ? kMaxParts32 : kMaxParts) * 64 || rmax > 64 || y_product_plan(a.Q, a.P, kp, out16, &n2) != LRC_OK) return LRC_OK;
     const size_t smem = side_smem(sh, a);
     if (smem > 200 * 1024) return LRC_OK;
     *handled = true;
@@ -472,7 +553,11 @@ lrc_status launch_split_t(const TTShape& sh, bool out16, void* out, cudaStream_t
     e = launch_pdl(tt_side_kernel<TC, true>, dim3((unsigned)(a.wunits + uunits)), dim3(256), smem, s, a);
     if (e != cudaSuccess) return cuda_fail(e, "tt_side_kernel launch");
     if ((st = after_launch("tt_side_kernel")) != LRC_OK) return st;
-    return launch_y_product(a.Wimg, kp, a.Uimg, kp, a.Q, a.P, out16, out, a.esc_w, a.esc_u, s, false, kBF);
+    st = launch_y_product(a.Wimg, kp, a.Uimg, kp, a.Q, a.P, out16, out, a.esc_w, a.esc_u, s, false, kBF);
+    if (!kF32 || st != LRC_OK) return st;
+    e = launch_pdl(tt_repair_kernel, dim3((unsigned)(2 * sm_count())), dim3(256), 0, s, a, static_cast<float*>(out));
+    if (e != cudaSuccess) return cuda_fail(e, "tt_repair_kernel launch");
+    return after_launch("tt_repair_kernel");
 }
 
 }  // namespace
@@ -481,7 +566,7 @@ lrc_status launch_tt_split_f16(const TTShape& sh, bool out16, void* out, cudaStr
     return launch_split_t<__half>(sh, out16, out, s, handled);
 }
 
-lrc_status launch_tt_split_f32tc(const TTShape& sh, float* out, cudaStream_t s, bool* handled) {
+lrc_status launch_tt_split_f32(const TTShape& sh, float* out, cudaStream_t s, bool* handled) {
     return launch_split_t<float>(sh, false, out, s, handled);
 }
 

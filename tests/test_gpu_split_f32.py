@@ -108,3 +108,45 @@ def test_repeat_is_the_same_bits(lrc, cuda):
     f = W.random_factors(m, n, k, seed=14)
     X = W.gaussian((b, n), 15)
     assert np.array_equal(run(lrc, cuda, f.U, f.s, f.Vt, X), run(lrc, cuda, f.U, f.s, f.Vt, X))
+
+
+def chain(cores, dims):
+    z = cores[0].reshape(dims[0], -1)
+    with np.errstate(invalid="ignore", over="ignore"):
+        for c in cores[1:]:
+            z = (z @ c.reshape(c.shape[0], -1)).reshape(-1, c.shape[2])
+    return z.reshape(-1)
+
+
+# small cores (the side kernel's images), and an output product large enough for
+# the parts of split_gemm32.cu, with and without a 16-byte row pitch
+TT_SHAPES = [((16, 16, 16, 16), (1, 16, 26, 16, 1)), ((33, 17, 29, 31), (1, 30, 40, 20, 1)), ((64, 70, 60), (1, 12, 60, 1)),
+             ((400, 100, 1000), (1, 9, 36, 1)), ((300, 130, 1001), (1, 40, 33, 1))]
+
+
+@pytest.mark.parametrize("fmt,bad", [("f32", None), ("f32tc", None), ("f32", np.inf), ("f32", np.nan),
+                                     ("f32", -3.4028234e38)])
+@pytest.mark.parametrize("dims,ranks", TT_SHAPES)
+def test_tt(lrc, cuda, dims, ranks, fmt, bad):
+    """An infinity among positive cores makes its entries infinite, a NaN NaN,
+    whatever the order of the chain."""
+    rng = np.random.default_rng(5)
+    d = len(dims)
+    cores = [oracle.rounded(rng.standard_normal((ranks[l], dims[l], ranks[l + 1])), "f32") for l in range(d)]
+    if bad is not None:
+        cores = [oracle.rounded(np.abs(c) * 1e-3 + 1e-6, "f32") for c in cores]
+        cores[0][0, 3, 1] = bad
+        cores[-1][2, 5, 0] = bad if abs(bad) == np.inf else cores[-1][2, 5, 0]
+    dev = [torch.from_numpy(c).float().to(cuda) for c in cores]
+    out = torch.empty(int(np.prod(dims)), dtype=torch.float32, device=cuda)
+    lrc.tt_reconstruct(dev, dims, ranks, fmt, out)
+    torch.cuda.synchronize()
+    assert lrc.lrc_device_status() == 0
+    want, got = chain(cores, dims), out.double().cpu().numpy()
+    assert np.array_equal(np.isnan(got), np.isnan(want))
+    inf = np.isinf(want)
+    assert np.array_equal(got[inf], want[inf])
+    ok = np.isfinite(want)
+    # roundings of the chain's sums, relative to the sums of magnitudes
+    bound = chain([np.where(np.isfinite(c), np.abs(c), 1.0) for c in cores], dims)
+    assert np.all(np.abs(got[ok] - want[ok]) <= 8 * np.sqrt(max(ranks)) * U32 * bound[ok] * d)
