@@ -3,9 +3,12 @@
 //
 // Rounding is the hardware conversion cvt.rn.{f32,f16,bf16}.f64: IEEE 754
 // round-to-nearest-even directly from binary64 (no intermediate format),
-// subnormals kept (no .ftz), overflow to infinity.  The kernels are
-// HBM-bound streams: each thread converts a group of 8 consecutive elements
-// of one row with 128-bit loads and stores where the row pitch allows it.
+// subnormals kept (no .ftz), overflow to infinity; the 16-bit formats take it
+// only where the result is no normal number, and integer operations with the
+// same result elsewhere (round16).  The kernels are HBM-bound streams: each
+// thread converts a group of 8 consecutive elements of one row with 128-bit
+// loads and stores where the row pitch allows it; a matrix whose elements lie
+// in one run is converted without row arithmetic (round_run_kernel).
 #include <cuda_fp16.h>
 
 #include "common.cuh"
@@ -37,6 +40,67 @@ __device__ __forceinline__ double widen_f16(uint16_t h) {
     return d;
 }
 
+// Rounding to a 16-bit format by integer operations, for zeros and for results
+// in the normal exponents (or that overflow by rounding up): the dropped bits of
+// the significand's upper word, with one bit for whether the lower word is zero,
+// rounded to nearest even into the encoding, whose carry reaches the exponent as
+// it should.  MANT: stored significand bits, BIAS: exponent bias; `special` is
+// set for every other input.
+template <int MANT, int BIAS>
+__device__ __forceinline__ uint32_t round16(double x, bool* special) {
+    const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+    constexpr int drop = 20 - MANT;
+    const uint32_t a = hi & 0x7fffffffu;
+    const uint32_t s = a | (lo != 0 ? 1u : 0u);
+    const uint32_t h = ((s + (1u << (drop - 1)) - 1u + ((s >> drop) & 1u)) >> drop) - ((uint32_t)(1023 - BIAS) << MANT);
+    *special |= s != 0 && (a >> 20) - (uint32_t)(1024 - BIAS) >= (uint32_t)(2 * BIAS);
+    return (s != 0 ? h : 0u) | ((hi >> 16) & 0x8000u);
+}
+
+// A group in a 16-bit format (FMT 2 or 3).  The conversion instructions from
+// binary64 issue about two a clock on an SM: 4096 x 16384 elements took 117 us
+// with them however they were loaded, and take 96 us (7.0 TB/s) without.  The
+// vote makes the branch a real one: with `special` alone the conversions are
+// issued for every group, switched off by a predicate, and the kernel takes
+// 130 us.  With a special value in every warp it takes the 117 us.
+template <int FMT>
+__device__ __forceinline__ void round_group(const double* v, uint32_t* h) {
+    bool special = false;
+#pragma unroll
+    for (int j = 0; j < kGroup; ++j)
+        h[j] = FMT == 2 ? round16<10, 15>(v[j], &special) : round16<7, 127>(v[j], &special);
+    if (__any_sync(__activemask(), special)) {
+#pragma unroll
+        for (int j = 0; j < kGroup; ++j) h[j] = FMT == 2 ? cvt_f16(v[j]) : cvt_bf16(v[j]);
+    }
+}
+__device__ __forceinline__ uint4 pack_group(const uint32_t* h) {
+    return make_uint4(h[0] | (h[1] << 16), h[2] | (h[3] << 16), h[4] | (h[5] << 16), h[6] | (h[7] << 16));
+}
+
+// Four doubles in one 32-byte load (p on a 32-byte boundary), read once.
+__device__ __forceinline__ void load4(const double* p, double* v) {
+    asm volatile("ld.global.L1::no_allocate.v4.f64 {%0,%1,%2,%3}, [%4];"
+                 : "=d"(v[0]), "=d"(v[1]), "=d"(v[2]), "=d"(v[3]) : "l"(p));
+}
+
+// A source whose elements lie in one run of whole groups, to a 16-bit format:
+// one group a thread and as many blocks as that takes.  Two or four groups in
+// flight in a thread gave nothing (96.0 us either way), a grid of resident
+// blocks that strides over the groups cost 4 us.
+template <int FMT>
+__global__ void __launch_bounds__(kThreads)
+round_run_kernel(const double* __restrict__ src, uint16_t* __restrict__ dst, int64_t groups) {
+    const int64_t g = (int64_t)blockIdx.x * kThreads + threadIdx.x;
+    if (g >= groups) return;
+    double v[kGroup];
+    load4(src + g * kGroup, v);
+    load4(src + g * kGroup + 4, v + 4);
+    uint32_t h[kGroup];
+    round_group<FMT>(v, h);
+    __stcs(reinterpret_cast<uint4*>(dst) + g, pack_group(h));
+}
+
 // FMT: 0 = binary64 copy, 1 = binary32, 2 = binary16, 3 = bfloat16
 template <int FMT>
 __global__ void __launch_bounds__(kThreads)
@@ -63,19 +127,13 @@ round_pack_kernel(const double* __restrict__ src, int64_t cols, int64_t ld_src,
         const bool full = vec_dst && (c0 + kGroup <= ld_dst);
         if (FMT == 2 || FMT == 3) {
             uint16_t* drow = static_cast<uint16_t*>(dst) + r * ld_dst;
-            uint16_t h[kGroup];
-#pragma unroll
-            for (int j = 0; j < kGroup; ++j) h[j] = FMT == 2 ? cvt_f16(v[j]) : cvt_bf16(v[j]);
+            uint32_t h[kGroup];
+            round_group<FMT == 3 ? 3 : 2>(v, h);
             if (full) {
-                uint4 q;
-                q.x = (uint32_t)h[0] | ((uint32_t)h[1] << 16);
-                q.y = (uint32_t)h[2] | ((uint32_t)h[3] << 16);
-                q.z = (uint32_t)h[4] | ((uint32_t)h[5] << 16);
-                q.w = (uint32_t)h[6] | ((uint32_t)h[7] << 16);
-                __stcs(reinterpret_cast<uint4*>(drow + c0), q);
+                __stcs(reinterpret_cast<uint4*>(drow + c0), pack_group(h));
             } else {
                 for (int j = 0; j < kGroup; ++j)
-                    if (c0 + j < ld_dst) drow[c0 + j] = h[j];
+                    if (c0 + j < ld_dst) drow[c0 + j] = (uint16_t)h[j];
             }
         } else if (FMT == 1) {
             float* drow = static_cast<float*>(dst) + r * ld_dst;
@@ -197,6 +255,15 @@ lrc_status launch_round(const double* src, int64_t rows, int64_t cols, int64_t l
     const int64_t total = rows * gpr;
     const bool vec_src = (ld_src % 2) == 0;
     const int grid = grid_for(total);
+    const int64_t run_blocks = (total + kThreads - 1) / kThreads;
+    if (storage_bytes(fmt) == 2 && cols == ld_src && cols == ld_dst && cols % kGroup == 0 && total > 0 &&
+        run_blocks <= 0x7fffffff && reinterpret_cast<uintptr_t>(src) % 32 == 0 &&
+        reinterpret_cast<uintptr_t>(dst) % 16 == 0) {
+        uint16_t* out = static_cast<uint16_t*>(dst);
+        if (fmt == LRC_BF16) round_run_kernel<3><<<(unsigned)run_blocks, kThreads, 0, s>>>(src, out, total);
+        else round_run_kernel<2><<<(unsigned)run_blocks, kThreads, 0, s>>>(src, out, total);
+        return after_launch("round_run_kernel");
+    }
     switch (fmt) {
         case LRC_F64:
             round_pack_kernel<0><<<grid, kThreads, 0, s>>>(src, cols, ld_src, dst, ld_dst, gpr, total,
