@@ -730,8 +730,12 @@ __global__ void __launch_bounds__(kThreads, 1) product_kernel(const __grid_const
 }
 
 // The partial tiles of a split reduction, added in the order of the groups.
-constexpr int kManyParts = 24;
 // (Of a listed, symmetric product the entries above the diagonal, both ways.)
+// MANY: kManyParts and more (one tile spread over all SMs: 152, 27 us one after
+// the other): eight warps take an eighth each, their sums are added in order
+// (12.5 us with the leftovers of an unrolled loop, 7.7 us by sum_parts).
+constexpr int kManyParts = 24;
+template <bool MANY>
 __global__ void __launch_bounds__(256) part_sum_kernel(const __grid_constant__ GemmArgs a, int NT, int64_t Q, int64_t G,
                                                        double* __restrict__ C, const double* __restrict__ rscale,
                                                        const double* __restrict__ cscale, int* __restrict__ clear,
@@ -754,24 +758,17 @@ __global__ void __launch_bounds__(256) part_sum_kernel(const __grid_constant__ G
         if (a.listed) C[col * a.cr + row * a.cc] = s;
         if (mirror) mirror[col * a.cr + row * a.cc] = s;
     };
-    if (p1 - p0 < kManyParts) {
+    if (!MANY) {
         for (int e = blockIdx.y * 256 + threadIdx.x; e < 128 * NT; e += 256 * gridDim.y) {
-            double s = 0.0;
-#pragma unroll 4
-            for (int64_t p = p0; p <= p1; ++p) s += part[p * step + e];
-            put(e, s);
+            put(e, sum_parts<4>(0.0, part + e, step, p0, p1 + 1));   // eight: 7.6 -> 10 us at 17 parts
         }
         return;
     }
-    // many partial tiles (one tile spread over all SMs: 152, 27 us one after the
-    // other): eight warps take an eighth each, their sums are added in order
     __shared__ double sm[8][32];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t np = p1 - p0 + 1, q0 = p0 + np * w / 8, q1 = p0 + np * (w + 1) / 8;
     for (int e0 = blockIdx.y * 32; e0 < 128 * NT; e0 += 32 * gridDim.y) {
-        double s = 0.0;
-#pragma unroll 4
-        for (int64_t p = q0; p < q1; ++p) s += part[p * step + e0 + lane];
+        double s = sum_parts<8>(0.0, part + e0 + lane, step, q0, q1);
         __syncthreads();
         sm[w][lane] = s;
         __syncthreads();
@@ -1049,8 +1046,8 @@ lrc_status run_product(const Operand64& A0, const Operand64& B0, const Out64& ou
     if (split) {
         const bool many = groups / (tiles / a.group) >= kManyParts;
         const unsigned gy = (unsigned)std::max<int64_t>(1, std::min<int64_t>(128 * NT / (many ? 32 : 256), (many ? 8 : 4) * sms / tiles));
-        e = launch_pdl(part_sum_kernel, dim3((unsigned)tiles, gy), dim3(256), 0, s, a, NT, Q, groups, out.C, out.rscale,
-                       out.cscale, out.clear, out.mirror);
+        e = launch_pdl(many ? part_sum_kernel<true> : part_sum_kernel<false>, dim3((unsigned)tiles, gy), dim3(256), 0,
+                       s, a, NT, Q, groups, out.C, out.rscale, out.cscale, out.clear, out.mirror);
         if (e != cudaSuccess) return cuda_fail(e, "part_sum_kernel launch");
         if ((st = after_launch("part_sum_kernel")) != LRC_OK) return st;
     }

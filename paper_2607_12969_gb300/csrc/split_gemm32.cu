@@ -419,9 +419,7 @@ __global__ void __launch_bounds__(256) part_sum32_kernel(const float* __restrict
     for (int q = blockIdx.y; q < blocks; q += gridDim.y) {
         const int rb = (q & 3) * 32, cb = (q >> 2) * 8;
         const float* src = part + tile * (128 * NT) + (cb + ty) * 128 + rb + tx;
-        float s = 0.0f;
-#pragma unroll 8
-        for (int64_t p = p0; p <= p1; ++p) s = __fadd_rn(s, __ldg(src + p * group * (128 * NT)));
+        const float s = sg::sum_parts<8>(0.0f, src, (int64_t)group * (128 * NT), p0, p1 + 1);
         __syncthreads();
         sm[ty][tx] = s;
         __syncthreads();

@@ -59,5 +59,23 @@ __host__ __device__ __forceinline__ int64_t group_of_chunk(int64_t u, int64_t Q,
     return ((u + 1) * G + Q - 1) / Q - 1;
 }
 
+// p0 .. p1 - 1 of the partial tiles added to s in order, kAhead loads in flight
+// also for the last ones (an unrolled loop takes what is left over one at a
+// time: the 38 partial tiles of an entry were ten loads waited for in turn).
+// Past the end the last load is repeated and zero added; a condition on the load
+// or the sum makes the compiler wait for each load in turn.
+template <int kAhead, typename T>
+__device__ __forceinline__ T sum_parts(T s, const T* __restrict__ part, int64_t step, int64_t p0, int64_t p1) {
+    int left = (int)(p1 - p0);
+    for (const T* at = part + p0 * step; left > 0; left -= kAhead, at += kAhead * step) {
+        T v[kAhead];
+#pragma unroll
+        for (int i = 0; i < kAhead; ++i) v[i] = __ldg(at + min(i, left - 1) * step);   // no branch between the loads
+#pragma unroll
+        for (int i = 0; i < kAhead; ++i) s += i < left ? v[i] : T(0);
+    }
+    return s;
+}
+
 }  // namespace sg
 }  // namespace lrc
