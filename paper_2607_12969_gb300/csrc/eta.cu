@@ -130,20 +130,6 @@ __global__ void eta_tt_blocks_kernel(const double* __restrict__ G, const T* __re
     }
 }
 
-// Weights of the digits of an interior level's products (split_gemm.cuh): 2^(2
-// shift) for the entries of the rounding error dG, 1 for those of G.  dG lies
-// about 2^-shift below G, and M's entries for it the same way: weighing one up and
-// the other down keeps the entries of a row close together.  w1[a] for the 2 ra
-// rows of CD, w2[a n + i] for its rows as the Gram matrices read them.
-__global__ void eta_tt_weights_kernel(int ra, int64_t n, double w, double* __restrict__ w1, double* __restrict__ w2) {
-    const int64_t total = 2 * (int64_t)ra * n;
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t a = e / n;
-        w2[e] = a < ra ? 1.0 : w;
-        if (e - a * n == 0) w1[a] = a < ra ? 1.0 : w;
-    }
-}
-
 // ---- C = A^T B over a long reduction, split over CTAs --------------------
 // Up to three products per launch.  Product j: A (L x p, pitch lda), B (L x p,
 // pitch ldb), binary64; C (p x p, pitch ldc).  Output tiles are T x T with
@@ -686,80 +672,6 @@ void interior_gram_specs(int ra, int64_t n, int rb, const double* CD, const doub
     sp[2] = {CZ, XZ + L1 * rb, rb, rb, L1, rb, true, Mn + (int64_t)rb * ld + rb, nullptr, ld};   // M'_ZZ
 }
 
-// An interior level through digits: the operands of its two products and three
-// Gram products, where they live, and its weights.
-struct DigitLevel {
-    sg::Operand64 m, cd, mz, cz;             // X_D = M CD, X_Z = M[:, Z] CZ
-    sg::Operand64 gd, xd, xz, gz, xzz;       // M'_DD = gd xd, M'_DZ = gd xz, M'_ZZ = gz xzz
-    double* w1;
-    double* w2;
-    double* part;
-    size_t bytes;
-};
-DigitLevel digit_level(int ra, int64_t n, int rb, const double* M, const double* CD, const double* CZ, const double* XD,
-                       const double* XZ, unsigned char* ws) {
-    DigitLevel g{};
-    const int64_t N = n * rb, L2 = 2 * (int64_t)ra * n, L1 = (int64_t)ra * n;
-    size_t off = 0;
-    auto take = [&](size_t bytes) {
-        unsigned char* p = ws + off;
-        off += align_up(bytes);
-        return p;
-    };
-    g.w1 = reinterpret_cast<double*>(take((size_t)2 * ra * 8));
-    g.w2 = reinterpret_cast<double*>(take((size_t)L2 * 8));
-    g.part = reinterpret_cast<double*>(take(sg::part_bytes(rb, rb)));
-    auto set = [&](sg::Operand64& o, const double* p, int64_t rs, int64_t cs, int64_t rows, int64_t K, const double* w,
-                   int sign) {
-        o.src = sg::Src64{p, rs, cs, w, sign};
-        o.rows = rows;
-        o.K = K;
-        sg::operand_carve(&o, take(sg::operand_bytes(rows, K)));
-    };
-    set(g.m, M, 2 * ra, 1, 2 * ra, 2 * ra, g.w1, -1);
-    set(g.cd, CD, 1, N, N, 2 * ra, g.w1, 1);
-    set(g.mz, M + ra, 2 * ra, 1, 2 * ra, ra, nullptr, 0);
-    set(g.cz, CZ, 1, N, N, ra, nullptr, 0);
-    set(g.gd, CD, 1, rb, rb, L2, g.w2, 1);
-    set(g.xd, XD, 1, rb, rb, L2, g.w2, -1);
-    set(g.xz, XZ, 1, rb, rb, L2, g.w2, -1);
-    set(g.gz, CZ, 1, rb, rb, L1, nullptr, 0);
-    set(g.xzz, XZ + L1 * rb, 1, rb, rb, L1, nullptr, 0);
-    g.bytes = off;
-    return g;
-}
-// Binary64 FMAs of an interior level, and from how many on digits pay: 256^3,
-// rank 34 (1.9e8 multiply-adds): the FMA kernels took 228 us.
-double level_work(int ra, int64_t n, int rb) {
-    return 6.0 * ra * ra * (double)n * rb + 3.5 * ra * (double)n * rb * rb;
-}
-constexpr double kDigitLevelWork = 6e7;
-
-lrc_status run_digit_level(const DigitLevel& g, int ra, int64_t n, int rb, double w, double* XD, double* XZ, double* Mn,
-                           cudaStream_t s) {
-    const int64_t N = n * rb, ld = 2 * (int64_t)rb;
-    eta_tt_weights_kernel<<<grid_for(2 * (int64_t)ra * n, 256), 256, 0, s>>>(ra, n, w, g.w1, g.w2);
-    lrc_status st = after_launch("eta_tt_weights_kernel");
-    if (st != LRC_OK) return st;
-    const sg::Operand64* first[4] = {&g.m, &g.cd, &g.mz, &g.cz};
-    if ((st = sg::slice(first, 4, s)) != LRC_OK) return st;
-    if ((st = sg::product(g.m, g.cd, sg::Out64{XD, N, 1, nullptr, nullptr}, false, nullptr, s)) != LRC_OK) return st;
-    if ((st = sg::product(g.mz, g.cz, sg::Out64{XZ, N, 1, nullptr, nullptr}, false, nullptr, s)) != LRC_OK) return st;
-    const sg::Operand64* second[5] = {&g.gd, &g.xd, &g.xz, &g.gz, &g.xzz};
-    if ((st = sg::slice(second, 5, s)) != LRC_OK) return st;
-    if ((st = sg::product(g.gd, g.xd, sg::Out64{Mn, ld, 1, nullptr, nullptr}, true, g.part, s)) != LRC_OK) return st;
-    sg::Out64 dz{Mn + rb, ld, 1, nullptr, nullptr};
-    dz.mirror = Mn + (int64_t)rb * ld;
-    if ((st = sg::product(g.gd, g.xz, dz, true, g.part, s)) != LRC_OK) return st;
-    return sg::product(g.gz, g.xzz, sg::Out64{Mn + (int64_t)rb * ld + rb, ld, 1, nullptr, nullptr}, true, g.part, s);
-}
-
-// 2^(2 shift) of the weights: shift is the format's precision.
-template <typename T>
-constexpr double digit_weight() {
-    return sizeof(T) == 8 ? 1.0 : sizeof(T) == 4 ? 281474976710656.0 : std::is_same<T, __half>::value ? 4194304.0 : 65536.0;
-}
-
 template <typename T>
 lrc_status tt_eta_t(const TTShape& sh, const void* const* hats, double* eta_out, double* norm_out,
                     cudaStream_t s) {
@@ -789,26 +701,9 @@ lrc_status tt_eta_t(const TTShape& sh, const void* const* hats, double* eta_out,
     const size_t o_m0 = c.take((size_t)4 * rmax * rmax * 8), o_m1 = c.take((size_t)4 * rmax * rmax * 8);
     const size_t o_part = c.take((size_t)slots * 8);
     const size_t o_cp = c.take((size_t)2 * kCombineBlocks * 8);
-    // digits of the largest interior level that goes through them
-    const size_t plain = c.off;
-    size_t dig_max = 0;
-    auto wants_digits = [&](int l) {
-        return level_work((int)sh.ranks[l], sh.dims[l], (int)sh.ranks[l + 1]) >= kDigitLevelWork &&
-               2 * sh.ranks[l] * sh.dims[l] <= sg::kMaxK && 2 * sh.ranks[l] <= sg::kMaxK;
-    };
-    for (int l = 1; l < d - 1; ++l)
-        if (wants_digits(l))
-            dig_max = std::max(dig_max, digit_level((int)sh.ranks[l], sh.dims[l], (int)sh.ranks[l + 1], nullptr, nullptr,
-                                                    nullptr, nullptr, nullptr, nullptr).bytes);
     void* ws = nullptr;
-    lrc_status st = LRC_OK;
-    const size_t o_dig = c.take(dig_max);
-    bool digits = dig_max > 0;
-    if (digits) {
-        if ((st = stream_workspace_try(s, c.off, &ws)) != LRC_OK) return st;
-        digits = ws != nullptr;
-    }
-    if (!digits && (st = stream_workspace(s, plain, &ws)) != LRC_OK) return st;
+    lrc_status st = stream_workspace(s, c.off, &ws);
+    if (st != LRC_OK) return st;
     char* base = (char*)ws;
     double* Pk = (double*)(base + o_pk);
     double* lev = (double*)(base + o_lev);
@@ -835,12 +730,9 @@ lrc_status tt_eta_t(const TTShape& sh, const void* const* hats, double* eta_out,
         eta_tt_blocks_kernel<T><<<grid_for(cnt, 256), 256, 0, s>>>((const double*)sh.cores[l], (const T*)hats[l],
                                                                     cnt, CD, CZ);
         if ((st = after_launch("eta_tt_blocks_kernel")) != LRC_OK) return st;
-        if (digits && wants_digits(l)) {
-            const DigitLevel g = digit_level(ra, n, rb, Mcur, CD, CZ, XD, XZ, (unsigned char*)base + o_dig);
-            if ((st = run_digit_level(g, ra, n, rb, digit_weight<T>(), XD, XZ, Mnext, s)) != LRC_OK) return st;
-            std::swap(Mcur, Mnext);
-            continue;
-        }
+        // (Not through digits: with left-orthogonal cores M is close to the identity,
+        // its rows lie far below their largest entry and are recomputed one by one;
+        // 512 x 512 x 224, ranks 70 and 52: 200 ms instead of 1.1.)
         // X_D = M [G; dG], X_Z = M[:, Z] Gh  (2ra x n rb each)
         MmSpec mm[2] = {{Mcur, CD, XD, 2 * ra, N, N, N, 2 * ra, 2 * ra},
                         {Mcur + ra, CZ, XZ, 2 * ra, N, N, N, 2 * ra, ra}};

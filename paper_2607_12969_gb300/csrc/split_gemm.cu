@@ -738,8 +738,7 @@ constexpr int kManyParts = 24;
 template <bool MANY>
 __global__ void __launch_bounds__(256) part_sum_kernel(const __grid_constant__ GemmArgs a, int NT, int64_t Q, int64_t G,
                                                        double* __restrict__ C, const double* __restrict__ rscale,
-                                                       const double* __restrict__ cscale, int* __restrict__ clear,
-                                                       double* __restrict__ mirror) {
+                                                       const double* __restrict__ cscale, int* __restrict__ clear) {
     pdl_wait();
     pdl_trigger();
     if (clear && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *clear = 0;
@@ -756,7 +755,6 @@ __global__ void __launch_bounds__(256) part_sum_kernel(const __grid_constant__ G
         if (cscale) s *= __ldg(cscale + col);
         C[row * a.cr + col * a.cc] = s;
         if (a.listed) C[col * a.cr + row * a.cc] = s;
-        if (mirror) mirror[col * a.cr + row * a.cc] = s;
     };
     if (!MANY) {
         for (int e = blockIdx.y * 256 + threadIdx.x; e < 128 * NT; e += 256 * gridDim.y) {
@@ -782,76 +780,140 @@ __global__ void __launch_bounds__(256) part_sum_kernel(const __grid_constant__ G
 }
 
 // ---------------------------------------------------------------- repair
-// Rows listed as hard: their part of C by binary64 FMAs, 64 x 64 tiles of
-// gathered rows, 4 x 4 entries a thread.
-__global__ void __launch_bounds__(256) repair_kernel(View64 A, const int* __restrict__ ha, int64_t M, View64 B,
-                                                     const int* __restrict__ hb, int64_t N, int64_t K,
-                                                     double* __restrict__ C, int64_t cr, int64_t cc,
-                                                     const double* __restrict__ rscale,
-                                                     const double* __restrict__ cscale, double* __restrict__ mirror) {
-    __shared__ double As[16][65];
-    __shared__ double Bs[16][65];
-    pdl_wait();
-    pdl_trigger();
-    const int64_t na = ha[0], nb = hb[0];
-    const int64_t ta = (na + 63) / 64 * ((N + 63) / 64), tb = (nb + 63) / 64 * ((M + 63) / 64);
-    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-    for (int64_t t = blockIdx.x; t < ta + tb; t += gridDim.x) {
+// Rows listed as hard: their part of C by binary64 FMAs.  The binary64 pipe (two
+// FMAs a clock on an SM) is the bound, as for the FMA kernels of the other paths;
+// with every row listed (factors whose entries decay over many binades) a product
+// should take what it takes there.  So the tile follows from how many there are:
+// R x R entries a thread in tiles of 16 R, and for few entries (R = 0) tiles of
+// 8 x 8 whose reduction is split over four threads.  With entries over 60 binades
+// in both operands: apply 16384 x 8192, k = 128, b = 2048 11.7 ms (FMA kernels
+// 11.2), 12287 x 16384, k = 272, b = 250 4.1 ms (4.2); 64 x 64 tiles alone took
+// 100 ms and more for results of 100 x 100 with a reduction of 30000.
+struct RepairArgs {
+    View64 A, B;
+    const int* ha;
+    const int* hb;
+    int64_t M, N, K;
+    double* C;
+    int64_t cr, cc;
+    const double* rscale;
+    const double* cscale;
+    int sym;                  // A and B are the same operand, C symmetric
+};
+constexpr int kRepairWords = 128 * 9;        // staged entries of an operand, with padding (the largest of all R)
+
+template <int R>
+__host__ __device__ constexpr int repair_tile() { return R == 0 ? 8 : 16 * R; }
+
+__device__ __forceinline__ int64_t repair_tiles(int64_t na, int64_t nb, int64_t M, int64_t N, int T) {
+    return (na + T - 1) / T * ((N + T - 1) / T) + (nb + T - 1) / T * ((M + T - 1) / T);
+}
+
+template <int R>
+__device__ __forceinline__ void repair_body(const RepairArgs& a, int64_t na, int64_t nb, double* As, double* Bs) {
+    constexpr int T = repair_tile<R>(), KS = 1024 / T, P = T + 1, E = R == 0 ? 1 : R, W = R == 0 ? 8 : 16;
+    const int64_t ta = (na + T - 1) / T * ((a.N + T - 1) / T), tiles = repair_tiles(na, nb, a.M, a.N, T);
+    const int tid = threadIdx.x;
+    const int part = R == 0 ? tid / 64 : 0;                        // quarter of the reduction
+    const int tx = tid % W, ty = R == 0 ? tid / 8 % 8 : tid / 16;
+    const bool all = na == a.M;                                    // every row of A: in order, not by the list
+    for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
         // tile of C rows (first list entry or row) and columns
         const bool ga = t < ta;
         const int64_t u = ga ? t : t - ta;
-        const int64_t other = ga ? (N + 63) / 64 : (M + 63) / 64;
-        const int64_t l0 = u / other * 64, o0 = (u % other) * 64;
+        const int64_t other = ((ga ? a.N : a.M) + T - 1) / T;
+        const int64_t l0 = u / other * T, o0 = (u % other) * T;
         const int64_t i0 = ga ? l0 : o0, j0 = ga ? o0 : l0;
-        const int64_t ni = ga ? na : M, nj = ga ? N : nb;
-        auto row_of = [&](int i) { return i0 + i < ni ? (ga ? (int64_t)ha[1 + i0 + i] : i0 + i) : (int64_t)-1; };
-        auto col_of = [&](int j) { return j0 + j < nj ? (ga ? j0 + j : (int64_t)hb[1 + j0 + j]) : (int64_t)-1; };
-        double acc[4][4];
+        if (a.sym && all && i0 > j0) continue;                     // written with the tile above the diagonal
+        const int64_t ni = ga ? na : a.M, nj = ga ? a.N : nb;
+        auto row_of = [&](int i) {
+            return i0 + i >= ni ? -1 : ga && !all ? __ldg(a.ha + 1 + i0 + i) : (int)(i0 + i);
+        };
+        auto col_of = [&](int j) { return j0 + j >= nj ? -1 : ga ? (int)(j0 + j) : __ldg(a.hb + 1 + j0 + j); };
+        // a thread stages four entries of each operand, neighbours along k
+        const int kk = tid % KS, x0 = tid / KS;
+        constexpr int XS = 256 / KS > 0 ? 256 / KS : 1;
+        static_assert(KS <= 256, "");
+        int ri[4], cj[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+        for (int q = 0; q < 4; ++q) {
+            ri[q] = row_of(x0 + q * XS);
+            cj[q] = col_of(x0 + q * XS);
+        }
+        double acc[E][E];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
-        for (int64_t k0 = 0; k0 < K; k0 += 16) {
+        for (int i = 0; i < E; ++i)
+#pragma unroll
+            for (int j = 0; j < E; ++j) acc[i][j] = 0.0;
+        double va[4], vb[4];
+        auto load = [&](int64_t k0) {
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                const int e = tid + 256 * q;
-                const int kk = e & 15, x = e >> 4;
-                const int64_t ri = row_of(x), cj = col_of(x);
-                As[kk][x] = (ri >= 0 && k0 + kk < K) ? A.at(ri, k0 + kk) : 0.0;
-                Bs[kk][x] = (cj >= 0 && k0 + kk < K) ? B.at(cj, k0 + kk) : 0.0;
+                va[q] = ri[q] >= 0 && k0 + kk < a.K ? a.A.at(ri[q], k0 + kk) : 0.0;
+                vb[q] = cj[q] >= 0 && k0 + kk < a.K ? a.B.at(cj[q], k0 + kk) : 0.0;
+            }
+        };
+        load(0);
+        for (int64_t k0 = 0; k0 < a.K; k0 += KS) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                As[kk * P + x0 + q * XS] = va[q];
+                Bs[kk * P + x0 + q * XS] = vb[q];
             }
             __syncthreads();
-            const int kn = (int)min((int64_t)16, K - k0);
+            if (k0 + KS < a.K) load(k0 + KS);                      // in flight over this slab's FMAs
+            const int kn = (int)min((int64_t)KS, a.K - k0);
+            const int kb = R == 0 ? part * (KS / 4) : 0, ke = R == 0 ? min(kn, kb + KS / 4) : kn;
 #pragma unroll 4
-            for (int kk = 0; kk < kn; ++kk) {
-                double x[4], y[4];
+            for (int k = kb; k < ke; ++k) {
+                double x[E], y[E];
 #pragma unroll
-                for (int i = 0; i < 4; ++i) x[i] = As[kk][ty + 16 * i];
+                for (int i = 0; i < E; ++i) x[i] = As[k * P + ty + W * i];
 #pragma unroll
-                for (int j = 0; j < 4; ++j) y[j] = Bs[kk][tx + 16 * j];
+                for (int j = 0; j < E; ++j) y[j] = Bs[k * P + tx + W * j];
 #pragma unroll
-                for (int i = 0; i < 4; ++i)
+                for (int i = 0; i < E; ++i)
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) acc[i][j] = fma(x[i], y[j], acc[i][j]);
+                    for (int j = 0; j < E; ++j) acc[i][j] = fma(x[i], y[j], acc[i][j]);
             }
             __syncthreads();
         }
+        if (R == 0) {
+            As[tid] = acc[0][0];
+            __syncthreads();
+            acc[0][0] = ((As[tid & 63] + As[64 + (tid & 63)]) + As[128 + (tid & 63)]) + As[192 + (tid & 63)];
+            __syncthreads();
+            if (part != 0) continue;
+        }
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int64_t row = row_of(ty + 16 * i);
+        for (int i = 0; i < E; ++i) {
+            const int64_t row = row_of(ty + W * i);
             if (row < 0) continue;
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int64_t col = col_of(tx + 16 * j);
+            for (int j = 0; j < E; ++j) {
+                const int64_t col = col_of(tx + W * j);
                 if (col < 0) continue;
                 double s = acc[i][j];
-                if (rscale) s *= __ldg(rscale + row);
-                if (cscale) s *= __ldg(cscale + col);
-                C[row * cr + col * cc] = s;
-                if (mirror) mirror[col * cr + row * cc] = s;
+                if (a.rscale) s *= __ldg(a.rscale + row);
+                if (a.cscale) s *= __ldg(a.cscale + col);
+                a.C[row * a.cr + col * a.cc] = s;
+                if (a.sym && all) a.C[col * a.cr + row * a.cc] = s;
             }
         }
     }
+}
+
+__global__ void __launch_bounds__(256, 2) repair_kernel(const __grid_constant__ RepairArgs a) {
+    __shared__ double As[kRepairWords], Bs[kRepairWords];
+    pdl_wait();
+    pdl_trigger();
+    const int64_t na = a.ha[0], nb = na == a.M ? 0 : a.hb[0];      // every row of A: all of C
+    if (na + nb == 0) return;
+    const int64_t grid = gridDim.x;
+    if (repair_tiles(na, nb, a.M, a.N, 64) >= 2 * grid) repair_body<4>(a, na, nb, As, Bs);
+    else if (repair_tiles(na, nb, a.M, a.N, 32) >= 2 * grid) repair_body<2>(a, na, nb, As, Bs);
+    else if (repair_tiles(na, nb, a.M, a.N, 16) >= 4 * grid) repair_body<1>(a, na, nb, As, Bs);
+    else repair_body<0>(a, na, nb, As, Bs);
 }
 
 size_t up256(size_t v) { return (v + 255) & ~(size_t)255; }
@@ -1047,13 +1109,13 @@ lrc_status run_product(const Operand64& A0, const Operand64& B0, const Out64& ou
         const bool many = groups / (tiles / a.group) >= kManyParts;
         const unsigned gy = (unsigned)std::max<int64_t>(1, std::min<int64_t>(128 * NT / (many ? 32 : 256), (many ? 8 : 4) * sms / tiles));
         e = launch_pdl(many ? part_sum_kernel<true> : part_sum_kernel<false>, dim3((unsigned)tiles, gy), dim3(256), 0,
-                       s, a, NT, Q, groups, out.C, out.rscale, out.cscale, out.clear, out.mirror);
+                       s, a, NT, Q, groups, out.C, out.rscale, out.cscale, out.clear);
         if (e != cudaSuccess) return cuda_fail(e, "part_sum_kernel launch");
         if ((st = after_launch("part_sum_kernel")) != LRC_OK) return st;
     }
-    e = launch_pdl(repair_kernel, dim3((unsigned)(2 * sms)), dim3(256), 0, s, View64{A.src}, (const int*)A.hard, A.rows,
-                   View64{B.src}, (const int*)B.hard, B.rows, A.K, out.C, out.cr, out.cc, out.rscale, out.cscale,
-                   out.mirror);
+    const RepairArgs r{View64{A.src}, View64{B.src}, A.hard, B.hard, A.rows, B.rows, A.K, out.C, out.cr, out.cc,
+                       out.rscale, out.cscale, sym ? 1 : 0};
+    e = launch_pdl(repair_kernel, dim3((unsigned)(2 * sms)), dim3(256), 0, s, r);
     if (e != cudaSuccess) return cuda_fail(e, "repair_kernel launch");
     return after_launch("repair_kernel");
 }

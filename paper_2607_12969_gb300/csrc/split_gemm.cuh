@@ -75,7 +75,6 @@ struct Out64 {
     const double* rscale;
     const double* cscale;
     int* clear = nullptr;    // a later operand's hard[0], set to 0 on the way (split only)
-    double* mirror = nullptr;    // C(i, j) also at mirror[j cr + i cc] (split only)
 };
 size_t part_bytes(int64_t M, int64_t N);
 lrc_status product(const Operand64& A, const Operand64& B, const Out64& out, bool split, double* part, cudaStream_t s);

@@ -166,3 +166,46 @@ def test_eta_through_digit_gram_matrices(lrc, cuda, fmt, m, n, k):
     want = np.sqrt(np.sum((M.T @ (Pu.T @ Pu) @ M) * (Pv @ Pv.T)))
     assert abs(eta - float(want)) <= 1e-13 * float(want)
     assert abs(norm - float(np.linalg.norm(f.s))) <= 1e-12 * norm or k > min(m, n)
+
+
+@pytest.mark.parametrize("m,n,k,b", [(4100, 600, 33, 700), (2050, 700, 40, 330), (1300, 2500, 70, 65), (130, 9000, 17, 65)])
+def test_every_row_wide(lrc, cuda, m, n, k, b):
+    """Every row of V^T and U recomputed: both products in the tiles that the
+    repair takes for many, fewer and few entries, with partial tiles."""
+    rng = np.random.default_rng(m)
+    wide = lambda *s: rng.standard_normal(s) * 2.0 ** -rng.integers(0, 60, s)
+    U, Vt, X, s = wide(m, k), wide(k, n), W.gaussian((b, n), 5), rng.uniform(0.5, 2.0, k)
+    got = run(lrc, cuda, U, s, Vt, X)
+    want = oracle.apply(U, s, Vt, X)
+    bound = (np.abs(X) @ np.abs(Vt).T * np.abs(s)) @ np.abs(U).T
+    assert np.all(np.abs(got - want) <= 2 * (n + k + 2) * U64 * bound)
+
+
+@pytest.mark.parametrize("m,n,k", [(3000, 1700, 61), (16384, 8192, 144)])
+def test_eta_of_wide_columns(lrc, cuda, m, n, k):
+    """The Gram matrices of eta with every column recomputed (upper tiles,
+    written both ways): against a power of two times the same factors, whose
+    digits and FMAs are the same, and against plain matrix products."""
+    g = torch.Generator(device=cuda).manual_seed(m)
+    rand = lambda *s: torch.randn(*s, generator=g, device=cuda, dtype=torch.float64)
+    wide = lambda *s: rand(*s) * torch.exp2(-torch.randint(0, 40, s, generator=g, device=cuda).double())
+    ld = lrc.lrc_packed_ld
+    U = torch.zeros(m, ld(k), dtype=torch.float64, device=cuda)
+    Vt = torch.zeros(k, ld(n), dtype=torch.float64, device=cuda)
+    U[:, :k], Vt[:, :n] = wide(m, k), wide(k, n)
+    s = rand(ld(k)).abs() + 0.1
+    hats = [a.float() for a in (U, s, Vt)]
+    eta, norm = lrc.lrc_lowrank_eta(U, s, Vt, *hats, "f32", m, n, k)
+    # the trace forms with the rounding errors explicit, as in the header
+    u, uh, v, vh = U[:, :k], hats[0][:, :k].double(), Vt[:, :n].T, hats[2][:, :n].double().T
+    S, Sh = s[:k], hats[1][:k].double()
+    P, Q = torch.cat([u - uh, uh], 1), torch.cat([v - vh, vh], 1)
+    D = torch.diag
+    M = torch.cat([torch.cat([D(S), D(S)], 1), torch.cat([D(S), D(S - Sh)], 1)], 0)
+    Gu, Gv = P.T @ P, Q.T @ Q
+    want = float(torch.sum((M.T @ Gu @ M) * Gv)) ** 0.5
+    wnorm = float(torch.sum((D(S) @ (u.T @ u) @ D(S)) * (v.T @ v))) ** 0.5
+    # a Gram entry has relative error (m + 2) u of its sum of magnitudes, and so
+    # have eta^2's two factors; its terms (all of one size) nearly add up
+    assert abs(eta - want) <= 8 * (m + n) * U64 * want
+    assert abs(norm - wnorm) <= 8 * (m + n) * U64 * wnorm
