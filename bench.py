@@ -115,11 +115,7 @@ def rank_set(fmt: str) -> str:
 # DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) from
 # one ncu capture of the call type's kernels as they stand; an entry is
 # removed when its kernels change.
-MEASURED_TRAFFIC: dict = {
-    # eta_matrix@sweep (lrc_lowrank_eta, m = n = 16384, k' = 272, binary16):
-    # all six kernels of one call, profiles/eta_matrix_lowrank_16384x16384_k272.md
-    "eta_matrix@sweep": 1_858_600_000,
-}
+MEASURED_TRAFFIC: dict = {}
 
 
 def work_round(rows, cols, ld, fmt):

@@ -30,7 +30,6 @@
 #include <cuda_fp16.h>
 
 #include <algorithm>
-#include <type_traits>
 #include <vector>
 
 #include "common.cuh"
@@ -604,7 +603,7 @@ DigitGram digit_gram(const double* A, int p, int64_t L, unsigned char* ws) {
 // Multiply-adds from which the Gram matrices of a matrix eta go through digits:
 // their eight launches cost about 60 us, the DFMA kernel 2 us per 1e6 until it
 // fills the GPU and 1.6 us per 1e6 from there (16384 x 8192, k = 144: 2.0e9,
-// 1887 -> 324 us with the rounding of the factors).
+// 1887 -> 255 us with the rounding of the factors).
 constexpr double kDigitGramWork = 3e7;
 
 template <typename T>
@@ -732,7 +731,7 @@ lrc_status tt_eta_t(const TTShape& sh, const void* const* hats, double* eta_out,
         if ((st = after_launch("eta_tt_blocks_kernel")) != LRC_OK) return st;
         // (Not through digits: with left-orthogonal cores M is close to the identity,
         // its rows lie far below their largest entry and are recomputed one by one;
-        // 512 x 512 x 224, ranks 70 and 52: 200 ms instead of 1.1.)
+        // 512 x 512 x 224, ranks 70 and 52: 200 ms a call instead of 2.2.)
         // X_D = M [G; dG], X_Z = M[:, Z] Gh  (2ra x n rb each)
         MmSpec mm[2] = {{Mcur, CD, XD, 2 * ra, N, N, N, 2 * ra, 2 * ra},
                         {Mcur + ra, CZ, XZ, 2 * ra, N, N, N, 2 * ra, ra}};

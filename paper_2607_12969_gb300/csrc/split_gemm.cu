@@ -786,9 +786,9 @@ __global__ void __launch_bounds__(256) part_sum_kernel(const __grid_constant__ G
 // should take what it takes there.  So the tile follows from how many there are:
 // R x R entries a thread in tiles of 16 R, and for few entries (R = 0) tiles of
 // 8 x 8 whose reduction is split over four threads.  With entries over 60 binades
-// in both operands: apply 16384 x 8192, k = 128, b = 2048 11.7 ms (FMA kernels
-// 11.2), 12287 x 16384, k = 272, b = 250 4.1 ms (4.2); 64 x 64 tiles alone took
-// 100 ms and more for results of 100 x 100 with a reduction of 30000.
+// in both operands: apply 16384 x 8192, k = 128, b = 2048 11.3 ms (FMA kernels
+// 11.2), 12287 x 16384, k = 272, b = 250 4.1 ms (4.2); 64 x 64 tiles alone
+// took about 100 ms for results of 140 x 104 with a reduction of 71680.
 struct RepairArgs {
     View64 A, B;
     const int* ha;
