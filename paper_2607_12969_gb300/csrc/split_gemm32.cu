@@ -436,76 +436,119 @@ struct RepairSide {
     const int* hard;
 };
 
-// Rows listed as hard: their part of C by binary32 FMAs, 64 x 64 tiles of
-// gathered rows, 4 x 4 entries a thread, sums of at most 1024 terms added up.
-__global__ void __launch_bounds__(256) repair32_kernel(RepairSide A, RepairSide B, int64_t K, float* __restrict__ C,
-                                                       int64_t ldc, const float* __restrict__ cscale) {
-    __shared__ float As[16][65];
-    __shared__ float Bs[16][65];
-    pdl_wait();
-    pdl_trigger();
-    const int64_t M = A.rows, N = B.rows, na = A.hard[0], nb = B.hard[0];
-    const int64_t ta = (na + 63) / 64 * ((N + 63) / 64), tb = (nb + 63) / 64 * ((M + 63) / 64);
-    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+// Rows listed as hard: their part of C by binary32 FMAs, sums of at most 1024
+// terms added up.  The tile follows from how many there are, so that a small
+// result with a long reduction keeps the GPU at work: R x R entries a thread in
+// tiles of 16 R, and for few entries (R = 0) tiles of 8 x 8 whose reduction is
+// split over four threads.
+template <int R>
+__device__ __forceinline__ void repair32_body(const RepairSide& A, const RepairSide& B, int64_t K, float* C, int64_t ldc,
+                                              const float* cscale, int64_t na, int64_t nb, float* As, float* Bs) {
+    constexpr int T = R == 0 ? 8 : 16 * R, KS = 1024 / T, P = T + 1, E = R == 0 ? 1 : R, W = R == 0 ? 8 : 16;
+    constexpr int XS = 256 / KS;
+    const int64_t M = A.rows, N = B.rows;
+    const int64_t ta = (na + T - 1) / T * ((N + T - 1) / T), tb = (nb + T - 1) / T * ((M + T - 1) / T);
+    const int tid = threadIdx.x;
+    const int part = R == 0 ? tid / 64 : 0;                        // quarter of a slab
+    const int tx = tid % W, ty = R == 0 ? tid / 8 % 8 : tid / 16;
     for (int64_t t = blockIdx.x; t < ta + tb; t += gridDim.x) {
         const bool ga = t < ta;
         const int64_t u = ga ? t : t - ta;
-        const int64_t other = ga ? (N + 63) / 64 : (M + 63) / 64;
-        const int64_t l0 = u / other * 64, o0 = (u % other) * 64;
+        const int64_t other = ((ga ? N : M) + T - 1) / T;
+        const int64_t l0 = u / other * T, o0 = (u % other) * T;
         const int64_t i0 = ga ? l0 : o0, j0 = ga ? o0 : l0;
         const int64_t ni = ga ? na : M, nj = ga ? N : nb;
-        auto row_of = [&](int i) { return i0 + i < ni ? (ga ? (int64_t)A.hard[1 + i0 + i] : i0 + i) : (int64_t)-1; };
-        auto col_of = [&](int j) { return j0 + j < nj ? (ga ? j0 + j : (int64_t)B.hard[1 + j0 + j]) : (int64_t)-1; };
-        float acc[4][4], tot[4][4];
+        auto row_of = [&](int i) { return i0 + i >= ni ? -1 : ga ? __ldg(A.hard + 1 + i0 + i) : (int)(i0 + i); };
+        auto col_of = [&](int j) { return j0 + j >= nj ? -1 : ga ? (int)(j0 + j) : __ldg(B.hard + 1 + j0 + j); };
+        const int kk = tid % KS, x0 = tid / KS;                    // a thread stages four entries of each operand
+        int ri[4], cj[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+        for (int q = 0; q < 4; ++q) {
+            ri[q] = row_of(x0 + q * XS);
+            cj[q] = col_of(x0 + q * XS);
+        }
+        float acc[E][E], tot[E][E];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) acc[i][j] = tot[i][j] = 0.0f;
-        for (int64_t k0 = 0; k0 < K; k0 += 16) {
+        for (int i = 0; i < E; ++i)
+#pragma unroll
+            for (int j = 0; j < E; ++j) acc[i][j] = tot[i][j] = 0.0f;
+        float va[4], vb[4];
+        auto load = [&](int64_t k0) {
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                const int e = tid + 256 * q;
-                const int kk = e & 15, x = e >> 4;
-                const int64_t ri = row_of(x), cj = col_of(x);
-                As[kk][x] = (ri >= 0 && k0 + kk < K) ? __ldg(A.p + ri * A.rs + (k0 + kk) * A.cs) : 0.0f;
-                Bs[kk][x] = (cj >= 0 && k0 + kk < K) ? __ldg(B.p + cj * B.rs + (k0 + kk) * B.cs) : 0.0f;
+                va[q] = ri[q] >= 0 && k0 + kk < K ? __ldg(A.p + ri[q] * A.rs + (k0 + kk) * A.cs) : 0.0f;
+                vb[q] = cj[q] >= 0 && k0 + kk < K ? __ldg(B.p + cj[q] * B.rs + (k0 + kk) * B.cs) : 0.0f;
+            }
+        };
+        load(0);
+        for (int64_t k0 = 0; k0 < K; k0 += KS) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                As[kk * P + x0 + q * XS] = va[q];
+                Bs[kk * P + x0 + q * XS] = vb[q];
             }
             __syncthreads();
-            const int kn = (int)min((int64_t)16, K - k0);
+            if (k0 + KS < K) load(k0 + KS);                        // in flight over this slab's FMAs
+            const int kn = (int)min((int64_t)KS, K - k0);
+            const int kb = R == 0 ? part * (KS / 4) : 0, ke = R == 0 ? min(kn, kb + KS / 4) : kn;
 #pragma unroll 4
-            for (int kk = 0; kk < kn; ++kk) {
-                float x[4], y[4];
+            for (int k = kb; k < ke; ++k) {
+                float x[E], y[E];
 #pragma unroll
-                for (int i = 0; i < 4; ++i) x[i] = As[kk][ty + 16 * i];
+                for (int i = 0; i < E; ++i) x[i] = As[k * P + ty + W * i];
 #pragma unroll
-                for (int j = 0; j < 4; ++j) y[j] = Bs[kk][tx + 16 * j];
+                for (int j = 0; j < E; ++j) y[j] = Bs[k * P + tx + W * j];
 #pragma unroll
-                for (int i = 0; i < 4; ++i)
+                for (int i = 0; i < E; ++i)
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(x[i], y[j], acc[i][j]);
+                    for (int j = 0; j < E; ++j) acc[i][j] = fmaf(x[i], y[j], acc[i][j]);
             }
             __syncthreads();
-            if ((k0 & 1023) == 1008 || k0 + 16 >= K) {
+            if (((k0 + KS) & 1023) == 0 || k0 + KS >= K) {
 #pragma unroll
-                for (int i = 0; i < 4; ++i)
+                for (int i = 0; i < E; ++i)
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) {
+                    for (int j = 0; j < E; ++j) {
                         tot[i][j] += acc[i][j];
                         acc[i][j] = 0.0f;
                     }
             }
         }
+        if (R == 0) {
+            As[tid] = tot[0][0];
+            __syncthreads();
+            tot[0][0] = ((As[tid & 63] + As[64 + (tid & 63)]) + As[128 + (tid & 63)]) + As[192 + (tid & 63)];
+            __syncthreads();
+            if (part != 0) continue;
+        }
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int64_t row = row_of(ty + 16 * i);
+        for (int i = 0; i < E; ++i) {
+            const int64_t row = row_of(ty + W * i);
             if (row < 0) continue;
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int64_t col = col_of(tx + 16 * j);
+            for (int j = 0; j < E; ++j) {
+                const int64_t col = col_of(tx + W * j);
                 if (col >= 0) C[row * ldc + col] = cscale ? tot[i][j] * __ldg(cscale + col) : tot[i][j];
             }
         }
     }
+}
+
+__global__ void __launch_bounds__(256, 2) repair32_kernel(const __grid_constant__ RepairSide A,
+                                                          const __grid_constant__ RepairSide B, int64_t K,
+                                                          float* __restrict__ C, int64_t ldc,
+                                                          const float* __restrict__ cscale) {
+    __shared__ float As[128 * 9], Bs[128 * 9];                     // the largest of all R, with padding
+    pdl_wait();
+    pdl_trigger();
+    const int64_t M = A.rows, N = B.rows, na = A.hard[0], nb = na == M ? 0 : B.hard[0];   // every row of A: all of C
+    if (na + nb == 0) return;
+    auto tiles = [&](int T) { return (na + T - 1) / T * ((N + T - 1) / T) + (nb + T - 1) / T * ((M + T - 1) / T); };
+    const int64_t grid = gridDim.x;
+    if (tiles(64) >= grid) repair32_body<4>(A, B, K, C, ldc, cscale, na, nb, As, Bs);
+    else if (tiles(32) >= grid) repair32_body<2>(A, B, K, C, ldc, cscale, na, nb, As, Bs);
+    else if (tiles(16) >= 4 * grid) repair32_body<1>(A, B, K, C, ldc, cscale, na, nb, As, Bs);
+    else repair32_body<0>(A, B, K, C, ldc, cscale, na, nb, As, Bs);
 }
 
 int64_t n_tiles(int64_t rows, bool splitk) { return (rows + n_tile(rows, splitk) - 1) / n_tile(rows, splitk); }

@@ -150,3 +150,19 @@ def test_tt(lrc, cuda, dims, ranks, fmt, bad):
     # roundings of the chain's sums, relative to the sums of magnitudes
     bound = chain([np.where(np.isfinite(c), np.abs(c), 1.0) for c in cores], dims)
     assert np.all(np.abs(got[ok] - want[ok]) <= 8 * np.sqrt(max(ranks)) * U32 * bound[ok] * d)
+
+
+@pytest.mark.parametrize("m,n,k,b", [(4100, 600, 136, 1100), (2050, 8300, 40, 520), (12000, 9000, 33, 250)])
+def test_every_row_recomputed(lrc, cuda, m, n, k, b):
+    """Entries below the parts' range in every row of V^T and U: both products
+    in the tiles that the repair takes for many and few entries."""
+    rng = np.random.default_rng(m)
+    f32 = lambda a: a.astype(np.float32).astype(np.float64)
+    small = lambda a: f32(np.where(np.arange(a.shape[1]) % 5 == 0, a * 1e-34, a))
+    U, Vt = small(rng.standard_normal((m, k))), small(rng.standard_normal((k, n)))
+    X, s = f32(rng.standard_normal((b, n))), f32(rng.uniform(0.5, 2.0, k))
+    got = run(lrc, cuda, U, s, Vt, X)
+    want = ((X @ Vt.T) * s) @ U.T
+    bound = (np.abs(X) @ np.abs(Vt).T * s) @ np.abs(U).T
+    # sums of at most 1024 terms and of their sums, two products, one scaling
+    assert np.all(np.abs(got - want) <= 2 * (min(n, 1024) + n / 1024 + k + 4) * U32 * bound)
