@@ -57,7 +57,7 @@ extern "C" {
 typedef enum {
     LRC_F64 = 0,      /* binary64 storage and output; binary64 FMAs, or on larger problems
                          exact products of 9-bit digits on the tensor cores rounded to
-                         binary64 once (no less accurate; see lrc_apply)                    */
+                         binary64 once where they carry an entry (see lrc_apply)            */
     LRC_F32 = 1,      /* binary32 storage and output; binary32 FMAs, or in larger applies
                          products of three bfloat16 parts of every operand on the tensor
                          cores, accumulated in binary32 (no less accurate)                   */
@@ -148,12 +148,16 @@ LRC_API lrc_status lrc_widen_factors(const void* src, lrc_fmt fmt, int64_t rows,
  * aligned.  k may exceed min(m, n).  Asynchronous on `stream`.
  *
  * LRC_F64: larger problems form both products from digits of the operands'
- * rows.  A result is within about 2^-61 of (largest entry of the row of one
- * operand) (largest entry of the row of the other) per term of the sum, plus
- * one rounding; rows whose entries lie further apart than the digits reach
- * (on average more than 2^-12 below the largest), or that hold an infinity, a
- * NaN or a largest entry outside 2^-480 ... 2^495, are formed by binary64
- * FMAs.  The digits (14 bytes an element, of at most 1 GiB of queries at a
+ * rows.  With B_i the power of two above the largest entry of row i of one
+ * operand and B_j of row j of the other, an entry of a product is as a rule
+ * within 2^-61 B_i B_j a term of the sum, with signs of their own, and at worst
+ * within about 2^-57 B_i B_j a term, plus one rounding.  Entries whose sum of
+ * magnitudes S_ij = sum_k |a_ik b_jk| is below about 2^-5 B_i B_j, where that
+ * would be less than binary64 FMAs give, are formed by binary64 FMAs, so that
+ * every entry is as a rule within 0.1 sqrt(K) 2^-53 S_ij of the exact sum of K
+ * terms, and at worst within K 2^-50 S_ij (FMA sums: K 2^-53 S_ij).  Rows that
+ * hold an infinity, a NaN or a largest entry outside 2^-480 ... 2^495 are formed
+ * by FMAs too.  The digits (14 bytes an element, of at most 1 GiB of queries at a
  * time) live in the stream's workspace; without memory for them, or while the
  * stream is being captured with a smaller workspace, the FMA kernels run.
  *

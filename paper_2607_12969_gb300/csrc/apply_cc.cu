@@ -39,6 +39,8 @@
 // entry by the inverse scales (exact).
 #include <cuda_fp16.h>
 
+#include <algorithm>
+
 #include "common.cuh"
 #include "split_gemm.cuh"
 #include "split_gemm32.cuh"
@@ -532,11 +534,14 @@ static lrc_status launch_apply_f64_tc(const double* U, const double* S, const do
     size_t pbytes = sg::part_bytes(pb, k);
     if (b % pb) pbytes = sg::part_bytes(b % pb, k) > pbytes ? sg::part_bytes(b % pb, k) : pbytes;     // the last panel
     const size_t o_p = take(pbytes);
+    const size_t o_f = take(std::max(sg::fix_bytes(pb, k), sg::fix_bytes(pb, m))), o_n = take(2 * sizeof(int));
     void* ws = nullptr;
     lrc_status st = stream_workspace_try(s, off, &ws);
     if (st != LRC_OK || !ws) return st;
     *handled = true;
     unsigned char* base = static_cast<unsigned char*>(ws);
+    sg::Listed* list = reinterpret_cast<sg::Listed*>(base + o_f);      // of one product after the other
+    int* counts = reinterpret_cast<int*>(base + o_n);
     double* W = reinterpret_cast<double*>(base + o_wd);
     double* part = reinterpret_cast<double*>(base + o_p);
     sg::operand_carve(&oV, base + o_v);
@@ -548,14 +553,14 @@ static lrc_status launch_apply_f64_tc(const double* U, const double* S, const do
         oX.rows = oW.rows = rows;
         sg::operand_carve(&oX, base + o_x);
         sg::operand_carve(&oW, base + o_w);
-        oW.cleared = true;
         const sg::Operand64* px[3] = {&oX, &oV, &oU};      // V and U with the first panel
         const sg::Operand64* pw[1] = {&oW};
-        if ((st = sg::slice(px, r0 == 0 ? 3 : 1, s)) != LRC_OK) return st;
-        if ((st = sg::product(oX, oV, sg::Out64{W, ldk, 1, nullptr, S, oW.hard}, true, part, s)) != LRC_OK) return st;
-        if ((st = sg::slice(pw, 1, s)) != LRC_OK) return st;
-        if ((st = sg::product(oW, oU, sg::Out64{Y + r0 * m, m, 1, nullptr, nullptr}, false, nullptr, s)) != LRC_OK)
+        const sg::Out64 oy{Y + r0 * m, m, 1, nullptr, nullptr};
+        if ((st = sg::slice(px, r0 == 0 ? 3 : 1, counts, 2, s)) != LRC_OK) return st;
+        if ((st = sg::product(oX, oV, sg::Out64{W, ldk, 1, nullptr, S}, true, part, {list, counts}, s)) != LRC_OK)
             return st;
+        if ((st = sg::slice(pw, 1, nullptr, 0, s)) != LRC_OK) return st;
+        if ((st = sg::product(oW, oU, oy, false, nullptr, {list, counts + 1}, s)) != LRC_OK) return st;
     }
     return LRC_OK;
 }

@@ -588,8 +588,11 @@ struct Carve {
 struct DigitGram {
     sg::Operand64 a;
     double* part;
+    sg::Listed* list;
 };
-size_t digit_gram_bytes(int p, int64_t L) { return sg::operand_bytes(p, L) + sg::part_bytes(p, p); }
+size_t digit_gram_bytes(int p, int64_t L) {
+    return sg::operand_bytes(p, L) + sg::part_bytes(p, p) + sg::fix_bytes(p, p);
+}
 DigitGram digit_gram(const double* A, int p, int64_t L, unsigned char* ws) {
     DigitGram g{};
     g.a.src = sg::Src64{A, 1, p, nullptr, 0};
@@ -597,6 +600,7 @@ DigitGram digit_gram(const double* A, int p, int64_t L, unsigned char* ws) {
     g.a.K = L;
     sg::operand_carve(&g.a, ws);
     g.part = reinterpret_cast<double*>(ws + sg::operand_bytes(p, L));
+    g.list = reinterpret_cast<sg::Listed*>(ws + sg::operand_bytes(p, L) + sg::part_bytes(p, p));
     return g;
 }
 
@@ -625,6 +629,7 @@ lrc_status lowrank_eta_t(const double* U, const double* S, const double* Vt, con
     lrc_status st = LRC_OK;
     bool digits = (double)(m + n) * w * w >= kDigitGramWork && m <= sg::kMaxK && n <= sg::kMaxK;
     const size_t o_du = c.take(digit_gram_bytes(w, m)), o_dv = c.take(digit_gram_bytes(w, n));
+    const size_t o_n = c.take(2 * sizeof(int));
     if (digits) {
         if ((st = stream_workspace_try(s, c.off, &ws)) != LRC_OK) return st;
         digits = ws != nullptr;
@@ -647,9 +652,10 @@ lrc_status lowrank_eta_t(const double* U, const double* S, const double* Vt, con
         const DigitGram g[2] = {digit_gram(Pu, w, m, (unsigned char*)base + o_du),
                                 digit_gram(Pv, w, n, (unsigned char*)base + o_dv)};
         const sg::Operand64* ops[2] = {&g[0].a, &g[1].a};
-        if ((st = sg::slice(ops, 2, s)) != LRC_OK) return st;
+        int* counts = (int*)(base + o_n);
+        if ((st = sg::slice(ops, 2, counts, 2, s)) != LRC_OK) return st;
         for (int i = 0; i < 2; ++i) {
-            if ((st = sg::gram(g[i].a, sp[i].C, w, g[i].part, s)) != LRC_OK) return st;
+            if ((st = sg::gram(g[i].a, sp[i].C, w, g[i].part, {g[i].list, counts + i}, s)) != LRC_OK) return st;
         }
     } else if ((st = run_gram(sp, 2, (double*)(base + o_part), s)) != LRC_OK) {
         return st;

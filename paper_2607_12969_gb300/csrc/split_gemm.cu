@@ -18,23 +18,33 @@
 //     2^24, so the tensor cores' binary32 accumulation forms them without
 //     error; those of classes 5 and 6 are as a rule, and where not the error
 //     is 2^-24 of a class that lies 2^-45 below the first.  Classes from 7 on
-//     are below 2^-62 and are left out (28 products of 49).
+//     are left out (28 products of 49).
 //   * every 64 terms (`period`: less often where the bound allows) the
 //     accumulators are drained into two 64-bit integers per entry, and the
 //     whole sum is rounded to binary64 once.
 //
-// So the result is as close as the best rounded one for rows whose entries
-// lie within about 2^-9 of each other's scale, and the error never exceeds
-// about 2^-61 of (largest of row i)(largest of row j) per term.  Rows that
-// this does not describe well -- their entries lie on average more than
-// 2^-kMaxGap below the largest, or they hold an infinity, a NaN or a largest
-// entry outside 2^-480 ... 2^495 -- get zero digits and are
-// recomputed by a kernel of binary64 FMAs (`repair`).
+// The error, in units of B_i B_j (B: the power of two above a row's largest
+// entry), is as a rule below 2^-61 a term with a sign of its own, and at worst
+// about 2^-57 a term, where the digits are all at their limits and of one sign
+// (the six products of class 7 alone then reach 2^-58.4).  That is small beside
+// S_ij = sum_k |a_ik b_jk| unless the large entries of one row meet zeros or
+// small entries of the other, where binary64 FMAs would be more exact.  So
+// S_ij is estimated from the first digits, sum_k |d_0 e_0| 2^-14, and an entry
+// of C for which that stays below 2^-5 (kMinSum) is listed and recomputed by
+// binary64 FMAs (repair_kernel).  The others are as a rule within
+// 0.1 sqrt(K) 2^-53 S_ij, and at worst (first digits rounded up from halves
+// besides) within K 2^-50 S_ij; FMA sums of K terms are bounded by K 2^-53 S_ij.
+// Rows of Gaussian entries reach the limit within 16 terms for all but 1e-6 of
+// the entries, also with columns scaled by j^-1.5 or 0.9^j.
+//
+// Rows that hold an infinity, a NaN or a largest entry outside 2^-480 ...
+// 2^495 get zero digits, so that all their entries are listed.
 //
 // Kernels: row statistics (row_stats_kernel), digits (slice_kernel, which
-// writes them as images that either side of a product loads by bulk copies), the product (product_kernel,
-// persistent, one CTA a SM), the ordered sum of split reductions
-// (part_sum_kernel) and the repair (repair_kernel).
+// writes them as images that either side of a product loads by bulk copies),
+// the product and the estimates of S (product_kernel, persistent, one CTA a
+// SM), the ordered sum of split reductions (part_sum_kernel) and the
+// recomputed entries (repair_kernel).
 #include <algorithm>
 #include <utility>
 
@@ -52,10 +62,14 @@ using namespace tc;
 __device__ unsigned int g_err_split;
 
 constexpr int64_t kOwnStatsK = 512;    // reductions up to this long: slice_kernel takes the row statistics itself
-constexpr int kMaxGap = 12;            // mean distance (in bits) of a row's entries below its largest
 constexpr int kNonFinite = 1 << 20;    // marks a row with an infinity or NaN in its statistics
+constexpr int kNoEntry = -(1 << 20);   // ... one without nonzero entries
+// In the exponents' place for a row whose digits are all zero: because it holds
+// nothing else, or because the digits cannot carry it.
+constexpr int kZeroRow = -1, kHardRow = -2;
+constexpr float kMinSum = 512.0f;      // 2^-5 in units of products of first digits
 // Biased exponents of a row's largest entry that digits carry: with both rows
-// inside, every result is zero or a normal number (round96).
+// inside, every result is zero or a normal number (round_pq).
 constexpr int kMinExp = 544, kMaxExp = 1518;
 
 // ---------------------------------------------------------------- sources
@@ -77,27 +91,16 @@ __device__ __forceinline__ int biased_exp(uint64_t bits) {
 }
 
 // ---------------------------------------------------------------- statistics
-// Per row: the largest biased exponent, the sum of the exponents of the
-// nonzero entries and their number.
-struct RowStat {
-    int mx = -(1 << 20), sum = 0, cnt = 0;
-    __device__ __forceinline__ void add(double x, int shift) {
-        const uint32_t h = (uint32_t)__double2hiint(x) & 0x7fffffffu, e = h >> 20;
-        int v = (int)e + shift, one = 1;
-        if (e - 1u >= 0x7feu) {            // zero, subnormal, infinity or NaN
-            one = (h | (uint32_t)__double2loint(x)) != 0 ? 1 : 0;
-            v = one ? biased_exp(((uint64_t)h << 32) | (uint32_t)__double2loint(x)) + shift : -(1 << 20);
-        }
-        mx = max(mx, v);
-        sum += one && v < kNonFinite / 2 ? v : 0;
-        cnt += one;
+// The largest biased exponent of a row's nonzero entries.
+__device__ __forceinline__ void stat_add(int& mx, double x, int shift) {
+    const uint32_t h = (uint32_t)__double2hiint(x) & 0x7fffffffu, e = h >> 20;
+    int v = (int)e + shift;
+    if (e - 1u >= 0x7feu) {            // zero, subnormal, infinity or NaN
+        const uint32_t lo = (uint32_t)__double2loint(x);
+        v = (h | lo) != 0 ? biased_exp(((uint64_t)h << 32) | lo) + shift : kNoEntry;
     }
-    __device__ __forceinline__ void merge(int4 o) {
-        mx = max(mx, o.x);
-        sum += o.y;
-        cnt += o.z;
-    }
-};
+    mx = max(mx, v);
+}
 
 // What the kernels below take of an operand, and its share of the blocks.
 struct Job {
@@ -106,15 +109,15 @@ struct Job {
     int64_t b0;              // first block
     int64_t kchunk;          // columns a block takes
     int kparts, splits, vec;
-    int4* stats;             // splits > 0: statistics per slice of K; else slice_kernel takes its own
+    int* stats;              // splits > 0: statistics per slice of K; else slice_kernel takes its own
     unsigned char* img;
     int* exps;
-    int* hard;
 };
 struct Jobs {
     Job j[kMaxOps];
     int n;
-    int* clear[kMaxOps];     // row lists to empty
+    int nclear;
+    int* clear;              // counters to set to zero
 };
 __device__ __forceinline__ const Job& job_of(const Jobs& js, int64_t block) {
     int i = 0;
@@ -126,15 +129,15 @@ __device__ __forceinline__ const Job& job_of(const Jobs& js, int64_t block) {
 // in warp 0.  K contiguous: a warp per row, lanes along K; else a lane per
 // row, so that either way a warp reads consecutive addresses.
 template <bool SCALED>
-__device__ __forceinline__ RowStat block_stats(const View64& v, int64_t r0, int64_t rows, int64_t k0, int64_t k1,
-                                               bool vec, int4 (&sm)[8][32]) {
+__device__ __forceinline__ int block_stats(const View64& v, int64_t r0, int64_t rows, int64_t k0, int64_t k1, bool vec,
+                                           int (&sm)[8][32]) {
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     auto shift = [&](int64_t k) { return SCALED ? v.shift(k) : 0; };
     if (v.s.cs == 1) {
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const int64_t r = r0 + warp + 8 * q;
-            RowStat a;
+            int a = kNoEntry;
             if (r < rows) {
                 int64_t k = k0 + 2 * lane;
                 if (vec) {
@@ -145,24 +148,22 @@ __device__ __forceinline__ RowStat block_stats(const View64& v, int64_t r0, int6
                             x[u] = __ldg(reinterpret_cast<const double2*>(v.s.p + r * v.s.rs + k + 64 * u));
 #pragma unroll
                         for (int u = 0; u < 4; ++u) {
-                            a.add(x[u].x, shift(k + 64 * u));
-                            a.add(x[u].y, shift(k + 64 * u + 1));
+                            stat_add(a, x[u].x, shift(k + 64 * u));
+                            stat_add(a, x[u].y, shift(k + 64 * u + 1));
                         }
                     }
                 }
                 for (; k < k1; k += 64) {
-                    a.add(v.at(r, k), shift(k));
-                    if (k + 1 < k1) a.add(v.at(r, k + 1), shift(k + 1));
+                    stat_add(a, v.at(r, k), shift(k));
+                    if (k + 1 < k1) stat_add(a, v.at(r, k + 1), shift(k + 1));
                 }
             }
-            a.mx = __reduce_max_sync(0xffffffffu, a.mx);
-            a.sum = __reduce_add_sync(0xffffffffu, a.sum);
-            a.cnt = __reduce_add_sync(0xffffffffu, a.cnt);
-            if (lane == 0) sm[0][warp + 8 * q] = make_int4(a.mx, a.sum, a.cnt, 0);
+            a = __reduce_max_sync(0xffffffffu, a);
+            if (lane == 0) sm[0][warp + 8 * q] = a;
         }
     } else {
         const int64_t r = r0 + lane;
-        RowStat a;
+        int a = kNoEntry;
         if (r < rows) {
             int64_t k = k0 + warp;
             for (; k + 24 < k1; k += 32) {
@@ -170,37 +171,36 @@ __device__ __forceinline__ RowStat block_stats(const View64& v, int64_t r0, int6
 #pragma unroll
                 for (int u = 0; u < 4; ++u) x[u] = v.at(r, k + 8 * u);
 #pragma unroll
-                for (int u = 0; u < 4; ++u) a.add(x[u], shift(k + 8 * u));
+                for (int u = 0; u < 4; ++u) stat_add(a, x[u], shift(k + 8 * u));
             }
-            for (; k < k1; k += 8) a.add(v.at(r, k), shift(k));
+            for (; k < k1; k += 8) stat_add(a, v.at(r, k), shift(k));
         }
-        sm[warp][lane] = make_int4(a.mx, a.sum, a.cnt, 0);
+        sm[warp][lane] = a;
     }
     __syncthreads();
-    RowStat t;
+    int t = kNoEntry;
     if (warp == 0) {
-        t.merge(sm[0][lane]);
+        t = sm[0][lane];
         if (v.s.cs != 1) {
 #pragma unroll
-            for (int w = 1; w < 8; ++w) t.merge(sm[w][lane]);
+            for (int w = 1; w < 8; ++w) t = max(t, sm[w][lane]);
         }
     }
     return t;
 }
 
 __global__ void __launch_bounds__(256) row_stats_kernel(const __grid_constant__ Jobs js) {
-    __shared__ int4 sm[8][32];
+    __shared__ int sm[8][32];
     pdl_wait();
     pdl_trigger();
     const Job& o = job_of(js, blockIdx.x);
     const int64_t lb = (int64_t)blockIdx.x - o.b0, rg = lb / o.splits, z = lb - rg * o.splits;
     const int64_t r0 = rg * 32, k0 = z * o.kchunk;
-    if (blockIdx.x == 0 && threadIdx.x < kMaxOps && js.clear[threadIdx.x]) *js.clear[threadIdx.x] = 0;
+    if (blockIdx.x == 0 && threadIdx.x < js.nclear) js.clear[threadIdx.x] = 0;
     const int64_t k1 = min(o.K, k0 + o.kchunk);
-    const RowStat a = o.v.s.scale ? block_stats<true>(o.v, r0, o.rows, k0, k1, o.vec != 0, sm)
-                                  : block_stats<false>(o.v, r0, o.rows, k0, k1, o.vec != 0, sm);
-    if (threadIdx.x < 32 && r0 + threadIdx.x < o.rows)
-        o.stats[z * o.rows + r0 + threadIdx.x] = make_int4(a.mx, a.sum, a.cnt, 0);
+    const int a = o.v.s.scale ? block_stats<true>(o.v, r0, o.rows, k0, k1, o.vec != 0, sm)
+                              : block_stats<false>(o.v, r0, o.rows, k0, k1, o.vec != 0, sm);
+    if (threadIdx.x < 32 && r0 + threadIdx.x < o.rows) o.stats[z * o.rows + r0 + threadIdx.x] = a;
 }
 
 // ---------------------------------------------------------------- digits
@@ -245,7 +245,7 @@ __device__ __forceinline__ void digits8(const double (&x)[8], const int (&sh)[8]
 // takes the row statistics itself); a lane is a row, so that a warp's 16-byte
 // stores of one digit are four runs of 128 bytes.
 __global__ void __launch_bounds__(256) slice_kernel(const __grid_constant__ Jobs js) {
-    __shared__ int4 sm[8][32];
+    __shared__ int sm[8][32];
     __shared__ int s_em[32];
     pdl_wait();
     pdl_trigger();
@@ -255,28 +255,17 @@ __global__ void __launch_bounds__(256) slice_kernel(const __grid_constant__ Jobs
     const int64_t lb = (int64_t)blockIdx.x - o.b0, rg = lb / o.kparts, kp = lb - rg * o.kparts;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int64_t r0 = rg * 32;
-    RowStat own;
+    int own = kNoEntry;
     if (o.splits == 0) own = block_stats<true>(v, r0, rows, 0, K, o.vec != 0, sm);
     if (tid < 32) {
         const int64_t r = r0 + lane;
-        int em = 1023;
-        bool zero = true;
+        int em = kZeroRow;
         if (r < rows) {
-            int mx = own.mx;
-            int64_t sum = own.sum, cnt = own.cnt;
-            for (int z = 0; z < o.splits; ++z) {
-                const int4 a = o.stats[(int64_t)z * rows + r];
-                mx = max(mx, a.x);
-                sum += a.y;
-                cnt += a.z;
-            }
-            if (cnt > 0) {
-                zero = mx < kMinExp || mx > kMaxExp || (int64_t)mx * cnt - sum > (int64_t)kMaxGap * cnt;
-                if (!zero) em = mx;
-                else if (kp == 0) o.hard[1 + atomicAdd(o.hard, 1)] = (int)r;
-            }
+            int mx = own;
+            for (int z = 0; z < o.splits; ++z) mx = max(mx, o.stats[(int64_t)z * rows + r]);
+            if (mx != kNoEntry) em = mx < kMinExp || mx > kMaxExp ? kHardRow : mx;
         }
-        s_em[lane] = zero ? -1 : em;
+        s_em[lane] = em;
         if (kp == 0 && r < o.img_rows) o.exps[r] = em;
     }
     __syncthreads();
@@ -331,6 +320,8 @@ struct GemmArgs {
     int split, group, stages, tma;
     int64_t a_block, b_block;    // bytes of a block of either image
     uint32_t a_bytes, b_bytes;   // of a tile's part of it
+    Listed* fix;                 // entries to recompute, and the number of blocks of them
+    int* nfix;
     int listed;                  // > 0: the tiles are list[0 ... listed), row << 8 | column
     uint16_t list[kMaxListed];
     uint32_t tmem_cols;
@@ -342,7 +333,8 @@ struct GemmArgs {
 // chunks took 26000 clocks, its MMAs 10750).
 constexpr int kEpiWarps = 16;
 constexpr int kThreads = 32 * (4 + kEpiWarps);
-// Registers: the first four warps (producer, MMA issuer, two idle) hand some
+// Registers: the first four warps (producer, MMA issuer, two that estimate the
+// sums of magnitudes) hand some
 // of theirs to the epilogue's, which keep two 64-bit sums per entry: 128 x 64
 // + 512 x 104 = 61440, the 640 x 96 = 61440 of the launch.
 constexpr int kRegsLow = 64, kRegsEpi = 104;
@@ -462,6 +454,115 @@ __device__ __forceinline__ void issue(uint32_t tmem, uint32_t col3, uint32_t fre
                                                                                                   blo, bhi);
 }
 
+// Four bytes of an image's first digits: those of row `lane` / 4 of a group and
+// columns 2 (lane % 4) + {0, 1} of an octet, without their signs.
+__device__ __forceinline__ uint32_t first_digits(const unsigned char* group, int octet, int lane) {
+    return __ldg(reinterpret_cast<const uint32_t*>(group + octet * 128 + lane * 4)) & 0x7fff7fffu;
+}
+// The same as an A fragment of m16n8k16: two row groups, both octets.
+__device__ __forceinline__ void first_digits_a(const unsigned char* p, int lane, uint32_t (&d)[4]) {
+    d[0] = first_digits(p, 0, lane);
+    d[1] = first_digits(p + kGroupBytes, 0, lane);
+    d[2] = first_digits(p, 1, lane);
+    d[3] = first_digits(p + kGroupBytes, 1, lane);
+}
+// d = a b + c (16 x 8, 16 terms)
+__device__ __forceinline__ void mma_16x8(float (&d)[4], const uint32_t (&a)[4], const uint32_t (&b)[2],
+                                         float c0, float c1, float c2, float c3) {
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, "
+                 "{%8, %9}, {%10, %11, %12, %13};"
+                 : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]), "f"(c0), "f"(c1), "f"(c2), "f"(c3));
+}
+
+// Lists the entries of half a tile's columns whose sums of magnitudes, estimated
+// from the first digits, do not reach kMinSum, 16 rows at a time, straight from
+// the images, whose octets have the layout of m16n8k16 fragments.  On most data
+// the first 16 terms pass for all entries: two warps have the time of the tile's
+// MMAs and epilogue for them, if the loads are not waited for one by one
+// (16384 x 8192, k = 128, b = 8192: 1577 us without the estimates, 2016 with each
+// load waited for, 1575 like this).  Where they do not, the sums go on over at
+// most kLookBlocks, and what then is below the limit is listed: repair_kernel
+// looks at the rest of the reduction with more warps.
+constexpr int kLookBlocks = 8;
+template <int NT>
+__device__ __forceinline__ void list_small_sums(const GemmArgs& a, int mt, int nt, int half, int lane) {
+    constexpr int J = NT / 16, kBatch = 4;
+    const int row_t = mt * 128, col0 = nt * NT + half * (NT / 2);
+    if (col0 >= a.N) return;
+    auto columns = [&](int kb, uint32_t (&d)[J][2]) {      // (what lies past the last row is not defined)
+        const unsigned char* p = a.B + kb * a.b_block + (int64_t)(col0 >> 3) * kGroupBytes;
+#pragma unroll
+        for (int j = 0; j < J; ++j) {
+            const bool in = col0 + 8 * j < a.N;
+            d[j][0] = in ? first_digits(p + j * kGroupBytes, 0, lane) : 0u;
+            d[j][1] = in ? first_digits(p + j * kGroupBytes, 1, lane) : 0u;
+        }
+    };
+    // rows lane / 4 (0, 1) and lane / 4 + 8 (2, 3), columns 8 j + 2 (lane % 4) + {0, 1}
+    float acc[J][4];
+    auto reached = [&]() {
+        float least = acc[0][0];
+#pragma unroll
+        for (int j = 0; j < J; ++j)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) least = fminf(least, acc[j][i]);
+        return __all_sync(0xffffffffu, least >= kMinSum) != 0;
+    };
+    uint32_t b[J][2];
+    columns(0, b);
+    uint32_t failed = 0;                                   // strips whose first terms do not suffice
+    for (int s0 = 0; s0 < 8; s0 += kBatch) {
+        const unsigned char* rows = a.A + (int64_t)((row_t >> 3) + 2 * s0) * kGroupBytes;
+        uint32_t x[kBatch][4];
+#pragma unroll
+        for (int s = 0; s < kBatch; ++s)                   // (rows are padded to 16)
+            if (row_t + 16 * (s0 + s) < a.M) first_digits_a(rows + s * 2 * kGroupBytes, lane, x[s]);
+#pragma unroll
+        for (int s = 0; s < kBatch; ++s) {
+            if (row_t + 16 * (s0 + s) >= a.M) break;
+#pragma unroll
+            for (int j = 0; j < J; ++j) mma_16x8(acc[j], x[s], b[j], 0.0f, 0.0f, 0.0f, 0.0f);
+            failed |= reached() ? 0u : 1u << (s0 + s);
+        }
+    }
+    for (; failed; failed &= failed - 1) {
+        const int row0 = row_t + 16 * (__ffs((int)failed) - 1);
+        // Entries that need no sum: past the edges, a row of zeros with one that holds
+        // no infinity or NaN, what a symmetric product leaves out.
+#pragma unroll
+        for (int i = 0; i < 4 * J; ++i) {
+            const int r = row0 + (lane >> 2) + 8 * ((i >> 1) & 1), c = col0 + 8 * (i >> 2) + 2 * (lane & 3) + (i & 1);
+            const int er = r < a.M ? a.ea[r] : 0, ec = c < a.N ? a.eb[c] : 0;
+            const bool zero = (er == kZeroRow && ec != kHardRow) || (ec == kZeroRow && er != kHardRow);
+            acc[i >> 2][i & 3] = zero || r >= a.M || c >= a.N || (a.listed && r > c) ? kMinSum : 0.0f;
+        }
+        const int last = min(a.kblocks, kLookBlocks);
+        bool done = reached();
+        for (int kb = 0; kb < last && !done; ++kb) {
+            uint32_t y[4];
+            first_digits_a(a.A + kb * a.a_block + (int64_t)(row0 >> 3) * kGroupBytes, lane, y);
+            columns(kb, b);
+#pragma unroll
+            for (int j = 0; j < J; ++j) mma_16x8(acc[j], y, b[j], acc[j][0], acc[j][1], acc[j][2], acc[j][3]);
+            done = reached();
+        }
+        if (done) continue;
+        int at = 0;
+        if (lane == 0) at = atomicAdd(a.nfix, 1);
+        Listed* f = a.fix + __shfl_sync(0xffffffffu, at, 0);
+        if (lane == 0) {
+            f->row0 = row0;
+            f->col0 = col0;
+        }
+#pragma unroll
+        for (int i = 0; i < 4 * J; ++i) {
+            const uint32_t m = __ballot_sync(0xffffffffu, !(acc[i >> 2][i & 3] >= kMinSum));
+            if (lane == 0) f->mask[i] = m;
+        }
+    }
+}
+
 template <int NT>
 __global__ void __launch_bounds__(kThreads, 1) product_kernel(const __grid_constant__ GemmArgs a,
                                                               const __grid_constant__ CUtensorMap tm_c) {
@@ -521,7 +622,7 @@ __global__ void __launch_bounds__(kThreads, 1) product_kernel(const __grid_const
         };
         while (ok && pc.next(a, &tile, &c0, &c1)) {
             const int2 at = tile_at(a, tile);
-                const int mt = at.x, nt = at.y;
+            const int mt = at.x, nt = at.y;
             const int64_t row = (int64_t)mt * 128 + r, col0 = (int64_t)nt * NT + quarter * HC;
             // exponents: of the thread's row, and of column `lane`
             const int ea = row < a.M ? a.ea[row] : 0;
@@ -621,7 +722,7 @@ __global__ void __launch_bounds__(kThreads, 1) product_kernel(const __grid_const
             bool ok = true;
             while (ok && pc.next(a, &tile, &c0, &c1)) {
                 const int2 at = tile_at(a, tile);
-            const int mt = at.x, nt = at.y;
+                const int mt = at.x, nt = at.y;
                 const int b1 = min(kChunkBlocks * c1, a.kblocks);
                 for (int kb = kChunkBlocks * c0; kb < b1; ++kb, ++it) {
                     if (!(ok = mbar_wait(&empty[slot], phase, abort, err, 1u))) break;
@@ -720,6 +821,15 @@ __global__ void __launch_bounds__(kThreads, 1) product_kernel(const __grid_const
         __syncwarp();
         volatile int no_abort = 0;
         mbar_wait(mma_done, 0, &no_abort, err, 2u, 100000000ull);
+    } else {
+        // ------------------------------------------------------------ sums of magnitudes
+        Pieces<GemmArgs> pc(a);
+        int tile, c0, c1;
+        while (pc.next(a, &tile, &c0, &c1)) {
+            if (c0 != 0) continue;             // the tile's first piece looks at all of the reduction
+            const int2 at = tile_at(a, tile);
+            list_small_sums<NT>(a, at.x, at.y, warp - 2, lane);
+        }
     }
     }
     __syncwarp();
@@ -738,10 +848,9 @@ constexpr int kManyParts = 24;
 template <bool MANY>
 __global__ void __launch_bounds__(256) part_sum_kernel(const __grid_constant__ GemmArgs a, int NT, int64_t Q, int64_t G,
                                                        double* __restrict__ C, const double* __restrict__ rscale,
-                                                       const double* __restrict__ cscale, int* __restrict__ clear) {
+                                                       const double* __restrict__ cscale) {
     pdl_wait();
     pdl_trigger();
-    if (clear && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *clear = 0;
     const int tile = blockIdx.x;
     const int2 at = tile_at(a, tile);
     const int64_t u = (int64_t)(tile / a.group) * a.chunks;
@@ -780,140 +889,174 @@ __global__ void __launch_bounds__(256) part_sum_kernel(const __grid_constant__ G
 }
 
 // ---------------------------------------------------------------- repair
-// Rows listed as hard: their part of C by binary64 FMAs.  The binary64 pipe (two
-// FMAs a clock on an SM) is the bound, as for the FMA kernels of the other paths;
-// with every row listed (factors whose entries decay over many binades) a product
-// should take what it takes there.  So the tile follows from how many there are:
-// R x R entries a thread in tiles of 16 R, and for few entries (R = 0) tiles of
-// 8 x 8 whose reduction is split over four threads.  With entries over 60 binades
-// in both operands: apply 16384 x 8192, k = 128, b = 2048 11.3 ms (FMA kernels
-// 11.2), 12287 x 16384, k = 272, b = 250 4.1 ms (4.2); 64 x 64 tiles alone
-// took about 100 ms for results of 140 x 104 with a reduction of 71680.
+// Listed entries by binary64 FMAs, whose rate (two a clock on an SM) is the bound
+// where there are many.
+//  * Reductions from kLongK on: a warp takes 8 x 8 entries, finishes the sums of
+//    their magnitudes, and recomputes those that stay below the limit, 8 x 4 at a
+//    time with the lanes along the reduction, or where there are few one after
+//    the other.
+//  * Shorter ones: a warp takes 16 x 8 entries, four a lane.
 struct RepairArgs {
     View64 A, B;
-    const int* ha;
-    const int* hb;
-    int64_t M, N, K;
+    const Listed* fix;
+    const int* nfix;
+    int64_t K;
     double* C;
     int64_t cr, cc;
     const double* rscale;
     const double* cscale;
-    int sym;                  // A and B are the same operand, C symmetric
+    int sym;                  // C symmetric, the entries above the diagonal are listed
+    int words;                // of a mask
+    const unsigned char* ia;  // the images, for longer sums of first digits
+    const unsigned char* ib;
+    int64_t a_block, b_block;
+    int kblocks;
 };
-constexpr int kRepairWords = 128 * 9;        // staged entries of an operand, with padding (the largest of all R)
+constexpr int kLongK = 96, kFew = 4;
 
-template <int R>
-__host__ __device__ constexpr int repair_tile() { return R == 0 ? 8 : 16 * R; }
-
-__device__ __forceinline__ int64_t repair_tiles(int64_t na, int64_t nb, int64_t M, int64_t N, int T) {
-    return (na + T - 1) / T * ((N + T - 1) / T) + (nb + T - 1) / T * ((M + T - 1) / T);
+__device__ __forceinline__ void put_entry(const RepairArgs& a, int64_t row, int64_t col, double s) {
+    if (a.rscale) s *= __ldg(a.rscale + row);
+    if (a.cscale) s *= __ldg(a.cscale + col);
+    a.C[row * a.cr + col * a.cc] = s;
+    if (a.sym) a.C[col * a.cr + row * a.cc] = s;
 }
 
-template <int R>
-__device__ __forceinline__ void repair_body(const RepairArgs& a, int64_t na, int64_t nb, double* As, double* Bs) {
-    constexpr int T = repair_tile<R>(), KS = 1024 / T, P = T + 1, E = R == 0 ? 1 : R, W = R == 0 ? 8 : 16;
-    const int64_t ta = (na + T - 1) / T * ((a.N + T - 1) / T), tiles = repair_tiles(na, nb, a.M, a.N, T);
-    const int tid = threadIdx.x;
-    const int part = R == 0 ? tid / 64 : 0;                        // quarter of the reduction
-    const int tx = tid % W, ty = R == 0 ? tid / 8 % 8 : tid / 16;
-    const bool all = na == a.M;                                    // every row of A: in order, not by the list
-    for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
-        // tile of C rows (first list entry or row) and columns
-        const bool ga = t < ta;
-        const int64_t u = ga ? t : t - ta;
-        const int64_t other = ((ga ? a.N : a.M) + T - 1) / T;
-        const int64_t l0 = u / other * T, o0 = (u % other) * T;
-        const int64_t i0 = ga ? l0 : o0, j0 = ga ? o0 : l0;
-        if (a.sym && all && i0 > j0) continue;                     // written with the tile above the diagonal
-        const int64_t ni = ga ? na : a.M, nj = ga ? a.N : nb;
-        auto row_of = [&](int i) {
-            return i0 + i >= ni ? -1 : ga && !all ? __ldg(a.ha + 1 + i0 + i) : (int)(i0 + i);
-        };
-        auto col_of = [&](int j) { return j0 + j >= nj ? -1 : ga ? (int)(j0 + j) : __ldg(a.hb + 1 + j0 + j); };
-        // a thread stages four entries of each operand, neighbours along k
-        const int kk = tid % KS, x0 = tid / KS;
-        constexpr int XS = 256 / KS > 0 ? 256 / KS : 1;
-        static_assert(KS <= 256, "");
-        int ri[4], cj[4];
+// One entry: lanes along the reduction, eight loads of either operand in flight.
+__device__ __forceinline__ void repair_dot(const RepairArgs& a, int64_t row, int64_t col, int lane) {
+    double s = 0.0;
+    for (int64_t k0 = 0; k0 < a.K; k0 += 256) {
+        double x[8], y[8];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            ri[q] = row_of(x0 + q * XS);
-            cj[q] = col_of(x0 + q * XS);
-        }
-        double acc[E][E];
-#pragma unroll
-        for (int i = 0; i < E; ++i)
-#pragma unroll
-            for (int j = 0; j < E; ++j) acc[i][j] = 0.0;
-        double va[4], vb[4];
-        auto load = [&](int64_t k0) {
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                va[q] = ri[q] >= 0 && k0 + kk < a.K ? a.A.at(ri[q], k0 + kk) : 0.0;
-                vb[q] = cj[q] >= 0 && k0 + kk < a.K ? a.B.at(cj[q], k0 + kk) : 0.0;
-            }
-        };
-        load(0);
-        for (int64_t k0 = 0; k0 < a.K; k0 += KS) {
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                As[kk * P + x0 + q * XS] = va[q];
-                Bs[kk * P + x0 + q * XS] = vb[q];
-            }
-            __syncthreads();
-            if (k0 + KS < a.K) load(k0 + KS);                      // in flight over this slab's FMAs
-            const int kn = (int)min((int64_t)KS, a.K - k0);
-            const int kb = R == 0 ? part * (KS / 4) : 0, ke = R == 0 ? min(kn, kb + KS / 4) : kn;
-#pragma unroll 4
-            for (int k = kb; k < ke; ++k) {
-                double x[E], y[E];
-#pragma unroll
-                for (int i = 0; i < E; ++i) x[i] = As[k * P + ty + W * i];
-#pragma unroll
-                for (int j = 0; j < E; ++j) y[j] = Bs[k * P + tx + W * j];
-#pragma unroll
-                for (int i = 0; i < E; ++i)
-#pragma unroll
-                    for (int j = 0; j < E; ++j) acc[i][j] = fma(x[i], y[j], acc[i][j]);
-            }
-            __syncthreads();
-        }
-        if (R == 0) {
-            As[tid] = acc[0][0];
-            __syncthreads();
-            acc[0][0] = ((As[tid & 63] + As[64 + (tid & 63)]) + As[128 + (tid & 63)]) + As[192 + (tid & 63)];
-            __syncthreads();
-            if (part != 0) continue;
+        for (int u = 0; u < 8; ++u) {
+            const int64_t k = k0 + 32 * u + lane;
+            x[u] = k < a.K ? a.A.at(row, k) : 0.0;
+            y[u] = k < a.K ? a.B.at(col, k) : 0.0;
         }
 #pragma unroll
-        for (int i = 0; i < E; ++i) {
-            const int64_t row = row_of(ty + W * i);
-            if (row < 0) continue;
+        for (int u = 0; u < 8; ++u) s = fma(x[u], y[u], s);
+    }
 #pragma unroll
-            for (int j = 0; j < E; ++j) {
-                const int64_t col = col_of(tx + W * j);
-                if (col < 0) continue;
-                double s = acc[i][j];
-                if (a.rscale) s *= __ldg(a.rscale + row);
-                if (a.cscale) s *= __ldg(a.cscale + col);
-                a.C[row * a.cr + col * a.cc] = s;
-                if (a.sym && all) a.C[col * a.cr + row * a.cc] = s;
-            }
+    for (int o = 16; o > 0; o /= 2) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) put_entry(a, row, col, s);
+}
+
+// Rows r0 ... r0 + 7 and columns c0, c0 + 2, c0 + 4, c0 + 6, bit 4 row + column / 2 of `mask`.
+__device__ __forceinline__ void repair_word(const RepairArgs& a, int64_t r0, int64_t c0, uint32_t mask, int lane) {
+    // an entry that is not listed may lie past the edge: the last listed one's row or column instead
+    const uint32_t cols = (mask | mask >> 4 | mask >> 8 | mask >> 12 | mask >> 16 | mask >> 20 | mask >> 24 | mask >> 28) & 15u;
+    const int rmax = (31 - __clz((int)mask)) / 4, cmax = 31 - __clz((int)cols);
+    double acc[32];
+#pragma unroll
+    for (int i = 0; i < 32; ++i) acc[i] = 0.0;
+    for (int64_t k = lane; k < a.K; k += 32) {
+        double x[8], y[4];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) x[i] = a.A.at(r0 + min(i, rmax), k);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) y[j] = a.B.at(c0 + 2 * min(j, cmax), k);
+#pragma unroll
+        for (int i = 0; i < 32; ++i) acc[i] = fma(x[i / 4], y[i % 4], acc[i]);
+    }
+    // the lanes' sums: lane l ends with entry l's
+#pragma unroll
+    for (int o = 16; o > 0; o /= 2) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int i = 0; i < o; ++i) {
+            const double mine = up ? acc[i + o] : acc[i], other = up ? acc[i] : acc[i + o];
+            acc[i] = mine + __shfl_xor_sync(0xffffffffu, other, o);
         }
     }
+    if ((mask >> lane) & 1) put_entry(a, r0 + lane / 4, c0 + 2 * (lane & 3), acc[0]);
+}
+
+// Which of 8 x 8 listed entries (words m0, m1) stay below the limit over all of
+// the reduction: eight blocks' digits in flight.
+__device__ __forceinline__ void still_small(const RepairArgs& a, int64_t r0, int64_t c0, int lane, uint32_t& m0,
+                                            uint32_t& m1) {
+    const unsigned char* pa = a.ia + (r0 >> 3) * kGroupBytes;
+    const unsigned char* pb = a.ib + (c0 >> 3) * kGroupBytes;
+    const bool on0 = (m0 >> lane) & 1, on1 = (m1 >> lane) & 1;
+    float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    for (int kb = 0; kb < a.kblocks; kb += 8) {
+        uint32_t x[8][4], y[8][2];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const bool in = kb + u < a.kblocks;
+            x[u][1] = x[u][3] = 0u;
+            x[u][0] = in ? first_digits(pa + (kb + u) * a.a_block, 0, lane) : 0u;
+            x[u][2] = in ? first_digits(pa + (kb + u) * a.a_block, 1, lane) : 0u;
+            y[u][0] = in ? first_digits(pb + (kb + u) * a.b_block, 0, lane) : 0u;
+            y[u][1] = in ? first_digits(pb + (kb + u) * a.b_block, 1, lane) : 0u;
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) mma_16x8(acc, x[u], y[u], acc[0], acc[1], acc[2], acc[3]);
+        if (__all_sync(0xffffffffu, (!on0 || acc[0] >= kMinSum) && (!on1 || acc[1] >= kMinSum))) break;
+    }
+    m0 &= __ballot_sync(0xffffffffu, !(acc[0] >= kMinSum));
+    m1 &= __ballot_sync(0xffffffffu, !(acc[1] >= kMinSum));
 }
 
 __global__ void __launch_bounds__(256, 2) repair_kernel(const __grid_constant__ RepairArgs a) {
-    __shared__ double As[kRepairWords], Bs[kRepairWords];
     pdl_wait();
     pdl_trigger();
-    const int64_t na = a.ha[0], nb = na == a.M ? 0 : a.hb[0];      // every row of A: all of C
-    if (na + nb == 0) return;
-    const int64_t grid = gridDim.x;
-    if (repair_tiles(na, nb, a.M, a.N, 64) >= 2 * grid) repair_body<4>(a, na, nb, As, Bs);
-    else if (repair_tiles(na, nb, a.M, a.N, 32) >= 2 * grid) repair_body<2>(a, na, nb, As, Bs);
-    else if (repair_tiles(na, nb, a.M, a.N, 16) >= 4 * grid) repair_body<1>(a, na, nb, As, Bs);
-    else repair_body<0>(a, na, nb, As, Bs);
+    const int64_t n = *a.nfix;
+    if (n == 0) return;
+    const int lane = threadIdx.x & 31;
+    const int64_t w0 = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5), warps = (int64_t)gridDim.x * 8;
+    if (a.K >= kLongK) {
+        // Few blocks: several warps a block, each with a word or with its share of the entries.
+        const int pairs = a.words / 2;
+        const int64_t blocks = n * pairs;
+        const int share = blocks * 32 <= warps ? 32 : blocks * 8 <= warps ? 8 : blocks * 2 <= warps ? 2 : 1;
+        for (int64_t u = w0; u < blocks * share; u += warps) {
+            const Listed& f = a.fix[u / share / pairs];
+            const int i = 2 * (int)(u / share % pairs), mine = (int)(u % share);
+            uint32_t m[2] = {f.mask[i], f.mask[i + 1]};
+            if (!(m[0] | m[1])) continue;
+            const int64_t r0 = f.row0 + 8 * ((i >> 1) & 1), c0 = f.col0 + 8 * (i >> 2);
+            if (a.kblocks > kLookBlocks) still_small(a, r0, c0, lane, m[0], m[1]);
+            int e = 0;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                if (share == 2 && mine != h) continue;
+                if (share <= 2 && __popc(m[h]) > kFew) {
+                    repair_word(a, r0, c0 + h, m[h], lane);
+                } else {
+                    for (uint32_t w = m[h]; w; w &= w - 1, ++e) {
+                        const int bit = __ffs((int)w) - 1;
+                        if (share <= 2 || e % share == mine) repair_dot(a, r0 + bit / 4, c0 + h + 2 * (bit & 3), lane);
+                    }
+                }
+            }
+        }
+        return;
+    }
+    const int groups = a.words / 4;
+    for (int64_t u = w0; u < n * groups; u += warps) {
+        const Listed& f = a.fix[u / groups];
+        const int j = (int)(u % groups);
+        bool on[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) on[i] = (f.mask[4 * j + i] >> lane) & 1;
+        const bool top = on[0] || on[1], low = on[2] || on[3], left = on[0] || on[2], right = on[1] || on[3];
+        if (!top && !low) continue;
+        // an entry that is not listed may lie past the edge: a listed one's row or column instead
+        const int64_t r = f.row0 + lane / 4, c = f.col0 + 8 * j + 2 * (lane & 3);
+        const int64_t r0 = top ? r : r + 8, r1 = low ? r + 8 : r, c0 = left ? c : c + 1, c1 = right ? c + 1 : c;
+        double acc[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 4
+        for (int64_t k = 0; k < a.K; ++k) {
+            const double x0 = a.A.at(r0, k), x1 = a.A.at(r1, k), y0 = a.B.at(c0, k), y1 = a.B.at(c1, k);
+            acc[0] = fma(x0, y0, acc[0]);
+            acc[1] = fma(x0, y1, acc[1]);
+            acc[2] = fma(x1, y0, acc[2]);
+            acc[3] = fma(x1, y1, acc[3]);
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            if (on[i]) put_entry(a, r + 8 * (i >> 1), c + (i & 1), acc[i]);
+    }
 }
 
 size_t up256(size_t v) { return (v + 255) & ~(size_t)255; }
@@ -940,7 +1083,7 @@ lrc_status launch_product(const GemmArgs& a, const CUtensorMap& tm, int64_t grid
 size_t operand_bytes(int64_t rows, int64_t K) {
     const int64_t ir = image_rows(rows);
     return up256((size_t)(ir / 8) * image_blocks(K) * kGroupBytes + kTailBytes) + up256((size_t)ir * 4) +
-           up256((size_t)rows * (K > kOwnStatsK ? kStatSplits : 0) * sizeof(int4)) + hard_bytes(rows);
+           up256((size_t)rows * (K > kOwnStatsK ? kStatSplits : 0) * 4);
 }
 
 void operand_carve(Operand64* o, unsigned char* ws) {
@@ -949,13 +1092,13 @@ void operand_carve(Operand64* o, unsigned char* ws) {
     ws += up256((size_t)(ir / 8) * image_blocks(o->K) * kGroupBytes + kTailBytes);
     o->exps = reinterpret_cast<int*>(ws);
     ws += up256((size_t)ir * 4);
-    o->stats = reinterpret_cast<int4*>(ws);
-    ws += up256((size_t)o->rows * (o->K > kOwnStatsK ? kStatSplits : 0) * sizeof(int4));
-    o->hard = reinterpret_cast<int*>(ws);
+    o->stats = reinterpret_cast<int*>(ws);
 }
 
-lrc_status slice(const Operand64* const* ops, int count, cudaStream_t s) {
+lrc_status slice(const Operand64* const* ops, int count, int* clear, int nclear, cudaStream_t s) {
     Jobs st{}, sl{};
+    st.clear = clear;
+    st.nclear = nclear;
     int64_t bs = 0, bl = 0;
     for (int i = 0; i < count; ++i) {
         const Operand64& o = *ops[i];
@@ -969,7 +1112,6 @@ lrc_status slice(const Operand64* const* ops, int count, cudaStream_t s) {
         j.stats = o.stats;
         j.img = o.img;
         j.exps = o.exps;
-        j.hard = o.hard;
         if (o.K > kOwnStatsK) {
             const int z = stat_splits(o.rows, o.K);
             j.kchunk = ((o.K + z - 1) / z + 31) / 32 * 32;
@@ -985,7 +1127,6 @@ lrc_status slice(const Operand64* const* ops, int count, cudaStream_t s) {
         j.b0 = bl;
         bl += (j.img_rows + 31) / 32 * j.kparts;
         sl.j[sl.n++] = j;
-        if (!o.cleared) st.clear[i] = o.hard;
     }
     if (bs > 0x7fffffff || bl > 0x7fffffff) {
         set_error("split product: operand too large");
@@ -994,9 +1135,8 @@ lrc_status slice(const Operand64* const* ops, int count, cudaStream_t s) {
     lrc_status r;
     cudaError_t e;
     if (st.n == 0) {
-        for (int i = 0; i < count; ++i)
-            if (st.clear[i] && (e = cudaMemsetAsync(st.clear[i], 0, sizeof(int), s)) != cudaSuccess)
-                return cuda_fail(e, "cudaMemsetAsync (row list)");
+        if (nclear > 0 && (e = cudaMemsetAsync(clear, 0, nclear * sizeof(int), s)) != cudaSuccess)
+            return cuda_fail(e, "cudaMemsetAsync (counters)");
     } else {
         e = launch_pdl(row_stats_kernel, dim3((unsigned)bs), dim3(256), 0, s, st);
         if (e != cudaSuccess) return cuda_fail(e, "row_stats_kernel launch");
@@ -1022,10 +1162,15 @@ size_t part_bytes(int64_t M, int64_t N) {
     return up256((size_t)(tiles_of(M, N) + sm_count()) * 128 * n_tile(N) * 8);
 }
 
+size_t fix_bytes(int64_t M, int64_t N) {
+    if (tiles_of(N, M) < tiles_of(M, N)) std::swap(M, N);
+    return up256((size_t)((M + 15) / 16) * (size_t)(2 * n_tiles(N)) * sizeof(Listed));
+}
+
 namespace {
 
-lrc_status run_product(const Operand64& A0, const Operand64& B0, const Out64& out0, bool split, double* part, bool sym,
-                       cudaStream_t s) {
+lrc_status run_product(const Operand64& A0, const Operand64& B0, const Out64& out0, bool split, double* part,
+                       const Fix& fix, bool sym, cudaStream_t s) {
     const bool swap = tiles_of(B0.rows, A0.rows) < tiles_of(A0.rows, B0.rows);
     const Operand64& A = swap ? B0 : A0;
     const Operand64& B = swap ? A0 : B0;
@@ -1041,6 +1186,8 @@ lrc_status run_product(const Operand64& A0, const Operand64& B0, const Out64& ou
     a.ea = A.exps;
     a.eb = B.exps;
     a.C = split ? part : out.C;
+    a.fix = fix.list;
+    a.nfix = fix.count;
     a.cr = out.cr;
     a.cc = out.cc;
     a.M = A.rows;
@@ -1101,20 +1248,20 @@ lrc_status run_product(const Operand64& A0, const Operand64& B0, const Out64& ou
         case 32: st = launch_product<32>(a, tm, grid, smem, s); break;
         case 48: st = launch_product<48>(a, tm, grid, smem, s); break;
         default: st = launch_product<64>(a, tm, grid, smem, s); break;
-        
     }
     if (st != LRC_OK) return st;
     cudaError_t e;
     if (split) {
         const bool many = groups / (tiles / a.group) >= kManyParts;
-        const unsigned gy = (unsigned)std::max<int64_t>(1, std::min<int64_t>(128 * NT / (many ? 32 : 256), (many ? 8 : 4) * sms / tiles));
+        const int64_t most = 128 * NT / (many ? 32 : 256), want = (many ? 8 : 4) * sms / tiles;
+        const unsigned gy = (unsigned)std::max<int64_t>(1, std::min(most, want));
         e = launch_pdl(many ? part_sum_kernel<true> : part_sum_kernel<false>, dim3((unsigned)tiles, gy), dim3(256), 0,
-                       s, a, NT, Q, groups, out.C, out.rscale, out.cscale, out.clear);
+                       s, a, NT, Q, groups, out.C, out.rscale, out.cscale);
         if (e != cudaSuccess) return cuda_fail(e, "part_sum_kernel launch");
         if ((st = after_launch("part_sum_kernel")) != LRC_OK) return st;
     }
-    const RepairArgs r{View64{A.src}, View64{B.src}, A.hard, B.hard, A.rows, B.rows, A.K, out.C, out.cr, out.cc,
-                       out.rscale, out.cscale, sym ? 1 : 0};
+    const RepairArgs r{View64{A.src}, View64{B.src}, fix.list, fix.count, A.K, out.C, out.cr, out.cc,
+                       out.rscale, out.cscale, a.listed ? 1 : 0, NT / 4, a.A, a.B, a.a_block, a.b_block, a.kblocks};
     e = launch_pdl(repair_kernel, dim3((unsigned)(2 * sms)), dim3(256), 0, s, r);
     if (e != cudaSuccess) return cuda_fail(e, "repair_kernel launch");
     return after_launch("repair_kernel");
@@ -1122,12 +1269,13 @@ lrc_status run_product(const Operand64& A0, const Operand64& B0, const Out64& ou
 
 }  // namespace
 
-lrc_status product(const Operand64& A, const Operand64& B, const Out64& out, bool split, double* part, cudaStream_t s) {
-    return run_product(A, B, out, split, part, false, s);
+lrc_status product(const Operand64& A, const Operand64& B, const Out64& out, bool split, double* part, const Fix& fix,
+                   cudaStream_t s) {
+    return run_product(A, B, out, split, part, fix, false, s);
 }
 
-lrc_status gram(const Operand64& A, double* C, int64_t ldc, double* part, cudaStream_t s) {
-    return run_product(A, A, Out64{C, ldc, 1, nullptr, nullptr}, true, part, true, s);
+lrc_status gram(const Operand64& A, double* C, int64_t ldc, double* part, const Fix& fix, cudaStream_t s) {
+    return run_product(A, A, Out64{C, ldc, 1, nullptr, nullptr}, true, part, fix, true, s);
 }
 
 }  // namespace sg

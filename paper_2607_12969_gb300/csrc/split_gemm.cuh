@@ -42,9 +42,7 @@ struct Operand64 {
     int64_t rows, K;
     unsigned char* img;      // digits
     int* exps;               // exponent of every row (image rows)
-    int4* stats;             // row statistics per slice of K
-    int* hard;               // hard[0] = rows that the digits cannot carry; then their indices
-    bool cleared = false;    // an earlier kernel of the call has set hard[0] = 0
+    int* stats;              // row statistics per slice of K
 };
 constexpr int kMaxOps = 5;   // operands per slice()
 
@@ -56,31 +54,44 @@ inline int64_t image_rows(int64_t rows) { return (rows + 15) / 16 * 16; }
 constexpr int kTailBytes = 16 * kGroupBytes;
 inline int64_t image_blocks(int64_t K) { return (K + kKB - 1) / kKB; }
 size_t operand_bytes(int64_t rows, int64_t K);
-// Carves an operand's buffers out of `ws` (256-byte aligned); its row list is
-// the last part, hard_bytes() of it.
+// Carves an operand's buffers out of `ws` (256-byte aligned).
 void operand_carve(Operand64* o, unsigned char* ws);
-inline size_t hard_bytes(int64_t rows) { return ((size_t)(rows + 1) * 4 + 255) & ~(size_t)255; }
 
 // Digits of up to kMaxOps operands (at most two launches for all of them).
-lrc_status slice(const Operand64* const* ops, int count, cudaStream_t s);
+// clear[0 ... nclear), at most 256 counters, are set to zero on the way.
+lrc_status slice(const Operand64* const* ops, int count, int* clear, int nclear, cudaStream_t s);
+
+// Entries of a product that the digits do not carry, of 16 rows and half a tile's
+// columns: bit 4 r + c of mask[4 j + 2 h + i] is entry (row0 + 8 h + r, col0 + 8 j
+// + 2 c + i).
+struct Listed {
+    int row0, col0;
+    uint32_t mask[16];
+};
+// `list` holds fix_bytes(M, N) for an M x N product, *count is zero before it.
+struct Fix {
+    Listed* list;
+    int* count;
+};
+size_t fix_bytes(int64_t M, int64_t N);
 
 // C(i, j) at C[i cr + j cc], i < A.rows, j < B.rows: the product A B^T times
 // rscale[i] cscale[j] (each may be null, and both are with `split` false).  `split` splits the reduction over
 // the CTAs (few, deep tiles); its partial sums are added in a fixed order.
-// `part` holds part_bytes() bytes.  Rows that the digits cannot carry are
+// `part` holds part_bytes() bytes.  Entries that the digits do not carry are
 // recomputed with binary64 FMAs.
 struct Out64 {
     double* C;
     int64_t cr, cc;
     const double* rscale;
     const double* cscale;
-    int* clear = nullptr;    // a later operand's hard[0], set to 0 on the way (split only)
 };
 size_t part_bytes(int64_t M, int64_t N);
-lrc_status product(const Operand64& A, const Operand64& B, const Out64& out, bool split, double* part, cudaStream_t s);
-// C(i, j) = C(j, i) at C[i ldc + j]: A A^T, `part` as above.  Tiles below the
-// diagonal are left out.
-lrc_status gram(const Operand64& A, double* C, int64_t ldc, double* part, cudaStream_t s);
+lrc_status product(const Operand64& A, const Operand64& B, const Out64& out, bool split, double* part, const Fix& fix,
+                   cudaStream_t s);
+// C(i, j) = C(j, i) at C[i ldc + j]: A A^T, `part` and `fix` as above.  Tiles
+// below the diagonal are left out.
+lrc_status gram(const Operand64& A, double* C, int64_t ldc, double* part, const Fix& fix, cudaStream_t s);
 
 }  // namespace sg
 }  // namespace lrc

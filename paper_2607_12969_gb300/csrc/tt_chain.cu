@@ -17,6 +17,7 @@
 // workspace (two buffers per side, alternating).
 #include <math.h>
 
+#include <algorithm>
 #include <vector>
 
 #include "common.cuh"
@@ -202,7 +203,7 @@ lrc_status launch_tt_chain_f64_tc(const TTShape& sh, double* out, cudaStream_t s
         size_t oa, ob, oc;
     };
     std::vector<Step> steps;
-    size_t off = 0;
+    size_t off = 0, fix = 0;
     auto take = [&](size_t bytes) {
         const size_t o = off;
         off += round256(bytes);
@@ -214,8 +215,9 @@ lrc_status launch_tt_chain_f64_tc(const TTShape& sh, double* out, cudaStream_t s
         t.a.rows = M;
         t.b.rows = N;
         t.a.K = t.b.K = K;
-        t.oa = take(sg::operand_bytes(M, K) - sg::hard_bytes(M));
-        t.ob = take(sg::operand_bytes(N, K) - sg::hard_bytes(N));
+        t.oa = take(sg::operand_bytes(M, K));
+        t.ob = take(sg::operand_bytes(N, K));
+        fix = std::max(fix, sg::fix_bytes(M, N));
         t.oc = last ? 0 : take((size_t)M * (size_t)N * 8);
         steps.push_back(t);
     };
@@ -231,17 +233,13 @@ lrc_status launch_tt_chain_f64_tc(const TTShape& sh, double* out, cudaStream_t s
     }
     const int right = (int)steps.size();
     add(left ? nullptr : G[0], right > left ? nullptr : G[d - 1], P, Q, sh.ranks[c], true);
-    // the row lists of all operands side by side, emptied at once
-    const size_t o_hard = off;
-    for (const Step& t : steps) off += sg::hard_bytes(t.M) + sg::hard_bytes(t.N);
+    const size_t o_f = take(fix), o_n = take(steps.size() * sizeof(int));      // list of one product after the other
     void* p = nullptr;
     lrc_status st = stream_workspace_try(s, off, &p);
     if (st != LRC_OK || !p) return st;
     *handled = true;
     unsigned char* ws = static_cast<unsigned char*>(p);
-    cudaError_t e = cudaMemsetAsync(ws + o_hard, 0, off - o_hard, s);
-    if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync (row lists)");
-    size_t hard = o_hard;
+    int* counts = reinterpret_cast<int*>(ws + o_n);
     for (int i = 0; i < (int)steps.size(); ++i) {
         Step& t = steps[i];
         const bool last = i + 1 == (int)steps.size();
@@ -250,16 +248,12 @@ lrc_status launch_tt_chain_f64_tc(const TTShape& sh, double* out, cudaStream_t s
         t.C = last ? out : reinterpret_cast<double*>(ws + t.oc);
         sg::operand_carve(&t.a, ws + t.oa);
         sg::operand_carve(&t.b, ws + t.ob);
-        t.a.hard = reinterpret_cast<int*>(ws + hard);
-        hard += sg::hard_bytes(t.M);
-        t.b.hard = reinterpret_cast<int*>(ws + hard);
-        hard += sg::hard_bytes(t.N);
-        t.a.cleared = t.b.cleared = true;
         t.a.src = sg::Src64{A, t.K, 1, nullptr, 0};
         t.b.src = sg::Src64{B, 1, t.N, nullptr, 0};
         const sg::Operand64* ops[2] = {&t.a, &t.b};
-        if ((st = sg::slice(ops, 2, s)) != LRC_OK) return st;
-        if ((st = sg::product(t.a, t.b, sg::Out64{t.C, t.N, 1, nullptr, nullptr}, false, nullptr, s)) != LRC_OK)
+        const sg::Out64 o{t.C, t.N, 1, nullptr, nullptr};
+        if ((st = sg::slice(ops, 2, counts, i == 0 ? (int)steps.size() : 0, s)) != LRC_OK) return st;
+        if ((st = sg::product(t.a, t.b, o, false, nullptr, {reinterpret_cast<sg::Listed*>(ws + o_f), counts + i}, s)) != LRC_OK)
             return st;
     }
     return LRC_OK;

@@ -209,3 +209,97 @@ def test_eta_of_wide_columns(lrc, cuda, m, n, k):
     # have eta^2's two factors; its terms (all of one size) nearly add up
     assert abs(eta - want) <= 8 * (m + n) * U64 * want
     assert abs(norm - wnorm) <= 8 * (m + n) * U64 * wnorm
+
+
+@pytest.mark.parametrize("m,n,k,b,share,gap", [(300, 64, 600, 300, 0.5, 16), (257, 1000, 64, 300, 0.45, 18), (257, 1000, 64, 300, 0.27, 40),
+                                               (130, 4099, 40, 200, 0.19, 59), (700, 1024, 33, 1000, 0.03, 70),
+                                               (2050, 300, 130, 1100, 0.15, 25)])
+def test_small_entries_that_are_all_that_counts(lrc, cuda, m, n, k, b, share, gap):
+    """A share of every row's entries lies 2^-gap below the others, and the other
+    operand is zero beside them: digits below the large entries hold little or
+    nothing of the result.  Both products, against the sums of magnitudes."""
+    rng = np.random.default_rng(gap)
+
+    def scaled(rows, cols):
+        small = rng.permutation(cols) < max(1, int(share * cols))
+        return rng.standard_normal((rows, cols)) * np.where(small, 2.0 ** -gap, 1.0), small
+    Vt, small = scaled(k, n)
+    X = rng.standard_normal((b, n)) * small
+    U, small_k = scaled(m, k)
+    s = np.where(small_k, rng.uniform(0.5, 2.0, k), 0.0)
+    for args in ((rng.standard_normal((m, k)), np.ones(k), Vt, X), (U, s, rng.standard_normal((k, n)), rng.standard_normal((b, n))),
+                 (U, s, Vt, X)):
+        want = oracle.apply(*args)
+        u, t, v, x = (np.abs(a) for a in args)
+        bound = ((x @ v.T) * t) @ u.T
+        assert np.all(np.abs(run(lrc, cuda, *args) - want) <= 2 * (n + k + 2) * U64 * bound)
+
+
+@pytest.mark.parametrize("m,n,k,b", [(70, 4096, 64, 64), (301, 600, 130, 2003), (4100, 100, 33, 300), (3001, 95, 97, 171)])
+def test_every_entry_listed(lrc, cuda, m, n, k, b):
+    """Disjoint large entries in every row of both products: blocks and single
+    entries, few and many, partial blocks at both edges, short and long sums."""
+    rng = np.random.default_rng(n)
+    even, even_k = np.arange(n) % 2 == 0, np.arange(k) % 2 == 0
+    X = rng.standard_normal((b, n)) * even
+    Vt = rng.standard_normal((k, n)) * np.where(even, 2.0 ** -30, 1.0) * even_k[:, None]
+    U = rng.standard_normal((m, k)) * np.where(even_k, 2.0 ** -30, 1.0)
+    s = rng.uniform(0.5, 2.0, k)
+    want = oracle.apply(U, s, Vt, X)
+    bound = ((np.abs(X) @ np.abs(Vt).T) * s) @ np.abs(U).T
+    assert np.all(np.abs(run(lrc, cuda, U, s, Vt, X) - want) <= 2 * (n + k + 2) * U64 * bound)
+
+
+def test_unit_and_zero_queries(lrc, cuda):
+    """One entry a query: Y is a column of A, whatever the size of its entries;
+    zero queries make zeros beside an infinite factor entry that they meet NaN."""
+    m, n, k, b = 500, 1100, 64, 400
+    f = W.random_factors(m, n, k, seed=31)
+    X = np.zeros((b, n))
+    X[np.arange(b), (np.arange(b) * 7) % n] = 3.0
+    X[5] = X[77] = 0.0
+    got = run(lrc, cuda, f.U, f.s, f.Vt, X)
+    want = oracle.apply(f.U, f.s, f.Vt, X)
+    bound = ((np.abs(X) @ np.abs(f.Vt).T) * f.s) @ np.abs(f.U).T
+    assert np.all(np.abs(got - want) <= 2 * (k + 4) * U64 * bound)
+    U = f.U.copy()
+    U[9, 2] = np.inf
+    got = run(lrc, cuda, U, f.s, f.Vt, X)
+    assert np.all(np.isnan(got[[5, 77], 9])) and np.all(got[5, :9] == 0) and np.all(got[77, 10:] == 0)
+
+
+def test_digits_at_their_limits(lrc, cuda):
+    """Constant rows of the value whose digits are 65, -256, ..., -256: what the
+    classes left out add has one sign and its largest size, below 2^-57 of the
+    power of two above the entries, squared, a term."""
+    n, k, b, m = 2048, 128, 64, 64
+    v = (65 * 2 ** 54 - sum(256 << (54 - 9 * i) for i in range(1, 7))) / 2.0 ** 61
+    got = run(lrc, cuda, np.full((m, k), v), np.ones(k), np.full((k, n), v), np.full((b, n), v))
+    L = np.longdouble
+    want = L(v) ** 3 * n * k
+    assert np.all(np.abs(got.astype(L) - want) <= (2 * U64 + 2 * 2.0 ** -57 / v ** 2) * want)
+
+
+@pytest.mark.parametrize("dims,ranks", TT_SHAPES)
+def test_tt_chain_of_blocks_of_different_size(lrc, cuda, dims, ranks):
+    """Half of every bond's slices 2^-20 ... 2^-60 below the others on one side,
+    and zero or larger on the other."""
+    rng = np.random.default_rng(8)
+    d = len(dims)
+    cores = [rng.standard_normal((ranks[l], dims[l], ranks[l + 1])) for l in range(d)]
+    for l in range(1, d):
+        half = np.arange(ranks[l]) % 2 == 0
+        cores[l - 1] = cores[l - 1] * np.where(half, 2.0 ** -(20 * l), 1.0)
+        cores[l] = cores[l] * np.where(half, 1.0, 0.0)[:, None, None] if l % 2 else cores[l] * np.where(half, 1.0, 2.0 ** -30)[:, None, None]
+    dev = [torch.from_numpy(np.ascontiguousarray(c)).to(cuda) for c in cores]
+    out = torch.empty(int(np.prod(dims)), dtype=torch.float64, device=cuda)
+    lrc.tt_reconstruct(dev, dims, ranks, "f64", out)
+    torch.cuda.synchronize()
+
+    def chain(cs):
+        z = cs[0].reshape(dims[0], -1)
+        for c in cs[1:]:
+            z = (z @ c.reshape(c.shape[0], -1)).reshape(-1, c.shape[2])
+        return z.reshape(-1)
+    bound = chain([np.abs(c) for c in cores])
+    assert np.all(np.abs(out.cpu().numpy() - chain(cores)) <= (sum(ranks) + 2 * d) * U64 * bound)

@@ -74,3 +74,48 @@ def test_three_products_meet_the_binary32_tolerance():
     assert rel.max() <= 1e-6, rel.max()
     # the dropped term W_lo U_lo is below 2^-22 of the product's scale
     assert np.max(np.abs(f(Wl) @ f(Ul).T)) <= 2.0 ** -22 * np.max(np.abs(f(Wh) @ f(Uh).T)) * 4
+
+
+# ---- binary64 from seven 9-bit digits (split_gemm.cu)
+
+def digits(x):
+    """Digits (rows, 7, columns) of rows of binary64 numbers, as Python integers,
+    and the exponents of the power of two above each row's largest entry."""
+    top = np.array([np.frexp(np.max(np.abs(r)))[1] for r in x])
+    v = np.array([[int(np.rint(np.ldexp(e, 61 - t))) for e in r] for r, t in zip(x, top)], dtype=object)
+    bias = sum(256 << (54 - 9 * i) for i in range(1, 7))
+    t = v + bias
+    d = [t >> 54] + [((t >> (54 - 9 * i)) & 511) - 256 for i in range(1, 7)]
+    return np.stack(d, 1), top
+
+
+def check_unlisted(a, b, far_off=False):
+    """Entries whose first digits' sum of magnitudes reaches 2^9 are within
+    K 2^-50 of the exact sum of magnitudes; the others are left to FMAs."""
+    K = a.shape[1]
+    (da, ta), (db, tb) = digits(a), digits(b)
+    kept = sum((da[:, i] @ db[:, j].T) * (1 << (9 * (6 - i - j))) for i in range(7) for j in range(7 - i))
+    est = abs(da[:, 0]) @ abs(db[:, 0]).T
+    ia, ib = (np.array([[int(np.ldexp(e, 61 - t + 200)) for e in r] for r, t in zip(x, top)], dtype=object)
+              for x, top in ((a, ta), (b, tb)))
+    exact, mags = ia @ ib.T, abs(ia) @ abs(ib).T              # in units of 2^-400 of the digits' square
+    err = abs(kept * (1 << 54) * (1 << 400) - exact)
+    on = np.asarray(est >= 512, bool)
+    assert np.all(err[on] * (1 << 50) <= K * mags[on])
+    if far_off:        # what the limit is for: digits alone would miss the FMA bound
+        assert np.any(err[~on] * (1 << 53) > 64 * K * mags[~on])
+    return on
+
+
+def test_digits_carry_what_the_estimate_passes():
+    rng = np.random.default_rng(3)
+    g = lambda *s: rng.standard_normal(s)
+    assert check_unlisted(g(12, 64), g(9, 64)).all()
+    assert check_unlisted(g(12, 40) * np.arange(1, 41) ** -0.75, g(9, 40) * np.arange(1, 41) ** -0.75).all()
+    limits = np.full((2, 48), (65 * 2 ** 54 - sum(256 << (54 - 9 * i) for i in range(1, 7))) / 2.0 ** 61)
+    assert check_unlisted(limits, limits).all()
+    for gap in (12, 20, 40, 70):
+        small = np.arange(64) % 4 == 0
+        a = g(12, 64) * np.where(small, 2.0 ** -gap, 1.0)
+        check_unlisted(a, np.vstack([g(5, 64) * small, g(4, 64)]), gap >= 20)
+    check_unlisted(g(12, 64) * 2.0 ** -rng.integers(0, 60, (12, 64)), g(9, 64) * 2.0 ** -rng.integers(0, 60, (9, 64)))
