@@ -60,7 +60,7 @@ typedef enum {
                          binary64 once where they carry an entry (see lrc_apply)            */
     LRC_F32 = 1,      /* binary32 storage and output; binary32 FMAs, or in larger applies
                          products of three bfloat16 parts of every operand on the tensor
-                         cores, accumulated in binary32 (no less accurate)                   */
+                         cores, accumulated in binary32 (see lrc_apply)                      */
     LRC_F16 = 2,      /* binary16 storage, binary32 accumulation, binary32 output           */
     LRC_F16_O16 = 3,  /* binary16 storage, binary32 accumulation, binary16 workspaces and
                          output: the method-precision FP16 path of Sec. 3.4                 */
@@ -182,10 +182,11 @@ LRC_API lrc_status lrc_widen_factors(const void* src, lrc_fmt fmt, int64_t rows,
  */
 /* LRC_F32: larger problems form both products from bfloat16 parts (x = hi +
  * mid + lo exactly; the six largest of the nine products of parts, which leaves
- * out 2^-26 of a term); a row that holds a nonzero entry outside 2^-100 ...
- * 2^126, an infinity or a NaN is formed by binary32 FMAs.  The parts (6 bytes
- * an element, of at most 1 GiB of queries at a time) live in the stream's
- * workspace; without it (see above) the FMA kernels run.
+ * out at most 2^-24 of a term and 2^-26 as a rule); a row with an infinity, a NaN
+ * or an entry above 2^40 (of X and of the b x k intermediate) or 2^32 (of U and
+ * V^T) is formed by binary32 FMAs.  The parts (6 bytes an element, of at most
+ * 1 GiB of queries at a time) live in the stream's workspace; without it (see
+ * above) the FMA kernels run.
  * LRC_F32_TC: the same; on smaller problems as LRC_F32 with the second product
  * (W U^T) on the tensor cores when b > 32 and k <= 192. */
 LRC_API lrc_status lrc_apply(const void* U, const void* S, const void* Vt, const void* X, void* Y,

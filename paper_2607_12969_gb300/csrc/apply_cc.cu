@@ -599,8 +599,8 @@ static lrc_status launch_apply_f32_tc(const float* U, const float* S, const floa
     int64_t pb = kPanelBytes / (sg32::kParts * 2 * sg32::kKB * sg32::image_blocks(n)) / 256 * 256;
     if (pb < 256) pb = 256;
     if (pb > b) pb = b;
-    sg32::Operand oV{Vt, ldn, 1, k, n, nullptr, nullptr}, oU{U, ldk, 1, m, k, nullptr, nullptr};
-    sg32::Operand oX{X, ldn, 1, pb, n, nullptr, nullptr}, oW{nullptr, ldk, 1, pb, k, nullptr, nullptr};
+    sg32::Operand oV{Vt, ldn, 1, k, n, true, nullptr, nullptr}, oU{U, ldk, 1, m, k, true, nullptr, nullptr};
+    sg32::Operand oX{X, ldn, 1, pb, n, false, nullptr, nullptr}, oW{nullptr, ldk, 1, pb, k, false, nullptr, nullptr};
     size_t off = 0;
     auto take = [&](size_t bytes) {
         const size_t o = off;

@@ -2,11 +2,11 @@
 //
 // The CUDA cores reach 42 to 47 TFLOP/s on these products; the tensor cores
 // multiply bfloat16 numbers at 1700.  A binary32 value is the exact sum of three
-// bfloat16 numbers, x = hi + mid + lo (each the nearest to what is left), so of
-// the nine products of parts the six largest,
+// bfloat16 numbers, x = hi + mid + lo (each the nearest to what is left: mid at
+// most 2^-8 of x, lo 2^-17), so of the nine products of parts the six largest,
 //     hi hi + (hi mid + mid hi) + (mid mid + hi lo + lo hi),
-// leave out only what lies 2^-26 below a term, less than binary32's own
-// rounding.  Each value is split by itself: nothing depends on its neighbours.
+// leave out at most 2^-24 of a term, binary32's own rounding of it, and 2^-26 as a
+// rule.  Each value is split by itself: nothing depends on its neighbours.
 //
 // The tensor cores' binary32 accumulation cuts sums off (about 0.4 units of the
 // last place a step of 16 terms, all in one direction), so hi hi runs for only
@@ -16,9 +16,14 @@
 // from binary64 of the apply (16384 x 8192, k = 136, b = 8192): 2.4e-7, with
 // binary32 FMAs 6.5e-7.
 //
-// Entries between 2^-100 and 2^126 in magnitude (and zero) are carried; a row
-// that holds another (its mid or lo part would fall below bfloat16's range, or
-// hi overflow), or an infinity or NaN, is recomputed with binary32 FMAs.
+// The parts are those of 2^24 x (2^48 comes off as an accumulator is added to the
+// running sum): every binary32 number is a multiple of 2^-149, so its scaled parts
+// are multiples of 2^-125, zero or normal bfloat16 numbers, and none is lost
+// however small x is.  Entries are bounded, 2^40 on the first side and 2^32 on the
+// second, so that no accumulator leaves binary32's range: a row with a larger one,
+// an infinity or a NaN is recomputed with binary32 FMAs.  (Without such a bound two
+// entries of 2^71 made hi hi infinite, hi mid the other infinity, and their sum a
+// NaN.)
 //
 // Kernels: parts_kernel (the images), product32_kernel (persistent, one CTA a
 // SM: 128 x up to 256 tiles), part_sum32_kernel (split reductions) and
@@ -44,6 +49,7 @@ struct Job {
     int64_t rs, cs, rows, K, img_rows, kblocks;
     int64_t b0;              // first block
     int kparts, vec;
+    float limit;             // largest magnitude carried
     unsigned char* img;
     int* hard;
 };
@@ -52,9 +58,15 @@ struct Jobs {
     int n;
 };
 constexpr int kJobCols = 256;      // columns a block takes
+constexpr float kUp = 0x1p24f, kDown = 0x1p-48f;
 
-// The bits of the three parts of x, each in the upper half of its word.
-__device__ __forceinline__ void parts_of(float x, uint32_t (&h)[kParts]) {
+// Largest entry carried on either side: 64 products of 2^48 times these stay
+// below 2^126.
+constexpr float kFirstLimit = 0x1p40f, kSecondLimit = 0x1p32f;
+
+// The bits of the three parts of 2^24 x, each in the upper half of its word.
+__device__ __forceinline__ void parts_of(float x0, uint32_t (&h)[kParts]) {
+    const float x = __fmul_rn(x0, kUp);
     const float hi = __uint_as_float((uint32_t)to_bf16_bits(x) << 16);
     const float r1 = __fsub_rn(x, hi);
     const float mid = __uint_as_float((uint32_t)to_bf16_bits(r1) << 16);
@@ -109,10 +121,7 @@ __global__ void __launch_bounds__(256) parts_kernel(const __grid_constant__ Jobs
             for (int i = 0; i < kParts; ++i) w[i][q] = __byte_perm(a[i], b[i], 0x7632);
         }
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const float m = fabsf(x[j]);
-            bad |= !(m >= 0x1p-100f && m <= 0x1p126f) && x[j] != 0.0f;
-        }
+        for (int j = 0; j < 8; ++j) bad |= !(fabsf(x[j]) <= o.limit);
         unsigned char* dst = row_base + (size_t)(oc >> 1) * block_bytes + (size_t)(oc & 1) * 128;
 #pragma unroll
         for (int i = 0; i < kParts; ++i)
@@ -219,8 +228,8 @@ __global__ void __launch_bounds__(kThreads, 1) product32_kernel(const __grid_con
                         tmem_ld_wait();
 #pragma unroll
                         for (int j = 0; j < 8; ++j) {
-                            sum[j0 + j] = __fadd_rn(sum[j0 + j], __uint_as_float(u[j]));
-                            sum[j0 + 8 + j] = __fadd_rn(sum[j0 + 8 + j], __uint_as_float(v[j]));
+                            sum[j0 + j] = __fmaf_rn(__uint_as_float(u[j]), kDown, sum[j0 + j]);
+                            sum[j0 + 8 + j] = __fmaf_rn(__uint_as_float(v[j]), kDown, sum[j0 + 8 + j]);
                         }
                     }
                 }
@@ -242,7 +251,7 @@ __global__ void __launch_bounds__(kThreads, 1) product32_kernel(const __grid_con
             }
             if (!ok) break;
             const int mt = tile / a.ntiles, nt = tile - mt * a.ntiles;
-            const int64_t row = (int64_t)mt * 128 + r, col0 = (int64_t)nt * NT + quarter * hc;
+            const int64_t col0 = (int64_t)nt * NT + quarter * hc;
             if (a.split) {
                 float* dst = a.C + sg::part_slot(a, tile) * (128 * NT) + (int64_t)(quarter * hc) * 128 + r;
 #pragma unroll
@@ -569,6 +578,7 @@ lrc_status split(const Operand* const* ops, int count, cudaStream_t s) {
         j.img_rows = image_rows(o.rows);
         j.kblocks = image_blocks(o.K);
         j.vec = o.cs == 1 && o.rs % 4 == 0 && aligned16(o.p);
+        j.limit = o.second ? kSecondLimit : kFirstLimit;
         j.img = o.img;
         j.hard = o.hard;
         j.kparts = (int)((j.kblocks * kKB + kJobCols - 1) / kJobCols);

@@ -20,12 +20,13 @@ inline int n_tile(int64_t rows, bool splitk) {
     return (int)(((rows + tiles - 1) / tiles + 15) / 16 * 16);
 }
 
-// One operand of a product, `rows` x K: entry (r, c) is p[r rs + c cs].  The
-// image is [block of kKB columns][group of 8 rows][part][column octet][8 rows x
+// One operand of a product, `rows` x K: entry (r, c) is p[r rs + c cs]; `second`
+// the side it is on.  The image is [block of kKB columns][group of 8 rows][part][column octet][8 rows x
 // 16 bytes] and serves as either side of a product.
 struct Operand {
     const float* p;
     int64_t rs, cs, rows, K;
+    bool second;
     unsigned char* img;
     int* hard;               // hard[0] = rows the parts cannot carry, hard[1 ...] their indices, then a mark per row
 };

@@ -108,7 +108,8 @@ lrc_status launch_chain(const TTShape& sh, T* out, cudaStream_t s, bool tc_final
     const size_t sides = lsz[0] + lsz[1] + rsz[0] + rsz[1];
     // binary32: a large output product in bfloat16 parts (split_gemm32.cu), where
     // there is workspace for them
-    sg32::Operand oz{nullptr, rc, 1, P[c], rc, nullptr, nullptr}, os{nullptr, 1, Q[c], Q[c], rc, nullptr, nullptr};
+    sg32::Operand oz{nullptr, rc, 1, P[c], rc, false, nullptr, nullptr};
+    sg32::Operand os{nullptr, 1, Q[c], Q[c], rc, true, nullptr, nullptr};
     const size_t zi = round256(sg32::image_bytes(P[c], rc)), si = round256(sg32::image_bytes(Q[c], rc));
     bool parts = sizeof(T) == 4 && 2.0 * (double)P[c] * (double)Q[c] * (double)rc >= kPartsFlops;
     if (parts) {

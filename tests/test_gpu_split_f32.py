@@ -166,3 +166,47 @@ def test_every_row_recomputed(lrc, cuda, m, n, k, b):
     bound = (np.abs(X) @ np.abs(Vt).T * s) @ np.abs(U).T
     # sums of at most 1024 terms and of their sums, two products, one scaling
     assert np.all(np.abs(got - want) <= 2 * (min(n, 1024) + n / 1024 + k + 4) * U32 * bound)
+
+
+@pytest.mark.parametrize("fmt", ["f32", "f32tc"])
+def test_products_near_the_ends_of_the_range(lrc, cuda, fmt):
+    """Products beyond binary32's range are infinite (not a NaN from parts that
+    overflow apart), those inside it finite, and those of entries down to the
+    smallest subnormal numbers as close as FMA sums."""
+    m, n, k, b = 300, 5000, 64, 600
+    f32 = lambda a: np.asarray(a, np.float64).astype(np.float32).astype(np.float64)
+    rng = np.random.default_rng(17)
+    X, Vt, U = f32(rng.standard_normal((b, n))), f32(rng.standard_normal((k, n))), f32(rng.standard_normal((m, k)))
+    s = np.ones(k)
+    X[3] = X[4] = X[5] = X[6] = 0.0
+    X[3, 9], Vt[7, 9] = f32(1.99 * 2.0 ** 70), f32(1.99 * 2.0 ** 70)
+    X[4, 11], Vt[8, 11] = f32(1.998 * 2.0 ** 64), f32(0.9989 * 2.0 ** 63)          # 0.998 2^128
+    X[5, 13], Vt[9, 13] = 2.0 ** -60, f32(1.7 * 2.0 ** -85)
+    X[6] = f32(rng.standard_normal(n) * 2.0 ** -rng.integers(100, 149, n))
+    U[:, 7:10] = 0.0
+    U[10, 7], U[11, 8], U[12, 9] = 1.0, f32(0.9), 1.0
+    U[13] = f32(rng.standard_normal(k) * 2.0 ** -rng.integers(100, 149, k))
+    got = run(lrc, cuda, U, s, Vt, X, fmt)
+    assert got[3, 10] == np.inf and np.isnan(got[3, 9])          # (0 times infinity)
+    W1 = X @ Vt.T
+    W1 = f32(np.where(np.abs(W1) < 2.0 ** 128, W1, np.inf))
+    rows = np.arange(b) != 3
+    want, bound = W1[rows] @ U.T, (np.abs(X[rows]) @ np.abs(Vt).T) @ np.abs(U).T
+    assert np.isfinite(got[4, 11]) and np.isfinite(want).all()
+    assert np.all(np.abs(got[rows] - want) <= 64 * U32 * bound + k * 2.0 ** -149)
+
+
+@pytest.mark.parametrize("m,n,k,b", [(4100, 600, 136, 1100), (2050, 8300, 40, 520), (12000, 9000, 33, 250)])
+def test_every_row_above_the_limit(lrc, cuda, m, n, k, b):
+    """Entries above the parts' limit in every row of V^T and U: both products in
+    the tiles that the repair takes for many and few entries."""
+    rng = np.random.default_rng(m)
+    f32 = lambda a: a.astype(np.float32).astype(np.float64)
+    large = lambda a: f32(np.where(np.arange(a.shape[1]) % 5 == 0, a * 2.0 ** 40, a))
+    U, Vt = large(rng.standard_normal((m, k))), large(rng.standard_normal((k, n)))
+    X, s = f32(rng.standard_normal((b, n))), f32(rng.uniform(0.5, 2.0, k))
+    got = run(lrc, cuda, U, s, Vt, X)
+    want = ((X @ Vt.T) * s) @ U.T
+    bound = (np.abs(X) @ np.abs(Vt).T * s) @ np.abs(U).T
+    # sums of at most 1024 terms and of their sums, two products, one scaling
+    assert np.all(np.abs(got - want) <= 2 * (min(n, 1024) + n / 1024 + k + 4) * U32 * bound)
