@@ -530,7 +530,6 @@ lrc_status launch_split_t(const TTShape& sh, bool out16, void* out, cudaStream_t
     if (kp > (kF32 ? kMaxParts32 : kMaxParts) * 64 || rmax > 64 || y_product_plan(a.Q, a.P, kp, out16, &n2) != LRC_OK) return LRC_OK;
     const size_t smem = side_smem(sh, a);
     if (smem > 200 * 1024) return LRC_OK;
-    *handled = true;
     a.pw = pw;
     a.pu = pu;
     a.scale_w = z_core ? 0 : 1;
@@ -540,8 +539,15 @@ lrc_status launch_split_t(const TTShape& sh, bool out16, void* out, cudaStream_t
     const size_t w_bytes = r256((size_t)btiles * BM * kp * 2), u_bytes = r256((size_t)a.Q * kp * 2);
     const size_t e_bytes = r256((size_t)(a.wunits + uunits) * sizeof(int));
     void* wsp = nullptr;
-    lrc_status st = stream_workspace(s, w_bytes + u_bytes + e_bytes, &wsp);
-    if (st != LRC_OK) return st;
+    lrc_status st;
+    if (kF32) {      // the FMA chain does with less workspace, with two cores without any
+        st = stream_workspace_try(s, w_bytes + u_bytes + e_bytes, &wsp);
+        if (st != LRC_OK || !wsp) return st;
+        *handled = true;
+    } else {
+        *handled = true;
+        if ((st = stream_workspace(s, w_bytes + u_bytes + e_bytes, &wsp)) != LRC_OK) return st;
+    }
     unsigned char* ws = static_cast<unsigned char*>(wsp);
     a.Wimg = ws;
     a.Uimg = reinterpret_cast<uint16_t*>(ws + w_bytes);

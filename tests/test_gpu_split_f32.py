@@ -210,3 +210,22 @@ def test_every_row_above_the_limit(lrc, cuda, m, n, k, b):
     bound = (np.abs(X) @ np.abs(Vt).T * s) @ np.abs(U).T
     # sums of at most 1024 terms and of their sums, two products, one scaling
     assert np.all(np.abs(got - want) <= 2 * (min(n, 1024) + n / 1024 + k + 4) * U32 * bound)
+
+
+@pytest.mark.parametrize("dims,ranks", [((300, 200), (1, 20, 1)), ((4096, 4096), (1, 48, 1))])
+def test_two_cores_captured_without_workspace(lrc, cuda, dims, ranks):
+    """A two-core binary32 chain needs no workspace: as the first call on its
+    stream it can be captured, and gives what FMA sums give."""
+    g = torch.Generator(device=cuda).manual_seed(3)
+    cores = [torch.randn(ranks[l], dims[l], ranks[l + 1], generator=g, device=cuda) for l in range(2)]
+    out = torch.zeros(dims, device=cuda)
+    torch.cuda.synchronize()
+    lrc.lrc_shutdown()                      # no stream has a workspace
+    st = torch.cuda.Stream()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=st):
+        lrc.tt_reconstruct(cores, dims, ranks, "f32", out, stream=st)
+    graph.replay()
+    torch.cuda.synchronize()
+    a, b = (c.reshape(-1, c.shape[2]).double() if l == 0 else c.reshape(c.shape[0], -1).double() for l, c in enumerate(cores))
+    assert torch.all((out.double() - a @ b).abs() <= (ranks[1] + 2) * U32 * (a.abs() @ b.abs()))
