@@ -244,7 +244,9 @@ LRC_API lrc_status lrc_apply_batched(int count, const void* const* U, const void
  */
 /* LRC_F32: chains whose cores fit the one-pass side kernel (bond rank <= 64)
  * and output products of at least 2.5e9 flops run on the tensor cores from
- * bfloat16 parts (see lrc_apply), others on FMAs.
+ * bfloat16 parts (see lrc_apply; in the former, entries of the partial products
+ * above 2^27 cost others of their group of 32 rows bits that lie 2^-150 and more
+ * below them), others on FMAs.
  * LRC_F32_TC: the same; other output products from scaled binary16 parts. */
 LRC_API lrc_status tt_reconstruct(const void* const* cores, const int64_t* dims, const int64_t* ranks,
                           int d, lrc_fmt fmt, void* out, lrc_stream_t stream);

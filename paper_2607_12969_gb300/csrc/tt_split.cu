@@ -69,6 +69,19 @@ __device__ __forceinline__ int scale_exp(float maxabs) {
     return e < -60 ? -60 : (e > 60 ? 60 : e);
 }
 
+// The exponent for binary32 chains' parts: max * 2^e in [2^50, 2^51), e in [-60,
+// 60].  Scaled by 2^23 and more every binary32 number is a multiple of 2^-126, so
+// that none of its parts falls below bfloat16's normal numbers: with a largest
+// entry below 2^27 nothing is lost, above that only bits 2^-150 and more below the
+// largest.  64 products of 2^51 with 2^68 (the largest that [-60, 60] leaves) stay
+// in range.  (With 2^14, as for binary16, entries 2^-125 below the unit's largest
+// lost their lower parts.)
+__device__ __forceinline__ int scale_exp32(float maxabs) {
+    if (!(maxabs > 0.0f) || !isfinite(maxabs)) return 0;
+    const int e = 50 - ilogbf(maxabs);
+    return e < -60 ? -60 : (e > 60 ? 60 : e);
+}
+
 // Does a unit of a binary32 chain with this largest magnitude hold an infinity or
 // a NaN (or come so near the range's end that hi would overflow)?
 template <typename TC>
@@ -342,7 +355,7 @@ tt_side_kernel(const SideArgs a) {
         for (int e = threadIdx.x; e < nrow * a.r; e += blockDim.x)
             mx = max_mag<TC>(mx, z[(e / a.r) * a.ldb + e % a.r]);
         const float tmax = block_max(mx, red);
-        const int ex = a.scale_w ? scale_exp(tmax) : 0;
+        const int ex = std::is_same_v<TC, float> ? scale_exp32(tmax) : a.scale_w ? scale_exp(tmax) : 0;
         const float f = pow2(ex);
         tc::pdl_trigger();
         if (threadIdx.x == 0) a.esc_w[t] = marked<TC>(tmax) ? kBadUnit : ex;
@@ -382,7 +395,7 @@ tt_side_kernel(const SideArgs a) {
         for (int e = threadIdx.x; e < nq * a.r; e += blockDim.x)
             mx = max_mag<TC>(mx, sc[(base + e / a.r) * a.ldb + e % a.r]);
         const float tmax = block_max(mx, red);
-        const int ex = a.scale_u ? scale_exp(tmax) : 0;
+        const int ex = std::is_same_v<TC, float> ? scale_exp32(tmax) : a.scale_u ? scale_exp(tmax) : 0;
         const float f = pow2(ex);
         tc::pdl_trigger();
         if (threadIdx.x == 0) a.esc_u[t] = marked<TC>(tmax) ? kBadUnit : ex;

@@ -229,3 +229,34 @@ def test_two_cores_captured_without_workspace(lrc, cuda, dims, ranks):
     torch.cuda.synchronize()
     a, b = (c.reshape(-1, c.shape[2]).double() if l == 0 else c.reshape(c.shape[0], -1).double() for l, c in enumerate(cores))
     assert torch.all((out.double() - a @ b).abs() <= (ranks[1] + 2) * U32 * (a.abs() @ b.abs()))
+
+
+def test_tt_rows_of_very_different_size(lrc, cuda):
+    """Rows of 2^18 down to 2^-124 in every group of 32, on either side: a row times
+    a unit column comes out as it is; and entries near both ends of the range."""
+    m, q = 96, 160
+    rng = np.random.default_rng(2)
+    f32 = lambda a: a.astype(np.float32)
+    scale = 2.0 ** np.floor(18 - 142 / 31 * (np.arange(m) % 32))
+    for flip in (False, True):
+        A = f32(np.stack([rng.standard_normal(m) * scale, rng.standard_normal(m) * 1e-3], 1))
+        B = np.zeros((2, q), np.float32)
+        B[0] = 2.0 ** (np.arange(q) % 3)
+        if flip:
+            A, B = np.ascontiguousarray(B.T), np.ascontiguousarray(A.T)
+        dims = (A.shape[0], B.shape[1])
+        out = torch.empty(dims, device=cuda)
+        cores = [torch.from_numpy(A)[None].to(cuda), torch.from_numpy(B)[:, :, None].to(cuda)]
+        lrc.tt_reconstruct(cores, dims, (1, 2, 1), "f32", out)
+        torch.cuda.synchronize()
+        assert np.array_equal(out.cpu().numpy(), f32(A.astype(np.float64) @ B.astype(np.float64)))
+    A = f32(rng.uniform(1, 2, (40, 2)) * np.array([2.0 ** 126, 0.0]))
+    B = f32(rng.uniform(1, 2, (2, 40)) * 2.0 ** -np.linspace(0, 140, 40)[None, :])
+    out = torch.empty((40, 40), device=cuda)
+    lrc.tt_reconstruct([torch.from_numpy(A)[None].to(cuda), torch.from_numpy(B)[:, :, None].to(cuda)], (40, 40), (1, 2, 1), "f32", out)
+    with np.errstate(over="ignore"):
+        want = f32(A.astype(np.float64) @ B.astype(np.float64)).astype(np.float64)
+    got = out.double().cpu().numpy()
+    assert np.array_equal(np.isinf(got), np.isinf(want))
+    ok = np.isfinite(want)
+    assert np.all(np.abs(got[ok] - want[ok]) <= 4 * U32 * np.abs(want[ok]))
