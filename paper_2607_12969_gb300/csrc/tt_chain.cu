@@ -111,7 +111,8 @@ lrc_status launch_chain(const TTShape& sh, T* out, cudaStream_t s, bool tc_final
     sg32::Operand oz{nullptr, rc, 1, P[c], rc, false, nullptr, nullptr};
     sg32::Operand os{nullptr, 1, Q[c], Q[c], rc, true, nullptr, nullptr};
     const size_t zi = round256(sg32::image_bytes(P[c], rc)), si = round256(sg32::image_bytes(Q[c], rc));
-    bool parts = sizeof(T) == 4 && 2.0 * (double)P[c] * (double)Q[c] * (double)rc >= kPartsFlops;
+    bool parts = sizeof(T) == 4 && 2.0 * (double)P[c] * (double)Q[c] * (double)rc >= kPartsFlops &&
+                 std::max(P[c], Q[c]) < ((int64_t)1 << 31);      // (rows are numbered in 32 bits)
     if (parts) {
         void* p = nullptr;
         const lrc_status st = stream_workspace_try(
@@ -262,10 +263,20 @@ lrc_status launch_tt_chain_f64_tc(const TTShape& sh, double* out, cudaStream_t s
 
 // Where the digits' fixed cost (three launches a product, about 20 us a chain)
 // pays: the FMA kernels take about 1 us per 1e6 flops (256^3, rank 34: 1.2e9
-// flops, 1.1 ms -> 0.15 ms).
+// flops, 1.1 ms -> 0.14 ms).  Rows are numbered in 32 bits.
 bool tt_chain_f64_tc_takes(const TTShape& sh) {
     constexpr double kTTDigitFlops = 4e7;
-    return plan_chain(sh).flops >= kTTDigitFlops;
+    constexpr int64_t kMost = (int64_t)1 << 31;
+    const ChainPlan p = plan_chain(sh);
+    if (p.flops < kTTDigitFlops) return false;
+    int64_t P = 1, Q = 1;
+    for (int j = 0; j < sh.d; ++j) {
+        (j < p.c ? P : Q) *= sh.dims[j];
+        // the products' other sides: core j's columns on the left, rows on the right
+        if (j < p.c && sh.dims[j] * sh.ranks[j + 1] >= kMost) return false;
+        if (j >= p.c && sh.ranks[j] * sh.dims[j] >= kMost) return false;
+    }
+    return P < kMost && Q < kMost;
 }
 
 bool tt_chain_saves(const TTShape& sh) { return plan_chain(sh).flops <= 0.8 * chain_flops(sh, sh.d - 1); }
