@@ -1162,6 +1162,8 @@ size_t part_bytes(int64_t M, int64_t N) {
     return up256((size_t)(tiles_of(M, N) + sm_count()) * 128 * n_tile(N) * 8);
 }
 
+int product_tile(int64_t M, int64_t N) { return tiles_of(N, M) < tiles_of(M, N) ? n_tile(M) : n_tile(N); }
+
 size_t fix_bytes(int64_t M, int64_t N) {
     if (tiles_of(N, M) < tiles_of(M, N)) std::swap(M, N);
     return up256((size_t)((M + 15) / 16) * (size_t)(2 * n_tiles(N)) * sizeof(Listed));

@@ -87,6 +87,8 @@ struct Out64 {
     const double* cscale;
 };
 size_t part_bytes(int64_t M, int64_t N);
+// Columns of the tiles that an M x N product takes.
+int product_tile(int64_t M, int64_t N);
 lrc_status product(const Operand64& A, const Operand64& B, const Out64& out, bool split, double* part, const Fix& fix,
                    cudaStream_t s);
 // C(i, j) = C(j, i) at C[i ldc + j]: A A^T, `part` and `fix` as above.  Tiles

@@ -263,10 +263,16 @@ lrc_status launch_tt_chain_f64_tc(const TTShape& sh, double* out, cudaStream_t s
 
 // Where the digits' fixed cost (three launches a product, about 20 us a chain)
 // pays: the FMA kernels take about 1 us per 1e6 flops (256^3, rank 34: 1.2e9
-// flops, 1.1 ms -> 0.14 ms).  Rows are numbered in 32 bits.
+// flops, 1.1 ms -> 0.14 ms).  A tile of the product (128 x NT) costs about the
+// same, 7 us of an SM, whatever its width and for all ranks up to 64, so the
+// output product has to have enough to do in one: bond rank times NT from
+// kTTDigitTile on.  Measured, digits / FMA kernels: 10^6 x 16 (NT = 16), rank 16
+// 377 / 432 us, rank 4 365 / 116; 300^3 (NT = 64), ranks 8 215 / 425, 4 254 / 219,
+// 2 411 / 116; 4096^2, rank 4 128 / 347, 2 231 / 195; 1000 x 1000 x 8, ranks 8 and
+// 4 (NT = 16) 382 / 128.  Rows are numbered in 32 bits.
 bool tt_chain_f64_tc_takes(const TTShape& sh) {
     constexpr double kTTDigitFlops = 4e7;
-    constexpr int64_t kMost = (int64_t)1 << 31;
+    constexpr int64_t kTTDigitTile = 192, kMost = (int64_t)1 << 31;
     const ChainPlan p = plan_chain(sh);
     if (p.flops < kTTDigitFlops) return false;
     int64_t P = 1, Q = 1;
@@ -276,7 +282,7 @@ bool tt_chain_f64_tc_takes(const TTShape& sh) {
         if (j < p.c && sh.dims[j] * sh.ranks[j + 1] >= kMost) return false;
         if (j >= p.c && sh.ranks[j] * sh.dims[j] >= kMost) return false;
     }
-    return P < kMost && Q < kMost;
+    return P < kMost && Q < kMost && sh.ranks[p.c] * sg::product_tile(P, Q) >= kTTDigitTile;
 }
 
 bool tt_chain_saves(const TTShape& sh) { return plan_chain(sh).flops <= 0.8 * chain_flops(sh, sh.d - 1); }

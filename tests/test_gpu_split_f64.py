@@ -303,3 +303,24 @@ def test_tt_chain_of_blocks_of_different_size(lrc, cuda, dims, ranks):
         return z.reshape(-1)
     bound = chain([np.abs(c) for c in cores])
     assert np.all(np.abs(out.cpu().numpy() - chain(cores)) <= (sum(ranks) + 2 * d) * U64 * bound)
+
+
+@pytest.mark.parametrize("dims,ranks", [((3000, 2500), (1, 3, 1)), ((3000, 2500), (1, 2, 1)), ((200000, 16), (1, 11, 1)),
+                                        ((200000, 16), (1, 12, 1)), ((16, 90000), (1, 16, 1)), ((1500, 70, 90), (1, 4, 3, 1)),
+                                        ((1500, 70, 48), (1, 8, 4, 1))])
+def test_tt_low_ranks_and_thin_sides(lrc, cuda, dims, ranks):
+    """Both sides of the rule on bond rank times tile width."""
+    g = torch.Generator(device=cuda).manual_seed(6)
+    d = len(dims)
+    cores = [torch.randn(ranks[l], dims[l], ranks[l + 1], generator=g, device=cuda, dtype=torch.float64) for l in range(d)]
+    out = torch.empty(int(np.prod(dims)), dtype=torch.float64, device=cuda)
+    lrc.tt_reconstruct(cores, dims, ranks, "f64", out)
+
+    def full(cs):
+        z = cs[0].reshape(dims[0], -1)
+        for c in cs[1:]:
+            z = (z @ c.reshape(c.shape[0], -1)).reshape(-1, c.shape[2])
+        return z.reshape(-1)
+    want, bound = full(cores), full([c.abs() for c in cores])
+    # a few roundings here, the reference's sums
+    assert torch.all((out - want).abs() <= 2 * (sum(ranks) + 2 * d) * U64 * bound)
