@@ -260,3 +260,26 @@ def test_tt_rows_of_very_different_size(lrc, cuda):
     assert np.array_equal(np.isinf(got), np.isinf(want))
     ok = np.isfinite(want)
     assert np.all(np.abs(got[ok] - want[ok]) <= 4 * U32 * np.abs(want[ok]))
+
+
+@pytest.mark.parametrize("fmt", ["f32", "f32tc"])
+@pytest.mark.parametrize("dims,ranks", [((20000, 16), (1, 16, 1)), ((16, 20001), (1, 5, 1)), ((200, 100, 8), (1, 8, 4, 1)),
+                                        ((9600, 96), (1, 16, 1)), ((9600, 97), (1, 16, 1)), ((8, 50, 60, 5), (1, 8, 20, 5, 1)),
+                                        ((2100, 500), (1, 17, 1)), ((700, 1500), (1, 64, 1))])
+def test_tt_thin_sides(lrc, cuda, dims, ranks, fmt):
+    """Both sides of the rule that sends thin tensors past the images."""
+    g = torch.Generator(device=cuda).manual_seed(5)
+    d = len(dims)
+    cores = [torch.randn(ranks[l], dims[l], ranks[l + 1], generator=g, device=cuda) for l in range(d)]
+    out = torch.empty(int(np.prod(dims)), device=cuda)
+    lrc.tt_reconstruct(cores, dims, ranks, fmt, out)
+
+    def full(cs):
+        z = cs[0].reshape(dims[0], -1)
+        for c in cs[1:]:
+            z = (z @ c.reshape(c.shape[0], -1)).reshape(-1, c.shape[2])
+        return z.reshape(-1)
+    want, bound = full([c.double() for c in cores]), full([c.double().abs() for c in cores])
+    # f32tc: 22 bits an operand of the largest of 32 rows, four times a rounding each
+    assert torch.all((out.double() - want).abs() <= (sum(ranks) + 2 * d + (64 if fmt == "f32tc" else 0)) * U32 * bound + (
+        8 * U32 * bound.max() if fmt == "f32tc" else 0))
