@@ -878,6 +878,8 @@ __device__ __forceinline__ void y_body(const CUtensorMap* tm_u, const CUtensorMa
                                     full(std::false_type{}, std::false_type{});
                                 }
                             } else {
+                                // (a branch a row for aligned pairs is slower: 100001 x
+                                // 33000, k = 48, b = 30 24.9 -> 30.9 us)
 #pragma unroll
                                 for (int rr = 0; rr < 32; ++rr) {
                                     if (rr >= nrows) break;

@@ -40,7 +40,6 @@
 #include <cuda_fp16.h>
 
 #include <algorithm>
-
 #include <type_traits>
 
 #include "common.cuh"
@@ -548,10 +547,10 @@ lrc_status launch_split_t(const TTShape& sh, bool out16, void* out, cudaStream_t
     if (kF32) {
         // Six parts of every row of Z and column of S are written and read, 24 rp bytes,
         // beside 4 P Q of output: not for tensors with a thin side, where the products of
-        // tt_chain.cu move less.  Measured, images / products: 10^6 x 16, rank 16 403 /
-        // 154 us, 10^5 x 64, ranks 16 and 48 52 / 30 and 93 / 40, 1000 x 1000 x 8, ranks 8
-        // and 4 1249 / 112; 200^3, rank 20 28 / 31, 2000 x 2000 x 16, rank 16 85 / 84,
-        // 4096^2, rank 64 45 / 58, 30^3, rank 8 (launches only) 22 / 25.
+        // tt_chain.cu move less.  Measured, images / products: 10^6 x 16, rank 16 396 /
+        // 155 us, 10^5 x 64, ranks 16 and 48 53 / 21 and 92 / 39, 1000 x 1000 x 8, ranks 8
+        // and 4 1235 / 113; 200^3, rank 20 28 / 33, 2000 x 2000 x 16, rank 16 81 / 84,
+        // 4096^2, rank 64 46 / 59, 30^3, rank 8 (launches only) 22 / 29.
         const double images = 6.0 * rp * ((double)a.P + (double)a.Q), out = (double)a.P * (double)a.Q;
         if (images > std::max(out, 1048576.0)) return LRC_OK;
     }
