@@ -226,7 +226,7 @@ void release_scratch();
 lrc_status stream_workspace(cudaStream_t s, size_t bytes, void** out);
 // The same where another path can do without: *out = nullptr when the buffer
 // cannot be made (no memory, or the stream is being captured and the present
-// one is too small).
+// one is too small); the present one then stays as it is.
 lrc_status stream_workspace_try(cudaStream_t s, size_t bytes, void** out);
 // Per-(device, stream) arrival counters, zero between kernels: kStreamCounters
 // of them, made (and zeroed in stream order) on first use.

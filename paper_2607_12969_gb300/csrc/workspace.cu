@@ -36,6 +36,8 @@ struct Slot {
 };
 std::map<std::pair<int, cudaStream_t>, Slot> g_slot;
 
+size_t whole_mib(size_t bytes) { return (bytes + ((size_t)1 << 20) - 1) & ~(((size_t)1 << 20) - 1); }
+
 }  // namespace
 
 lrc_status stream_workspace(cudaStream_t s, size_t bytes, void** out) {
@@ -52,7 +54,7 @@ lrc_status stream_workspace(cudaStream_t s, size_t bytes, void** out) {
             b.ptr = nullptr;
             b.bytes = 0;
         }
-        const size_t want = (bytes + ((size_t)1 << 20) - 1) & ~(((size_t)1 << 20) - 1);   // whole MiB
+        const size_t want = whole_mib(bytes);
         e = cudaMalloc(&b.ptr, want);
         if (e != cudaSuccess) {
             b.ptr = nullptr;
@@ -71,21 +73,32 @@ lrc_status stream_workspace_try(cudaStream_t s, size_t bytes, void** out) {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return cuda_fail(e, "cudaGetDevice");
-    bool grow = true;
-    {
-        std::lock_guard<std::mutex> lock(g_ws_mu);
-        const auto it = g_ws.find(std::make_pair(dev, s));
-        grow = it == g_ws.end() || it->second.bytes < bytes;
-    }
-    if (grow) {
+    std::lock_guard<std::mutex> lock(g_ws_mu);
+    Buf& b = g_ws[std::make_pair(dev, s)];
+    if (b.bytes < bytes) {
         // a buffer cannot be made or replaced while the stream is being captured
         cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
         if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) cudaGetLastError();
         if (cap != cudaStreamCaptureStatusNone) return LRC_OK;
+        // The new buffer first: where there is no memory for it the call goes on
+        // without, and the present one, whose address graphs may hold, stays.
+        const size_t want = whole_mib(bytes);
+        void* p = nullptr;
+        if (cudaMalloc(&p, want) != cudaSuccess) {
+            cudaGetLastError();
+            return LRC_OK;
+        }
+        if (b.ptr) {
+            if ((e = cudaStreamSynchronize(s)) != cudaSuccess) {
+                cudaFree(p);
+                return cuda_fail(e, "cudaStreamSynchronize (workspace growth)");
+            }
+            cudaFree(b.ptr);
+        }
+        b = Buf{p, want};
     }
-    const lrc_status st = stream_workspace(s, bytes, out);
-    if (st == LRC_ERR_NOMEM) *out = nullptr;
-    return st == LRC_ERR_NOMEM ? LRC_OK : st;
+    *out = b.ptr;
+    return LRC_OK;
 }
 
 lrc_status stream_counters(cudaStream_t s, unsigned int** out) {
