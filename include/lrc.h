@@ -155,7 +155,9 @@ LRC_API lrc_status lrc_widen_factors(const void* src, lrc_fmt fmt, int64_t rows,
  * magnitudes S_ij = sum_k |a_ik b_jk| is below about 2^-5 B_i B_j, where that
  * would be less than binary64 FMAs give, are formed by binary64 FMAs, so that
  * every entry is as a rule within 0.1 sqrt(K) 2^-53 S_ij of the exact sum of K
- * terms, and at worst within K 2^-50 S_ij (FMA sums: K 2^-53 S_ij).  Rows that
+ * terms, and at worst within K 2^-50 S_ij (FMA sums: K 2^-53 S_ij).  (2^-9 where
+ * the entries of a row are whole multiples of 2^-7 B_i, as the identity's are:
+ * then within 2^-52 S_ij for every term that is not zero.)  Rows that
  * hold an infinity, a NaN or a largest entry outside 2^-480 ... 2^495 are formed
  * by FMAs too.  The digits (14 bytes an element, of at most 1 GiB of queries at a
  * time) live in the stream's workspace; without memory for them, or while the

@@ -540,7 +540,7 @@ static lrc_status launch_apply_f64_tc(const double* U, const double* S, const do
     if (st != LRC_OK || !ws) return st;
     *handled = true;
     unsigned char* base = static_cast<unsigned char*>(ws);
-    sg::Listed* list = reinterpret_cast<sg::Listed*>(base + o_f);      // of one product after the other
+    int2* list = reinterpret_cast<int2*>(base + o_f);      // of one product after the other
     int* counts = reinterpret_cast<int*>(base + o_n);
     double* W = reinterpret_cast<double*>(base + o_wd);
     double* part = reinterpret_cast<double*>(base + o_p);

@@ -588,7 +588,7 @@ struct Carve {
 struct DigitGram {
     sg::Operand64 a;
     double* part;
-    sg::Listed* list;
+    int2* list;
 };
 size_t digit_gram_bytes(int p, int64_t L) {
     return sg::operand_bytes(p, L) + sg::part_bytes(p, p) + sg::fix_bytes(p, p);
@@ -600,7 +600,7 @@ DigitGram digit_gram(const double* A, int p, int64_t L, unsigned char* ws) {
     g.a.K = L;
     sg::operand_carve(&g.a, ws);
     g.part = reinterpret_cast<double*>(ws + sg::operand_bytes(p, L));
-    g.list = reinterpret_cast<sg::Listed*>(ws + sg::operand_bytes(p, L) + sg::part_bytes(p, p));
+    g.list = reinterpret_cast<int2*>(ws + sg::operand_bytes(p, L) + sg::part_bytes(p, p));
     return g;
 }
 

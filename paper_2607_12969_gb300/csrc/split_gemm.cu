@@ -35,7 +35,10 @@
 // 0.1 sqrt(K) 2^-53 S_ij, and at worst (first digits rounded up from halves
 // besides) within K 2^-50 S_ij; FMA sums of K terms are bounded by K 2^-53 S_ij.
 // Rows of Gaussian entries reach the limit within 16 terms for all but 1e-6 of
-// the entries, also with columns scaled by j^-1.5 or 0.9^j.
+// the entries, also with columns scaled by j^-1.5 or 0.9^j.  Where one of the rows
+// has first digits only (units, signs, small integers) no class is left out, the
+// other row's rounding (2^-62 of its B a term) is all there is, and the limit is
+// 2^-9 (kMinShort).
 //
 // Rows that hold an infinity, a NaN or a largest entry outside 2^-480 ...
 // 2^495 get zero digits, so that all their entries are listed.
@@ -64,10 +67,10 @@ __device__ unsigned int g_err_split;
 constexpr int64_t kOwnStatsK = 512;    // reductions up to this long: slice_kernel takes the row statistics itself
 constexpr int kNonFinite = 1 << 20;    // marks a row with an infinity or NaN in its statistics
 constexpr int kNoEntry = -(1 << 20);   // ... one without nonzero entries
-// In the exponents' place for a row whose digits are all zero: because it holds
-// nothing else, or because the digits cannot carry it.
-constexpr int kZeroRow = -1, kHardRow = -2;
-constexpr float kMinSum = 512.0f;      // 2^-5 in units of products of first digits
+// Kinds of rows: with digits past the first; with first digits only; with none,
+// because it holds nothing but zeros, or because the digits cannot carry it.
+enum RowKind : unsigned char { kDeepRow, kShortRow, kZeroRow, kHardRow };
+constexpr float kMinSum = 512.0f, kMinShort = 32.0f;     // 2^-5 and 2^-9 in units of products of first digits
 // Biased exponents of a row's largest entry that digits carry: with both rows
 // inside, every result is zero or a normal number (round_pq).
 constexpr int kMinExp = 544, kMaxExp = 1518;
@@ -112,6 +115,7 @@ struct Job {
     int* stats;              // splits > 0: statistics per slice of K; else slice_kernel takes its own
     unsigned char* img;
     int* exps;
+    unsigned char* kind;
 };
 struct Jobs {
     Job j[kMaxOps];
@@ -189,7 +193,7 @@ __device__ __forceinline__ int block_stats(const View64& v, int64_t r0, int64_t 
     return t;
 }
 
-__global__ void __launch_bounds__(256) row_stats_kernel(const __grid_constant__ Jobs js) {
+__global__ void __launch_bounds__(256, 6) row_stats_kernel(const __grid_constant__ Jobs js) {
     __shared__ int sm[8][32];
     pdl_wait();
     pdl_trigger();
@@ -200,7 +204,10 @@ __global__ void __launch_bounds__(256) row_stats_kernel(const __grid_constant__ 
     const int64_t k1 = min(o.K, k0 + o.kchunk);
     const int a = o.v.s.scale ? block_stats<true>(o.v, r0, o.rows, k0, k1, o.vec != 0, sm)
                               : block_stats<false>(o.v, r0, o.rows, k0, k1, o.vec != 0, sm);
-    if (threadIdx.x < 32 && r0 + threadIdx.x < o.rows) o.stats[z * o.rows + r0 + threadIdx.x] = a;
+    if (threadIdx.x < 32 && r0 + threadIdx.x < o.rows) {
+        o.stats[z * o.rows + r0 + threadIdx.x] = a;
+        if (z == 0) o.kind[r0 + threadIdx.x] = kShortRow;
+    }
 }
 
 // ---------------------------------------------------------------- digits
@@ -209,8 +216,9 @@ __global__ void __launch_bounds__(256) row_stats_kernel(const __grid_constant__ 
 // largest entry.  The value is rounded to a multiple of 2^-61 of 2^(em -
 // 1022), the power of two above it, and the digits are those of that integer
 // plus 256 at every place but the first, minus 256 again: a number read with
-// digits in [-256, 255].
-__device__ __forceinline__ void digits8(const double (&x)[8], const int (&sh)[8], int em, uint32_t (&w)[kParts64][4]) {
+// digits in [-256, 255].  `any` collects the integers' bits.
+__device__ __forceinline__ void digits8(const double (&x)[8], const int (&sh)[8], int em, uint32_t (&w)[kParts64][4],
+                                        uint64_t& any) {
     constexpr uint64_t kBias = 256ull * (1ull + (1ull << 9) + (1ull << 18) + (1ull << 27) + (1ull << 36) + (1ull << 45));
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
@@ -225,6 +233,7 @@ __device__ __forceinline__ void digits8(const double (&x)[8], const int (&sh)[8]
             if (s >= 0) v = mant << s;
             else v = s > -55 ? (mant + (1ll << (-s - 1))) >> -s : 0;
             if (b < 0) v = -v;
+            any |= (uint64_t)v;
             const uint64_t t = (uint64_t)v + kBias;
             const int d0 = (int)((int64_t)t >> 54);
             f[h][0] = __int_as_float(0x4b400000 + d0) - 12582912.0f;
@@ -244,9 +253,9 @@ __device__ __forceinline__ void digits8(const double (&x)[8], const int (&sh)[8]
 // and `kchunk` columns (of an operand with a short reduction all of them, and
 // takes the row statistics itself); a lane is a row, so that a warp's 16-byte
 // stores of one digit are four runs of 128 bytes.
-__global__ void __launch_bounds__(256) slice_kernel(const __grid_constant__ Jobs js) {
+__global__ void __launch_bounds__(256, 4) slice_kernel(const __grid_constant__ Jobs js) {
     __shared__ int sm[8][32];
-    __shared__ int s_em[32];
+    __shared__ int s_em[32], s_deep[32];
     pdl_wait();
     pdl_trigger();
     const Job& o = job_of(js, blockIdx.x);
@@ -259,22 +268,24 @@ __global__ void __launch_bounds__(256) slice_kernel(const __grid_constant__ Jobs
     if (o.splits == 0) own = block_stats<true>(v, r0, rows, 0, K, o.vec != 0, sm);
     if (tid < 32) {
         const int64_t r = r0 + lane;
-        int em = kZeroRow;
-        if (r < rows) {
-            int mx = own;
+        int mx = own;
+        if (r < rows)
             for (int z = 0; z < o.splits; ++z) mx = max(mx, o.stats[(int64_t)z * rows + r]);
-            if (mx != kNoEntry) em = mx < kMinExp || mx > kMaxExp ? kHardRow : mx;
+        const bool none = r >= rows || mx == kNoEntry, hard = !none && (mx < kMinExp || mx > kMaxExp);
+        s_em[lane] = none || hard ? -1 : mx;
+        s_deep[lane] = 0;
+        if (kp == 0 && r < o.img_rows) {
+            o.exps[r] = none || hard ? 1023 : mx;
+            if (none || hard) o.kind[r] = none ? kZeroRow : kHardRow;
         }
-        s_em[lane] = em;
-        if (kp == 0 && r < o.img_rows) o.exps[r] = em;
     }
     __syncthreads();
     const int64_t r = r0 + lane;
-    if (r >= o.img_rows) return;
     const int em = s_em[lane];
+    uint64_t any = 0;
     const size_t block_bytes = (size_t)(o.img_rows / 8) * kGroupBytes;
     unsigned char* row_base = o.img + (size_t)(r >> 3) * kGroupBytes + (r & 7) * 16;
-    const int64_t o1 = min((kp + 1) * o.kchunk, o.kblocks * kKB) / 8;
+    const int64_t o1 = r < o.img_rows ? min((kp + 1) * o.kchunk, o.kblocks * kKB) / 8 : 0;
     for (int64_t oc = kp * o.kchunk / 8 + warp; oc < o1; oc += 8) {
         double x[8];
         int sh[8];
@@ -297,11 +308,18 @@ __global__ void __launch_bounds__(256) slice_kernel(const __grid_constant__ Jobs
 #pragma unroll
         for (int j = 0; j < 8; ++j) sh[j] = (v.s.scale && k0 + j < K) ? v.shift(k0 + j) : 0;
         uint32_t w[kParts64][4];
-        digits8(x, sh, em < 0 ? 1023 : em, w);
+        digits8(x, sh, em < 0 ? 1023 : em, w, any);
         unsigned char* dst = row_base + (size_t)(oc >> 1) * block_bytes + (size_t)(oc & 1) * 128;
 #pragma unroll
         for (int i = 0; i < kParts64; ++i)
             *reinterpret_cast<uint4*>(dst + i * (8 * kKB * 2)) = make_uint4(w[i][0], w[i][1], w[i][2], w[i][3]);
+    }
+    if (any & ((1ull << 54) - 1)) s_deep[lane] = 1;        // digits past the first
+    __syncthreads();
+    if (tid < 32 && r < rows && em >= 0) {
+        // (row_stats_kernel has made it kShortRow where several CTAs have a part of the row)
+        if (s_deep[lane]) o.kind[r] = kDeepRow;
+        else if (o.splits == 0) o.kind[r] = kShortRow;
     }
 }
 
@@ -320,7 +338,7 @@ struct GemmArgs {
     int split, group, stages, tma;
     int64_t a_block, b_block;    // bytes of a block of either image
     uint32_t a_bytes, b_bytes;   // of a tile's part of it
-    Listed* fix;                 // entries to recompute, and the number of blocks of them
+    int2* fix;                   // listed blocks (first row, first column), and their number
     int* nfix;
     int listed;                  // > 0: the tiles are list[0 ... listed), row << 8 | column
     uint16_t list[kMaxListed];
@@ -475,43 +493,31 @@ __device__ __forceinline__ void mma_16x8(float (&d)[4], const uint32_t (&a)[4], 
                  : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]), "f"(c0), "f"(c1), "f"(c2), "f"(c3));
 }
 
-// Lists the entries of half a tile's columns whose sums of magnitudes, estimated
-// from the first digits, do not reach kMinSum, 16 rows at a time, straight from
-// the images, whose octets have the layout of m16n8k16 fragments.  On most data
-// the first 16 terms pass for all entries: two warps have the time of the tile's
-// MMAs and epilogue for them, if the loads are not waited for one by one
-// (16384 x 8192, k = 128, b = 8192: 1577 us without the estimates, 2016 with each
-// load waited for, 1575 like this).  Where they do not, the sums go on over at
-// most kLookBlocks, and what then is below the limit is listed: repair_kernel
-// looks at the rest of the reduction with more warps.
-constexpr int kLookBlocks = 8;
+// Lists the blocks (16 rows, half a tile's columns) in which an entry's sum of
+// magnitudes, estimated from the first digits of the first 16 terms, does not reach
+// kMinSum; repair_kernel looks at those more closely.  Straight from the images,
+// whose octets have the layout of m16n8k16 fragments.  Two warps have the time of a
+// tile's MMAs and epilogue for this, if the loads are not waited for one by one and
+// the registers that the first warps keep suffice (16384 x 8192, k = 128, b = 8192:
+// 1577 us without the estimates, 2016 with each load waited for, 1616 with the
+// longer sums here too).
 template <int NT>
 __device__ __forceinline__ void list_small_sums(const GemmArgs& a, int mt, int nt, int half, int lane) {
     constexpr int J = NT / 16, kBatch = 4;
+    constexpr uint32_t kBeyond = 0x49804980u;              // 2^20, twice: past the edges every sum is large
     const int row_t = mt * 128, col0 = nt * NT + half * (NT / 2);
     if (col0 >= a.N) return;
-    auto columns = [&](int kb, uint32_t (&d)[J][2]) {      // (what lies past the last row is not defined)
-        const unsigned char* p = a.B + kb * a.b_block + (int64_t)(col0 >> 3) * kGroupBytes;
+    uint32_t b[J][2];
+    {
+        const unsigned char* p = a.B + (int64_t)(col0 >> 3) * kGroupBytes;
 #pragma unroll
         for (int j = 0; j < J; ++j) {
-            const bool in = col0 + 8 * j < a.N;
-            d[j][0] = in ? first_digits(p + j * kGroupBytes, 0, lane) : 0u;
-            d[j][1] = in ? first_digits(p + j * kGroupBytes, 1, lane) : 0u;
+            const bool in = col0 + 8 * j + (lane >> 2) < a.N;
+            b[j][0] = in ? first_digits(p + j * kGroupBytes, 0, lane) : kBeyond;
+            b[j][1] = in ? first_digits(p + j * kGroupBytes, 1, lane) : kBeyond;
         }
-    };
-    // rows lane / 4 (0, 1) and lane / 4 + 8 (2, 3), columns 8 j + 2 (lane % 4) + {0, 1}
-    float acc[J][4];
-    auto reached = [&]() {
-        float least = acc[0][0];
-#pragma unroll
-        for (int j = 0; j < J; ++j)
-#pragma unroll
-            for (int i = 0; i < 4; ++i) least = fminf(least, acc[j][i]);
-        return __all_sync(0xffffffffu, least >= kMinSum) != 0;
-    };
-    uint32_t b[J][2];
-    columns(0, b);
-    uint32_t failed = 0;                                   // strips whose first terms do not suffice
+    }
+    uint32_t failed = 0;
     for (int s0 = 0; s0 < 8; s0 += kBatch) {
         const unsigned char* rows = a.A + (int64_t)((row_t >> 3) + 2 * s0) * kGroupBytes;
         uint32_t x[kBatch][4];
@@ -520,46 +526,26 @@ __device__ __forceinline__ void list_small_sums(const GemmArgs& a, int mt, int n
             if (row_t + 16 * (s0 + s) < a.M) first_digits_a(rows + s * 2 * kGroupBytes, lane, x[s]);
 #pragma unroll
         for (int s = 0; s < kBatch; ++s) {
-            if (row_t + 16 * (s0 + s) >= a.M) break;
+            const int row0 = row_t + 16 * (s0 + s);
+            if (row0 >= a.M) break;
+            if (row0 + 16 > a.M) {
+                if (row0 + (lane >> 2) >= a.M) x[s][0] = x[s][2] = kBeyond;
+                if (row0 + (lane >> 2) + 8 >= a.M) x[s][1] = x[s][3] = kBeyond;
+            }
+            float acc[J][4], least;
 #pragma unroll
             for (int j = 0; j < J; ++j) mma_16x8(acc[j], x[s], b[j], 0.0f, 0.0f, 0.0f, 0.0f);
-            failed |= reached() ? 0u : 1u << (s0 + s);
+            least = acc[0][0];
+#pragma unroll
+            for (int j = 0; j < J; ++j)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) least = fminf(least, acc[j][i]);
+            failed |= __all_sync(0xffffffffu, least >= kMinSum) ? 0u : 1u << (s0 + s);
         }
     }
-    for (; failed; failed &= failed - 1) {
-        const int row0 = row_t + 16 * (__ffs((int)failed) - 1);
-        // Entries that need no sum: past the edges, a row of zeros with one that holds
-        // no infinity or NaN, what a symmetric product leaves out.
-#pragma unroll
-        for (int i = 0; i < 4 * J; ++i) {
-            const int r = row0 + (lane >> 2) + 8 * ((i >> 1) & 1), c = col0 + 8 * (i >> 2) + 2 * (lane & 3) + (i & 1);
-            const int er = r < a.M ? a.ea[r] : 0, ec = c < a.N ? a.eb[c] : 0;
-            const bool zero = (er == kZeroRow && ec != kHardRow) || (ec == kZeroRow && er != kHardRow);
-            acc[i >> 2][i & 3] = zero || r >= a.M || c >= a.N || (a.listed && r > c) ? kMinSum : 0.0f;
-        }
-        const int last = min(a.kblocks, kLookBlocks);
-        bool done = reached();
-        for (int kb = 0; kb < last && !done; ++kb) {
-            uint32_t y[4];
-            first_digits_a(a.A + kb * a.a_block + (int64_t)(row0 >> 3) * kGroupBytes, lane, y);
-            columns(kb, b);
-#pragma unroll
-            for (int j = 0; j < J; ++j) mma_16x8(acc[j], y, b[j], acc[j][0], acc[j][1], acc[j][2], acc[j][3]);
-            done = reached();
-        }
-        if (done) continue;
-        int at = 0;
-        if (lane == 0) at = atomicAdd(a.nfix, 1);
-        Listed* f = a.fix + __shfl_sync(0xffffffffu, at, 0);
-        if (lane == 0) {
-            f->row0 = row0;
-            f->col0 = col0;
-        }
-#pragma unroll
-        for (int i = 0; i < 4 * J; ++i) {
-            const uint32_t m = __ballot_sync(0xffffffffu, !(acc[i >> 2][i & 3] >= kMinSum));
-            if (lane == 0) f->mask[i] = m;
-        }
+    if (lane == 0 && failed) {
+        int2* list = a.fix + atomicAdd(a.nfix, __popc(failed));
+        for (; failed; failed &= failed - 1) *list++ = make_int2(row_t + 16 * (__ffs((int)failed) - 1), col0);
     }
 }
 
@@ -889,26 +875,27 @@ __global__ void __launch_bounds__(256) part_sum_kernel(const __grid_constant__ G
 }
 
 // ---------------------------------------------------------------- repair
-// Listed entries by binary64 FMAs, whose rate (two a clock on an SM) is the bound
-// where there are many.
-//  * Reductions from kLongK on: a warp takes 8 x 8 entries, finishes the sums of
-//    their magnitudes, and recomputes those that stay below the limit, 8 x 4 at a
-//    time with the lanes along the reduction, or where there are few one after
-//    the other.
-//  * Shorter ones: a warp takes 16 x 8 entries, four a lane.
+// Of the listed blocks the entries whose sums of magnitudes stay below the limit
+// over all of the reduction, by binary64 FMAs, whose rate (two a clock on an SM) is
+// the bound where there are many.  A warp takes 16 x 8 entries.
+//  * Reductions from kLongK on: 8 x 4 entries at a time with the lanes along the
+//    reduction, or where there are few one after the other.
+//  * Shorter ones: four entries a lane.
 struct RepairArgs {
     View64 A, B;
-    const Listed* fix;
+    const int2* fix;
     const int* nfix;
-    int64_t K;
+    int64_t M, N, K;
     double* C;
     int64_t cr, cc;
     const double* rscale;
     const double* cscale;
-    int sym;                  // C symmetric, the entries above the diagonal are listed
-    int words;                // of a mask
-    const unsigned char* ia;  // the images, for longer sums of first digits
+    int sym;                  // C symmetric, the entries above the diagonal are formed
+    int groups;               // of 8 columns in a block
+    const unsigned char* ia;  // images and kinds of rows
     const unsigned char* ib;
+    const unsigned char* ka;
+    const unsigned char* kb;
     int64_t a_block, b_block;
     int kblocks;
 };
@@ -970,92 +957,104 @@ __device__ __forceinline__ void repair_word(const RepairArgs& a, int64_t r0, int
     if ((mask >> lane) & 1) put_entry(a, r0 + lane / 4, c0 + 2 * (lane & 3), acc[0]);
 }
 
-// Which of 8 x 8 listed entries (words m0, m1) stay below the limit over all of
-// the reduction: eight blocks' digits in flight.
-__device__ __forceinline__ void still_small(const RepairArgs& a, int64_t r0, int64_t c0, int lane, uint32_t& m0,
-                                            uint32_t& m1) {
+// What a sum of first digits starts from, so that kMinSum is the limit for all: a
+// row of zeros makes zeros, unless the other holds an infinity or a NaN.
+__device__ __forceinline__ float first_sum(int ka, int kb) {
+    if ((ka == kZeroRow && kb != kHardRow) || (kb == kZeroRow && ka != kHardRow)) return kMinSum;
+    return ka == kDeepRow && kb == kDeepRow ? 0.0f : kMinSum - kMinShort;
+}
+
+// The entries of rows r0 ... r0 + 15 and columns c0 ... c0 + 7 that stay below the
+// limit: bit `lane` of m[2 h + i] is row r0 + 8 h + lane / 4, column c0 + 2 (lane %
+// 4) + i.  Eight blocks' digits in flight.
+__device__ __forceinline__ void small_sums(const RepairArgs& a, int64_t r0, int64_t c0, int lane, uint32_t (&m)[4]) {
     const unsigned char* pa = a.ia + (r0 >> 3) * kGroupBytes;
     const unsigned char* pb = a.ib + (c0 >> 3) * kGroupBytes;
-    const bool on0 = (m0 >> lane) & 1, on1 = (m1 >> lane) & 1;
-    float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-    for (int kb = 0; kb < a.kblocks; kb += 8) {
+    float acc[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int64_t r = r0 + 8 * (i >> 1) + lane / 4, c = c0 + 2 * (lane & 3) + (i & 1);
+        const bool in = r < a.M && c < a.N && !(a.sym && r > c);
+        acc[i] = in ? first_sum(a.ka[r], a.kb[c]) : kMinSum;
+    }
+    auto least = [&]() { return fminf(fminf(acc[0], acc[1]), fminf(acc[2], acc[3])); };
+    bool done = __all_sync(0xffffffffu, least() >= kMinSum) != 0;
+    for (int kb = 0; kb < a.kblocks && !done; kb += 8) {
         uint32_t x[8][4], y[8][2];
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
             const bool in = kb + u < a.kblocks;
-            x[u][1] = x[u][3] = 0u;
-            x[u][0] = in ? first_digits(pa + (kb + u) * a.a_block, 0, lane) : 0u;
-            x[u][2] = in ? first_digits(pa + (kb + u) * a.a_block, 1, lane) : 0u;
-            y[u][0] = in ? first_digits(pb + (kb + u) * a.b_block, 0, lane) : 0u;
-            y[u][1] = in ? first_digits(pb + (kb + u) * a.b_block, 1, lane) : 0u;
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                x[u][i] = in ? first_digits(pa + (kb + u) * a.a_block + (i & 1) * kGroupBytes, i >> 1, lane) : 0u;
+#pragma unroll
+            for (int i = 0; i < 2; ++i) y[u][i] = in ? first_digits(pb + (kb + u) * a.b_block, i, lane) : 0u;
         }
 #pragma unroll
         for (int u = 0; u < 8; ++u) mma_16x8(acc, x[u], y[u], acc[0], acc[1], acc[2], acc[3]);
-        if (__all_sync(0xffffffffu, (!on0 || acc[0] >= kMinSum) && (!on1 || acc[1] >= kMinSum))) break;
+        done = __all_sync(0xffffffffu, least() >= kMinSum) != 0;
     }
-    m0 &= __ballot_sync(0xffffffffu, !(acc[0] >= kMinSum));
-    m1 &= __ballot_sync(0xffffffffu, !(acc[1] >= kMinSum));
+#pragma unroll
+    for (int i = 0; i < 4; ++i) m[i] = __ballot_sync(0xffffffffu, !(acc[i] >= kMinSum));
 }
 
 __global__ void __launch_bounds__(256, 2) repair_kernel(const __grid_constant__ RepairArgs a) {
     pdl_wait();
     pdl_trigger();
-    const int64_t n = *a.nfix;
-    if (n == 0) return;
+    const int64_t units = (int64_t)*a.nfix * a.groups;
+    if (units == 0) return;
     const int lane = threadIdx.x & 31;
     const int64_t w0 = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5), warps = (int64_t)gridDim.x * 8;
-    if (a.K >= kLongK) {
-        // Few blocks: several warps a block, each with a word or with its share of the entries.
-        const int pairs = a.words / 2;
-        const int64_t blocks = n * pairs;
-        const int share = blocks * 32 <= warps ? 32 : blocks * 8 <= warps ? 8 : blocks * 2 <= warps ? 2 : 1;
-        for (int64_t u = w0; u < blocks * share; u += warps) {
-            const Listed& f = a.fix[u / share / pairs];
-            const int i = 2 * (int)(u / share % pairs), mine = (int)(u % share);
-            uint32_t m[2] = {f.mask[i], f.mask[i + 1]};
-            if (!(m[0] | m[1])) continue;
-            const int64_t r0 = f.row0 + 8 * ((i >> 1) & 1), c0 = f.col0 + 8 * (i >> 2);
-            if (a.kblocks > kLookBlocks) still_small(a, r0, c0, lane, m[0], m[1]);
+    // Few units with a long reduction: several warps each, with a word or with their
+    // share of the entries.
+    const int share = a.K < kLongK || units * 4 > warps ? 1 : units * 8 > warps ? 4 : units * 32 > warps ? 8 : 32;
+    for (int64_t u = w0; u < units * share; u += warps) {
+        const int mine = (int)(u % share), j = (int)(u / share % a.groups);
+        const int2 f = a.fix[u / share / a.groups];
+        const int64_t r0 = f.x, c0 = f.y + 8 * j;
+        if (c0 >= a.N) continue;
+        uint32_t m[4];
+        small_sums(a, r0, c0, lane, m);
+        if (!(m[0] | m[1] | m[2] | m[3])) continue;
+        if (a.K >= kLongK) {
             int e = 0;
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                if (share == 2 && mine != h) continue;
-                if (share <= 2 && __popc(m[h]) > kFew) {
-                    repair_word(a, r0, c0 + h, m[h], lane);
+            for (int i = 0; i < 4; ++i) {
+                if (share == 4 && mine != i) continue;
+                const int64_t rw = r0 + 8 * (i >> 1), cw = c0 + (i & 1);
+                if (share <= 4 && __popc(m[i]) > kFew) {
+                    repair_word(a, rw, cw, m[i], lane);
                 } else {
-                    for (uint32_t w = m[h]; w; w &= w - 1, ++e) {
+                    for (uint32_t w = m[i]; w; w &= w - 1, ++e) {
                         const int bit = __ffs((int)w) - 1;
-                        if (share <= 2 || e % share == mine) repair_dot(a, r0 + bit / 4, c0 + h + 2 * (bit & 3), lane);
+                        if (share <= 4 || e % share == mine) repair_dot(a, rw + bit / 4, cw + 2 * (bit & 3), lane);
                     }
                 }
             }
+            continue;
         }
-        return;
-    }
-    const int groups = a.words / 4;
-    for (int64_t u = w0; u < n * groups; u += warps) {
-        const Listed& f = a.fix[u / groups];
-        const int j = (int)(u % groups);
         bool on[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) on[i] = (f.mask[4 * j + i] >> lane) & 1;
+        for (int i = 0; i < 4; ++i) on[i] = (m[i] >> lane) & 1;
         const bool top = on[0] || on[1], low = on[2] || on[3], left = on[0] || on[2], right = on[1] || on[3];
-        if (!top && !low) continue;
-        // an entry that is not listed may lie past the edge: a listed one's row or column instead
-        const int64_t r = f.row0 + lane / 4, c = f.col0 + 8 * j + 2 * (lane & 3);
-        const int64_t r0 = top ? r : r + 8, r1 = low ? r + 8 : r, c0 = left ? c : c + 1, c1 = right ? c + 1 : c;
-        double acc[4] = {0.0, 0.0, 0.0, 0.0};
+        if (top || low) {
+            // an entry that is not listed may lie past the edge: a listed one's row or column instead
+            const int64_t r = r0 + lane / 4, c = c0 + 2 * (lane & 3);
+            const int64_t ra = top ? r : r + 8, rb = low ? r + 8 : r, ca = left ? c : c + 1, cb = right ? c + 1 : c;
+            double acc[4] = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll 4
-        for (int64_t k = 0; k < a.K; ++k) {
-            const double x0 = a.A.at(r0, k), x1 = a.A.at(r1, k), y0 = a.B.at(c0, k), y1 = a.B.at(c1, k);
-            acc[0] = fma(x0, y0, acc[0]);
-            acc[1] = fma(x0, y1, acc[1]);
-            acc[2] = fma(x1, y0, acc[2]);
-            acc[3] = fma(x1, y1, acc[3]);
-        }
+            for (int64_t k = 0; k < a.K; ++k) {
+                const double x0 = a.A.at(ra, k), x1 = a.A.at(rb, k), y0 = a.B.at(ca, k), y1 = a.B.at(cb, k);
+                acc[0] = fma(x0, y0, acc[0]);
+                acc[1] = fma(x0, y1, acc[1]);
+                acc[2] = fma(x1, y0, acc[2]);
+                acc[3] = fma(x1, y1, acc[3]);
+            }
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
-            if (on[i]) put_entry(a, r + 8 * (i >> 1), c + (i & 1), acc[i]);
+            for (int i = 0; i < 4; ++i)
+                if (on[i]) put_entry(a, r + 8 * (i >> 1), c + (i & 1), acc[i]);
+        }
+        __syncwarp();
     }
 }
 
@@ -1082,7 +1081,7 @@ lrc_status launch_product(const GemmArgs& a, const CUtensorMap& tm, int64_t grid
 
 size_t operand_bytes(int64_t rows, int64_t K) {
     const int64_t ir = image_rows(rows);
-    return up256((size_t)(ir / 8) * image_blocks(K) * kGroupBytes + kTailBytes) + up256((size_t)ir * 4) +
+    return up256((size_t)(ir / 8) * image_blocks(K) * kGroupBytes + kTailBytes) + up256((size_t)ir * 4) + up256((size_t)ir) +
            up256((size_t)rows * (K > kOwnStatsK ? kStatSplits : 0) * 4);
 }
 
@@ -1092,6 +1091,8 @@ void operand_carve(Operand64* o, unsigned char* ws) {
     ws += up256((size_t)(ir / 8) * image_blocks(o->K) * kGroupBytes + kTailBytes);
     o->exps = reinterpret_cast<int*>(ws);
     ws += up256((size_t)ir * 4);
+    o->kind = ws;
+    ws += up256((size_t)ir);
     o->stats = reinterpret_cast<int*>(ws);
 }
 
@@ -1112,6 +1113,7 @@ lrc_status slice(const Operand64* const* ops, int count, int* clear, int nclear,
         j.stats = o.stats;
         j.img = o.img;
         j.exps = o.exps;
+        j.kind = o.kind;
         if (o.K > kOwnStatsK) {
             const int z = stat_splits(o.rows, o.K);
             j.kchunk = ((o.K + z - 1) / z + 31) / 32 * 32;
@@ -1166,7 +1168,7 @@ int product_tile(int64_t M, int64_t N) { return tiles_of(N, M) < tiles_of(M, N) 
 
 size_t fix_bytes(int64_t M, int64_t N) {
     if (tiles_of(N, M) < tiles_of(M, N)) std::swap(M, N);
-    return up256((size_t)((M + 15) / 16) * (size_t)(2 * n_tiles(N)) * sizeof(Listed));
+    return up256((size_t)((M + 15) / 16) * (size_t)(2 * n_tiles(N)) * sizeof(int2));
 }
 
 namespace {
@@ -1262,8 +1264,9 @@ lrc_status run_product(const Operand64& A0, const Operand64& B0, const Out64& ou
         if (e != cudaSuccess) return cuda_fail(e, "part_sum_kernel launch");
         if ((st = after_launch("part_sum_kernel")) != LRC_OK) return st;
     }
-    const RepairArgs r{View64{A.src}, View64{B.src}, fix.list, fix.count, A.K, out.C, out.cr, out.cc,
-                       out.rscale, out.cscale, a.listed ? 1 : 0, NT / 4, a.A, a.B, a.a_block, a.b_block, a.kblocks};
+    const RepairArgs r{View64{A.src}, View64{B.src}, fix.list, fix.count, A.rows, B.rows, A.K, out.C, out.cr, out.cc,
+                       out.rscale, out.cscale, a.listed ? 1 : 0, NT / 16, A.img, B.img, A.kind, B.kind,
+                       a.a_block, a.b_block, a.kblocks};
     e = launch_pdl(repair_kernel, dim3((unsigned)(2 * sms)), dim3(256), 0, s, r);
     if (e != cudaSuccess) return cuda_fail(e, "repair_kernel launch");
     return after_launch("repair_kernel");

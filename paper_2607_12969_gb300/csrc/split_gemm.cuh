@@ -42,6 +42,7 @@ struct Operand64 {
     int64_t rows, K;
     unsigned char* img;      // digits
     int* exps;               // exponent of every row (image rows)
+    unsigned char* kind;     // what every row's digits are (split_gemm.cu)
     int* stats;              // row statistics per slice of K
 };
 constexpr int kMaxOps = 5;   // operands per slice()
@@ -61,16 +62,10 @@ void operand_carve(Operand64* o, unsigned char* ws);
 // clear[0 ... nclear), at most 256 counters, are set to zero on the way.
 lrc_status slice(const Operand64* const* ops, int count, int* clear, int nclear, cudaStream_t s);
 
-// Entries of a product that the digits do not carry, of 16 rows and half a tile's
-// columns: bit 4 r + c of mask[4 j + 2 h + i] is entry (row0 + 8 h + r, col0 + 8 j
-// + 2 c + i).
-struct Listed {
-    int row0, col0;
-    uint32_t mask[16];
-};
-// `list` holds fix_bytes(M, N) for an M x N product, *count is zero before it.
+// Blocks of a product that may hold entries which the digits do not carry: `list`
+// holds fix_bytes(M, N) for an M x N product, *count is zero before it.
 struct Fix {
-    Listed* list;
+    int2* list;
     int* count;
 };
 size_t fix_bytes(int64_t M, int64_t N);

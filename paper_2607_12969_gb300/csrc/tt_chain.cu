@@ -255,7 +255,7 @@ lrc_status launch_tt_chain_f64_tc(const TTShape& sh, double* out, cudaStream_t s
         const sg::Operand64* ops[2] = {&t.a, &t.b};
         const sg::Out64 o{t.C, t.N, 1, nullptr, nullptr};
         if ((st = sg::slice(ops, 2, counts, i == 0 ? (int)steps.size() : 0, s)) != LRC_OK) return st;
-        if ((st = sg::product(t.a, t.b, o, false, nullptr, {reinterpret_cast<sg::Listed*>(ws + o_f), counts + i}, s)) != LRC_OK)
+        if ((st = sg::product(t.a, t.b, o, false, nullptr, {reinterpret_cast<int2*>(ws + o_f), counts + i}, s)) != LRC_OK)
             return st;
     }
     return LRC_OK;

@@ -324,3 +324,20 @@ def test_tt_low_ranks_and_thin_sides(lrc, cuda, dims, ranks):
     want, bound = full(cores), full([c.abs() for c in cores])
     # a few roundings here, the reference's sums
     assert torch.all((out - want).abs() <= 2 * (sum(ranks) + 2 * d) * U64 * bound)
+
+
+@pytest.mark.parametrize("m,n,k,b", [(300, 1100, 64, 1100), (200, 5000, 40, 700), (257, 300, 33, 2100)])
+def test_identity_and_sign_queries(lrc, cuda, m, n, k, b):
+    """Rows with first digits only lose nothing but the other row's rounding: the
+    identity gives the rows of V (to u of each), a few signs u of their sums."""
+    rng = np.random.default_rng(n)
+    Vt = rng.standard_normal((k, n)) * 2.0 ** -rng.integers(0, 12, (k, n))
+    U = np.eye(m, k)
+    X = np.zeros((b, n))
+    X[np.arange(b), np.arange(b) % n] = 1.0
+    few = np.arange(b) % 3 == 0
+    X[few] += (rng.random((few.sum(), n)) < 5 / n) * rng.choice([-1.0, 1.0, 3.0], (few.sum(), n))
+    got = run(lrc, cuda, U, np.ones(k), Vt, X)[:, :min(m, k)]
+    want = (X @ Vt.T)[:, :min(m, k)]
+    terms = np.count_nonzero(X, axis=1)[:, None]
+    assert np.all(np.abs(got - want) <= (2 * terms + 2) * U64 * (np.abs(X) @ np.abs(Vt).T)[:, :min(m, k)])

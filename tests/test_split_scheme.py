@@ -90,8 +90,9 @@ def digits(x):
 
 
 def check_unlisted(a, b, far_off=False):
-    """Entries whose first digits' sum of magnitudes reaches 2^9 are within
-    K 2^-50 of the exact sum of magnitudes; the others are left to FMAs."""
+    """Entries whose first digits' sum of magnitudes reaches 2^9, or 2^5 where a row
+    has first digits only, are within K 2^-50 of the exact sum of magnitudes (then
+    within 2^-52 for every term that is not zero); the others are left to FMAs."""
     K = a.shape[1]
     (da, ta), (db, tb) = digits(a), digits(b)
     kept = sum((da[:, i] @ db[:, j].T) * (1 << (9 * (6 - i - j))) for i in range(7) for j in range(7 - i))
@@ -100,8 +101,11 @@ def check_unlisted(a, b, far_off=False):
               for x, top in ((a, ta), (b, tb)))
     exact, mags = ia @ ib.T, abs(ia) @ abs(ib).T              # in units of 2^-400 of the digits' square
     err = abs(kept * (1 << 54) * (1 << 400) - exact)
-    on = np.asarray(est >= 512, bool)
+    short = np.logical_or.outer(np.all(da[:, 1:] == 0, (1, 2)), np.all(db[:, 1:] == 0, (1, 2)))
+    on = np.asarray(est >= np.where(short, 32, 512), bool)
     assert np.all(err[on] * (1 << 50) <= K * mags[on])
+    terms = np.asarray(ia != 0, int) @ np.asarray(ib != 0, int).T
+    assert np.all(err[on & short] * (1 << 52) <= terms[on & short] * mags[on & short])
     if far_off:        # what the limit is for: digits alone would miss the FMA bound
         assert np.any(err[~on] * (1 << 53) > 64 * K * mags[~on])
     return on
@@ -118,4 +122,6 @@ def test_digits_carry_what_the_estimate_passes():
         small = np.arange(64) % 4 == 0
         a = g(12, 64) * np.where(small, 2.0 ** -gap, 1.0)
         check_unlisted(a, np.vstack([g(5, 64) * small, g(4, 64)]), gap >= 20)
+    on = check_unlisted(np.vstack([np.eye(20, 64), rng.integers(-3, 4, (9, 64)).astype(float)]), g(9, 64))
+    assert 0.9 < on[:20].mean() < 1 and on[20:].all()
     check_unlisted(g(12, 64) * 2.0 ** -rng.integers(0, 60, (12, 64)), g(9, 64) * 2.0 ** -rng.integers(0, 60, (9, 64)))
