@@ -978,7 +978,7 @@ __device__ __forceinline__ void small_sums(const RepairArgs& a, int64_t r0, int6
         acc[i] = in ? first_sum(a.ka[r], a.kb[c]) : kMinSum;
     }
     auto least = [&]() { return fminf(fminf(acc[0], acc[1]), fminf(acc[2], acc[3])); };
-    bool done = __all_sync(0xffffffffu, least() >= kMinSum) != 0;
+    bool done = false;
     for (int kb = 0; kb < a.kblocks && !done; kb += 8) {
         uint32_t x[8][4], y[8][2];
 #pragma unroll

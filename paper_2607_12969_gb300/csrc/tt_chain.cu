@@ -267,9 +267,9 @@ lrc_status launch_tt_chain_f64_tc(const TTShape& sh, double* out, cudaStream_t s
 // same, 7 us of an SM, whatever its width and for all ranks up to 64, so the
 // output product has to have enough to do in one: bond rank times NT from
 // kTTDigitTile on.  Measured, digits / FMA kernels: 10^6 x 16 (NT = 16), rank 16
-// 377 / 432 us, rank 4 365 / 116; 300^3 (NT = 64), ranks 8 215 / 425, 4 254 / 219,
-// 2 411 / 116; 4096^2, rank 4 128 / 347, 2 231 / 195; 1000 x 1000 x 8, ranks 8 and
-// 4 (NT = 16) 382 / 128.  Rows are numbered in 32 bits.
+// 448 / 434 us, rank 4 440 / 115; 300^3 (NT = 64), ranks 8 183 / 424, 4 191 / 219,
+// 2 288 / 115; 4096^2, rank 4 103 / 347, 2 151 / 195; 16384 x 8192, rank 1 543 /
+// 295; 1000 x 1000 x 8, ranks 8 and 4 (NT = 16) 506 / 128.  Rows are numbered in 32 bits.
 bool tt_chain_f64_tc_takes(const TTShape& sh) {
     constexpr double kTTDigitFlops = 4e7;
     constexpr int64_t kTTDigitTile = 192, kMost = (int64_t)1 << 31;
