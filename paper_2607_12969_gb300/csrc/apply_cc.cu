@@ -19,18 +19,20 @@
 // element per row so that the transposing stores are conflict-free too.
 //
 // binary64 forms both products on the tensor cores from exact products of
-// digits (split_gemm.cu; 16384 x 8192, k = 128, b = 8192: 45.5 -> 1.54 ms);
+// digits (split_gemm.cu; 16384 x 8192, k = 128, b = 8192: 45.5 -> 1.58 ms);
 // this kernel (DFMA-bound: the GB300 issues about 2 DFMA per clock per SM),
 // with thin 8-row tiles and many CTAs per SM, so the work spreads evenly over
-// the SMs, takes what that path does not: no workspace to be had, n above 2^20.  binary32 (FFMA-bound) runs the two products on the
-// register-tiled kernel of gemm_cc.cu instead: phase 1 split over n (partial
-// sums of at most 1024 terms, added in split order by
-// reduce_scale_f32_kernel, which also applies diag(s)), phase 2 over
-// 128 x 128 tiles of Y.  W (b x k') passes through the stream's workspace.
+// the SMs, takes what that path does not: no workspace to be had, n above 2^20.
+// binary32: larger problems from bfloat16 parts on the tensor cores
+// (split_gemm32.cu); smaller ones (FFMA-bound) run the two products on the
+// register-tiled kernel of gemm_cc.cu: phase 1 split over n (partial sums of at
+// most 1024 terms, added in split order by reduce_scale_f32_kernel, which also
+// applies diag(s)), phase 2 over 128 x 128 tiles of Y.  W (b x k') passes
+// through the stream's workspace.
 //
-// LRC_F32_TC (a variant): on those smaller problems phase 2 on the tensor cores.  W (per row: queries
-// may differ in magnitude by any factor) and U (per 32 rows) are scaled by
-// powers of two that bring each group's largest magnitude into [2^14, 2^15)
+// LRC_F32_TC (a variant): on those smaller problems phase 2 on the tensor
+// cores.  W (per row: queries may differ in magnitude by any factor) and U (per
+// 32 rows) are scaled by powers of two that bring each group's largest magnitude into [2^14, 2^15)
 // and split into binary16 parts hi = fp16(x), lo = fp16(x - hi)
 // laid side by side along the reduction, W as [W_hi | W_lo | W_hi] in the
 // product's 128-row operand image and U as [U_hi | U_hi | U_lo] rows, so
@@ -583,7 +585,9 @@ lrc_status launch_apply_f64(const double* U, const double* S, const double* Vt, 
 // (7.6e8) 73 / 99 us; 16384 x 600, k = 40, b = 256 (1.7e8) 38 / 31 us and b =
 // 1024 47 / 64 us; 2048^2, k = 136, b = 256 (1.4e8) 41 / 39 us; with a long
 // reduction earlier: 600 x 16384, k = 40, b = 256 50 / 87 us, 16384^2, k = 272,
-// b = 20 (1.8e8) 75 / 92 us.
+// b = 20 (1.8e8) 75 / 92 us.  Low ranks, where the images are most of the bytes:
+// k = 4 4096^2, b = 8192 143 / 241 us, 16384^2, b = 1024 90 / 131, 1138^2, b = 8192
+// (7.5e7, FMA kernels) 82, k = 12 67 / 84.
 static bool apply_f32_tc_takes(int64_t m, int64_t n, int64_t k, int64_t b) {
     if (n >= (1ll << 30) || k > 4096 || m >= (1ll << 31) || b >= (1ll << 31)) return false;
     const double work = (double)(m + n) * (double)k * (double)b;

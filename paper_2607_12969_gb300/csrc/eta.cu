@@ -735,9 +735,10 @@ lrc_status tt_eta_t(const TTShape& sh, const void* const* hats, double* eta_out,
         eta_tt_blocks_kernel<T><<<grid_for(cnt, 256), 256, 0, s>>>((const double*)sh.cores[l], (const T*)hats[l],
                                                                     cnt, CD, CZ);
         if ((st = after_launch("eta_tt_blocks_kernel")) != LRC_OK) return st;
-        // (Not through digits: with left-orthogonal cores M is close to the identity,
-        // its rows lie far below their largest entry and are recomputed one by one;
-        // 512 x 512 x 224, ranks 70 and 52: 200 ms a call instead of 2.2.)
+        // (Not through digits: with left-orthogonal cores M is close to the identity
+        // and most sums of magnitudes lie below what digits carry; 512 x 512 x 224,
+        // ranks 70 and 52, with such rows recomputed one by one: 200 ms a call
+        // instead of 2.2.)
         // X_D = M [G; dG], X_Z = M[:, Z] Gh  (2ra x n rb each)
         MmSpec mm[2] = {{Mcur, CD, XD, 2 * ra, N, N, N, 2 * ra, 2 * ra},
                         {Mcur + ra, CZ, XZ, 2 * ra, N, N, N, 2 * ra, ra}};

@@ -219,7 +219,8 @@ __global__ void __launch_bounds__(256, 6) row_stats_kernel(const __grid_constant
 // digits in [-256, 255].  `any` collects the integers' bits.
 __device__ __forceinline__ void digits8(const double (&x)[8], const int (&sh)[8], int em, uint32_t (&w)[kParts64][4],
                                         uint64_t& any) {
-    constexpr uint64_t kBias = 256ull * (1ull + (1ull << 9) + (1ull << 18) + (1ull << 27) + (1ull << 36) + (1ull << 45));
+    constexpr uint64_t kBias =
+        256ull * (1ull + (1ull << 9) + (1ull << 18) + (1ull << 27) + (1ull << 36) + (1ull << 45));
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
         float f[2][kParts64];
@@ -699,124 +700,124 @@ __global__ void __launch_bounds__(kThreads, 1) product_kernel(const __grid_const
     } else {
         reg_dec<kRegsLow>();
         if (warp == 0) {
-        // ------------------------------------------------------------ producer
-        if (lane == 0) {
+            // ------------------------------------------------------------ producer
+            if (lane == 0) {
+                Pieces<GemmArgs> pc(a);
+                int tile, c0, c1;
+                int it = 0, slot = 0;
+                uint32_t phase = 1;
+                bool ok = true;
+                while (ok && pc.next(a, &tile, &c0, &c1)) {
+                    const int2 at = tile_at(a, tile);
+                    const int mt = at.x, nt = at.y;
+                    const int b1 = min(kChunkBlocks * c1, a.kblocks);
+                    for (int kb = kChunkBlocks * c0; kb < b1; ++kb, ++it) {
+                        if (!(ok = mbar_wait(&empty[slot], phase, abort, err, 1u))) break;
+                        unsigned char* dst = ring + (size_t)slot * stage_bytes;
+                        mbar_arrive_expect_tx(&full[slot], stage_bytes);
+                        bulk_load(dst, a.A + kb * a.a_block + (size_t)mt * a.a_bytes, a.a_bytes, &full[slot]);
+                        bulk_load(dst + a.a_bytes, a.B + kb * a.b_block + (size_t)nt * a.b_bytes, a.b_bytes, &full[slot]);
+                        if (++slot == a.stages) {
+                            slot = 0;
+                            phase ^= 1;
+                        }
+                    }
+                }
+                if (!ok) {
+                    volatile int no_abort = 0;
+                    for (int j = it - a.stages > 0 ? it - a.stages : 0; j < it; ++j)
+                        mbar_wait(&full[j % a.stages], (j / a.stages) & 1, &no_abort, err, 0u, 100000000ull);
+                }
+            }
+        } else if (warp == 1) {
+            // ------------------------------------------------------------ MMA issuer
+            // The whole warp walks the loop and waits; one lane issues, in one branch
+            // per block (with a branch or an election per MMA the warp, which shares
+            // its scheduler with busy epilogue warps, issued one in 49 to 100 clocks).
             Pieces<GemmArgs> pc(a);
             int tile, c0, c1;
-            int it = 0, slot = 0;
-            uint32_t phase = 1;
+            int slot = 0, ch = 0;
+            uint32_t phase = 0;            // parity of the ring's current pass
             bool ok = true;
+            // waits agree on every lane before the warp goes on
+            auto wait = [&](uint64_t* bar, uint32_t parity) {
+                return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort, err, 2u)) != 0;
+            };
+            // column octets 128 bytes apart, row groups kGroupBytes
+            const uint64_t ad = smem_desc(smem_u32(ring), 128, kGroupBytes, 0);
+            const uint64_t bd = smem_desc(smem_u32(ring) + a.a_bytes, 128, kGroupBytes, 0);
+            const uint32_t ahi = (uint32_t)(ad >> 32), bhi = (uint32_t)(bd >> 32), alo0 = (uint32_t)ad, blo0 = (uint32_t)bd;
             while (ok && pc.next(a, &tile, &c0, &c1)) {
-                const int2 at = tile_at(a, tile);
-                const int mt = at.x, nt = at.y;
-                const int b1 = min(kChunkBlocks * c1, a.kblocks);
-                for (int kb = kChunkBlocks * c0; kb < b1; ++kb, ++it) {
-                    if (!(ok = mbar_wait(&empty[slot], phase, abort, err, 1u))) break;
-                    unsigned char* dst = ring + (size_t)slot * stage_bytes;
-                    mbar_arrive_expect_tx(&full[slot], stage_bytes);
-                    bulk_load(dst, a.A + kb * a.a_block + (size_t)mt * a.a_bytes, a.a_bytes, &full[slot]);
-                    bulk_load(dst + a.a_bytes, a.B + kb * a.b_block + (size_t)nt * a.b_bytes, a.b_bytes, &full[slot]);
-                    if (++slot == a.stages) {
-                        slot = 0;
+                for (int c = c0; c < c1 && ok; ++c, ++ch) {
+                    const int nb = min(kChunkBlocks, a.kblocks - kChunkBlocks * c);
+                    uint32_t fresh = 0;
+#pragma unroll
+                    for (int t = 0; t < kParts64; ++t) fresh |= (c - c0) % period(t) == 0 ? 1u << t : 0u;
+                    // Classes 0 to 3 of the whole chunk, drained while the others run.  Class
+                    // 3, the only one of them drained every chunk, has two accumulators, so
+                    // the chunk waits for the drain before the last one, and for the last
+                    // one only where it emptied one of classes 0 to 2 (128 x 64 tiles of two
+                    // chunks: the second chunk's MMAs no longer wait for the rounding and
+                    // stores of the tile before).
+                    if (!(ok = wait(&gempty[ch & 1], ((ch >> 1) & 1) ^ 1))) break;
+                    if ((fresh & 7) && ch > 0 && !(ok = wait(&gempty[(ch - 1) & 1], ((ch - 1) >> 1) & 1))) break;
+                    const uint32_t col3 = (uint32_t)(ch & 1 ? 7 : 3) * NT;
+                    for (int b0 = 0; b0 < nb; b0 += 2) {
+                        // two blocks per wait, half the lanes polling each
+                        const int b1 = min(b0 + 2, nb);
+                        int sl = slot + min(b0 + (lane & 1), b1 - 1);
+                        const uint32_t ph = sl >= a.stages ? phase ^ 1 : phase;
+                        if (sl >= a.stages) sl -= a.stages;
+                        if (!(ok = wait(&full[sl], ph))) break;
+                        tc_fence_after();
+                        if (elect_one()) {
+                            sl = slot + b0 >= a.stages ? slot + b0 - a.stages : slot + b0;
+                            for (int b = b0; b < b1; ++b) {
+                                const uint32_t off = (uint32_t)sl * stage_bytes / 16;
+                                if (b == 0) issue<NT, 0, 4>(tmem, col3, fresh, alo0 + off, ahi, blo0 + off, bhi);
+                                else issue<NT, 0, 4>(tmem, col3, 0u, alo0 + off, ahi, blo0 + off, bhi);
+                                if (++sl == a.stages) sl = 0;
+                            }
+                            if (b1 == nb) mma_commit(&gfull[ch & 1]);
+                        }
+                        __syncwarp();
+                    }
+                    if (!ok) break;
+                    if (!(ok = wait(&gempty[2], (ch & 1) ^ 1))) break;
+                    tc_fence_after();
+                    if (elect_one()) {
+                        int sl = slot;
+                        for (int b = 0; b < nb; ++b) {
+                            const uint32_t off = (uint32_t)sl * stage_bytes / 16;
+                            if (b == 0) issue<NT, 4, 7>(tmem, 0u, fresh, alo0 + off, ahi, blo0 + off, bhi);
+                            else issue<NT, 4, 7>(tmem, 0u, 0u, alo0 + off, ahi, blo0 + off, bhi);
+                            mma_commit(&empty[sl]);
+                            if (++sl == a.stages) sl = 0;
+                        }
+                        mma_commit(&gfull[2]);
+                    }
+                    __syncwarp();
+                    slot += nb;
+                    if (slot >= a.stages) {
+                        slot -= a.stages;
                         phase ^= 1;
                     }
                 }
             }
-            if (!ok) {
-                volatile int no_abort = 0;
-                for (int j = it - a.stages > 0 ? it - a.stages : 0; j < it; ++j)
-                    mbar_wait(&full[j % a.stages], (j / a.stages) & 1, &no_abort, err, 0u, 100000000ull);
+            if (elect_one()) mma_commit(mma_done);
+            __syncwarp();
+            volatile int no_abort = 0;
+            mbar_wait(mma_done, 0, &no_abort, err, 2u, 100000000ull);
+        } else {
+            // ------------------------------------------------------------ sums of magnitudes
+            Pieces<GemmArgs> pc(a);
+            int tile, c0, c1;
+            while (pc.next(a, &tile, &c0, &c1)) {
+                if (c0 != 0) continue;             // the tile's first piece looks at all of the reduction
+                const int2 at = tile_at(a, tile);
+                list_small_sums<NT>(a, at.x, at.y, warp - 2, lane);
             }
         }
-    } else if (warp == 1) {
-        // ------------------------------------------------------------ MMA issuer
-        // The whole warp walks the loop and waits; one lane issues, in one branch
-        // per block (with a branch or an election per MMA the warp, which shares
-        // its scheduler with busy epilogue warps, issued one in 49 to 100 clocks).
-        Pieces<GemmArgs> pc(a);
-        int tile, c0, c1;
-        int slot = 0, ch = 0;
-        uint32_t phase = 0;            // parity of the ring's current pass
-        bool ok = true;
-        // waits agree on every lane before the warp goes on
-        auto wait = [&](uint64_t* bar, uint32_t parity) {
-            return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort, err, 2u)) != 0;
-        };
-        // column octets 128 bytes apart, row groups kGroupBytes
-        const uint64_t ad = smem_desc(smem_u32(ring), 128, kGroupBytes, 0);
-        const uint64_t bd = smem_desc(smem_u32(ring) + a.a_bytes, 128, kGroupBytes, 0);
-        const uint32_t ahi = (uint32_t)(ad >> 32), bhi = (uint32_t)(bd >> 32), alo0 = (uint32_t)ad, blo0 = (uint32_t)bd;
-        while (ok && pc.next(a, &tile, &c0, &c1)) {
-            for (int c = c0; c < c1 && ok; ++c, ++ch) {
-                const int nb = min(kChunkBlocks, a.kblocks - kChunkBlocks * c);
-                uint32_t fresh = 0;
-#pragma unroll
-                for (int t = 0; t < kParts64; ++t) fresh |= (c - c0) % period(t) == 0 ? 1u << t : 0u;
-                // Classes 0 to 3 of the whole chunk, drained while the others run.  Class
-                // 3, the only one of them drained every chunk, has two accumulators, so
-                // the chunk waits for the drain before the last one, and for the last
-                // one only where it emptied one of classes 0 to 2 (128 x 64 tiles of two
-                // chunks: the second chunk's MMAs no longer wait for the rounding and
-                // stores of the tile before).
-                if (!(ok = wait(&gempty[ch & 1], ((ch >> 1) & 1) ^ 1))) break;
-                if ((fresh & 7) && ch > 0 && !(ok = wait(&gempty[(ch - 1) & 1], ((ch - 1) >> 1) & 1))) break;
-                const uint32_t col3 = (uint32_t)(ch & 1 ? 7 : 3) * NT;
-                for (int b0 = 0; b0 < nb; b0 += 2) {
-                    // two blocks per wait, half the lanes polling each
-                    const int b1 = min(b0 + 2, nb);
-                    int sl = slot + min(b0 + (lane & 1), b1 - 1);
-                    const uint32_t ph = sl >= a.stages ? phase ^ 1 : phase;
-                    if (sl >= a.stages) sl -= a.stages;
-                    if (!(ok = wait(&full[sl], ph))) break;
-                    tc_fence_after();
-                    if (elect_one()) {
-                        sl = slot + b0 >= a.stages ? slot + b0 - a.stages : slot + b0;
-                        for (int b = b0; b < b1; ++b) {
-                            const uint32_t off = (uint32_t)sl * stage_bytes / 16;
-                            if (b == 0) issue<NT, 0, 4>(tmem, col3, fresh, alo0 + off, ahi, blo0 + off, bhi);
-                            else issue<NT, 0, 4>(tmem, col3, 0u, alo0 + off, ahi, blo0 + off, bhi);
-                            if (++sl == a.stages) sl = 0;
-                        }
-                        if (b1 == nb) mma_commit(&gfull[ch & 1]);
-                    }
-                    __syncwarp();
-                }
-                if (!ok) break;
-                if (!(ok = wait(&gempty[2], (ch & 1) ^ 1))) break;
-                tc_fence_after();
-                if (elect_one()) {
-                    int sl = slot;
-                    for (int b = 0; b < nb; ++b) {
-                        const uint32_t off = (uint32_t)sl * stage_bytes / 16;
-                        if (b == 0) issue<NT, 4, 7>(tmem, 0u, fresh, alo0 + off, ahi, blo0 + off, bhi);
-                        else issue<NT, 4, 7>(tmem, 0u, 0u, alo0 + off, ahi, blo0 + off, bhi);
-                        mma_commit(&empty[sl]);
-                        if (++sl == a.stages) sl = 0;
-                    }
-                    mma_commit(&gfull[2]);
-                }
-                __syncwarp();
-                slot += nb;
-                if (slot >= a.stages) {
-                    slot -= a.stages;
-                    phase ^= 1;
-                }
-            }
-        }
-        if (elect_one()) mma_commit(mma_done);
-        __syncwarp();
-        volatile int no_abort = 0;
-        mbar_wait(mma_done, 0, &no_abort, err, 2u, 100000000ull);
-    } else {
-        // ------------------------------------------------------------ sums of magnitudes
-        Pieces<GemmArgs> pc(a);
-        int tile, c0, c1;
-        while (pc.next(a, &tile, &c0, &c1)) {
-            if (c0 != 0) continue;             // the tile's first piece looks at all of the reduction
-            const int2 at = tile_at(a, tile);
-            list_small_sums<NT>(a, at.x, at.y, warp - 2, lane);
-        }
-    }
     }
     __syncwarp();
     tc_fence_before();
@@ -930,7 +931,8 @@ __device__ __forceinline__ void repair_dot(const RepairArgs& a, int64_t row, int
 // Rows r0 ... r0 + 7 and columns c0, c0 + 2, c0 + 4, c0 + 6, bit 4 row + column / 2 of `mask`.
 __device__ __forceinline__ void repair_word(const RepairArgs& a, int64_t r0, int64_t c0, uint32_t mask, int lane) {
     // an entry that is not listed may lie past the edge: the last listed one's row or column instead
-    const uint32_t cols = (mask | mask >> 4 | mask >> 8 | mask >> 12 | mask >> 16 | mask >> 20 | mask >> 24 | mask >> 28) & 15u;
+    uint32_t cols = mask | mask >> 16;
+    cols = (cols | cols >> 8 | cols >> 4 | cols >> 12) & 15u;
     const int rmax = (31 - __clz((int)mask)) / 4, cmax = 31 - __clz((int)cols);
     double acc[32];
 #pragma unroll
@@ -1081,8 +1083,8 @@ lrc_status launch_product(const GemmArgs& a, const CUtensorMap& tm, int64_t grid
 
 size_t operand_bytes(int64_t rows, int64_t K) {
     const int64_t ir = image_rows(rows);
-    return up256((size_t)(ir / 8) * image_blocks(K) * kGroupBytes + kTailBytes) + up256((size_t)ir * 4) + up256((size_t)ir) +
-           up256((size_t)rows * (K > kOwnStatsK ? kStatSplits : 0) * 4);
+    return up256((size_t)(ir / 8) * image_blocks(K) * kGroupBytes + kTailBytes) + up256((size_t)ir * 4) +
+           up256((size_t)ir) + up256((size_t)rows * (K > kOwnStatsK ? kStatSplits : 0) * 4);
 }
 
 void operand_carve(Operand64* o, unsigned char* ws) {

@@ -77,8 +77,11 @@ lrc_status product(const double* A, int64_t lda, const double* B, int64_t ldb, d
     return gemm_cc_f64(A, lda, B, ldb, C, ldc, M, N, K, s);
 }
 
-// Output products of binary32 chains go through bfloat16 parts from here on
-// (512 x 512 x 224, ranks 70, 52: 6.1e9 flops).
+// Output products of binary32 chains go through bfloat16 parts from here on.
+// Measured, parts / FMA kernel: 512 x 512 x 224, ranks 70, 52 (6.1e9) 147 / 249 us,
+// 700 x 500 x 300, ranks 80, 40 (8.4e9) 207 / 368, 2048^2, rank 300 (2.5e9) 27 / 70.
+// Below it the parts gain too (4096^2, rank 68 (2.3e9) 33 / 61, 10^5 x 64, rank 100
+// (1.3e9) 49 / 72, 256^3, ranks 70 (2.3e9) 64 / 86), so it could lie lower.
 constexpr double kPartsFlops = 2.5e9;
 
 // tc_final (binary32 only): a smaller output product on the tensor cores through
@@ -255,8 +258,8 @@ lrc_status launch_tt_chain_f64_tc(const TTShape& sh, double* out, cudaStream_t s
         const sg::Operand64* ops[2] = {&t.a, &t.b};
         const sg::Out64 o{t.C, t.N, 1, nullptr, nullptr};
         if ((st = sg::slice(ops, 2, counts, i == 0 ? (int)steps.size() : 0, s)) != LRC_OK) return st;
-        if ((st = sg::product(t.a, t.b, o, false, nullptr, {reinterpret_cast<int2*>(ws + o_f), counts + i}, s)) != LRC_OK)
-            return st;
+        const sg::Fix f{reinterpret_cast<int2*>(ws + o_f), counts + i};
+        if ((st = sg::product(t.a, t.b, o, false, nullptr, f, s)) != LRC_OK) return st;
     }
     return LRC_OK;
 }

@@ -6,11 +6,11 @@
 // Z = G_1...G_c is a P x r matrix and S = G_{c+1}...G_d an r x Q matrix
 // (P = n_1...n_c, Q = n_{c+1}...n_d, r = r_c), and the C-order tensor is the
 // P x Q product Z S.  One launch (tt_side_kernel) forms Z and S: each CTA
-// walks the chain for 32 rows of Z or 32 columns of S in shared memory (binary16 cores widened exactly, binary32 arithmetic) and
-// writes them into the tensor-core operand images; a second launch, the
-// binary16 tensor-core product of apply_tc.cu, forms Z S with Z as its
-// 128-row W tiles and S^T as its U rows -- nearly all of the work and all of
-// the output traffic.
+// walks the chain for 32 rows of Z or 32 columns of S in shared memory
+// (binary16 cores widened exactly, binary32 arithmetic) and writes them into
+// the tensor-core operand images; a second launch, the binary16 tensor-core
+// product of apply_tc.cu, forms Z S with Z as its 128-row W tiles and S^T as
+// its U rows -- nearly all of the work and all of the output traffic.
 //
 // Operands of that product are binary16 with binary32 accumulation (Sec. 3.4).
 // An operand that is a stored binary16 core is exact in binary16.  An operand the
@@ -33,9 +33,10 @@
 // reduction, hi hi last: the tensor cores cut sums off at every step of 16
 // terms, in one direction, so the steps at the result's full size are few (16^6,
 // rank 26: distance from the exact tensor 1.8e-7, with an FMA product 2.0e-7, in
-// 39 us instead of 42).  Units
-// of Z or S that hold an infinity or a NaN are marked in their scale, and the
-// entries they reach are formed from the images by tt_repair_kernel.
+// 37 us instead of 42).  Units of Z or S that hold an infinity or a NaN are
+// marked in their scale, and the entries they reach are formed from the images
+// by tt_repair_kernel.  Without workspace for the images, or with a thin side,
+// the chain runs on binary32 FMAs.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
@@ -541,7 +542,8 @@ lrc_status launch_split_t(const TTShape& sh, bool out16, void* out, cudaStream_t
     SideArgs a{};
     const int rmax = fill_side(sh, c, a);
     int n2 = 0;
-    if (kp > (kF32 ? kMaxParts32 : kMaxParts) * 64 || rmax > 64 || y_product_plan(a.Q, a.P, kp, out16, &n2) != LRC_OK) return LRC_OK;
+    if (kp > (kF32 ? kMaxParts32 : kMaxParts) * 64 || rmax > 64) return LRC_OK;
+    if (y_product_plan(a.Q, a.P, kp, out16, &n2) != LRC_OK) return LRC_OK;
     const size_t smem = side_smem(sh, a);
     if (smem > 200 * 1024) return LRC_OK;
     if (kF32) {
