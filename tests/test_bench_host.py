@@ -94,6 +94,14 @@ def test_roofline_takes_the_larger_bound():
     assert bench.bound_of(w64) == "alu"
 
 
+def test_parts_roofline_takes_the_tensor_rate_where_it_is_larger():
+    for fmt, parts in (("f64", 28), ("f32", 6), ("f16", 1)):
+        w = bench.work_apply(16384, 8192, 128, 8192, fmt)
+        want = max(w["bytes"] / bench.PEAKS["hbm"], w["flops"] * parts / bench.PEAKS["f16"])
+        assert bench.parts_roofline_time(w) == pytest.approx(want)
+        assert bench.parts_roofline_time(w) <= bench.roofline_time(w)
+
+
 def test_f32tc_bound_adds_the_two_engines():
     m, n, k, b = 16384, 8192, 136, 8192
     w = bench.work_apply(m, n, k, b, "f32tc")

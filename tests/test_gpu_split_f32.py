@@ -154,8 +154,8 @@ def test_tt(lrc, cuda, dims, ranks, fmt, bad):
 
 @pytest.mark.parametrize("m,n,k,b", [(4100, 600, 136, 1100), (2050, 8300, 40, 520), (12000, 9000, 33, 250)])
 def test_every_row_recomputed(lrc, cuda, m, n, k, b):
-    """Entries below the parts' range in every row of V^T and U: both products
-    in the tiles that the repair takes for many and few entries."""
+    """Entries of 1e-34 in every row of V^T and U, whose unscaled parts would fall
+    below bfloat16's range."""
     rng = np.random.default_rng(m)
     f32 = lambda a: a.astype(np.float32).astype(np.float64)
     small = lambda a: f32(np.where(np.arange(a.shape[1]) % 5 == 0, a * 1e-34, a))

@@ -3,8 +3,9 @@ chain, the Gram matrices of eta): values cut into seven 9-bit digits, 28 exact
 digit products, one rounding.
 
 Integer data whose sums stay below 2^53 must come out exactly, whatever the
-tiling; rows that the digits cannot carry (wide ranges, infinities, NaN,
-extreme magnitudes) go through binary64 FMAs and must come out as they do."""
+tiling; entries that the digits do not carry (sums of magnitudes far below the
+rows' largest entries, infinities, NaN, extreme magnitudes) go through binary64
+FMAs and must come out as they do."""
 import numpy as np
 import pytest
 import torch
@@ -170,8 +171,8 @@ def test_eta_through_digit_gram_matrices(lrc, cuda, fmt, m, n, k):
 
 @pytest.mark.parametrize("m,n,k,b", [(4100, 600, 33, 700), (2050, 700, 40, 330), (1300, 2500, 70, 65), (130, 9000, 17, 65)])
 def test_every_row_wide(lrc, cuda, m, n, k, b):
-    """Every row of V^T and U recomputed: both products in the tiles that the
-    repair takes for many, fewer and few entries, with partial tiles."""
+    """Entries over 60 binades in every row of V^T and U: digits over rows that
+    hold mostly small entries, and what of them is recomputed, with partial tiles."""
     rng = np.random.default_rng(m)
     wide = lambda *s: rng.standard_normal(s) * 2.0 ** -rng.integers(0, 60, s)
     U, Vt, X, s = wide(m, k), wide(k, n), W.gaussian((b, n), 5), rng.uniform(0.5, 2.0, k)
@@ -183,9 +184,9 @@ def test_every_row_wide(lrc, cuda, m, n, k, b):
 
 @pytest.mark.parametrize("m,n,k", [(3000, 1700, 61), (16384, 8192, 144)])
 def test_eta_of_wide_columns(lrc, cuda, m, n, k):
-    """The Gram matrices of eta with every column recomputed (upper tiles,
-    written both ways): against a power of two times the same factors, whose
-    digits and FMAs are the same, and against plain matrix products."""
+    """The Gram matrices of eta of columns over 40 binades (entries above the
+    diagonal recomputed where the digits do not carry them, written both ways),
+    against plain matrix products."""
     g = torch.Generator(device=cuda).manual_seed(m)
     rand = lambda *s: torch.randn(*s, generator=g, device=cuda, dtype=torch.float64)
     wide = lambda *s: rand(*s) * torch.exp2(-torch.randint(0, 40, s, generator=g, device=cuda).double())
@@ -341,3 +342,22 @@ def test_identity_and_sign_queries(lrc, cuda, m, n, k, b):
     want = (X @ Vt.T)[:, :min(m, k)]
     terms = np.count_nonzero(X, axis=1)[:, None]
     assert np.all(np.abs(got - want) <= (2 * terms + 2) * U64 * (np.abs(X) @ np.abs(Vt).T)[:, :min(m, k)])
+
+
+@pytest.mark.parametrize("m,n,k", [(3000, 1700, 61), (20000, 900, 40), (9000, 8192, 144)])
+def test_eta_of_columns_outside_the_digits_exponents(lrc, cuda, m, n, k):
+    """Every entry of one Gram matrix (upper tiles, written both ways) formed by
+    FMAs: the same eta as of the factors scaled into the digits' range."""
+    g = torch.Generator(device=cuda).manual_seed(k)
+    rand = lambda *s: torch.randn(*s, generator=g, device=cuda, dtype=torch.float64)
+    ld = lrc.lrc_packed_ld
+    U, Vt = rand(m, ld(k)), rand(k, ld(n))
+    s = rand(ld(k)).abs() + 0.1
+    hats = [a * (1 + 1e-6 * rand(*a.shape)) for a in (U, s, Vt)]
+    eta, norm = lrc.lrc_lowrank_eta(U, s, Vt, *hats, "f64", m, n, k)
+    down, up = 2.0 ** -485, 2.0 ** 400
+    e2, n2 = lrc.lrc_lowrank_eta(U * down, s * up, Vt, hats[0] * down, hats[1] * up, hats[2], "f64", m, n, k)
+    assert lrc.lrc_device_status() == 0
+    # m terms a Gram entry, each way of summing within (m + 2) u of its magnitudes
+    assert abs(e2 / (down * up) - eta) <= 4 * (m + n) * U64 * eta
+    assert abs(n2 / (down * up) - norm) <= 4 * (m + n) * U64 * norm
