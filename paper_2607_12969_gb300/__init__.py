@@ -220,11 +220,14 @@ _ARRAYS = {}
 
 
 def _array(ctype, xs):
-    """ctypes array of xs (the array types are made once per length)."""
+    """ctypes array of xs (the array types are kept, for at most 64 lengths)."""
     key = (ctype, len(xs))
     at = _ARRAYS.get(key)
     if at is None:
-        at = _ARRAYS[key] = ctype * max(len(xs), 1)
+        at = ctype * max(len(xs), 1)
+        if len(_ARRAYS) >= 64:
+            _ARRAYS.clear()
+        _ARRAYS[key] = at
     return at(*xs)
 
 

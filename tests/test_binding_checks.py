@@ -119,3 +119,10 @@ def test_tensor_on_another_gpu_is_refused():
     # a stream of cuda:1 with tensors on cuda:0
     with pytest.raises(ValueError, match="cuda:0, but the call runs on cuda:1"):
         lrc.lrc_fro_diff(h((100,), torch.float64), "f64", None, "f64", 100, stream=OnDevice1())
+
+
+def test_kept_array_types_are_bounded():
+    import ctypes
+    for n in range(200):
+        assert list(lrc._array(ctypes.c_int64, range(n)))[:n] == list(range(n))
+        assert len(lrc._ARRAYS) <= 64
